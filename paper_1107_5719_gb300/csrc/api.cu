@@ -72,6 +72,22 @@ struct rt_ctx {
     char* rec_mem = nullptr;
     long long rec_cap = 0;
     bool rec_valid = false;
+    // the recording assembled into an operator (rec_op), in the same block;
+    // its node lists (per quadrature) and the recording's working storage
+    bool rec_op = false;
+    OpMap op{};
+    OpLists ol{};
+    char* ol_mem = nullptr;
+    char* ow_mem = nullptr;
+    struct OpWork {
+        double* sp;             // padded source planes (also the length march's nodes)
+        int *lmax, *Lp, *rowbase, *cnt, *segb, *E, *rows, *poff;
+        long long *eb, *prow;
+        unsigned long long* steps;
+        double *c0s, *bcs;
+    } ow{};
+    std::vector<int> dord;      // directions by sign and decreasing |mu| (OpLists)
+    int dpos = 0;
 
     // device state, FP64
     double *chi = nullptr, *eps = nullptr, *B = nullptr, *J = nullptr, *S = nullptr;
@@ -190,12 +206,23 @@ void free_os_graphs(rt_ctx* c)
     }
 }
 
+// Working storage of the recording (freed with the grid or the directions).
+void free_op_work(rt_ctx* c)
+{
+    if (c->ow_mem) cudaFree(c->ow_mem);
+    c->ow_mem = nullptr;
+    c->ow = rt_ctx::OpWork{};
+    c->rec_valid = false;       // an operator's tables live there
+}
+
 void free_rec(rt_ctx* c)
 {
     if (c->rec_mem) cudaFree(c->rec_mem);
     c->rec_mem = nullptr;
     c->rec = FsRec{};
     c->rec32 = Rec32{};
+    c->op = OpMap{};
+    c->rec_op = false;
     c->spair = nullptr;
     c->rec_cap = 0;
     c->rec_valid = false;
@@ -217,6 +244,7 @@ void free_grid_buffers(rt_ctx* c)
     free_ng(c);
     c->partial_groups = 0;
     free_rec(c);
+    free_op_work(c);
 }
 
 void free_tables(rt_ctx* c)
@@ -225,6 +253,9 @@ void free_tables(rt_ctx* c)
     dfree(c->poff); dfree(c->poff32); dfree(c->bwdf);
     dfree(c->dn);
     dfree(c->d_mu); dfree(c->d_phi); dfree(c->d_w);
+    dfree(c->ol_mem);
+    c->ol = OpLists{};
+    free_op_work(c);
 }
 
 // Add the device time of the kernels bracketed since the last harvest;
@@ -273,24 +304,28 @@ int auto_groups(const rt_ctx* c)
     return G;
 }
 
-// Device memory for a recording of `need` bytes within the context's
-// budget (rec_mode): false when it does not fit or cannot be allocated.
+// The context's byte budget for a recording (rec_mode); 0 when the device
+// cannot be asked.
+long long rec_limit(const rt_ctx* c)
+{
+    if (c->rec_mode >= 0) return c->rec_mode;
+    size_t fr = 0, tot = 0;
+    if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
+        cudaGetLastError();
+        return 0;
+    }
+    // at most 60% of the device, leaving 2 GiB free
+    const long long limit = (long long)(0.6 * (double)tot);
+    const long long avail = (long long)fr + c->rec_cap - (2LL << 30);
+    return avail < limit ? avail : limit;
+}
+
+// Device memory for a recording of `need` bytes within that budget: false
+// when it does not fit or cannot be allocated.
 bool rec_reserve(rt_ctx* c, long long need)
 {
     if (need <= c->rec_cap) return true;
-    long long limit = c->rec_mode;
-    if (limit < 0) {
-        size_t fr = 0, tot = 0;
-        if (cudaMemGetInfo(&fr, &tot) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
-        // at most 60% of the device, leaving 2 GiB free
-        limit = (long long)(0.6 * (double)tot);
-        const long long avail = (long long)fr + c->rec_cap - (2LL << 30);
-        if (avail < limit) limit = avail;
-    }
-    if (need > limit) return false;
+    if (need > rec_limit(c)) return false;
     if (cudaStreamSynchronize(c->stream) != cudaSuccess) return false;
     free_rec(c);
     if (cudaMalloc((void**)&c->rec_mem, (size_t)need) != cudaSuccess) {
@@ -304,11 +339,8 @@ bool rec_reserve(rt_ctx* c, long long need)
 
 long long up256(long long b) { return (b + 255) / 256 * 256; }
 
-// The recorded march: whether this context records and replays it (FP64
-// with long characteristics and the linear source, or the FP32 sweep; a
-// byte budget that admits it), with its buffers carved from one block.
-// When it does not fit, the march runs as it is every time.
-// Bytes a recording of this context's march takes (0: its form does not record).
+// Bytes a ray-by-ray recording of this context's march takes (0: its form
+// does not record).
 long long rec_need(const rt_ctx* c)
 {
     if (c->fs_method != RT_FS_LONG || c->g.nz < 2 ||
@@ -331,6 +363,9 @@ long long rec_need(const rt_ctx* c)
            up256(pair_records(c->g) * (long long)sizeof(float4));
 }
 
+// The ray-by-ray recording: whether this context records and replays its
+// march (a form that records, within the byte budget), its buffers carved
+// from one block.  When it does not fit, the march runs every time.
 int ensure_rec(rt_ctx* c, bool& use)
 {
     use = false;
@@ -380,6 +415,297 @@ int ensure_rec(rt_ctx* c, bool& use)
         c->rec32.nwp = (int)nwp;
         c->spair = reinterpret_cast<float4*>(q + b_coef + b_lmax + 2 * b_slot);
     }
+    use = true;
+    return RT_OK;
+}
+
+// ---- assembled operator (op.cu) ------------------------------------------
+
+// Grids and quadratures it handles: offsets in 31 bits, per-plane tables of
+// 2 nz entries, a block's lengths in shared memory.
+bool op_fits(const rt_ctx* c)
+{
+    return 4 * c->g.N < (1LL << 31) && c->g.nz <= 1024 && c->g.ndir <= 24 * 1024;
+}
+
+// The most entries and chunk rows the planes can have (every ray alive up
+// to the boundary): eb, prow (exclusive prefix sums) and their totals.
+void op_bounds(const rt_ctx* c, bool para, std::vector<long long>* eb, std::vector<long long>* prow,
+               long long& entries, long long& rows)
+{
+    const long long nxy = (long long)c->g.nx * c->g.ny;
+    const long long Dp = c->dpos, Dm = c->g.ndir - Dp;
+    const long long up = std::min(nxy, 4 * Dp), um = std::min(nxy, 4 * Dm);
+    const long long u2p = (up + 1) & ~1LL, u2m = (um + 1) & ~1LL;
+    entries = rows = 0;
+    for (int k = 0; k < c->g.nz; ++k) {
+        const long long M = k, Mm = c->g.nz - 1 - k;
+        if (eb) (*eb)[k] = entries;
+        if (prow) (*prow)[k] = rows;
+        long long e = M * u2p + Mm * u2m;
+        if (para) e += (Mm > 0 ? u2p : 0) + (M > 0 ? u2m : 0);
+        entries += (e + kOpPad - 1) / kOpPad * kOpPad;
+        rows += Dp * M + Dm * Mm + (para ? c->g.ndir : 0);
+    }
+}
+
+long long op_tiles(const rt_ctx* c) { return ((long long)c->g.nx * c->g.ny + 31) / 32; }
+
+// Bytes of an operator of `entries` entries (its own terms included).
+long long op_bytes(const rt_ctx* c, long long entries)
+{
+    return up256(entries * op_tiles(c) * 32 * (long long)sizeof(double)) +
+           up256(entries * (long long)sizeof(int)) + 2 * up256(c->g.N * (long long)sizeof(double));
+}
+
+// Memory an operator may take with its chunk buffer: what the ray-by-ray
+// recording takes, or somewhat more where that is small (33^3 with 256
+// directions: 1.25 GB against 1.18).
+long long op_budget(const rt_ctx* c, long long need)
+{
+    const long long extra = std::min(std::max(need / 4, 2LL << 30), 8LL << 30);
+    return need + extra;
+}
+
+// The most memory a recording of this context asks for.
+long long rec_ask(const rt_ctx* c, long long need)
+{
+    if (!op_fits(c)) return need;
+    long long entries, rows;
+    op_bounds(c, c->src_order == RT_SRC_PARABOLIC, nullptr, nullptr, entries, rows);
+    const long long most = op_bytes(c, entries) +
+                           up256(rows * c->g.nx * c->g.ny * (long long)sizeof(double));
+    return std::max(need, std::min(most, op_budget(c, need)));
+}
+
+// Node lists of the context's directions, built at the first recording.
+int ensure_op_lists(rt_ctx* c)
+{
+    if (c->ol_mem) return RT_OK;
+    const Geometry& g = c->g;
+    const long long nxy = (long long)g.nx * g.ny, Q = 2LL * g.nz;
+    const int Dmax = std::max(c->dpos, g.ndir - c->dpos);
+    OpLists L{};
+    L.dpos = c->dpos;
+    L.icap = 4 * Dmax;
+    L.ucap = (int)std::min(nxy, (long long)L.icap);
+    const long long b_dord = up256(4LL * g.ndir), b_cnt = up256(4 * Q),
+                    b_node = up256(4 * Q * L.ucap), b_start = up256(4 * Q * (L.ucap + 1)),
+                    b_item = up256(4 * Q * L.icap), b_pos = up256(4LL * g.ndir * g.nz),
+                    b_con = up256((long long)sizeof(OpContrib) * Q * L.icap), b_l = 256;
+    const long long total = b_dord + b_cnt + b_node + b_start + b_item + b_pos + b_con + b_l;
+    char* m = nullptr;
+    CK(cudaMalloc((void**)&m, (size_t)total));
+    char* q = m;
+    int* dord = reinterpret_cast<int*>(q); q += b_dord;
+    L.dord = dord;
+    L.ucount = reinterpret_cast<int*>(q); q += b_cnt;
+    L.unode = reinterpret_cast<int*>(q); q += b_node;
+    L.ustart = reinterpret_cast<int*>(q); q += b_start;
+    L.uofi = reinterpret_cast<int*>(q); q += b_item;
+    L.posmax = reinterpret_cast<int*>(q); q += b_pos;
+    L.contrib = reinterpret_cast<OpContrib*>(q); q += b_con;
+    L.lpos = reinterpret_cast<int*>(q);
+    int* scratch = nullptr;
+    const long long ns = op_list_scratch(g);
+    cudaError_t e = ns ? cudaMalloc((void**)&scratch, sizeof(int) * (size_t)ns) : cudaSuccess;
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(dord, c->dord.data(), sizeof(int) * g.ndir, cudaMemcpyHostToDevice,
+                            c->stream);
+    if (e == cudaSuccess)
+        e = launch_op_lists(g, c->info, c->off, c->bw, c->dn, L, scratch, c->stream);
+    if (scratch) {
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        cudaFree(scratch);
+    }
+    if (e != cudaSuccess) {
+        cudaFree(m);
+        return fail(c, e == cudaErrorMemoryAllocation ? RT_ENOMEM : RT_ECUDA,
+                    "building the operator's node lists: %s", cudaGetErrorString(e));
+    }
+    c->ol = L;
+    c->ol_mem = m;
+    c->stats.launches += 1;
+    return RT_OK;
+}
+
+int ensure_op_work(rt_ctx* c)
+{
+    if (c->ow_mem) return RT_OK;
+    const Geometry& g = c->g;
+    const long long nwp = op_tiles(c), T = (long long)g.ndir * g.nz, Q = 2LL * g.nz * g.nz;
+    const long long b_sp = up256(32 * g.N), b_lmax = up256(4 * T * nwp), b_t = up256(4 * T),
+                    b_q = up256(4 * Q), b_z = up256(8LL * g.nz),
+                    b_slot = up256(8LL * kSlots * g.N);
+    char* m = nullptr;
+    CK(cudaMalloc((void**)&m, (size_t)(b_sp + b_lmax + 3 * b_t + 2 * b_q + 4 * b_z + 256 + 2 * b_slot)));
+    c->ow_mem = m;
+    auto& w = c->ow;
+    w.sp = reinterpret_cast<double*>(m); m += b_sp;
+    w.lmax = reinterpret_cast<int*>(m); m += b_lmax;
+    w.Lp = reinterpret_cast<int*>(m); m += b_t;
+    w.rowbase = reinterpret_cast<int*>(m); m += b_t;
+    w.poff = reinterpret_cast<int*>(m); m += b_t;
+    w.cnt = reinterpret_cast<int*>(m); m += b_q;
+    w.segb = reinterpret_cast<int*>(m); m += b_q;
+    w.E = reinterpret_cast<int*>(m); m += b_z;
+    w.rows = reinterpret_cast<int*>(m); m += b_z;
+    w.eb = reinterpret_cast<long long*>(m); m += b_z;
+    w.prow = reinterpret_cast<long long*>(m); m += b_z;
+    w.steps = reinterpret_cast<unsigned long long*>(m); m += 256;
+    w.c0s = reinterpret_cast<double*>(m); m += b_slot;
+    w.bcs = reinterpret_cast<double*>(m);
+    CK(launch_pad_offsets(g, c->info, c->off, 2LL * g.ny, w.poff, c->stream));
+    c->stats.launches += 1;
+    return RT_OK;
+}
+
+double cut_of(const rt_ctx* c);
+
+// Below this bound on an operator's bytes its exact size is not asked for:
+// the recording runs without a host wait.
+constexpr long long kOpNoWait = 256LL << 20;
+
+// Record the FP64 march of the current source (linear or parabolic) and
+// assemble its operator, or keep it ray by ray where the operator would take
+// more memory (op_budget).  use: whether a recording is held afterwards.
+int ensure_rec64(rt_ctx* c, int G, bool& use)
+{
+    use = false;
+    const long long need = rec_need(c);
+    if (c->rec_mode == 0 || need == 0) return RT_OK;
+    if (c->rec_valid) {
+        use = true;
+        return RT_OK;
+    }
+    const long long limit = std::max(rec_limit(c), c->rec_cap);
+    if (need > limit) return RT_OK;
+    int rc;
+    if ((rc = ensure_op_work(c))) return rc;
+    const Geometry& g = c->g;
+    const bool para = c->src_order == RT_SRC_PARABOLIC;
+    const long long nxy = (long long)g.nx * g.ny, nwp = op_tiles(c);
+    auto& w = c->ow;
+    cudaStream_t st = c->stream;
+    CK(launch_op_lengths(g, c->chi, c->S, c->scal + 0, c->info, w.poff, c->bw32,
+                         cut_of(c) * kRecCutMargin, para ? kParaCutBits : 0, G,
+                         reinterpret_cast<float2*>(w.sp), w.lmax, (int)nwp, w.Lp, w.steps, st));
+    c->stats.launches += 3;
+    bool op = op_fits(c);
+    std::vector<long long> eb(g.nz), prow(g.nz);
+    std::vector<int> order(g.nz);
+    for (int k = 0; k < g.nz; ++k) order[k] = k;
+    std::vector<int> first{0, g.nz};    // ranks of the chunks' first planes
+    long long entries = 0, rows = 0, chunk = 0;
+    if (op) {
+        if ((rc = ensure_op_lists(c))) return rc;
+        CK(launch_op_counts(g, c->ol, para, w.Lp, w.rowbase, w.cnt, w.segb, w.E, w.rows, st));
+        c->stats.launches += 1;
+        op_bounds(c, para, &eb, &prow, entries, rows);
+        chunk = up256(rows * nxy * (long long)sizeof(double));
+        const long long room = std::max(std::min(limit, op_budget(c, need)), c->rec_cap);
+        if (op_bytes(c, entries) + chunk > std::min(room, kOpNoWait)) {
+            // the size it really has, and chunks of planes
+            std::vector<int> E(g.nz), R(g.nz);
+            CK(cudaMemcpyAsync(E.data(), w.E, sizeof(int) * g.nz, cudaMemcpyDeviceToHost, st));
+            CK(cudaMemcpyAsync(R.data(), w.rows, sizeof(int) * g.nz, cudaMemcpyDeviceToHost, st));
+            if (g.zorder)
+                CK(cudaMemcpyAsync(order.data(), g.zorder, sizeof(int) * g.nz,
+                                   cudaMemcpyDeviceToHost, st));
+            CK(cudaStreamSynchronize(st));
+            c->stats.host_syncs += 1;
+            entries = rows = 0;
+            long long most = 0;
+            for (int k = 0; k < g.nz; ++k) {
+                eb[k] = entries;
+                entries += E[k];
+                rows += R[k];
+                most = std::max(most, (long long)R[k]);
+            }
+            const long long row = nxy * (long long)sizeof(double), own = op_bytes(c, entries);
+            // a chunk large enough to fill the GPU a few times over: an
+            // eighth of the ray-by-ray recording, the whole if it fits
+            long long cb = std::min(rows, std::max(most, std::max(need / 8, 2LL << 30) / row)) * row;
+            if (own + up256(cb) > room) cb = most * row;
+            if (own + up256(cb) > room) {
+                op = false;
+            } else {
+                first.assign(1, 0);
+                long long at = 0;
+                for (int r = 0; r < g.nz; ++r) {
+                    if ((at + R[order[r]]) * row > cb) {
+                        first.push_back(r);
+                        at = 0;
+                    }
+                    prow[order[r]] = at;
+                    at += R[order[r]];
+                }
+                first.push_back(g.nz);
+                chunk = up256(cb);
+            }
+        }
+    }
+    if (op) {
+        const long long own = op_bytes(c, entries);
+        long long want = own + chunk;
+        if (want > c->rec_cap) {
+            // a little to spare, so that the next opacity fits as well
+            const long long more = want + own / 64;
+            if (!rec_reserve(c, more <= limit ? more : want)) op = false;
+        }
+    }
+    if (!op) {
+        if (!rec_reserve(c, need)) return RT_OK;
+        if ((rc = ensure_rec(c, use))) return rc;
+        if (!use) return RT_OK;
+        CK(cudaMemcpyAsync(c->rec.lmax, w.lmax, sizeof(int) * (size_t)g.ndir * g.nz * nwp,
+                           cudaMemcpyDeviceToDevice, st));
+    } else {
+        const long long b_A = up256(entries * nwp * 32 * (long long)sizeof(double)),
+                        b_off = up256(entries * (long long)sizeof(int)), b_n = up256(8 * g.N);
+        char* q = c->rec_mem;
+        c->op.A = reinterpret_cast<double*>(q); q += b_A;
+        c->op.off = reinterpret_cast<int*>(q); q += b_off;
+        c->op.c0 = reinterpret_cast<double*>(q); q += b_n;
+        c->op.bc = reinterpret_cast<double*>(q); q += b_n;
+        c->op.E = w.E;
+        c->op.eb = w.eb;
+        c->op.steps = w.steps;
+        c->op.nwp = (int)nwp;
+        CK(cudaMemcpyAsync(w.eb, eb.data(), sizeof(long long) * g.nz, cudaMemcpyHostToDevice, st));
+        CK(cudaMemcpyAsync(w.prow, prow.data(), sizeof(long long) * g.nz, cudaMemcpyHostToDevice, st));
+        CK(launch_op_offsets(g, c->ol, w.cnt, w.segb, c->op, st));
+        c->stats.launches += 1;
+    }
+    RecOut ro{};
+    ro.base = op ? reinterpret_cast<double*>(c->rec_mem + op_bytes(c, entries)) : c->rec.coef;
+    ro.rowbase = op ? w.rowbase : nullptr;
+    ro.prow = op ? w.prow : nullptr;
+    ro.para = op && para ? 1 : 0;
+    ro.cdn = op ? nullptr : c->rec.cdn;
+    double* c0s = op ? w.c0s : c->rec.c0;
+    double* bcs = op ? w.bcs : c->rec.bc;
+    for (size_t i = 0; i + 1 < first.size(); ++i) {
+        const int r0 = first[i], np = first[i + 1] - r0;
+        if (para)
+            CK(launch_rec64p(g, r0, np, c->chi, c->B, c->gdiff, c->info, c->off, c->bw, c->bwh, c->dn,
+                             ro, w.lmax, (int)nwp, G, c0s, bcs, st));
+        else
+            CK(launch_rec64(g, r0, np, c->chi, c->B, c->gdiff, c->info, c->off, c->bw, c->bwh, ro,
+                            w.lmax, (int)nwp, G, c0s, bcs, st));
+        c->stats.launches += 1;
+        if (op) {
+            CK(launch_op_assemble(g, r0, np, c->ol, ro, w.lmax, w.cnt, w.segb, c->op, st));
+            c->stats.launches += 1;
+        }
+    }
+    if (op) {
+        CK(launch_op_own(g.N, w.c0s, w.bcs, const_cast<double*>(c->op.c0),
+                         const_cast<double*>(c->op.bc), st));
+        c->stats.launches += 1;
+    }
+    c->rec_op = op;
+    c->rec_valid = true;
     use = true;
     return RT_OK;
 }
@@ -548,19 +874,31 @@ int fs_prepare(rt_ctx* c)
     return RT_OK;
 }
 
-double cut_of(const rt_ctx* c) { return c->cut >= 0 ? c->cut : default_cut(c->precision); }
-
-int fs_finish(rt_ctx* c, double* Jout)
+double cut_of(const rt_ctx* c)
 {
-    if (c->precision == RT_FP64)
+    return c->cut >= 0 ? c->cut : default_cut(c->precision);
+}
+
+// Lambda* is read off the operator (its own and nearest-node entries are the
+// exact elements; 0.05 against 25 ms for the kernel on the 65^3 slab) unless
+// the recording was cut so early that the cut shows in them.
+constexpr double kOpLstarCut = 1e-16;
+
+// direct: Jout holds J already (the assembled operator)
+int fs_finish(rt_ctx* c, double* Jout, bool direct)
+{
+    if (direct) {
+    } else if (c->precision == RT_FP64)
         CK(launch_sum_groups(c->g.N, c->partial, Jout, c->stream));
     else if (c->precision == RT_FP32_SWEEP && c->fin == 2)
         CK(launch_sum_groups_ref(c->g.N, c->partial, c->dS, c->wsum, c->J_ref, Jout, c->stream));
     else
         CK(launch_sum_groups_src(c->g.N, c->partial, c->S, c->wsum, Jout, c->stream));
-    c->stats.launches += 1;
+    c->stats.launches += direct ? 0 : 1;
     if (!c->lstar_valid) {
-        if (c->src_order == RT_SRC_PARABOLIC) {
+        if (direct && cut_of(c) <= kOpLstarCut) {
+            CK(launch_op_lstar(c->g, c->ol, c->op, c->ow.cnt, c->ow.segb, c->lstar, c->stream));
+        } else if (c->src_order == RT_SRC_PARABOLIC) {
             CK(launch_lstar64p(c->g, c->chi, c->info, c->off, c->bw, c->dn, c->lstar, c->stream));
         } else if (c->precision == RT_FP64) {
             CK(launch_lstar64(c->g, c->chi, c->info, c->off, c->bw, c->lstar, c->stream));
@@ -676,6 +1014,33 @@ int df_formal(rt_ctx* c, int G, unsigned long long* steps, cudaStream_t st)
     return RT_OK;
 }
 
+// The FP64 formal solution of a context: recorded in the first one after
+// the opacities, directions or boundary change (J then comes from the
+// recording like every later one, so that it does not depend on which
+// formal solution recorded), or marched when the recording does not fit.
+// direct: J is in Jout, else in the slots of c->partial.
+int fs64_formal(rt_ctx* c, int G, double* Jout, unsigned long long* steps, bool& direct)
+{
+    bool use = false;
+    int rc = ensure_rec64(c, G, use);
+    if (rc) return rc;
+    direct = use && c->rec_op;
+    cudaStream_t st = c->stream;
+    if (direct) {
+        CK(launch_op_apply64(c->g, c->S, c->ow.sp, c->op, Jout, steps, st));
+        c->stats.launches += 1;
+    } else if (use) {
+        CK(launch_fs64rep(c->g, c->S, c->info, c->off, c->bw, c->rec, G, c->partial, steps, st));
+    } else if (c->src_order == RT_SRC_PARABOLIC) {
+        CK(launch_fs64p(c->g, c->chi, c->S, c->B, c->gdiff, c->info, c->off, c->bw, c->dn,
+                        c->scal + 0, cut_of(c), G, c->partial, steps, st));
+    } else {
+        CK(launch_fs64(c->g, c->chi, c->S, c->B, c->gdiff, c->info, c->off, c->bw, c->bwh,
+                       c->scal + 0, cut_of(c), G, c->partial, steps, st));
+    }
+    return RT_OK;
+}
+
 int run_fs(rt_ctx* c, double* Jout, bool count_steps)
 {
     if (c->fs_method == RT_FS_SHORT) return run_fs_short(c, Jout, count_steps);
@@ -685,44 +1050,9 @@ int run_fs(rt_ctx* c, double* Jout, bool count_steps)
     if (count_steps) CK(cudaMemsetAsync(c->d_steps, 0, sizeof(unsigned long long), c->stream));
     const double cut = cut_of(c);
     if (c->profiling) CK(cudaEventRecord(c->ev[0], c->stream));
-    if (c->precision == RT_FP64 && c->src_order == RT_SRC_PARABOLIC) {
-        // recorded like the linear source (with the downstream point's
-        // coefficients), else marched
-        bool use = false;
-        if ((rc = ensure_rec(c, use))) return rc;
-        unsigned long long* sp = count_steps ? c->d_steps : nullptr;
-        if (use && !c->rec_valid) {
-            CK(launch_fs64p(c->g, c->chi, c->S, c->B, c->gdiff, c->info, c->off, c->bw, c->dn,
-                            c->scal + 0, cut, G, c->partial, sp, c->stream, &c->rec));
-            c->rec_valid = true;
-            c->stats.launches += 1;
-        }
-        if (use)
-            CK(launch_fs64rep(c->g, c->S, c->info, c->off, c->bw, c->rec, G, c->partial, sp,
-                              c->stream));
-        else
-            CK(launch_fs64p(c->g, c->chi, c->S, c->B, c->gdiff, c->info, c->off, c->bw, c->dn,
-                            c->scal + 0, cut, G, c->partial, sp, c->stream));
-    } else if (c->precision == RT_FP64) {
-        bool use = false;
-        if ((rc = ensure_rec(c, use))) return rc;
-        if (use && !c->rec_valid) {
-            // record; J then comes from the replay like every later one, so
-            // that it does not depend on which formal solution recorded
-            CK(launch_fs64(c->g, c->chi, c->S, c->B, c->gdiff, c->info, c->off, c->bw, c->bwh,
-                           c->scal + 0, cut, G, c->partial, count_steps ? c->d_steps : nullptr,
-                           c->stream, &c->rec));
-            c->rec_valid = true;
-            c->stats.launches += 1;
-        }
-        if (use) {
-            CK(launch_fs64rep(c->g, c->S, c->info, c->off, c->bw, c->rec, G, c->partial,
-                              count_steps ? c->d_steps : nullptr, c->stream));
-        } else {
-            CK(launch_fs64(c->g, c->chi, c->S, c->B, c->gdiff, c->info, c->off, c->bw, c->bwh,
-                           c->scal + 0, cut, G, c->partial, count_steps ? c->d_steps : nullptr,
-                           c->stream));
-        }
+    bool direct = false;
+    if (c->precision == RT_FP64) {
+        if ((rc = fs64_formal(c, G, Jout, count_steps ? c->d_steps : nullptr, direct))) return rc;
     } else if (c->precision == RT_DF64) {
         if ((rc = df_formal(c, G, count_steps ? c->d_steps : nullptr, c->stream))) return rc;
     } else if (c->fin == 1) {
@@ -756,7 +1086,7 @@ int run_fs(rt_ctx* c, double* Jout, bool count_steps)
     }
     c->stats.fs_launches += 1;
     c->stats.launches += 1;
-    if ((rc = fs_finish(c, Jout))) return rc;
+    if ((rc = fs_finish(c, Jout, direct))) return rc;
     if (c->precision == RT_FP32_SWEEP && c->fin == 1 && (rc = fin_record(c, Jout, c->stream)))
         return rc;
     if (count_steps) {
@@ -1366,7 +1696,11 @@ int batch_admit(rt_batch* b, int max_iter)
     for (int p : b->order) {
         rt_ctx* c = b->ctx[p];
         if (b->admitted[p] || b->converged[p] || b->iters[p] >= max_iter) continue;
-        const long long need = rec_need(c);
+        // room for the assembled operator of an FP64 problem where the
+        // budget allows it at all, else for the ray-by-ray recording
+        long long need = rec_need(c);
+        if (need > 0 && c->precision == RT_FP64 && rec_ask(c, need) <= limit)
+            need = rec_ask(c, need);
         // a pooled block that holds the recording
         int pick = -1;
         for (size_t i = 0; i < b->rec_pool.size(); ++i)
@@ -1419,8 +1753,14 @@ void batch_release(rt_batch* b, int p)
         c->rec_cap = 0;
         c->rec = FsRec{};
         c->rec32 = Rec32{};
+        c->op = OpMap{};
+        c->rec_op = false;
         c->spair = nullptr;
         c->rec_valid = false;
+    }
+    if (c->ow_mem) {
+        cudaStreamSynchronize(b->stream);
+        free_op_work(c);
     }
 }
 
@@ -1554,6 +1894,7 @@ cudaError_t build_batch_os_graph(rt_batch* b, const std::vector<int>& act, doubl
 int batch_fs(rt_batch* b, const std::vector<int>& act)
 {
     int rc;
+    std::vector<char> direct(b->ctx.size(), 0);     // J is in c->Jfs already
     for (int p : act) {
         rt_ctx* c = b->ctx[p];
         if ((rc = bpass(b, p, prepare_source(c, nullptr, true)))) return rc;
@@ -1652,24 +1993,12 @@ int batch_fs(rt_batch* b, const std::vector<int>& act)
     } else {
         for (int p : act) {
             rt_ctx* c = b->ctx[p];
-            bool use = false;
-            if (b->precision == RT_FP64 && (rc = bpass(b, p, ensure_rec(c, use)))) return rc;
             if (b->precision == RT_DF64) {
                 if ((rc = bpass(b, p, df_formal(c, G, b->d_steps, b->stream)))) return rc;
-            } else if (use) {
-                if (!c->rec_valid) {
-                    BCK(launch_fs64(c->g, c->chi, c->S, c->B, c->gdiff, c->info, c->off, c->bw,
-                                    c->bwh, c->scal + 0, cut_of(c), G, c->partial, b->d_steps,
-                                    b->stream, &c->rec));
-                    c->rec_valid = true;
-                    b->stats.launches += 1;
-                }
-                BCK(launch_fs64rep(c->g, c->S, c->info, c->off, c->bw, c->rec, G, c->partial,
-                                   b->d_steps, b->stream));
             } else {
-                BCK(launch_fs64(c->g, c->chi, c->S, c->B, c->gdiff, c->info, c->off, c->bw,
-                                c->bwh, c->scal + 0, cut_of(c), G, c->partial, b->d_steps,
-                                b->stream));
+                bool d = false;
+                if ((rc = bpass(b, p, fs64_formal(c, G, c->Jfs, b->d_steps, d)))) return rc;
+                direct[p] = d;
             }
             b->stats.fs_launches += 1;
             b->stats.launches += 1;
@@ -1678,7 +2007,7 @@ int batch_fs(rt_batch* b, const std::vector<int>& act)
     if (b->profiling) BCK(cudaEventRecord(b->ev[1], b->stream));
     for (int p : act) {
         rt_ctx* c = b->ctx[p];
-        if ((rc = bpass(b, p, fs_finish(c, c->Jfs)))) return rc;
+        if ((rc = bpass(b, p, fs_finish(c, c->Jfs, direct[p])))) return rc;
         if (c->precision == RT_FP32_SWEEP && c->fin == 1 &&
             (rc = bpass(b, p, fin_record(c, c->Jfs, b->stream))))
             return rc;
@@ -1994,6 +2323,14 @@ int rt_set_quadrature(rt_ctx* c, int ndir, const double* mu, const double* phi, 
         c->stats.launches += 1;
     }
     c->wsum = sw;
+    c->dord.resize(ndir);
+    for (int d = 0; d < ndir; ++d) c->dord[d] = d;
+    std::stable_sort(c->dord.begin(), c->dord.end(), [mu](int a, int b) {
+        if ((mu[a] > 0) != (mu[b] > 0)) return mu[a] > 0;
+        return std::fabs(mu[a]) > std::fabs(mu[b]);
+    });
+    c->dpos = 0;
+    for (int d = 0; d < ndir; ++d) c->dpos += mu[d] > 0;
     c->have_quad = true;
     if ((rc = form_buffers(c, c->precision))) {
         c->have_quad = false;

@@ -120,14 +120,15 @@ cudaError_t launch_dir_tables(const Geometry& g, double dx, double dy, double dz
 cudaError_t launch_plane_order(const Geometry& g, double dz, const double* chi, double* scratch,
                                int* order, cudaStream_t st);
 
-// The FP64 march recorded as a linear map of the source S (the opacities,
-// directions and boundary values fixed): J = sum_slots [c0 S_v + bc +
-// sum_{d in slot} w_d sum_{m=1..L} c_m S(p_m)].
+// The FP64 march recorded as a linear map of the source S, ray by ray (the
+// opacities, directions and boundary values fixed): J = sum_slots [c0 S_v +
+// bc + sum_{d in slot} w_d sum_{m=1..L} c_m S(p_m)].  Kept where the
+// assembled operator (OpMap, below) takes more memory than this.
 //   coef: c_m of voxel t of plane k0 and direction d at
 //     rec_base(g, d, k0, sgn_d) + (m-1) nx ny + t, m = 1..M (M the steps to
-//     the boundary plane), zero past the ray's own length;
+//     the boundary plane);
 //   lmax[(d nz + k0) nwp + t/32]: the longest ray of the warp, the length
-//     the replay runs (nwp = warps per plane);
+//     recorded and replayed for all its lanes (nwp = warps per plane);
 //   c0, bc [kSlots][N]: the voxel's own coefficient and the boundary term.
 struct FsRec {
     double* coef;
@@ -141,9 +142,9 @@ struct FsRec {
     double* cdn;
     const DownGeo* dn;
 };
-// The recording march cuts the characteristics at cut * kRecCutMargin, so
-// that the recorded lengths still meet the cutoff for sources whose
-// intensities are up to 1/kRecCutMargin times smaller.
+// The recorded lengths cut the characteristics at cut * kRecCutMargin, so
+// that they still meet the cutoff for sources whose intensities are up to
+// 1/kRecCutMargin times smaller.
 constexpr double kRecCutMargin = 1e-2;
 __host__ __device__ __forceinline__ long long rec_base(const Geometry& g, int d, int k0, int sgn)
 {
@@ -152,19 +153,15 @@ __host__ __device__ __forceinline__ long long rec_base(const Geometry& g, int d,
     const long long before = sgn > 0 ? k * (k - 1) / 2 : k * (g.nz - 1) - k * (k - 1) / 2;
     return ((long long)d * ((long long)g.nz * (g.nz - 1) / 2) + before) * nxy;
 }
-// Device bytes of an FsRec for grid g (coefficients, lengths, c0 and bc).
-long long rec_bytes(const Geometry& g);
 
 // FP64 formal solution: partial[kSlots][N]; `groups` (1..kSlots) is the
 // number of z-blocks walking the slots (a tuning knob, no effect on J).
 // G[ny][nx]: dB/dtau at the bottom nodes (LTE-diffusion inner boundary),
-// read only when bottom_bc == 2 (may be null otherwise).  rec != null:
-// also record the march into *rec (FsRec), cut at cut * kRecCutMargin.
+// read only when bottom_bc == 2 (may be null otherwise).
 cudaError_t launch_fs64(const Geometry& g, const double* chi, const double* S, const double* B,
                         const double* G, const DirInfo* info, const StepGeo* off,
                         const Bw4d* bw, const Bw4d* bwh, const double* smax, double cut,
-                        int groups, double* partial, unsigned long long* steps, cudaStream_t st,
-                        const FsRec* rec = nullptr);
+                        int groups, double* partial, unsigned long long* steps, cudaStream_t st);
 // The recorded march for source S: partial[kSlots][N] as launch_fs64.
 cudaError_t launch_fs64rep(const Geometry& g, const double* S, const DirInfo* info,
                            const StepGeo* off, const Bw4d* bw, const FsRec& rec, int groups,
@@ -177,16 +174,113 @@ cudaError_t launch_diffusion_grad(const Geometry& g, double dz, const double* ch
 // ---- parabolic source (para.cu) --------------------------------------------
 cudaError_t launch_down_tables(const Geometry& g, double dx, double dy, double dz,
                                const double* mu, const double* phi, DownGeo* dn, cudaStream_t st);
-// As launch_fs64 with the parabolic source (rec != null: also record it,
-// with rec->cdn, cut at cut * kRecCutMargin).
+// Parabolic weights exceed the linear ones in magnitude by a small factor:
+// more bits of margin in the transmission cutoff.
+constexpr int kParaCutBits = 4;
+// As launch_fs64 with the parabolic source.
 cudaError_t launch_fs64p(const Geometry& g, const double* chi, const double* S, const double* B,
                          const double* G, const DirInfo* info, const StepGeo* off,
                          const Bw4d* bw, const DownGeo* dn, const double* smax, double cut,
-                         int groups, double* partial, unsigned long long* steps, cudaStream_t st,
-                         const FsRec* rec = nullptr);
+                         int groups, double* partial, unsigned long long* steps, cudaStream_t st);
 cudaError_t launch_lstar64p(const Geometry& g, const double* chi, const DirInfo* info,
                             const StepGeo* off, const Bw4d* bw, const DownGeo* dn, double* lstar,
                             cudaStream_t st);
+
+// ---- assembled operator (op.cu) --------------------------------------------
+// One contribution of a direction to a node: w_d times the bilinear weight;
+// ul = 2 u + 1 on the last contribution of node u of its list, else 2 u.
+struct OpContrib {
+    double wb;
+    int d, ul;
+};
+// Per (sign, slot) q = sign * nz + m, sign 0 for mu > 0 and 1 for mu < 0, slot
+// m >= 1 the distance in planes, slot 0 the downstream point of the
+// parabolic source: the distinct nodes and their contributions.
+struct OpLists {
+    int dpos;           // directions with mu > 0
+    const int* dord;    // [ndir] directions, mu > 0 first, each sign by decreasing |mu|
+    int ucap, icap;     // strides: nodes and items (4 per direction) per list
+    int* ucount;        // [2 nz] distinct nodes
+    int* unode;         // [2 nz][ucap] node y nx + x relative to the voxel's, x < nx, y < ny
+    int* ustart;        // [2 nz][ucap + 1] first contribution of each node
+    int* uofi;          // [2 nz][icap] list position of item 4 rank + corner
+    int* posmax;        // [ndir][nz] length of the prefix that holds the direction's nodes
+    OpContrib* contrib; // [2 nz][icap]
+    int* lpos;          // [2][2][9] positions of the 3x3 nearest nodes of slots 0, 1 (-1: none)
+};
+// The operator: entries eb[k0] .. eb[k0] + E[k0] - 1 of plane k0, coefficient
+// of entry e for voxel t of the plane at
+//   A[eb[k0] nwp 32 + ((t/32) E[k0]/2 + e/2) 64 + (t%32) 2 + e%2],
+// its node at off[eb[k0] + e] from the voxel in planes padded to 2ny x 2nx.
+struct OpMap {
+    const double* A;
+    const int* off;
+    const int* E;           // [nz], multiples of kOpPad
+    const long long* eb;    // [nz]
+    const double* c0;       // [N] coefficient of the voxel's own S
+    const double* bc;       // [N] boundary term
+    const unsigned long long* steps;    // voxel-steps it stands for
+    int nwp;                // 32-voxel tiles per plane
+};
+constexpr int kOpPad = 32;
+// Where a recording march writes its coefficients: with rowbase, row m of
+// direction d and plane k0 (its slot-0 row first when para) in the buffer
+// of one chunk of planes; without, the layout of FsRec.
+struct RecOut {
+    double* base;
+    const int* rowbase;     // [nz][ndir]
+    const long long* prow;  // [nz] first row of the plane in its chunk
+    int para;
+    double* cdn;            // FsRec's downstream coefficients (rowbase == null)
+};
+// The coefficient of p_1 of voxel 0 of plane k0, direction d.
+template <typename T>
+__device__ __forceinline__ T* rec_rows(const Geometry& g, const RecOut& r, T* base, int d, int k0,
+                                       int s)
+{
+    const long long nxy = (long long)g.nx * g.ny;
+    if (!r.rowbase) return base + rec_base(g, d, k0, s);
+    return base + (r.prow[k0] + r.rowbase[(long long)k0 * g.ndir + d] + r.para) * nxy;
+}
+// Scratch ints of launch_op_lists (0: it works in shared memory).
+long long op_list_scratch(const Geometry& g);
+cudaError_t launch_op_lists(const Geometry& g, const DirInfo* info, const StepGeo* off,
+                            const Bw4d* bw, const DownGeo* dn, const OpLists& L, int* scratch,
+                            cudaStream_t st);
+// Ray lengths: lmax as FsRec, Lp[nz][ndir] the longest of each plane, *steps
+// the voxel-steps; node: 4N scratch, poff: launch_pad_offsets with 2ny rows;
+// extra_bits: margin in the cutoff besides cut.
+cudaError_t launch_op_lengths(const Geometry& g, const double* chi, const double* S,
+                              const double* smax, const DirInfo* info, const int* poff,
+                              const float4* bw32, double cut, int extra_bits, int groups,
+                              float2* node, int* lmax, int nwp, int* Lp, unsigned long long* steps,
+                              cudaStream_t st);
+// cnt, segb [nz][2 nz]: entries per (plane, list) and the first of them;
+// E, rows [nz]; rowbase [nz][ndir].
+cudaError_t launch_op_counts(const Geometry& g, const OpLists& L, bool para, const int* Lp,
+                             int* rowbase, int* cnt, int* segb, int* E, int* rows, cudaStream_t st);
+cudaError_t launch_op_offsets(const Geometry& g, const OpLists& L, const int* cnt, const int* segb,
+                              const OpMap& op, cudaStream_t st);
+// Recording march of the planes of rank r0 .. r0 + nplanes - 1.
+cudaError_t launch_rec64(const Geometry& g, int r0, int nplanes, const double* chi, const double* B,
+                         const double* G, const DirInfo* info, const StepGeo* off, const Bw4d* bw,
+                         const Bw4d* bwh, const RecOut& ro, const int* lmax, int nwp, int groups,
+                         double* c0s, double* bcs, cudaStream_t st);
+// The same with the parabolic source (para.cu).
+cudaError_t launch_rec64p(const Geometry& g, int r0, int nplanes, const double* chi, const double* B,
+                          const double* G, const DirInfo* info, const StepGeo* off, const Bw4d* bw,
+                          const Bw4d* bwh, const DownGeo* dn, const RecOut& ro, const int* lmax,
+                          int nwp, int groups, double* c0s, double* bcs, cudaStream_t st);
+cudaError_t launch_op_assemble(const Geometry& g, int r0, int nplanes, const OpLists& L,
+                               const RecOut& ro, const int* lmax, const int* cnt, const int* segb,
+                               const OpMap& op, cudaStream_t st);
+cudaError_t launch_op_own(long long N, const double* c0s, const double* bcs, double* c0, double* bc,
+                          cudaStream_t st);
+// J of source S; sp: 4N scratch doubles (S padded).
+cudaError_t launch_op_apply64(const Geometry& g, const double* S, double* sp, const OpMap& op,
+                              double* J, unsigned long long* steps, cudaStream_t st);
+cudaError_t launch_op_lstar(const Geometry& g, const OpLists& L, const OpMap& op, const int* cnt,
+                            const int* segb, double* lstar, cudaStream_t st);
 
 // ---- short characteristics (sc.cu) -----------------------------------------
 // Directions per march launch (the [directions][N] partial buffer holds

@@ -1,0 +1,760 @@
+// The recorded formal solution as an assembled operator.
+//
+// With the opacities, directions and boundary values fixed, the formal
+// solution is linear in the source S (Hauschildt & Baron 2011, Sect. 2.2: I is
+// a weighted sum of S along the characteristic plus the transmitted boundary
+// intensity).  Because voxel centres are lattice points, the upstream points
+// of a direction touch the same node offsets for every voxel of a plane, so
+// the contributions of all directions to one node offset add up to one
+// coefficient per voxel:
+//   J_v = c0_v S_v + bc_v + sum_e A[e][v] S[v + off_e],
+// the offsets e of plane k0 being, for each sign of mu and each distance m,
+// the distinct nodes the directions of that sign touch m planes away.  Per
+// replayed step (four nodes) the 65^3 slab with 32 x 32 directions holds 2.2
+// distinct nodes, so a formal solution is 2.2 FP64 operations per step
+// instead of the five of interpolating S at every step, and 8 bytes of
+// coefficient per operation.
+//
+// Recording, once per opacity:
+//   k_op_lists   (once per quadrature) per (sign, distance) the distinct
+//                nodes, the steepest directions' first (they are cut off
+//                last, so the nodes still in use are a prefix), and per node
+//                its contributions (direction, w_d times the bilinear weight)
+//   k_op_len     the length of every warp's rays, from an FP32 march
+//   k_op_counts  per (plane, sign, distance) the prefix of nodes in use
+//   k_rec64      the march's coefficients c_m of S(p_m) of one chunk of planes
+//   k_op_assemble  A[e][v] = sum over e's contributions of w_d b c_m
+// and k_op_apply64 evaluates J for a source.
+#include "internal.h"
+#include "weights.cuh"
+
+namespace rt3d {
+
+namespace {
+
+constexpr int kOpThreads = 128;      // march and length kernels
+constexpr int kListThreads = 256;
+
+struct OpNodes {
+    int a00, a10, a01, a11;
+};
+
+__device__ __forceinline__ OpNodes op_nodes(int i0, int j0, int ox, int oy, int nx, int ny)
+{
+    int x0 = i0 + ox;
+    x0 -= x0 >= nx ? nx : 0;
+    const int x1 = x0 + 1 == nx ? 0 : x0 + 1;
+    int y0 = j0 + oy;
+    y0 -= y0 >= ny ? ny : 0;
+    const int y1 = y0 + 1 == ny ? 0 : y0 + 1;
+    return OpNodes{y0 * nx + x0, y0 * nx + x1, y1 * nx + x0, y1 * nx + x1};
+}
+
+__device__ __forceinline__ int op_nmax(OpNodes n) { return max(max(n.a00, n.a10), max(n.a01, n.a11)); }
+__device__ __forceinline__ int op_nmin(OpNodes n) { return min(min(n.a00, n.a10), min(n.a01, n.a11)); }
+
+__device__ __forceinline__ double op_bilin(const double* __restrict__ p, OpNodes n, Bw4d b)
+{
+    return b.x * __ldg(p + n.a00) + b.y * __ldg(p + n.a10) + b.z * __ldg(p + n.a01) +
+           b.w * __ldg(p + n.a11);
+}
+
+// One block per (sign, slot m): the distinct nodes of the directions of that
+// sign at distance m (m >= 1), or at the downstream point (m = 0, when dn is
+// given), in the order of the direction list (decreasing |mu|); then each
+// node's contributions in the same order.  Item i of the block is corner
+// i & 3 of direction dl[i >> 2].
+__global__ void __launch_bounds__(kListThreads)
+k_op_lists(Geometry g, const DirInfo* __restrict__ info, const StepGeo* __restrict__ off,
+           const Bw4d* __restrict__ bw, const DownGeo* __restrict__ dn, OpLists L, int* gfirst)
+{
+    extern __shared__ int sfirst[];
+    __shared__ int wsum[kListThreads / 32];
+    const int nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny;
+    const int si = blockIdx.x / nz, m = blockIdx.x - si * nz;
+    const int D = si == 0 ? L.dpos : g.ndir - L.dpos;
+    const int* dl = L.dord + (si == 0 ? 0 : L.dpos);
+    const long long row = (long long)si * nz + m;
+    const int n = (m == 0 && !dn) ? 0 : 4 * D;
+    int* first = gfirst ? gfirst + row * nxy : sfirst;
+    int* unode = L.unode + row * L.ucap;
+    int* ustart = L.ustart + row * (L.ucap + 1);
+    int* uofi = L.uofi + row * L.icap;
+    OpContrib* ct = L.contrib + row * L.icap;
+    auto node = [&](int i) {
+        const int d = dl[i >> 2];
+        int x, y;
+        if (m == 0) {
+            x = dn[d].ox;
+            y = dn[d].oy;
+        } else {
+            const StepGeo o = off[(long long)d * nz + m];
+            x = o.ox;
+            y = o.oy;
+        }
+        x += i & 1;
+        x -= x == nx ? nx : 0;
+        y += (i >> 1) & 1;
+        y -= y == ny ? ny : 0;
+        return y * nx + x;
+    };
+    for (int t = threadIdx.x; t < nxy; t += kListThreads) first[t] = 0x7fffffff;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += kListThreads) atomicMin(&first[node(i)], i);
+    __syncthreads();
+    // ordered compaction of the items that are the first of their node; a
+    // node's entry then holds -(position + 1)
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int base = 0;
+    for (int i0 = 0; i0 < n; i0 += kListThreads) {
+        const int i = i0 + threadIdx.x;
+        const int nd = i < n ? node(i) : 0;
+        const bool f = i < n && first[nd] == i;
+        const unsigned b = __ballot_sync(0xffffffffu, f);
+        if (lane == 0) wsum[wid] = __popc(b);
+        __syncthreads();
+        int pre = base, tot = 0;
+        for (int w = 0; w < kListThreads / 32; ++w) {
+            if (w < wid) pre += wsum[w];
+            tot += wsum[w];
+        }
+        if (f) {
+            const int pos = pre + __popc(b & ((1u << lane) - 1));
+            first[nd] = -(pos + 1);
+            unode[pos] = nd;
+        }
+        base += tot;
+        __syncthreads();
+    }
+    const int U = base;
+    for (int i = threadIdx.x; i < n; i += kListThreads) uofi[i] = -first[node(i)] - 1;
+    // where the 27-point neighbourhood's nodes are in the list (m <= 1)
+    if (m <= 1 && threadIdx.x < 9) {
+        const int ox = threadIdx.x % 3 - 1, oy = threadIdx.x / 3 - 1;
+        const int f = n ? first[(oy < 0 ? ny - 1 : oy) * nx + (ox < 0 ? nx - 1 : ox)] : 0;
+        L.lpos[(si * 2 + m) * 9 + threadIdx.x] = f < 0 ? -f - 1 : -1;
+    }
+    __syncthreads();
+    // the prefix of the list that direction d needs
+    for (int q = threadIdx.x; 4 * q < n; q += kListThreads) {
+        const int* u = uofi + 4 * q;
+        L.posmax[(long long)dl[q] * nz + m] = max(max(u[0], u[1]), max(u[2], u[3])) + 1;
+    }
+    // contributions: counts, their prefix sums, then the entries
+    for (int u = threadIdx.x; u < U; u += kListThreads) {
+        int c = 0;
+        for (int i = 0; i < n; ++i) c += uofi[i] == u;
+        ustart[u + 1] = c;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        ustart[0] = 0;
+        int s = 0;
+        for (int u = 0; u < U; ++u) {
+            s += ustart[u + 1];
+            ustart[u + 1] = s;
+        }
+        L.ucount[row] = U;
+    }
+    __syncthreads();
+    for (int u = threadIdx.x; u < U; u += kListThreads) {
+        int j = ustart[u];
+        const int last = ustart[u + 1] - 1;
+        for (int i = 0; i < n; ++i) {
+            if (uofi[i] != u) continue;
+            const int d = dl[i >> 2], q = i & 3;
+            const Bw4d b = m == 0 ? dn[d].b : bw[(long long)d * nz + m];
+            const double v = q == 0 ? b.x : q == 1 ? b.y : q == 2 ? b.z : b.w;
+            ct[j] = OpContrib{info[d].w * v, d, 2 * u + (j == last)};
+            ++j;
+        }
+    }
+}
+
+// node2[k][y][x] = {chi, S / smax} in FP32, planes padded to 2ny x 2nx by
+// periodic copies.  chi is kept below 1e25 (opaque in any case) so that the
+// FP32 march forms no infinities.
+__global__ void k_op_pack_len(Geometry g, const double* __restrict__ chi,
+                              const double* __restrict__ S, const double* __restrict__ smax,
+                              float2* __restrict__ node)
+{
+    const int nx = g.nx, ny = g.ny;
+    const long long W = 2LL * nx, P = 4LL * nx * ny;
+    const double sm = *smax, inv = sm > 0.0 ? 1.0 / sm : 0.0;
+    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < g.N;
+         v += (long long)gridDim.x * blockDim.x) {
+        const int i = (int)(v % nx), j = (int)((v / nx) % ny);
+        const long long k = v / ((long long)nx * ny);
+        const float2 q = make_float2((float)fmin(chi[v], 1e25), (float)(S[v] * inv));
+        float2* p = node + k * P + (long long)j * W + i;
+        p[0] = q;
+        p[nx] = q;
+        p[(long long)ny * W] = q;
+        p[(long long)ny * W + nx] = q;
+    }
+}
+
+// Lengths of the rays: the march in FP32, a ray ending once the rest of it
+// can change I by less than 2^-lcut |I|, i.e. T smax <= 2^-lcut |I| (tested
+// on logarithms: tau log2 e + log2(|I| / smax) >= lcut).  The 32 lanes of a
+// warp share the longest of their rays.
+__global__ void __launch_bounds__(kOpThreads)
+k_op_len(Geometry g, const float2* __restrict__ node, const DirInfo* __restrict__ info,
+         const int* __restrict__ poff, const float4* __restrict__ bw, float lcut,
+         int* __restrict__ lmax, int nwp)
+{
+    constexpr float kLog2e = 1.4426950408889634f;
+    const int nx = g.nx, nz = g.nz, nxy = nx * g.ny;
+    const int t = blockIdx.x * kOpThreads + threadIdx.x;
+    const int k0 = plane_at(g, blockIdx.z);
+    const bool active = t < nxy;
+    const unsigned amask = __ballot_sync(0xffffffffu, active);
+    if (!active) return;
+    const int j0 = t / nx, i0 = t - j0 * nx;
+    const long long W = 2LL * nx, P = 4LL * nxy;
+    const long long base = k0 * P + j0 * W + i0;
+    const float2 me = node[base];
+    const float2* nb = node + base;
+    for (int d = blockIdx.y; d < g.ndir; d += gridDim.y) {
+        const int s = info[d].sgn;
+        const float hs = info[d].hs32;
+        const int M = s > 0 ? k0 : nz - 1 - k0;
+        const int* od = poff + (long long)d * nz;
+        const float4* bd = bw + (long long)d * nz;
+        float I = 0.f, T = 1.f, tau = 0.f, ca = me.x, sa = me.y;
+        int m = 0;
+        while (m < M) {
+            const int o = od[m + 1];
+            RT_GUARD(g, base + o, 4 * g.N, kSiteFs64) break;
+            RT_GUARD(g, base + o + W + 1, 4 * g.N, kSiteFs64) break;
+            const float4 b = bd[m + 1];
+            const float2* q = nb + o;
+            const float2 q00 = __ldg(q), q10 = __ldg(q + 1), q01 = __ldg(q + W), q11 = __ldg(q + W + 1);
+            const float cb = b.x * q00.x + b.y * q10.x + b.z * q01.x + b.w * q11.x;
+            const float sb = b.x * q00.y + b.y * q10.y + b.z * q01.y + b.w * q11.y;
+            const float x = hs * (ca + cb);
+            float wc, wu, e;
+            seg_weights32(x, wc, wu, e);
+            I = fmaf(T, fmaf(wc, sa, wu * sb), I);
+            tau += x;
+            T = ex2_approx(-tau * kLog2e);
+            ca = cb;
+            sa = sb;
+            ++m;
+            float lg;
+            asm("lg2.approx.f32 %0, %1;" : "=f"(lg) : "f"(fabsf(I)));
+            if (fmaf(tau, kLog2e, lg) >= lcut) break;
+        }
+        const int Lw = __reduce_max_sync(amask, m);
+        if ((threadIdx.x & 31) == 0) lmax[((long long)d * nz + k0) * nwp + (t >> 5)] = Lw;
+    }
+}
+
+// Per (plane k0, direction d): the longest warp, Lp; and the voxel-steps of
+// all of them into *steps.  One warp per (k0, d).
+__global__ void k_op_plane_len(Geometry g, const int* __restrict__ lmax, int nwp,
+                               int* __restrict__ Lp, unsigned long long* __restrict__ steps)
+{
+    const int lane = threadIdx.x & 31;
+    const int d = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), k0 = blockIdx.y;
+    if (d >= g.ndir) return;
+    const int last = g.nx * g.ny - 32 * (nwp - 1);      // lanes of the plane's last warp
+    int L = 0;
+    unsigned long long s = 0;
+    for (int w = lane; w < nwp; w += 32) {
+        const int l = lmax[((long long)d * g.nz + k0) * nwp + w];
+        L = max(L, l);
+        s += (unsigned long long)l * (w == nwp - 1 ? last : 32);
+    }
+    L = __reduce_max_sync(0xffffffffu, L);
+    for (int h = 16; h > 0; h >>= 1) s += __shfl_down_sync(0xffffffffu, s, h);
+    if (lane == 0) {
+        Lp[(long long)k0 * g.ndir + d] = L;
+        if (s) atomicAdd(steps, s);
+    }
+}
+
+// Per plane k0 (one block): the rows of the chunk buffer (row of (d, m) is
+// rowbase[k0][d] + m - 1, with one more row first for the downstream point
+// of the parabolic source), the entries per (sign, slot) rounded up to
+// pairs, their first entry and the plane's number of entries, rounded up to
+// kOpPad.
+__global__ void __launch_bounds__(kListThreads)
+k_op_counts(Geometry g, OpLists L, int para, const int* __restrict__ Lp, int* __restrict__ rowbase,
+            int* __restrict__ cnt, int* __restrict__ segb, int* __restrict__ E, int* __restrict__ rows)
+{
+    __shared__ int wsum[kListThreads / 32];
+    const int nz = g.nz, k0 = blockIdx.x;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int* lp = Lp + (long long)k0 * g.ndir;
+    int base = 0;
+    for (int d0 = 0; d0 < g.ndir; d0 += kListThreads) {
+        const int d = d0 + threadIdx.x;
+        const int v = d < g.ndir ? lp[d] + para : 0;
+        int x = v;
+        for (int h = 1; h < 32; h <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, h);
+            if (lane >= h) x += y;
+        }
+        if (lane == 31) wsum[wid] = x;
+        __syncthreads();
+        int pre = base, tot = 0;
+        for (int w = 0; w < kListThreads / 32; ++w) {
+            if (w < wid) pre += wsum[w];
+            tot += wsum[w];
+        }
+        if (d < g.ndir) rowbase[(long long)k0 * g.ndir + d] = pre + x - v;
+        base += tot;
+        __syncthreads();
+    }
+    if (threadIdx.x == 0) rows[k0] = base;
+    int* cn = cnt + (long long)k0 * 2 * nz;
+    for (int q = threadIdx.x; q < 2 * nz; q += kListThreads) {
+        const int si = q / nz, m = q - si * nz, s = si ? -1 : 1;
+        int n = 0;
+        if (m == 0) {
+            if (para && k0 + s >= 0 && k0 + s < nz) n = L.ucount[q];
+        } else if (m <= (s > 0 ? k0 : nz - 1 - k0)) {
+            const int D = si == 0 ? L.dpos : g.ndir - L.dpos;
+            const int* dl = L.dord + (si == 0 ? 0 : L.dpos);
+            for (int i = 0; i < D; ++i)
+                if (lp[dl[i]] >= m) n = max(n, L.posmax[(long long)dl[i] * nz + m]);
+        }
+        cn[q] = n;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int e = 0;
+        for (int q = 0; q < 2 * nz; ++q) {
+            segb[(long long)k0 * 2 * nz + q] = e;
+            e += (cn[q] + 1) & ~1;
+        }
+        E[k0] = (e + kOpPad - 1) / kOpPad * kOpPad;
+    }
+}
+
+// off[e]: the entry's node relative to the voxel in planes padded to
+// 2ny x 2nx (0 for the padding entries, whose coefficients are 0).
+__global__ void k_op_offsets(Geometry g, OpLists L, const int* __restrict__ cnt,
+                             const int* __restrict__ segb, const int* __restrict__ E,
+                             const long long* __restrict__ eb, int* __restrict__ off)
+{
+    const int nx = g.nx, nz = g.nz, k0 = blockIdx.y;
+    int* o = off + eb[k0];
+    for (int q = blockIdx.x; q <= 2 * nz; q += gridDim.x) {
+        if (q == 2 * nz) {          // the plane's tail
+            const int* sb = segb + (long long)k0 * 2 * nz;
+            const int last = sb[2 * nz - 1] + ((cnt[(long long)k0 * 2 * nz + 2 * nz - 1] + 1) & ~1);
+            for (int e = last + threadIdx.x; e < E[k0]; e += blockDim.x) o[e] = 0;
+            continue;
+        }
+        const int si = q / nz, m = q - si * nz, s = si ? -1 : 1;
+        const int n = cnt[(long long)k0 * 2 * nz + q], b = segb[(long long)k0 * 2 * nz + q];
+        const long long dk = m == 0 ? s : -(long long)m * s;
+        for (int u = threadIdx.x; u < ((n + 1) & ~1); u += blockDim.x) {
+            int v = 0;
+            if (u < n) {
+                const int nd = L.unode[(long long)q * L.ucap + u], y = nd / nx, x = nd - y * nx;
+                v = (int)((dk * 2 * g.ny + y) * 2 * nx + x);
+            }
+            o[b + u] = v;
+        }
+    }
+}
+
+// The march of the planes of rank r0 + blockIdx.z, its coefficients of S
+// recorded: c_m = T_{m-1} w_up,{m-1} + T_m w_cur,m at row (d, m) (the last
+// point: T_{L-1} w_up), and per voxel and slot sum_d w_d w_cur,0 and
+// sum_d w_d T_L I_bc (rays that reach the boundary plane).  The lengths are
+// given (k_op_len), so the march carries no intensity, no source and no
+// cutoff test: 24 of the 32 FP64 instructions per step of the march that
+// also forms I (the FP64 pipe bounds both).
+__global__ void __launch_bounds__(kOpThreads)
+k_rec64(Geometry g, int r0, const double* __restrict__ chi, const double* __restrict__ B,
+        const double* __restrict__ G, const DirInfo* __restrict__ info,
+        const StepGeo* __restrict__ off, const Bw4d* __restrict__ bw, const Bw4d* __restrict__ bwh,
+        RecOut ro, const int* __restrict__ lmax, int nwp, double* __restrict__ c0s,
+        double* __restrict__ bcs)
+{
+    const int nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny;
+    const int t = blockIdx.x * kOpThreads + threadIdx.x;
+    const int k0 = plane_at(g, r0 + blockIdx.z), zb = blockIdx.y, ZB = gridDim.y;
+    __shared__ double tab[kExpTable];
+    fill_exp_table(tab);
+    __syncthreads();
+    if (t >= nxy) return;
+    const int j0 = t / nx, i0 = t - j0 * nx;
+    const long long v = (long long)k0 * nxy + t;
+    const double chi0 = chi[v];
+    for (int slot = zb; slot < kSlots; slot += ZB) {
+        double C0 = 0.0, Bc = 0.0;
+        for (int d = slot; d < g.ndir; d += kSlots) {
+            const int s = info[d].sgn;
+            const double w = info[d].w;
+            const int M = s > 0 ? k0 : nz - 1 - k0;
+            const int L = lmax[((long long)d * nz + k0) * nwp + (t >> 5)];
+            const StepGeo* od = off + (long long)d * nz;
+            const Bw4d* bh = bwh + (long long)d * nz;
+            double* rc = rec_rows(g, ro, ro.base, d, k0, s) + t;
+            double T = 1.0, ca = info[d].hs * chi0, cprev = 0.0;
+            for (int m = 0; m < L; ++m) {
+                const long long pb = (long long)(k0 - (m + 1) * s) * nxy;
+                const StepGeo o = od[m + 1];
+                const OpNodes n = op_nodes(i0, j0, o.ox, o.oy, nx, ny);
+                RT_GUARD(g, pb + op_nmin(n), g.N, kSiteFs64) break;
+                RT_GUARD(g, pb + op_nmax(n), g.N, kSiteFs64) break;
+                const double cb = op_bilin(chi + pb, n, bh[m + 1]);
+                double wc, wu, e;
+                seg_weights64(ca + cb, tab, wc, wu, e);
+                if (m == 0) C0 = fma(w, wc, C0);
+                else rc[(long long)(m - 1) * nxy] = fma(T, wc, cprev);
+                cprev = T * wu;
+                T *= e;
+                ca = cb;
+            }
+            if (L > 0) rc[(long long)(L - 1) * nxy] = cprev;
+            const int bc = s > 0 ? g.top_bc : g.bottom_bc;
+            if (bc && L == M) {
+                const long long pb = (long long)(k0 - M * s) * nxy;
+                const StepGeo o = od[M];
+                const OpNodes n = op_nodes(i0, j0, o.ox, o.oy, nx, ny);
+                const Bw4d b = bw[(long long)d * nz + M];
+                double ibc = op_bilin(B + pb, n, b);
+                if (bc == 2) ibc = fma(info[d].amu, op_bilin(G, n, b), ibc);   // B + |mu| dB/dtau
+                Bc = fma(w, T * ibc, Bc);
+            }
+        }
+        c0s[(long long)slot * g.N + v] = C0;
+        bcs[(long long)slot * g.N + v] = Bc;
+    }
+}
+
+// A of the planes of rank r0 + blockIdx.y: one block per 32 voxels, the
+// lanes of its warps the voxels.  A warp takes a run of entries of a list and
+// walks their contributions, which are consecutive: 32 at a time, each lane
+// looks up one contribution's row, then the warp adds them eight by eight in
+// list order (eight coefficient loads in flight) and stores an entry when its
+// last contribution is in.  Rows past the warp's own rays hold nothing
+// (m > its length) and count as zero.
+constexpr int kAsmRun = 16;      // entries of a run (even)
+__global__ void __launch_bounds__(kListThreads)
+k_op_assemble(Geometry g, int r0, OpLists L, RecOut ro, const int* __restrict__ lmax, int nwp,
+              const int* __restrict__ cnt, const int* __restrict__ segb, const int* __restrict__ E,
+              const long long* __restrict__ eb, double* __restrict__ A)
+{
+    extern __shared__ int2 lr[];     // [ndir] {length, first row}
+    const int nz = g.nz, nxy = g.nx * g.ny;
+    const int k0 = plane_at(g, r0 + blockIdx.y), tile = blockIdx.x;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int t = tile * 32 + lane;
+    const bool live = t < nxy;
+    for (int d = threadIdx.x; d < g.ndir; d += blockDim.x)
+        lr[d] = make_int2(lmax[((long long)d * nz + k0) * nwp + tile],
+                          ro.rowbase[(long long)k0 * g.ndir + d]);
+    __syncthreads();
+    const double* c = ro.base + ro.prow[k0] * nxy + (live ? t : 0);
+    double2* out = reinterpret_cast<double2*>(A + eb[k0] * (long long)nwp * 32) +
+                   (long long)tile * (E[k0] / 2) * 32 + lane;
+    int run = wid;                   // runs go round the warps, across the lists
+    for (int q = blockIdx.z; q < 2 * nz; q += gridDim.z) {
+        const int n = cnt[(long long)k0 * 2 * nz + q];
+        if (n == 0) continue;
+        const int m = q < nz ? q : q - nz;
+        double2* oq = out + (long long)(segb[(long long)k0 * 2 * nz + q] / 2) * 32;
+        const int* us = L.ustart + (long long)q * (L.ucap + 1);
+        const OpContrib* ct = L.contrib + (long long)q * L.icap;
+        const int runs = (n + kAsmRun - 1) / kAsmRun;
+        for (; run < runs; run += nw) {
+            const int js = us[run * kAsmRun], je = us[min(n, (run + 1) * kAsmRun)];
+            double acc = 0.0, even = 0.0;
+            for (int jb = js; jb < je; jb += 32) {
+                OpContrib k{0.0, 0, 0};
+                int row = -1;
+                if (jb + lane < je) {
+                    k = ct[jb + lane];
+                    const int2 p = lr[k.d];
+                    if (m <= p.x || m == 0) row = p.y + m - 1 + ro.para;
+                }
+                const int nj = min(32, je - jb);
+                for (int i = 0; i < nj; i += 8) {
+                    double cv[8];
+#pragma unroll
+                    for (int h = 0; h < 8; ++h) {
+                        const int r = __shfl_sync(0xffffffffu, row, i + h);
+                        cv[h] = r >= 0 ? __ldg(c + (long long)r * nxy) : 0.0;
+                    }
+#pragma unroll
+                    for (int h = 0; h < 8; ++h) {
+                        acc = fma(__shfl_sync(0xffffffffu, k.wb, i + h), cv[h], acc);
+                        const int ul = __shfl_sync(0xffffffffu, k.ul, i + h);
+                        if (ul & 1) {       // entry ul >> 1 is complete
+                            if (!live) acc = 0.0;
+                            if (ul & 2) oq[(long long)(ul >> 2) * 32] = make_double2(even, acc);
+                            else even = acc;
+                            acc = 0.0;
+                        }
+                    }
+                }
+            }
+            if ((n & 1) && (run + 1) * kAsmRun >= n) oq[(long long)(n >> 1) * 32] = make_double2(even, 0.0);
+        }
+        run -= runs;
+    }
+    if (blockIdx.z) return;
+    const int qz = 2 * nz - 1;
+    const int tail = (segb[(long long)k0 * 2 * nz + qz] + cnt[(long long)k0 * 2 * nz + qz] + 1) / 2;
+    for (int p = tail + wid; p < E[k0] / 2; p += nw) out[(long long)p * 32] = make_double2(0.0, 0.0);
+}
+
+// c0[v] = sum over slots of c0s, bc[v] likewise (slot order fixed)
+__global__ void k_op_own(long long N, const double* __restrict__ c0s, const double* __restrict__ bcs,
+                         double* __restrict__ c0, double* __restrict__ bc)
+{
+    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < N;
+         v += (long long)gridDim.x * blockDim.x) {
+        double a = 0.0, b = 0.0;
+        for (int q = 0; q < kSlots; ++q) {
+            a += c0s[q * N + v];
+            b += bcs[q * N + v];
+        }
+        c0[v] = a;
+        bc[v] = b;
+    }
+}
+
+// S in planes padded to 2ny x 2nx by periodic copies, so that an entry's node
+// is at one offset from every voxel of the plane.
+__global__ void k_op_pack(Geometry g, const double* __restrict__ S, double* __restrict__ sp)
+{
+    const int nx = g.nx, ny = g.ny;
+    const long long W = 2LL * nx, P = 4LL * nx * ny;
+    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < g.N;
+         v += (long long)gridDim.x * blockDim.x) {
+        const int i = (int)(v % nx), j = (int)((v / nx) % ny);
+        const long long k = v / ((long long)nx * ny);
+        const double s = S[v];
+        double* p = sp + k * P + (long long)j * W + i;
+        p[0] = s;
+        p[nx] = s;
+        p[(long long)ny * W] = s;
+        p[(long long)ny * W + nx] = s;
+    }
+}
+
+// J of a source: one block per 32 voxels of a plane, its warps taking four
+// entries at a time in turn (the block streams its coefficients, 8 bytes per
+// FP64 FMA, in order), then the warps' sums and the voxel's own terms in
+// fixed order.
+template <int NW>
+__global__ void __launch_bounds__(NW * 32, NW < 24 ? 24 / NW : 1)
+k_op_apply64(Geometry g, const double* __restrict__ S, const double* __restrict__ sp, OpMap op,
+             double* __restrict__ J, unsigned long long* __restrict__ steps)
+{
+    __shared__ double red[NW][32];
+    const int nx = g.nx, nxy = nx * g.ny;
+    const int tile = blockIdx.x, k0 = plane_at(g, blockIdx.y);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int t = tile * 32 + lane, tc = t < nxy ? t : 0;
+    const int j0 = tc / nx, i0 = tc - j0 * nx;
+    const long long at = (long long)k0 * 4 * nxy + (long long)j0 * 2 * nx + i0;
+    const double* s = sp + at;
+    const int E = op.E[k0];
+    const long long eb = op.eb[k0];
+    const double2* A = reinterpret_cast<const double2*>(op.A + eb * op.nwp * 32) +
+                       (long long)tile * (E / 2) * 32 + lane;
+    const int4* off = reinterpret_cast<const int4*>(op.off + eb);
+    double acc0 = 0.0, acc1 = 0.0;
+    constexpr int kQ = 4;       // quads of entries in flight per warp
+    const int nq = E / 4;
+    int q = wid;
+    for (; q + (kQ - 1) * NW < nq; q += kQ * NW) {
+        int4 o[kQ];
+        double2 a[kQ], b[kQ];
+#pragma unroll
+        for (int i = 0; i < kQ; ++i) {
+            o[i] = __ldg(off + q + i * NW);
+            a[i] = __ldcs(A + (long long)(q + i * NW) * 64);
+            b[i] = __ldcs(A + (long long)(q + i * NW) * 64 + 32);
+        }
+#pragma unroll
+        for (int i = 0; i < kQ; ++i) {
+            RT_GUARD(g, at + min(min(o[i].x, o[i].y), min(o[i].z, o[i].w)), 4 * g.N, kSiteFs64) continue;
+            RT_GUARD(g, at + max(max(o[i].x, o[i].y), max(o[i].z, o[i].w)), 4 * g.N, kSiteFs64) continue;
+            acc0 = fma(a[i].x, __ldg(s + o[i].x), acc0);
+            acc1 = fma(a[i].y, __ldg(s + o[i].y), acc1);
+            acc0 = fma(b[i].x, __ldg(s + o[i].z), acc0);
+            acc1 = fma(b[i].y, __ldg(s + o[i].w), acc1);
+        }
+    }
+    for (; q < nq; q += NW) {
+        const int4 o = __ldg(off + q);
+        RT_GUARD(g, at + min(min(o.x, o.y), min(o.z, o.w)), 4 * g.N, kSiteFs64) break;
+        RT_GUARD(g, at + max(max(o.x, o.y), max(o.z, o.w)), 4 * g.N, kSiteFs64) break;
+        const double2 a = __ldcs(A + (long long)q * 64), b = __ldcs(A + (long long)q * 64 + 32);
+        acc0 = fma(a.x, __ldg(s + o.x), acc0);
+        acc1 = fma(a.y, __ldg(s + o.y), acc1);
+        acc0 = fma(b.x, __ldg(s + o.z), acc0);
+        acc1 = fma(b.y, __ldg(s + o.w), acc1);
+    }
+    red[wid][lane] = acc0 + acc1;
+    __syncthreads();
+    if (wid == 0 && t < nxy) {
+        const long long v = (long long)k0 * nxy + t;
+        double a = fma(op.c0[v], S[v], op.bc[v]);
+        for (int w = 0; w < NW; ++w) a += red[w][lane];
+        J[v] = a;
+    }
+    if (steps && tile == 0 && blockIdx.y == 0 && threadIdx.x == 0) atomicAdd(steps, *op.steps);
+}
+
+// Lambda* from the operator: the voxel's own coefficient and those of the
+// nearest nodes of the neighbouring planes (distance 1 upstream; for the
+// parabolic source also the downstream point).
+__global__ void k_op_lstar(Geometry g, OpLists L, OpMap op, const int* __restrict__ cnt,
+                           const int* __restrict__ segb, double* __restrict__ lstar)
+{
+    const int nxy = g.nx * g.ny, nz = g.nz;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, k0 = blockIdx.y, o = blockIdx.z;
+    if (t >= nxy) return;
+    const long long v = (long long)k0 * nxy + t;
+    const int oz = o / 9 - 1;
+    double r = 0.0;
+    if (oz == 0) {
+        if (o == 13) r = op.c0[v];
+    } else {
+        const double* A = op.A + op.eb[k0] * (long long)op.nwp * 32 +
+                          (long long)(t >> 5) * op.E[k0] * 32;
+        for (int m = 1; m >= 0; --m) {
+            // upstream (m = 1): plane k0 - s; downstream (m = 0): plane k0 + s
+            const int si = (m == 1) == (oz < 0) ? 0 : 1;
+            const int u = L.lpos[(si * 2 + m) * 9 + o % 9];
+            const long long q = (long long)k0 * 2 * nz + (long long)si * nz + m;
+            if (u < 0 || u >= cnt[q]) continue;
+            const int e = segb[q] + u;
+            r += A[((long long)(e >> 1) * 32 + (t & 31)) * 2 + (e & 1)];
+        }
+    }
+    lstar[(long long)o * g.N + v] = r;
+}
+
+unsigned op_grid1d(long long n, int threads)
+{
+    long long b = (n + threads - 1) / threads;
+    if (b > 152LL * 32) b = 152LL * 32;
+    if (b < 1) b = 1;
+    return (unsigned)b;
+}
+
+}  // namespace
+
+// Nodes of a plane that fit in shared memory while its list is built.
+constexpr int kListSmemNodes = 24 * 1024;
+
+long long op_list_scratch(const Geometry& g)
+{
+    const long long nxy = (long long)g.nx * g.ny;
+    return nxy <= kListSmemNodes ? 0 : 2 * nxy * g.nz;
+}
+
+cudaError_t launch_op_lists(const Geometry& g, const DirInfo* info, const StepGeo* off,
+                            const Bw4d* bw, const DownGeo* dn, const OpLists& L, int* scratch,
+                            cudaStream_t st)
+{
+    const size_t shm = scratch ? 0 : sizeof(int) * (size_t)g.nx * g.ny;
+    if (shm > 40 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(k_op_lists, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)shm);
+        if (e != cudaSuccess) return e;
+    }
+    k_op_lists<<<2 * g.nz, kListThreads, shm, st>>>(g, info, off, bw, dn, L, scratch);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_op_lengths(const Geometry& g, const double* chi, const double* S,
+                              const double* smax, const DirInfo* info, const int* poff,
+                              const float4* bw32, double cut, int extra_bits, int groups,
+                              float2* node, int* lmax, int nwp, int* Lp, unsigned long long* steps,
+                              cudaStream_t st)
+{
+    k_op_pack_len<<<op_grid1d(g.N, 256), 256, 0, st>>>(g, chi, S, smax, node);
+    // two bits beyond the cutoff cover the FP32 rounding of tau and I
+    const float lcut = cut > 0.0 ? (float)(-log2(cut)) + 2.0f + (float)extra_bits : INFINITY;
+    const dim3 grid((g.nx * g.ny + kOpThreads - 1) / kOpThreads, groups, g.nz);
+    k_op_len<<<grid, kOpThreads, 0, st>>>(g, node, info, poff, bw32, lcut, lmax, nwp);
+    cudaError_t e = cudaMemsetAsync(steps, 0, sizeof(unsigned long long), st);
+    if (e != cudaSuccess) return e;
+    k_op_plane_len<<<dim3((g.ndir + 7) / 8, g.nz), 256, 0, st>>>(g, lmax, nwp, Lp, steps);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_op_counts(const Geometry& g, const OpLists& L, bool para, const int* Lp,
+                             int* rowbase, int* cnt, int* segb, int* E, int* rows, cudaStream_t st)
+{
+    k_op_counts<<<g.nz, kListThreads, 0, st>>>(g, L, para ? 1 : 0, Lp, rowbase, cnt, segb, E, rows);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_op_offsets(const Geometry& g, const OpLists& L, const int* cnt, const int* segb,
+                              const OpMap& op, cudaStream_t st)
+{
+    const dim3 grid(2 * g.nz + 1 < 64 ? 2 * g.nz + 1 : 64, g.nz);
+    k_op_offsets<<<grid, 128, 0, st>>>(g, L, cnt, segb, op.E, op.eb, const_cast<int*>(op.off));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_rec64(const Geometry& g, int r0, int nplanes, const double* chi, const double* B,
+                         const double* G, const DirInfo* info, const StepGeo* off, const Bw4d* bw,
+                         const Bw4d* bwh, const RecOut& ro, const int* lmax, int nwp, int groups,
+                         double* c0s, double* bcs, cudaStream_t st)
+{
+    const dim3 grid((g.nx * g.ny + kOpThreads - 1) / kOpThreads, groups, nplanes);
+    k_rec64<<<grid, kOpThreads, 0, st>>>(g, r0, chi, B, G, info, off, bw, bwh, ro, lmax, nwp, c0s,
+                                         bcs);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_op_assemble(const Geometry& g, int r0, int nplanes, const OpLists& L,
+                               const RecOut& ro, const int* lmax, const int* cnt, const int* segb,
+                               const OpMap& op, cudaStream_t st)
+{
+    const size_t shm = sizeof(int2) * (size_t)g.ndir;
+    if (shm > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(k_op_assemble, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)shm);
+        if (e != cudaSuccess) return e;
+    }
+    // few tiles: several blocks share a tile's lists, so that every SM has work
+    int split = 1;
+    while (split < 8 && (long long)op.nwp * nplanes * split < 152 * 8) split *= 2;
+    k_op_assemble<<<dim3(op.nwp, nplanes, split), kListThreads, shm, st>>>(
+        g, r0, L, ro, lmax, op.nwp, cnt, segb, op.E, op.eb, const_cast<double*>(op.A));
+    return cudaGetLastError();
+}
+
+cudaError_t launch_op_own(long long N, const double* c0s, const double* bcs, double* c0, double* bc,
+                          cudaStream_t st)
+{
+    k_op_own<<<op_grid1d(N, 256), 256, 0, st>>>(N, c0s, bcs, c0, bc);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_op_apply64(const Geometry& g, const double* S, double* sp, const OpMap& op,
+                              double* J, unsigned long long* steps, cudaStream_t st)
+{
+    k_op_pack<<<op_grid1d(g.N, 256), 256, 0, st>>>(g, S, sp);
+    const dim3 grid(op.nwp, g.nz);
+    if ((long long)op.nwp * g.nz < 152 * 3)
+        k_op_apply64<16><<<grid, 512, 0, st>>>(g, S, sp, op, J, steps);
+    else
+        k_op_apply64<8><<<grid, 256, 0, st>>>(g, S, sp, op, J, steps);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_op_lstar(const Geometry& g, const OpLists& L, const OpMap& op, const int* cnt,
+                            const int* segb, double* lstar, cudaStream_t st)
+{
+    k_op_lstar<<<dim3((g.nx * g.ny + 127) / 128, g.nz, 27), 128, 0, st>>>(g, L, op, cnt, segb, lstar);
+    return cudaGetLastError();
+}
+
+}  // namespace rt3d
