@@ -196,16 +196,21 @@ int rt_last_step_count(rt_ctx *ctx, unsigned long long *steps);
  * and also stores, per (voxel, direction, step), the coefficient of S at
  * that step's upstream point (the products of transmissions and segment
  * weights), cut at 1e-2 times the cutoff; every formal solution then
- * evaluates J from those coefficients and its S (FP64: five FP64
- * operations per step instead of the weights' exponential and division),
- * so J does not depend on which formal solution recorded.  The parabolic
+ * evaluates J from those coefficients and its S, so J does not depend on
+ * which formal solution recorded.  FP64 and double-float: the coefficients
+ * that the directions give the same node of the same voxel are added up
+ * once, and a formal solution is one multiply-add per (voxel, node) (Lambda*
+ * is read off them); where that takes more memory than the coefficients
+ * themselves and half as much again (at least 4, at most 24 GiB more), they
+ * are kept ray by ray and S is interpolated at every step.  The parabolic
  * source also keeps the coefficient of S at the downstream point per
  * (voxel, direction).  The FP32 sweep records FP32 coefficients of
  * S(p_m) - S_0 for its difference form and replays them with the
  * interpolated source differences of its march (its finishing stage
  * replays the same recording for the source change); the double-float
- * form records double-float coefficients of S(p_m) - S_0.  Memory, FP64
- * and double-float: 8 ndir nx ny nz (nz-1)/2 bytes of coefficients plus
+ * form records double-float coefficients of S(p_m) - S_0.  The memory
+ * max_bytes is compared with, FP64 and double-float:
+ * 8 ndir nx ny nz (nz-1)/2 bytes of coefficients plus
  * 4 ndir nz ceil(nx ny/32) + 128 N bytes (65^3 x 1024 directions: 72 GB;
  * parabolic: + 8 ndir N); FP32 sweep: about 8 ndir nx ceil(ny/2) nz (nz+6)/2
  * bytes of coefficients (blocks of four steps) plus 4 ndir nz nx ny/64 +

@@ -84,7 +84,7 @@ struct rt_ctx {
         int *lmax, *Lp, *rowbase, *cnt, *segb, *E, *rows, *poff;
         long long *eb, *prow;
         unsigned long long* steps;
-        double *c0s, *bcs;
+        double *c0s, *bcs, *tss;
     } ow{};
     std::vector<int> dord;      // directions by sign and decreasing |mu| (OpLists)
     int dpos = 0;
@@ -455,15 +455,15 @@ long long op_tiles(const rt_ctx* c) { return ((long long)c->g.nx * c->g.ny + 31)
 long long op_bytes(const rt_ctx* c, long long entries)
 {
     return up256(entries * op_tiles(c) * 32 * (long long)sizeof(double)) +
-           up256(entries * (long long)sizeof(int)) + 2 * up256(c->g.N * (long long)sizeof(double));
+           up256(entries * (long long)sizeof(int)) + 3 * up256(c->g.N * (long long)sizeof(double));
 }
 
 // Memory an operator may take with its chunk buffer: what the ray-by-ray
-// recording takes, or somewhat more where that is small (33^3 with 256
-// directions: 1.25 GB against 1.18).
+// recording takes and half as much again, at least 4 and at most 24 GiB (61 x
+// 45 x 52 with 384 directions in double-float: 13 GB against 11.2).
 long long op_budget(const rt_ctx* c, long long need)
 {
-    const long long extra = std::min(std::max(need / 4, 2LL << 30), 8LL << 30);
+    const long long extra = std::min(std::max(need / 2, 4LL << 30), 24LL << 30);
     return need + extra;
 }
 
@@ -538,7 +538,7 @@ int ensure_op_work(rt_ctx* c)
                     b_q = up256(4 * Q), b_z = up256(8LL * g.nz),
                     b_slot = up256(8LL * kSlots * g.N);
     char* m = nullptr;
-    CK(cudaMalloc((void**)&m, (size_t)(b_sp + b_lmax + 3 * b_t + 2 * b_q + 4 * b_z + 256 + 2 * b_slot)));
+    CK(cudaMalloc((void**)&m, (size_t)(b_sp + b_lmax + 3 * b_t + 2 * b_q + 4 * b_z + 256 + 3 * b_slot)));
     c->ow_mem = m;
     auto& w = c->ow;
     w.sp = reinterpret_cast<double*>(m); m += b_sp;
@@ -554,22 +554,25 @@ int ensure_op_work(rt_ctx* c)
     w.prow = reinterpret_cast<long long*>(m); m += b_z;
     w.steps = reinterpret_cast<unsigned long long*>(m); m += 256;
     w.c0s = reinterpret_cast<double*>(m); m += b_slot;
-    w.bcs = reinterpret_cast<double*>(m);
+    w.bcs = reinterpret_cast<double*>(m); m += b_slot;
+    w.tss = reinterpret_cast<double*>(m);
     CK(launch_pad_offsets(g, c->info, c->off, 2LL * g.ny, w.poff, c->stream));
     c->stats.launches += 1;
     return RT_OK;
 }
 
 double cut_of(const rt_ctx* c);
+ViewDF viewdf(rt_ctx* c);
 
 // Below this bound on an operator's bytes its exact size is not asked for:
 // the recording runs without a host wait.
-constexpr long long kOpNoWait = 256LL << 20;
+constexpr long long kOpNoWait = 64LL << 20;
 
-// Record the FP64 march of the current source (linear or parabolic) and
-// assemble its operator, or keep it ray by ray where the operator would take
-// more memory (op_budget).  use: whether a recording is held afterwards.
-int ensure_rec64(rt_ctx* c, int G, bool& use)
+// Record the march of the current source (FP64, linear or parabolic, or
+// double-float) and assemble its operator, or keep it ray by ray where the
+// operator would take more memory (op_budget).  use: whether a recording is
+// held afterwards.
+int ensure_op_rec(rt_ctx* c, int G, bool& use)
 {
     use = false;
     const long long need = rec_need(c);
@@ -583,12 +586,12 @@ int ensure_rec64(rt_ctx* c, int G, bool& use)
     int rc;
     if ((rc = ensure_op_work(c))) return rc;
     const Geometry& g = c->g;
-    const bool para = c->src_order == RT_SRC_PARABOLIC;
+    const bool para = c->src_order == RT_SRC_PARABOLIC, df = c->precision == RT_DF64;
     const long long nxy = (long long)g.nx * g.ny, nwp = op_tiles(c);
     auto& w = c->ow;
     cudaStream_t st = c->stream;
     CK(launch_op_lengths(g, c->chi, c->S, c->scal + 0, c->info, w.poff, c->bw32,
-                         cut_of(c) * kRecCutMargin, para ? kParaCutBits : 0, G,
+                         cut_of(c) * kRecCutMargin, para ? kParaCutBits : df ? 1 : 0, df, G,
                          reinterpret_cast<float2*>(w.sp), w.lmax, (int)nwp, w.Lp, w.steps, st));
     c->stats.launches += 3;
     bool op = op_fits(c);
@@ -626,7 +629,7 @@ int ensure_rec64(rt_ctx* c, int G, bool& use)
             // a chunk large enough to fill the GPU a few times over: an
             // eighth of the ray-by-ray recording, the whole if it fits
             long long cb = std::min(rows, std::max(most, std::max(need / 8, 2LL << 30) / row)) * row;
-            if (own + up256(cb) > room) cb = most * row;
+            if (own + up256(cb) > room) cb = std::max(most, rows / 12) * row;
             if (own + up256(cb) > room) {
                 op = false;
             } else {
@@ -658,7 +661,7 @@ int ensure_rec64(rt_ctx* c, int G, bool& use)
         if (!rec_reserve(c, need)) return RT_OK;
         if ((rc = ensure_rec(c, use))) return rc;
         if (!use) return RT_OK;
-        CK(cudaMemcpyAsync(c->rec.lmax, w.lmax, sizeof(int) * (size_t)g.ndir * g.nz * nwp,
+        CK(cudaMemcpyAsync(df ? c->rec32.lmax : c->rec.lmax, w.lmax, sizeof(int) * (size_t)g.ndir * g.nz * nwp,
                            cudaMemcpyDeviceToDevice, st));
     } else {
         const long long b_A = up256(entries * nwp * 32 * (long long)sizeof(double)),
@@ -668,6 +671,7 @@ int ensure_rec64(rt_ctx* c, int G, bool& use)
         c->op.off = reinterpret_cast<int*>(q); q += b_off;
         c->op.c0 = reinterpret_cast<double*>(q); q += b_n;
         c->op.bc = reinterpret_cast<double*>(q); q += b_n;
+        c->op.ts = reinterpret_cast<double*>(q);
         c->op.E = w.E;
         c->op.eb = w.eb;
         c->op.steps = w.steps;
@@ -678,16 +682,20 @@ int ensure_rec64(rt_ctx* c, int G, bool& use)
         c->stats.launches += 1;
     }
     RecOut ro{};
-    ro.base = op ? reinterpret_cast<double*>(c->rec_mem + op_bytes(c, entries)) : c->rec.coef;
+    ro.base = op ? reinterpret_cast<double*>(c->rec_mem + op_bytes(c, entries))  :
+              df ? reinterpret_cast<double*>(c->rec32.coef) : c->rec.coef;
     ro.rowbase = op ? w.rowbase : nullptr;
     ro.prow = op ? w.prow : nullptr;
     ro.para = op && para ? 1 : 0;
     ro.cdn = op ? nullptr : c->rec.cdn;
-    double* c0s = op ? w.c0s : c->rec.c0;
-    double* bcs = op ? w.bcs : c->rec.bc;
+    double* c0s = op ? w.c0s : df ? nullptr : c->rec.c0;
+    double* bcs = op ? w.bcs : df ? c->rec32.bc : c->rec.bc;
+    double* tss = op ? w.tss : c->rec32.tsum;
     for (size_t i = 0; i + 1 < first.size(); ++i) {
         const int r0 = first[i], np = first[i + 1] - r0;
-        if (para)
+        if (df)
+            CK(launch_recdf(viewdf(c), r0, np, ro, w.lmax, (int)nwp, G, c0s, bcs, tss, st));
+        else if (para)
             CK(launch_rec64p(g, r0, np, c->chi, c->B, c->gdiff, c->info, c->off, c->bw, c->bwh, c->dn,
                              ro, w.lmax, (int)nwp, G, c0s, bcs, st));
         else
@@ -695,13 +703,12 @@ int ensure_rec64(rt_ctx* c, int G, bool& use)
                             w.lmax, (int)nwp, G, c0s, bcs, st));
         c->stats.launches += 1;
         if (op) {
-            CK(launch_op_assemble(g, r0, np, c->ol, ro, w.lmax, w.cnt, w.segb, c->op, st));
+            CK(launch_op_assemble(g, df, r0, np, c->ol, ro, w.lmax, w.cnt, w.segb, c->op, st));
             c->stats.launches += 1;
         }
     }
     if (op) {
-        CK(launch_op_own(g.N, w.c0s, w.bcs, const_cast<double*>(c->op.c0),
-                         const_cast<double*>(c->op.bc), st));
+        CK(launch_op_own(g.N, w.c0s, w.bcs, df ? w.tss : nullptr, c->op, st));
         c->stats.launches += 1;
     }
     c->rec_op = op;
@@ -882,7 +889,7 @@ double cut_of(const rt_ctx* c)
 // Lambda* is read off the operator (its own and nearest-node entries are the
 // exact elements; 0.05 against 25 ms for the kernel on the 65^3 slab) unless
 // the recording was cut so early that the cut shows in them.
-constexpr double kOpLstarCut = 1e-16;
+constexpr double kOpLstarCut = 1e-15;
 
 // direct: Jout holds J already (the assembled operator)
 int fs_finish(rt_ctx* c, double* Jout, bool direct)
@@ -897,7 +904,7 @@ int fs_finish(rt_ctx* c, double* Jout, bool direct)
     c->stats.launches += direct ? 0 : 1;
     if (!c->lstar_valid) {
         if (direct && cut_of(c) <= kOpLstarCut) {
-            CK(launch_op_lstar(c->g, c->ol, c->op, c->ow.cnt, c->ow.segb, c->lstar, c->stream));
+            CK(launch_op_lstar(c->g, c->precision == RT_DF64, c->ol, c->op, c->ow.cnt, c->ow.segb, c->lstar, c->stream));
         } else if (c->src_order == RT_SRC_PARABOLIC) {
             CK(launch_lstar64p(c->g, c->chi, c->info, c->off, c->bw, c->dn, c->lstar, c->stream));
         } else if (c->precision == RT_FP64) {
@@ -995,22 +1002,21 @@ int run_fs_short(rt_ctx* c, double* Jout, bool count_steps)
 
 // The double-float formal solution of a context: recorded in the first one
 // after the opacities change and replayed, or marched when the recording
-// does not fit.
-int df_formal(rt_ctx* c, int G, unsigned long long* steps, cudaStream_t st)
+// does not fit.  direct: J is in Jout, else in the slots of c->partial.
+int df_formal(rt_ctx* c, int G, double* Jout, unsigned long long* steps, bool& direct)
 {
     bool use = false;
-    int rc = ensure_rec(c, use);
+    int rc = ensure_op_rec(c, G, use);
     if (rc) return rc;
-    const double cut = cut_of(c);
-    if (use && !c->rec_valid) {
-        CK(launch_fsdf(viewdf(c), cut * kRecCutMargin, G, steps, st, &c->rec32));
-        c->rec_valid = true;
+    direct = use && c->rec_op;
+    if (direct) {
+        CK(launch_op_apply_df(c->g, c->S, c->ow.sp, c->op, c->wsum, Jout, steps, c->stream));
         c->stats.launches += 1;
+    } else if (use) {
+        CK(launch_fsdfrep(viewdf(c), c->rec32, G, steps, c->stream));
+    } else {
+        CK(launch_fsdf(viewdf(c), cut_of(c), G, steps, c->stream));
     }
-    if (use)
-        CK(launch_fsdfrep(viewdf(c), c->rec32, G, steps, st));
-    else
-        CK(launch_fsdf(viewdf(c), cut, G, steps, st));
     return RT_OK;
 }
 
@@ -1022,7 +1028,7 @@ int df_formal(rt_ctx* c, int G, unsigned long long* steps, cudaStream_t st)
 int fs64_formal(rt_ctx* c, int G, double* Jout, unsigned long long* steps, bool& direct)
 {
     bool use = false;
-    int rc = ensure_rec64(c, G, use);
+    int rc = ensure_op_rec(c, G, use);
     if (rc) return rc;
     direct = use && c->rec_op;
     cudaStream_t st = c->stream;
@@ -1054,7 +1060,7 @@ int run_fs(rt_ctx* c, double* Jout, bool count_steps)
     if (c->precision == RT_FP64) {
         if ((rc = fs64_formal(c, G, Jout, count_steps ? c->d_steps : nullptr, direct))) return rc;
     } else if (c->precision == RT_DF64) {
-        if ((rc = df_formal(c, G, count_steps ? c->d_steps : nullptr, c->stream))) return rc;
+        if ((rc = df_formal(c, G, Jout, count_steps ? c->d_steps : nullptr, direct))) return rc;
     } else if (c->fin == 1) {
         if ((rc = fin_reference_march(c, G, count_steps ? c->d_steps : nullptr, c->stream)))
             return rc;
@@ -1126,6 +1132,8 @@ int prepare_source(rt_ctx* c, const double* S_in, bool device)
     } else if (c->precision == RT_FP32_SWEEP) {
         CK(launch_pack_pairs(c->g, c->chi, c->S, c->pair, c->plo, c->stream));
         c->stats.launches += 1;
+    } else if (c->precision == RT_DF64 && c->rec_valid && c->rec_op) {
+        // the operator packs its own source planes
     } else if (c->precision == RT_DF64) {
         CK(launch_packdf(c->g, c->chi, c->S, c->node4, c->stream));
         c->stats.launches += 1;
@@ -1699,7 +1707,7 @@ int batch_admit(rt_batch* b, int max_iter)
         // room for the assembled operator of an FP64 problem where the
         // budget allows it at all, else for the ray-by-ray recording
         long long need = rec_need(c);
-        if (need > 0 && c->precision == RT_FP64 && rec_ask(c, need) <= limit)
+        if (need > 0 && c->precision != RT_FP32_SWEEP && rec_ask(c, need) <= limit)
             need = rec_ask(c, need);
         // a pooled block that holds the recording
         int pick = -1;
@@ -1981,7 +1989,9 @@ int batch_fs(rt_batch* b, const std::vector<int>& act)
         for (int p : act) {
             rt_ctx* c = b->ctx[p];
             if (c->precision == RT_DF64) {
-                if ((rc = bpass(b, p, df_formal(c, G, b->d_steps, b->stream)))) return rc;
+                bool d = false;
+                if ((rc = bpass(b, p, df_formal(c, G, c->Jfs, b->d_steps, d)))) return rc;
+                direct[p] = d;
             } else if (c->fin == 1) {
                 if ((rc = bpass(b, p, fin_reference_march(c, G, b->d_steps, b->stream)))) return rc;
             } else {
@@ -1993,13 +2003,11 @@ int batch_fs(rt_batch* b, const std::vector<int>& act)
     } else {
         for (int p : act) {
             rt_ctx* c = b->ctx[p];
-            if (b->precision == RT_DF64) {
-                if ((rc = bpass(b, p, df_formal(c, G, b->d_steps, b->stream)))) return rc;
-            } else {
-                bool d = false;
-                if ((rc = bpass(b, p, fs64_formal(c, G, c->Jfs, b->d_steps, d)))) return rc;
-                direct[p] = d;
-            }
+            bool d = false;
+            rc = b->precision == RT_DF64 ? df_formal(c, G, c->Jfs, b->d_steps, d)
+                                         : fs64_formal(c, G, c->Jfs, b->d_steps, d);
+            if ((rc = bpass(b, p, rc))) return rc;
+            direct[p] = d;
             b->stats.fs_launches += 1;
             b->stats.launches += 1;
         }

@@ -134,15 +134,8 @@ __device__ __forceinline__ void add_steps_df(unsigned long long* steps, unsigned
     if ((threadIdx.x & 31) == 0 && n) atomicAdd(steps, n);
 }
 
-// REC: also record the march as a linear map of the source (Rec32 with the
-// FP64 layout of rec_base: per (direction, plane) [step][voxel], one
-// double-float pair per entry): the coefficient of S(p_m) - S_0,
-// T_{m-1} w_up + T_m w_cur in double-float, and per voxel and slot the
-// boundary sums sum_d w_d T_L and w_d T_L I_bc; partial is then not
-// written (J comes from the replay).
-template <bool REC>
 __global__ void __launch_bounds__(kThreadsDF)
-k_fsdf(ViewDF p, float cut, unsigned long long* __restrict__ steps, Rec32 rec)
+k_fsdf(ViewDF p, float cut, unsigned long long* __restrict__ steps)
 {
     __shared__ dfl tab[2 * kExpTableDF];
     fill_exp_table_df(tab);
@@ -151,10 +144,8 @@ k_fsdf(ViewDF p, float cut, unsigned long long* __restrict__ steps, Rec32 rec)
     const int nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny;
     const int t = blockIdx.x * kThreadsDF + threadIdx.x;
     const int k0 = blockIdx.y, zb = blockIdx.z, ZB = gridDim.z;
-    const bool active = t < nxy;
-    const unsigned amask = REC ? __ballot_sync(0xffffffffu, active) : 0u;
     unsigned long long nsteps = 0;
-    if (active) {
+    if (t < nxy) {
         const int j0 = t / nx, i0 = t - j0 * nx;
         const long long v = (long long)k0 * nxy + t;
         const long long W = 2LL * nx, P = 4LL * nxy;
@@ -167,7 +158,7 @@ k_fsdf(ViewDF p, float cut, unsigned long long* __restrict__ steps, Rec32 rec)
         const float tcut = smax > 0.f ? cut * S0.h / (2.0f * smax) : 0.f;
         const float4* nb = p.node + base;
         for (int slot = zb; slot < kSlots; slot += ZB) {
-            double Jp = 0.0, tsum = 0.0, bcs = 0.0;
+            double Jp = 0.0;
             for (int d = slot; d < g.ndir; d += kSlots) {
                 const DirInfo di = p.info[d];
                 const int s = di.sgn;
@@ -176,8 +167,6 @@ k_fsdf(ViewDF p, float cut, unsigned long long* __restrict__ steps, Rec32 rec)
                 const float4* bd = p.bw + (long long)d * nz * 2;
                 const dfl hs = df_make(di.hs32, di.hs32lo);
                 dfl I = df_make(0.f, 0.f), T = df_make(1.f, 0.f), ca = chi0, da = df_make(0.f, 0.f);
-                float2* rc = REC ? rec.coef + rec_base(g, d, k0, s) + t : nullptr;
-                dfl cprev = df_make(0.f, 0.f);
                 bool early = false;
                 int m = 0;
                 for (; m < M; ++m) {
@@ -195,14 +184,6 @@ k_fsdf(ViewDF p, float cut, unsigned long long* __restrict__ steps, Rec32 rec)
                     const dfl x = df_mul(hs, df_add_s(ca, cb));
                     dfl wc, wu, e;
                     seg_weights_df(x, tab, wc, wu, e);
-                    if (REC) {
-                        const dfl twu = df_mul(T, wu);
-                        if (m > 0) {
-                            const dfl c = df_add_s(cprev, df_mul(T, wc));
-                            rc[(long long)(m - 1) * nxy] = make_float2(c.h, c.l);
-                        }
-                        cprev = twu;
-                    }
                     I = df_add_s(I, df_mul(T, df_add_s(df_mul(wc, da), df_mul(wu, db))));
                     T = df_mul(T, e);
                     ca = cb;
@@ -232,33 +213,107 @@ k_fsdf(ViewDF p, float cut, unsigned long long* __restrict__ steps, Rec32 rec)
                                                     g01.y, g11.x, g11.y);
                             ibc = df_add_s(ibc, df_mul(df_make(di.amu32, di.amu32lo), gr));
                         }
-                        if (REC) bcs = fma(di.w * df_to_double(T), df_to_double(ibc), bcs);
                         ibc = df_sub_s(ibc, S0);
                     } else {
                         ibc = df_neg(S0);
                     }
                     I = df_add_s(I, df_mul(T, ibc));
-                    if (REC) tsum = fma(di.w, df_to_double(T), tsum);
-                }
-                if (REC) {
-                    if (m > 0) rc[(long long)(m - 1) * nxy] = make_float2(cprev.h, cprev.l);
-                    const int Lw = __reduce_max_sync(amask, m);
-                    for (int q = m; q < Lw; ++q) rc[(long long)q * nxy] = make_float2(0.f, 0.f);
-                    if ((threadIdx.x & 31) == __ffs(amask) - 1)
-                        rec.lmax[((long long)d * nz + k0) * rec.nwp + (t >> 5)] = Lw;
                 }
                 nsteps += (unsigned long long)m;
                 Jp = fma(di.w, df_to_double(I), Jp);
             }
-            if (REC) {
-                rec.tsum[(long long)slot * g.N + v] = tsum;
-                rec.bc[(long long)slot * g.N + v] = bcs;
-            } else {
-                p.partial[(long long)slot * g.N + v] = Jp;
-            }
+            p.partial[(long long)slot * g.N + v] = Jp;
         }
     }
     if (steps) add_steps_df(steps, nsteps);
+}
+
+// The recording march (see k_rec64 in op.cu): over the given lengths, chi
+// alone; the coefficient of S(p_m) - S_0 is T_{m-1} w_up + T_m w_cur.
+__global__ void __launch_bounds__(kThreadsDF)
+k_recdf(ViewDF p, int r0, RecOut ro, const int* __restrict__ lmax, int nwp,
+        double* __restrict__ c0s, double* __restrict__ bcs, double* __restrict__ tss)
+{
+    __shared__ dfl tab[2 * kExpTableDF];
+    fill_exp_table_df(tab);
+    __syncthreads();
+    const Geometry& g = p.g;
+    const int nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny;
+    const int t = blockIdx.x * kThreadsDF + threadIdx.x;
+    const int k0 = plane_at(g, r0 + blockIdx.z), zb = blockIdx.y, ZB = gridDim.y;
+    if (t >= nxy) return;
+    const int j0 = t / nx, i0 = t - j0 * nx;
+    const long long v = (long long)k0 * nxy + t;
+    const long long W = 2LL * nx, P = 4LL * nxy;
+    const long long base = k0 * P + j0 * W + i0;
+    // the chi parts {chi_hi, chi_lo} of the node records
+    const float2* nb = reinterpret_cast<const float2*>(p.node + base);
+    const dfl chi0 = df_make(nb[0].x, nb[0].y);
+    float2* cbase = reinterpret_cast<float2*>(ro.base);
+    for (int slot = zb; slot < kSlots; slot += ZB) {
+        double tsum = 0.0, bsum = 0.0;
+        dfl C0 = df_make(0.f, 0.f);
+        for (int d = slot; d < g.ndir; d += kSlots) {
+            const DirInfo di = p.info[d];
+            const int s = di.sgn;
+            const int M = s > 0 ? k0 : nz - 1 - k0;
+            const int L = lmax[((long long)d * nz + k0) * nwp + (t >> 5)];
+            const int* od = p.poff + (long long)d * nz;
+            const float4* bd = p.bw + (long long)d * nz * 2;
+            const dfl hs = df_make(di.hs32, di.hs32lo);
+            float2* rc = rec_rows(g, ro, cbase, d, k0, s) + t;
+            dfl T = df_make(1.f, 0.f), ca = chi0, cprev = df_make(0.f, 0.f);
+            for (int m = 0; m < L; ++m) {
+                const int o = od[m + 1];
+                RT_GUARD(g, base + o, 4 * g.N, kSiteFsdf) break;
+                RT_GUARD(g, base + o + W + 1, 4 * g.N, kSiteFsdf) break;
+                const float4 wh = bd[2 * (m + 1)], wl = bd[2 * (m + 1) + 1];
+                const float2* q = nb + 2LL * o;           // float2 stride: two per node
+                const float2 q00 = __ldg(q), q10 = __ldg(q + 2);
+                const float2 q01 = __ldg(q + 2 * W), q11 = __ldg(q + 2 * W + 2);
+                const dfl cb = bilin_df(wh, wl, q00.x, q00.y, q10.x, q10.y, q01.x, q01.y, q11.x, q11.y);
+                const dfl x = df_mul(hs, df_add_s(ca, cb));
+                dfl wc, wu, e;
+                seg_weights_df(x, tab, wc, wu, e);
+                if (m == 0) {
+                    C0 = df_add_s(C0, df_mul(df_from_double(di.w), wc));
+                } else {
+                    const dfl c = df_add_s(cprev, df_mul(T, wc));
+                    rc[(long long)(m - 1) * nxy] = make_float2(c.h, c.l);
+                }
+                cprev = df_mul(T, wu);
+                T = df_mul(T, e);
+                ca = cb;
+            }
+            if (L > 0) rc[(long long)(L - 1) * nxy] = make_float2(cprev.h, cprev.l);
+            if (L == M) {
+                const double Td = df_to_double(T);
+                tsum = fma(di.w, Td, tsum);
+                const int bc = s > 0 ? g.top_bc : g.bottom_bc;
+                if (bc) {
+                    const StepGeo o = p.off[(long long)d * nz + M];
+                    const float4 wh = bd[2 * M], wl = bd[2 * M + 1];
+                    long long ip = (j0 + o.oy) * W + (i0 + o.ox);
+                    RT_GUARD(g, ip, P - W - 1, kSiteFsdf) ip = 0;   // record, read a safe node
+                    const float2* pb = p.b2 + (s > 0 ? 0LL : P) + ip;
+                    const float2 c00 = pb[0], c10 = pb[1], c01 = pb[W], c11 = pb[W + 1];
+                    dfl ibc = bilin_df(wh, wl, c00.x, c00.y, c10.x, c10.y, c01.x, c01.y, c11.x, c11.y);
+                    if (bc == 2) {   // + |mu| dB/dtau (LTE diffusion)
+                        const float2* pg = p.g2df + ip;
+                        const float2 g00 = pg[0], g10 = pg[1], g01 = pg[W], g11 = pg[W + 1];
+                        const dfl gr = bilin_df(wh, wl, g00.x, g00.y, g10.x, g10.y, g01.x, g01.y,
+                                                g11.x, g11.y);
+                        ibc = df_add_s(ibc, df_mul(df_make(di.amu32, di.amu32lo), gr));
+                    }
+                    bsum = fma(di.w * Td, df_to_double(ibc), bsum);
+                }
+            }
+        }
+        const long long e = (long long)slot * g.N + v;
+        tss[e] = tsum;
+        bcs[e] = bsum;
+        if (c0s) c0s[e] = df_to_double(C0);
+    }
 }
 
 // Replay of the recorded double-float march for the source in p.node (its
@@ -621,16 +676,22 @@ cudaError_t launch_grad_df(const Geometry& g, const double* G, float2* out, cuda
 }
 
 cudaError_t launch_fsdf(const ViewDF& p, double cut, int groups, unsigned long long* steps,
-                        cudaStream_t st, const Rec32* rec)
+                        cudaStream_t st)
 {
     const int nxy = p.g.nx * p.g.ny;
     // planes in index order (g.zorder unused): 40.9 ms against 41.05 ms
     // with the order table on the 65^3 slab
     dim3 grid((nxy + kThreadsDF - 1) / kThreadsDF, p.g.nz, groups);
-    if (rec)
-        k_fsdf<true><<<grid, kThreadsDF, 0, st>>>(p, (float)cut, steps, *rec);
-    else
-        k_fsdf<false><<<grid, kThreadsDF, 0, st>>>(p, (float)cut, steps, Rec32{});
+    k_fsdf<<<grid, kThreadsDF, 0, st>>>(p, (float)cut, steps);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_recdf(const ViewDF& p, int r0, int nplanes, const RecOut& ro, const int* lmax,
+                         int nwp, int groups, double* c0s, double* bcs, double* tss, cudaStream_t st)
+{
+    const int nxy = p.g.nx * p.g.ny;
+    const dim3 grid((nxy + kThreadsDF - 1) / kThreadsDF, groups, nplanes);
+    k_recdf<<<grid, kThreadsDF, 0, st>>>(p, r0, ro, lmax, nwp, c0s, bcs, tss);
     return cudaGetLastError();
 }
 

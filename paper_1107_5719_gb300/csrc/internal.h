@@ -208,7 +208,8 @@ struct OpLists {
     OpContrib* contrib; // [2 nz][icap]
     int* lpos;          // [2][2][9] positions of the 3x3 nearest nodes of slots 0, 1 (-1: none)
 };
-// The operator: entries eb[k0] .. eb[k0] + E[k0] - 1 of plane k0, coefficient
+// The operator (double-float: each coefficient a pair of floats, of S(e) -
+// S_v): entries eb[k0] .. eb[k0] + E[k0] - 1 of plane k0, coefficient
 // of entry e for voxel t of the plane at
 //   A[eb[k0] nwp 32 + ((t/32) E[k0]/2 + e/2) 64 + (t%32) 2 + e%2],
 // its node at off[eb[k0] + e] from the voxel in planes padded to 2ny x 2nx.
@@ -219,6 +220,7 @@ struct OpMap {
     const long long* eb;    // [nz]
     const double* c0;       // [N] coefficient of the voxel's own S
     const double* bc;       // [N] boundary term
+    const double* ts;       // [N] double-float: sum_d w_d T_L of the rays that reach the boundary
     const unsigned long long* steps;    // voxel-steps it stands for
     int nwp;                // 32-voxel tiles per plane
 };
@@ -249,10 +251,11 @@ cudaError_t launch_op_lists(const Geometry& g, const DirInfo* info, const StepGe
                             cudaStream_t st);
 // Ray lengths: lmax as FsRec, Lp[nz][ndir] the longest of each plane, *steps
 // the voxel-steps; node: 4N scratch, poff: launch_pad_offsets with 2ny rows;
-// extra_bits: margin in the cutoff besides cut.
+// extra_bits: margin in the cutoff besides cut; own: the cutoff is relative to
+// the voxel's own source (double-float), not to its intensity.
 cudaError_t launch_op_lengths(const Geometry& g, const double* chi, const double* S,
                               const double* smax, const DirInfo* info, const int* poff,
-                              const float4* bw32, double cut, int extra_bits, int groups,
+                              const float4* bw32, double cut, int extra_bits, bool own, int groups,
                               float2* node, int* lmax, int nwp, int* Lp, unsigned long long* steps,
                               cudaStream_t st);
 // cnt, segb [nz][2 nz]: entries per (plane, list) and the first of them;
@@ -271,16 +274,20 @@ cudaError_t launch_rec64p(const Geometry& g, int r0, int nplanes, const double* 
                           const double* G, const DirInfo* info, const StepGeo* off, const Bw4d* bw,
                           const Bw4d* bwh, const DownGeo* dn, const RecOut& ro, const int* lmax,
                           int nwp, int groups, double* c0s, double* bcs, cudaStream_t st);
-cudaError_t launch_op_assemble(const Geometry& g, int r0, int nplanes, const OpLists& L,
+cudaError_t launch_op_assemble(const Geometry& g, bool df, int r0, int nplanes, const OpLists& L,
                                const RecOut& ro, const int* lmax, const int* cnt, const int* segb,
                                const OpMap& op, cudaStream_t st);
-cudaError_t launch_op_own(long long N, const double* c0s, const double* bcs, double* c0, double* bc,
-                          cudaStream_t st);
+// The voxels' own terms from the slots' (tss: null for FP64).
+cudaError_t launch_op_own(long long N, const double* c0s, const double* bcs, const double* tss,
+                          const OpMap& op, cudaStream_t st);
 // J of source S; sp: 4N scratch doubles (S padded).
 cudaError_t launch_op_apply64(const Geometry& g, const double* S, double* sp, const OpMap& op,
                               double* J, unsigned long long* steps, cudaStream_t st);
-cudaError_t launch_op_lstar(const Geometry& g, const OpLists& L, const OpMap& op, const int* cnt,
-                            const int* segb, double* lstar, cudaStream_t st);
+// The same in double-float: J = wsum S + sum_e A_e (S(e) - S) + bc - S ts.
+cudaError_t launch_op_apply_df(const Geometry& g, const double* S, double* sp, const OpMap& op,
+                               double wsum, double* J, unsigned long long* steps, cudaStream_t st);
+cudaError_t launch_op_lstar(const Geometry& g, bool df, const OpLists& L, const OpMap& op,
+                            const int* cnt, const int* segb, double* lstar, cudaStream_t st);
 
 // ---- short characteristics (sc.cu) -----------------------------------------
 // Directions per march launch (the [directions][N] partial buffer holds
@@ -450,11 +457,18 @@ cudaError_t launch_packdf(const Geometry& g, const double* chi, const double* S,
                           cudaStream_t st);
 cudaError_t launch_bw_df(long long n, const Bw4d* bw, float4* out, cudaStream_t st);
 cudaError_t launch_grad_df(const Geometry& g, const double* G, float2* out, cudaStream_t st);
-// rec != null: also record the march (Rec32 in the layout of rec_base, one
-// double-float pair per entry; lmax, tsum, bc as for the FP32 sweep).
 cudaError_t launch_fsdf(const ViewDF& p, double cut, int groups, unsigned long long* steps,
-                        cudaStream_t st, const Rec32* rec = nullptr);
-// The recorded double-float march for the source in p.node.
+                        cudaStream_t st);
+// Recording march of the planes of rank r0 .. r0 + nplanes - 1 (planes of
+// p.g.zorder): double-float coefficients of S(p_m) - S_0 into ro (its base
+// holding float2), per voxel and slot sum_d w_d w_cur,0 (c0s; null: not
+// wanted), w_d T_L (tss) and w_d T_L I_bc (bcs) of the rays that reach the
+// boundary.
+cudaError_t launch_recdf(const ViewDF& p, int r0, int nplanes, const RecOut& ro, const int* lmax,
+                         int nwp, int groups, double* c0s, double* bcs, double* tss, cudaStream_t st);
+// The march recorded ray by ray (Rec32 in the layout of rec_base, one
+// double-float pair per entry, where the operator does not fit) for the
+// source in p.node.
 cudaError_t launch_fsdfrep(const ViewDF& p, const Rec32& rec, int groups,
                            unsigned long long* steps, cudaStream_t st);
 

@@ -25,6 +25,7 @@
 //   k_rec64      the march's coefficients c_m of S(p_m) of one chunk of planes
 //   k_op_assemble  A[e][v] = sum over e's contributions of w_d b c_m
 // and k_op_apply64 evaluates J for a source.
+#include "df.cuh"
 #include "internal.h"
 #include "weights.cuh"
 
@@ -194,10 +195,12 @@ __global__ void k_op_pack_len(Geometry g, const double* __restrict__ chi,
     }
 }
 
-// Lengths of the rays: the march in FP32, a ray ending once the rest of it
+// Lengths of the rays, from a march in FP32.  A ray ends once the rest of it
 // can change I by less than 2^-lcut |I|, i.e. T smax <= 2^-lcut |I| (tested
-// on logarithms: tau log2 e + log2(|I| / smax) >= lcut).  The 32 lanes of a
-// warp share the longest of their rays.
+// on logarithms: tau log2 e + log2(|I| / smax) >= lcut); OWN (double-float):
+// by less than 2^-lcut of the voxel's own source, which takes no intensity.
+// The 32 lanes of a warp share the longest of their rays.
+template <bool OWN>
 __global__ void __launch_bounds__(kOpThreads)
 k_op_len(Geometry g, const float2* __restrict__ node, const DirInfo* __restrict__ info,
          const int* __restrict__ poff, const float4* __restrict__ bw, float lcut,
@@ -215,6 +218,8 @@ k_op_len(Geometry g, const float2* __restrict__ node, const DirInfo* __restrict_
     const long long base = k0 * P + j0 * W + i0;
     const float2 me = node[base];
     const float2* nb = node + base;
+    float own;      // NaN for S < 0, -inf for S = 0: never cut
+    asm("lg2.approx.f32 %0, %1;" : "=f"(own) : "f"(me.y));
     for (int d = blockIdx.y; d < g.ndir; d += gridDim.y) {
         const int s = info[d].sgn;
         const float hs = info[d].hs32;
@@ -231,18 +236,20 @@ k_op_len(Geometry g, const float2* __restrict__ node, const DirInfo* __restrict_
             const float2* q = nb + o;
             const float2 q00 = __ldg(q), q10 = __ldg(q + 1), q01 = __ldg(q + W), q11 = __ldg(q + W + 1);
             const float cb = b.x * q00.x + b.y * q10.x + b.z * q01.x + b.w * q11.x;
-            const float sb = b.x * q00.y + b.y * q10.y + b.z * q01.y + b.w * q11.y;
             const float x = hs * (ca + cb);
-            float wc, wu, e;
-            seg_weights32(x, wc, wu, e);
-            I = fmaf(T, fmaf(wc, sa, wu * sb), I);
+            float lg = own;
+            if (!OWN) {
+                const float sb = b.x * q00.y + b.y * q10.y + b.z * q01.y + b.w * q11.y;
+                float wc, wu, e;
+                seg_weights32(x, wc, wu, e);
+                I = fmaf(T, fmaf(wc, sa, wu * sb), I);
+                sa = sb;
+                asm("lg2.approx.f32 %0, %1;" : "=f"(lg) : "f"(fabsf(I)));
+            }
             tau += x;
-            T = ex2_approx(-tau * kLog2e);
+            if (!OWN) T = ex2_approx(-tau * kLog2e);
             ca = cb;
-            sa = sb;
             ++m;
-            float lg;
-            asm("lg2.approx.f32 %0, %1;" : "=f"(lg) : "f"(fabsf(I)));
             if (fmaf(tau, kLog2e, lg) >= lcut) break;
         }
         const int Lw = __reduce_max_sync(amask, m);
@@ -437,11 +444,46 @@ k_rec64(Geometry g, int r0, const double* __restrict__ chi, const double* __rest
 // last contribution is in.  Rows past the warp's own rays hold nothing
 // (m > its length) and count as zero.
 constexpr int kAsmRun = 16;      // entries of a run (even)
+
+// The two arithmetics of the coefficients: FP64, or double-float pairs.
+struct AsmF64 {
+    using V = double;
+    using Pair = double2;
+    static __device__ __forceinline__ V zero() { return 0.0; }
+    static __device__ __forceinline__ V weight(double w) { return w; }
+    static __device__ __forceinline__ V shfl(V w, int i) { return __shfl_sync(0xffffffffu, w, i); }
+    static __device__ __forceinline__ V fma(V w, V c, V a) { return ::fma(w, c, a); }
+    static __device__ __forceinline__ Pair pair(V a, V b) { return make_double2(a, b); }
+};
+struct AsmDF {
+    using V = float2;
+    using Pair = float4;
+    static __device__ __forceinline__ V zero() { return make_float2(0.f, 0.f); }
+    static __device__ __forceinline__ V weight(double w)
+    {
+        const dfl q = df_from_double(w);
+        return make_float2(q.h, q.l);
+    }
+    static __device__ __forceinline__ V shfl(V w, int i)
+    {
+        return make_float2(__shfl_sync(0xffffffffu, w.x, i), __shfl_sync(0xffffffffu, w.y, i));
+    }
+    static __device__ __forceinline__ V fma(V w, V c, V a)
+    {
+        const dfl r = df_add_s(df_make(a.x, a.y), df_mul(df_make(w.x, w.y), df_make(c.x, c.y)));
+        return make_float2(r.h, r.l);
+    }
+    static __device__ __forceinline__ Pair pair(V a, V b) { return make_float4(a.x, a.y, b.x, b.y); }
+};
+
+template <typename T>
 __global__ void __launch_bounds__(kListThreads)
 k_op_assemble(Geometry g, int r0, OpLists L, RecOut ro, const int* __restrict__ lmax, int nwp,
               const int* __restrict__ cnt, const int* __restrict__ segb, const int* __restrict__ E,
-              const long long* __restrict__ eb, double* __restrict__ A)
+              const long long* __restrict__ eb, typename T::V* __restrict__ A)
 {
+    using V = typename T::V;
+    using Pair = typename T::Pair;
     extern __shared__ int2 lr[];     // [ndir] {length, first row}
     const int nz = g.nz, nxy = g.nx * g.ny;
     const int k0 = plane_at(g, r0 + blockIdx.y), tile = blockIdx.x;
@@ -452,73 +494,81 @@ k_op_assemble(Geometry g, int r0, OpLists L, RecOut ro, const int* __restrict__ 
         lr[d] = make_int2(lmax[((long long)d * nz + k0) * nwp + tile],
                           ro.rowbase[(long long)k0 * g.ndir + d]);
     __syncthreads();
-    const double* c = ro.base + ro.prow[k0] * nxy + (live ? t : 0);
-    double2* out = reinterpret_cast<double2*>(A + eb[k0] * (long long)nwp * 32) +
-                   (long long)tile * (E[k0] / 2) * 32 + lane;
+    const V* c = reinterpret_cast<const V*>(ro.base) + ro.prow[k0] * nxy + (live ? t : 0);
+    Pair* out = reinterpret_cast<Pair*>(A + eb[k0] * (long long)nwp * 32) +
+                (long long)tile * (E[k0] / 2) * 32 + lane;
     int run = wid;                   // runs go round the warps, across the lists
     for (int q = blockIdx.z; q < 2 * nz; q += gridDim.z) {
         const int n = cnt[(long long)k0 * 2 * nz + q];
         if (n == 0) continue;
         const int m = q < nz ? q : q - nz;
-        double2* oq = out + (long long)(segb[(long long)k0 * 2 * nz + q] / 2) * 32;
+        Pair* oq = out + (long long)(segb[(long long)k0 * 2 * nz + q] / 2) * 32;
         const int* us = L.ustart + (long long)q * (L.ucap + 1);
         const OpContrib* ct = L.contrib + (long long)q * L.icap;
         const int runs = (n + kAsmRun - 1) / kAsmRun;
         for (; run < runs; run += nw) {
             const int js = us[run * kAsmRun], je = us[min(n, (run + 1) * kAsmRun)];
-            double acc = 0.0, even = 0.0;
+            V acc = T::zero(), even = T::zero();
             for (int jb = js; jb < je; jb += 32) {
-                OpContrib k{0.0, 0, 0};
-                int row = -1;
+                V wb = T::zero();
+                int row = -1, ul0 = 0;
                 if (jb + lane < je) {
-                    k = ct[jb + lane];
+                    const OpContrib k = ct[jb + lane];
                     const int2 p = lr[k.d];
                     if (m <= p.x || m == 0) row = p.y + m - 1 + ro.para;
+                    wb = T::weight(k.wb);
+                    ul0 = k.ul;
                 }
                 const int nj = min(32, je - jb);
                 for (int i = 0; i < nj; i += 8) {
-                    double cv[8];
+                    V cv[8];
 #pragma unroll
                     for (int h = 0; h < 8; ++h) {
                         const int r = __shfl_sync(0xffffffffu, row, i + h);
-                        cv[h] = r >= 0 ? __ldg(c + (long long)r * nxy) : 0.0;
+                        cv[h] = r >= 0 ? __ldg(c + (long long)r * nxy) : T::zero();
                     }
 #pragma unroll
                     for (int h = 0; h < 8; ++h) {
-                        acc = fma(__shfl_sync(0xffffffffu, k.wb, i + h), cv[h], acc);
-                        const int ul = __shfl_sync(0xffffffffu, k.ul, i + h);
+                        acc = T::fma(T::shfl(wb, i + h), cv[h], acc);
+                        const int ul = __shfl_sync(0xffffffffu, ul0, i + h);
                         if (ul & 1) {       // entry ul >> 1 is complete
-                            if (!live) acc = 0.0;
-                            if (ul & 2) oq[(long long)(ul >> 2) * 32] = make_double2(even, acc);
+                            if (!live) acc = T::zero();
+                            if (ul & 2) oq[(long long)(ul >> 2) * 32] = T::pair(even, acc);
                             else even = acc;
-                            acc = 0.0;
+                            acc = T::zero();
                         }
                     }
                 }
             }
-            if ((n & 1) && (run + 1) * kAsmRun >= n) oq[(long long)(n >> 1) * 32] = make_double2(even, 0.0);
+            if ((n & 1) && (run + 1) * kAsmRun >= n)
+                oq[(long long)(n >> 1) * 32] = T::pair(even, T::zero());
         }
         run -= runs;
     }
     if (blockIdx.z) return;
     const int qz = 2 * nz - 1;
     const int tail = (segb[(long long)k0 * 2 * nz + qz] + cnt[(long long)k0 * 2 * nz + qz] + 1) / 2;
-    for (int p = tail + wid; p < E[k0] / 2; p += nw) out[(long long)p * 32] = make_double2(0.0, 0.0);
+    for (int p = tail + wid; p < E[k0] / 2; p += nw)
+        out[(long long)p * 32] = T::pair(T::zero(), T::zero());
 }
 
-// c0[v] = sum over slots of c0s, bc[v] likewise (slot order fixed)
+// c0[v] = sum over slots of c0s; bc[v] and ts[v] (when given) likewise (slot
+// order fixed)
 __global__ void k_op_own(long long N, const double* __restrict__ c0s, const double* __restrict__ bcs,
-                         double* __restrict__ c0, double* __restrict__ bc)
+                         const double* __restrict__ tss, double* __restrict__ c0,
+                         double* __restrict__ bc, double* __restrict__ ts)
 {
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < N;
          v += (long long)gridDim.x * blockDim.x) {
-        double a = 0.0, b = 0.0;
+        double a = 0.0, b = 0.0, c = 0.0;
         for (int q = 0; q < kSlots; ++q) {
             a += c0s[q * N + v];
             b += bcs[q * N + v];
+            if (tss) c += tss[q * N + v];
         }
         c0[v] = a;
         bc[v] = b;
+        if (tss) ts[v] = c;
     }
 }
 
@@ -607,9 +657,105 @@ k_op_apply64(Geometry g, const double* __restrict__ S, const double* __restrict_
     if (steps && tile == 0 && blockIdx.y == 0 && threadIdx.x == 0) atomicAdd(steps, *op.steps);
 }
 
+// S as double-float pairs in the padded planes of k_op_pack.
+__global__ void k_op_pack_df(Geometry g, const double* __restrict__ S, float2* __restrict__ sp)
+{
+    const int nx = g.nx, ny = g.ny;
+    const long long W = 2LL * nx, P = 4LL * nx * ny;
+    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < g.N;
+         v += (long long)gridDim.x * blockDim.x) {
+        const int i = (int)(v % nx), j = (int)((v / nx) % ny);
+        const long long k = v / ((long long)nx * ny);
+        const dfl q = df_from_double(S[v]);
+        const float2 s = make_float2(q.h, q.l);
+        float2* p = sp + k * P + (long long)j * W + i;
+        p[0] = s;
+        p[nx] = s;
+        p[(long long)ny * W] = s;
+        p[(long long)ny * W + nx] = s;
+    }
+}
+
+// h + l += (ah + al) ((sh + sl) - (s0h + s0l)): the difference of the high
+// parts exact (TwoSum), the product's leading term split exactly, the sum of
+// the leading parts exact (TwoSum); everything below goes to l.  h and l are
+// not renormalised: l stays a sum of terms below 2^-23 of those in h.
+__device__ __forceinline__ void diff_add_df(float& h, float& l, float ah, float al, float2 s,
+                                            float s0h, float s0l)
+{
+    const dfl d = two_sum(s.x, -s0h);
+    const float dl = d.l + (s.y - s0l);
+    dfl p = two_prod(ah, d.h);
+    p.l = fmaf(ah, dl, fmaf(al, d.h, p.l));
+    const dfl t = two_sum(h, p.h);
+    h = t.h;
+    l += t.l + p.l;
+}
+
+// J of a source in double-float, as k_op_apply64 with the recording's
+// difference form: J = sum_e A_e (S_e - S_0) + bc + (wsum - ts) S_0.  22
+// FP32 operations and 8 coefficient bytes per entry: bound by memory.
+template <int NW>
+__global__ void __launch_bounds__(NW * 32, NW < 24 ? 32 / NW : 1)
+k_op_apply_df(Geometry g, const double* __restrict__ S, const float2* __restrict__ sp, OpMap op,
+              double wsum, double* __restrict__ J, unsigned long long* __restrict__ steps)
+{
+    __shared__ double red[NW][32];
+    const int nx = g.nx, nxy = nx * g.ny;
+    const int tile = blockIdx.x, k0 = plane_at(g, blockIdx.y);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int t = tile * 32 + lane, tc = t < nxy ? t : 0;
+    const int j0 = tc / nx, i0 = tc - j0 * nx;
+    const long long at = (long long)k0 * 4 * nxy + (long long)j0 * 2 * nx + i0;
+    const float2* s = sp + at;
+    const float2 s0 = s[0];
+    const int E = op.E[k0];
+    const long long eb = op.eb[k0];
+    const float4* A = reinterpret_cast<const float4*>(op.A + eb * op.nwp * 32) +
+                      (long long)tile * (E / 2) * 32 + lane;
+    const int4* off = reinterpret_cast<const int4*>(op.off + eb);
+    float h0 = 0.f, l0 = 0.f, h1 = 0.f, l1 = 0.f;
+    constexpr int kQ = 2;       // quads of entries in flight per warp
+    const int nq = E / 4;
+    auto quad = [&](int4 o, float4 a, float4 b) {
+        RT_GUARD(g, at + min(min(o.x, o.y), min(o.z, o.w)), 4 * g.N, kSiteFsdf) return;
+        RT_GUARD(g, at + max(max(o.x, o.y), max(o.z, o.w)), 4 * g.N, kSiteFsdf) return;
+        const float2 p0 = __ldg(s + o.x), p1 = __ldg(s + o.y), p2 = __ldg(s + o.z), p3 = __ldg(s + o.w);
+        diff_add_df(h0, l0, a.x, a.y, p0, s0.x, s0.y);
+        diff_add_df(h1, l1, a.z, a.w, p1, s0.x, s0.y);
+        diff_add_df(h0, l0, b.x, b.y, p2, s0.x, s0.y);
+        diff_add_df(h1, l1, b.z, b.w, p3, s0.x, s0.y);
+    };
+    int q = wid;
+    for (; q + (kQ - 1) * NW < nq; q += kQ * NW) {
+        int4 o[kQ];
+        float4 a[kQ], b[kQ];
+#pragma unroll
+        for (int i = 0; i < kQ; ++i) {
+            o[i] = __ldg(off + q + i * NW);
+            a[i] = __ldcs(A + (long long)(q + i * NW) * 64);
+            b[i] = __ldcs(A + (long long)(q + i * NW) * 64 + 32);
+        }
+#pragma unroll
+        for (int i = 0; i < kQ; ++i) quad(o[i], a[i], b[i]);
+    }
+    for (; q < nq; q += NW)
+        quad(__ldg(off + q), __ldcs(A + (long long)q * 64), __ldcs(A + (long long)q * 64 + 32));
+    red[wid][lane] = ((double)h0 + (double)l0) + ((double)h1 + (double)l1);
+    __syncthreads();
+    if (wid == 0 && t < nxy) {
+        const long long v = (long long)k0 * nxy + t;
+        double a = op.bc[v];
+        for (int w = 0; w < NW; ++w) a += red[w][lane];
+        J[v] = fma(wsum - op.ts[v], S[v], a);
+    }
+    if (steps && tile == 0 && blockIdx.y == 0 && threadIdx.x == 0) atomicAdd(steps, *op.steps);
+}
+
 // Lambda* from the operator: the voxel's own coefficient and those of the
 // nearest nodes of the neighbouring planes (distance 1 upstream; for the
 // parabolic source also the downstream point).
+template <bool DF>
 __global__ void k_op_lstar(Geometry g, OpLists L, OpMap op, const int* __restrict__ cnt,
                            const int* __restrict__ segb, double* __restrict__ lstar)
 {
@@ -631,7 +777,13 @@ __global__ void k_op_lstar(Geometry g, OpLists L, OpMap op, const int* __restric
             const long long q = (long long)k0 * 2 * nz + (long long)si * nz + m;
             if (u < 0 || u >= cnt[q]) continue;
             const int e = segb[q] + u;
-            r += A[((long long)(e >> 1) * 32 + (t & 31)) * 2 + (e & 1)];
+            const double* a = A + ((long long)(e >> 1) * 32 + (t & 31)) * 2 + (e & 1);
+            if (DF) {
+                const float2 p = *reinterpret_cast<const float2*>(a);
+                r += (double)p.x + (double)p.y;
+            } else {
+                r += *a;
+            }
         }
     }
     lstar[(long long)o * g.N + v] = r;
@@ -672,7 +824,7 @@ cudaError_t launch_op_lists(const Geometry& g, const DirInfo* info, const StepGe
 
 cudaError_t launch_op_lengths(const Geometry& g, const double* chi, const double* S,
                               const double* smax, const DirInfo* info, const int* poff,
-                              const float4* bw32, double cut, int extra_bits, int groups,
+                              const float4* bw32, double cut, int extra_bits, bool own, int groups,
                               float2* node, int* lmax, int nwp, int* Lp, unsigned long long* steps,
                               cudaStream_t st)
 {
@@ -680,7 +832,10 @@ cudaError_t launch_op_lengths(const Geometry& g, const double* chi, const double
     // two bits beyond the cutoff cover the FP32 rounding of tau and I
     const float lcut = cut > 0.0 ? (float)(-log2(cut)) + 2.0f + (float)extra_bits : INFINITY;
     const dim3 grid((g.nx * g.ny + kOpThreads - 1) / kOpThreads, groups, g.nz);
-    k_op_len<<<grid, kOpThreads, 0, st>>>(g, node, info, poff, bw32, lcut, lmax, nwp);
+    if (own)
+        k_op_len<true><<<grid, kOpThreads, 0, st>>>(g, node, info, poff, bw32, lcut, lmax, nwp);
+    else
+        k_op_len<false><<<grid, kOpThreads, 0, st>>>(g, node, info, poff, bw32, lcut, lmax, nwp);
     cudaError_t e = cudaMemsetAsync(steps, 0, sizeof(unsigned long long), st);
     if (e != cudaSuccess) return e;
     k_op_plane_len<<<dim3((g.ndir + 7) / 8, g.nz), 256, 0, st>>>(g, lmax, nwp, Lp, steps);
@@ -713,47 +868,77 @@ cudaError_t launch_rec64(const Geometry& g, int r0, int nplanes, const double* c
     return cudaGetLastError();
 }
 
-cudaError_t launch_op_assemble(const Geometry& g, int r0, int nplanes, const OpLists& L,
+cudaError_t launch_op_assemble(const Geometry& g, bool df, int r0, int nplanes, const OpLists& L,
                                const RecOut& ro, const int* lmax, const int* cnt, const int* segb,
                                const OpMap& op, cudaStream_t st)
 {
     const size_t shm = sizeof(int2) * (size_t)g.ndir;
     if (shm > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k_op_assemble, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)shm);
+        cudaError_t e = df ? cudaFuncSetAttribute(k_op_assemble<AsmDF>,
+                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm)
+                           : cudaFuncSetAttribute(k_op_assemble<AsmF64>,
+                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
         if (e != cudaSuccess) return e;
     }
-    // few tiles: several blocks share a tile's lists, so that every SM has work
+    // few tiles: several blocks share a tile's lists, so that every SM has
+    // work (17^3 with 256 directions: 93 against 258 us)
     int split = 1;
     while (split < 8 && (long long)op.nwp * nplanes * split < 152 * 8) split *= 2;
-    k_op_assemble<<<dim3(op.nwp, nplanes, split), kListThreads, shm, st>>>(
-        g, r0, L, ro, lmax, op.nwp, cnt, segb, op.E, op.eb, const_cast<double*>(op.A));
+    const dim3 grid(op.nwp, nplanes, split);
+    double* A = const_cast<double*>(op.A);
+    if (df)
+        k_op_assemble<AsmDF><<<grid, kListThreads, shm, st>>>(g, r0, L, ro, lmax, op.nwp, cnt, segb, op.E,
+                                                              op.eb, reinterpret_cast<float2*>(A));
+    else
+        k_op_assemble<AsmF64><<<grid, kListThreads, shm, st>>>(g, r0, L, ro, lmax, op.nwp, cnt, segb,
+                                                               op.E, op.eb, A);
     return cudaGetLastError();
 }
 
-cudaError_t launch_op_own(long long N, const double* c0s, const double* bcs, double* c0, double* bc,
-                          cudaStream_t st)
+cudaError_t launch_op_own(long long N, const double* c0s, const double* bcs, const double* tss,
+                          const OpMap& op, cudaStream_t st)
 {
-    k_op_own<<<op_grid1d(N, 256), 256, 0, st>>>(N, c0s, bcs, c0, bc);
+    k_op_own<<<op_grid1d(N, 256), 256, 0, st>>>(N, c0s, bcs, tss, const_cast<double*>(op.c0),
+                                                const_cast<double*>(op.bc), const_cast<double*>(op.ts));
     return cudaGetLastError();
 }
+
+// Below this many tiles 16 warps share one (17^3: 28 against 79 us)
+constexpr long long kFewTiles = 152 * 3;
 
 cudaError_t launch_op_apply64(const Geometry& g, const double* S, double* sp, const OpMap& op,
                               double* J, unsigned long long* steps, cudaStream_t st)
 {
     k_op_pack<<<op_grid1d(g.N, 256), 256, 0, st>>>(g, S, sp);
     const dim3 grid(op.nwp, g.nz);
-    if ((long long)op.nwp * g.nz < 152 * 3)
+    if ((long long)op.nwp * g.nz < kFewTiles)
         k_op_apply64<16><<<grid, 512, 0, st>>>(g, S, sp, op, J, steps);
     else
         k_op_apply64<8><<<grid, 256, 0, st>>>(g, S, sp, op, J, steps);
     return cudaGetLastError();
 }
 
-cudaError_t launch_op_lstar(const Geometry& g, const OpLists& L, const OpMap& op, const int* cnt,
-                            const int* segb, double* lstar, cudaStream_t st)
+cudaError_t launch_op_apply_df(const Geometry& g, const double* S, double* sp, const OpMap& op,
+                               double wsum, double* J, unsigned long long* steps, cudaStream_t st)
 {
-    k_op_lstar<<<dim3((g.nx * g.ny + 127) / 128, g.nz, 27), 128, 0, st>>>(g, L, op, cnt, segb, lstar);
+    float2* p = reinterpret_cast<float2*>(sp);
+    k_op_pack_df<<<op_grid1d(g.N, 256), 256, 0, st>>>(g, S, p);
+    const dim3 grid(op.nwp, g.nz);
+    if ((long long)op.nwp * g.nz < kFewTiles)
+        k_op_apply_df<16><<<grid, 512, 0, st>>>(g, S, p, op, wsum, J, steps);
+    else
+        k_op_apply_df<8><<<grid, 256, 0, st>>>(g, S, p, op, wsum, J, steps);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_op_lstar(const Geometry& g, bool df, const OpLists& L, const OpMap& op,
+                            const int* cnt, const int* segb, double* lstar, cudaStream_t st)
+{
+    const dim3 grid((g.nx * g.ny + 127) / 128, g.nz, 27);
+    if (df)
+        k_op_lstar<true><<<grid, 128, 0, st>>>(g, L, op, cnt, segb, lstar);
+    else
+        k_op_lstar<false><<<grid, 128, 0, st>>>(g, L, op, cnt, segb, lstar);
     return cudaGetLastError();
 }
 
