@@ -165,10 +165,10 @@ k_fs64(Geometry g, const double* __restrict__ chi, const double* __restrict__ S,
                     RT_GUARD(g, pb + nodes_max(n), g.N, kSiteFs64) { early = true; break; }
                     const double cb = bilin(chi + pb, n, bh[m + 1]);
                     const double sb = bilin(S + pb, n, bd[m + 1]);
-                    double wc, wu, e;
-                    seg_weights64(ca + cb, tab, wc, wu, e);
-                    I = fma(T, fma(wc, sa, wu * sb), I);
-                    T *= e;
+                    double b, gu, Tn;
+                    seg_step64(T, ca + cb, tab, b, gu, Tn);
+                    I = fma(gu, sb, fma(b, sa, I));
+                    T = Tn;
                     ca = cb;
                     sa = sb;
                     if (cut_now(T, I, need)) {

@@ -71,30 +71,69 @@ __device__ __forceinline__ void exp_neg_df(dfl x, const dfl* __restrict__ tab, d
     om = df_sub_s(c, tp);
 }
 
-// Segment weights in double-float (same definitions as weights.cuh).
-__device__ __forceinline__ void seg_weights_df(dfl x, const dfl* __restrict__ tab, dfl& wc, dfl& wu,
-                                               dfl& e)
+// c - x r, |x r| < |c|, r and the result unnormalised pairs (the low part a
+// few units of 2^-24 of the high one)
+__device__ __forceinline__ dfl horner_df(dfl x, dfl r, float ch, float cl)
 {
-    if (x.h < 0.05f) {
-        // phi2 series: E = 1/2 + z/24 + z^2/720 + ..., O = x (1/6 + z/120 + z^2/5040 + ...);
-        // from z^2 on the terms are below 9e-9 and are summed in FP32.
-        const dfl z = df_mul(x, x);
-        const float zf = z.h;
-        const float rE = zf * zf * fmaf(zf, fmaf(zf, 1.0f / 3628800.0f, 1.0f / 40320.0f), 1.0f / 720.0f);
-        const float rO = zf * zf * fmaf(zf, 1.0f / 362880.0f, 1.0f / 5040.0f);
-        const dfl c24 = df_make(0.0416666679084301f, -1.2417634698280722e-09f);    // 1/24
-        const dfl c120 = df_make(0.008333333767950535f, -4.34617203337595e-10f);   // 1/120
-        const dfl c6 = df_make(0.1666666716337204f, -4.967053879312289e-09f);      // 1/6
-        dfl E = df_add_f(df_mul(z, c24), rE);
-        E = df_add_f(E, 0.5f);
-        dfl Op = df_add_f(df_mul(z, c120), rO);
-        Op = df_add_s(c6, Op);
-        const dfl O = df_mul(x, Op);
-        wc = df_mul(x, df_add_s(E, df_neg(O)));
-        e = df_add_s(df_add_f(df_neg(x), 1.0f), df_mul(x, wc));
-        wu = df_mul(df_mul(x, e), df_add_s(E, O));
+    const dfl p = two_prod(x.h, r.h);
+    const float pl = fmaf(x.l, r.h, fmaf(x.h, r.l, p.l));
+    const float s = ch - p.h;
+    return dfl{s, ((ch - s) - p.h) + (cl - pl)};
+}
+
+// phi2(-x) = sum_k (-x)^k/(k+2)!, x < 1/2, by Horner; the terms below 2^-28 of
+// the sum in FP32 (their rounding is below 2^-52): from k = 3, 4 or 8 on.
+__device__ __forceinline__ dfl phi2_neg_df(dfl x)
+{
+    const float f = -x.h;
+    dfl r;
+    if (x.h < 0.03125f) {
+        if (x.h < 0.001953125f) {
+            r = dfl{fmaf(f, fmaf(f, 1.0f / 5040, 1.0f / 720), 1.0f / 120), 0.f};
+        } else {
+            r = dfl{fmaf(f, fmaf(f, fmaf(f, 1.0f / 362880, 1.0f / 40320), 1.0f / 5040), 1.0f / 720), 0.f};
+            r = horner_df(x, r, 0.00833333377f, -4.34617203e-10f);
+        }
     } else {
-        dfl om;
+        r = dfl{fmaf(f, fmaf(f, fmaf(f, fmaf(f, 1.0f / 87178291200.0f, 1.0f / 6227020800.0f),
+                                     1.0f / 479001600), 1.0f / 39916800), 1.0f / 3628800), 0.f};
+        r = horner_df(x, r, 2.75573188e-06f, 3.79357122e-14f);
+        r = horner_df(x, r, 2.48015876e-05f, -3.40699609e-13f);
+        r = horner_df(x, r, 0.000198412701f, -2.72559687e-12f);
+        r = horner_df(x, r, 0.00138888892f, -3.36310944e-11f);
+        r = horner_df(x, r, 0.00833333377f, -4.34617203e-10f);
+    }
+    r = horner_df(x, r, 0.0416666679f, -1.24176347e-09f);
+    r = horner_df(x, r, 0.166666672f, -4.96705388e-09f);
+    r = horner_df(x, r, 0.5f, 0.f);
+    return quick_two_sum(r.h, r.l);
+}
+
+// (a - b) + c with |a| >= |b|, |a - b| >= |c|
+__device__ __forceinline__ dfl sub_add_df(dfl a, dfl b, dfl c)
+{
+    const dfl s = quick_two_sum(a.h, -b.h);
+    const dfl u = quick_two_sum(s.h, c.h);
+    return quick_two_sum(u.h, ((a.l - b.l) + s.l) + (c.l + u.l));
+}
+
+// A segment of optical depth x with the transmission T at its near end:
+// b = T w_cur, g = T w_up, Tn = T e (definitions as weights.cuh).  Below
+// x = 1/2 from the series, a = T x: b = a phi2(-x), Tn = (T - a) + x b,
+// g = (a - b) - x b, about 100 FP32 operations and half of what the
+// exponential and the division of the closed form take.
+__device__ __forceinline__ void seg_step_df(dfl T, dfl x, const dfl* __restrict__ tab, dfl& b, dfl& g,
+                                            dfl& Tn)
+{
+    if (x.h < 0.5f) {
+        const dfl a = df_mul(T, x);
+        b = df_mul(a, phi2_neg_df(x));
+        dfl xb = two_prod(x.h, b.h);
+        xb.l = fmaf(x.l, b.h, fmaf(x.h, b.l, xb.l));
+        Tn = sub_add_df(T, a, xb);
+        g = sub_add_df(a, b, df_neg(xb));
+    } else {
+        dfl e, om;
         if (x.h <= 80.0f) {
             exp_neg_df(x, tab, e, om);
         } else {
@@ -102,11 +141,19 @@ __device__ __forceinline__ void seg_weights_df(dfl x, const dfl* __restrict__ ta
             om = df_make(1.f, 0.f);
         }
         // q = om / x: FP32 quotient and two corrections from the residual
-        // (one leaves a relative error near 2^-44, amplified up to 40x in 1 - q)
+        // (one leaves a relative error near 2^-44, amplified in 1 - q)
         const dfl q = df_div_s(om, x);
-        wc = df_add_f(df_neg(q), 1.0f);
-        wu = df_sub_s(q, e);
+        b = df_mul(T, df_add_f(df_neg(q), 1.0f));
+        g = df_mul(T, df_sub_s(q, e));
+        Tn = df_mul(T, e);
     }
+}
+
+// The same for T = 1: w_cur, w_up, e.
+__device__ __forceinline__ void seg_weights_df(dfl x, const dfl* __restrict__ tab, dfl& wc, dfl& wu,
+                                               dfl& e)
+{
+    seg_step_df(df_make(1.f, 0.f), x, tab, wc, wu, e);
 }
 
 // Bilinear interpolation of a double-float field: sum of four df products
@@ -182,10 +229,10 @@ k_fsdf(ViewDF p, float cut, unsigned long long* __restrict__ steps)
                                             q11.z, q11.w);
                     const dfl db = df_sub_s(sb, S0);
                     const dfl x = df_mul(hs, df_add_s(ca, cb));
-                    dfl wc, wu, e;
-                    seg_weights_df(x, tab, wc, wu, e);
-                    I = df_add_s(I, df_mul(T, df_add_s(df_mul(wc, da), df_mul(wu, db))));
-                    T = df_mul(T, e);
+                    dfl b, gu, Tn;
+                    seg_step_df(T, x, tab, b, gu, Tn);
+                    I = df_add_s(I, df_add_s(df_mul(b, da), df_mul(gu, db)));
+                    T = Tn;
                     ca = cb;
                     da = db;
                     if (T.h <= tcut) {
@@ -273,16 +320,16 @@ k_recdf(ViewDF p, int r0, RecOut ro, const int* __restrict__ lmax, int nwp,
                 const float2 q01 = __ldg(q + 2 * W), q11 = __ldg(q + 2 * W + 2);
                 const dfl cb = bilin_df(wh, wl, q00.x, q00.y, q10.x, q10.y, q01.x, q01.y, q11.x, q11.y);
                 const dfl x = df_mul(hs, df_add_s(ca, cb));
-                dfl wc, wu, e;
-                seg_weights_df(x, tab, wc, wu, e);
+                dfl b, gu, Tn;
+                seg_step_df(T, x, tab, b, gu, Tn);
                 if (m == 0) {
-                    C0 = df_add_s(C0, df_mul(df_from_double(di.w), wc));
+                    C0 = df_add_s(C0, df_mul(df_from_double(di.w), b));
                 } else {
-                    const dfl c = df_add_s(cprev, df_mul(T, wc));
+                    const dfl c = df_add_s(cprev, b);
                     rc[(long long)(m - 1) * nxy] = make_float2(c.h, c.l);
                 }
-                cprev = df_mul(T, wu);
-                T = df_mul(T, e);
+                cprev = gu;
+                T = Tn;
                 ca = cb;
             }
             if (L > 0) rc[(long long)(L - 1) * nxy] = make_float2(cprev.h, cprev.l);

@@ -411,12 +411,11 @@ k_rec64(Geometry g, int r0, const double* __restrict__ chi, const double* __rest
                 RT_GUARD(g, pb + op_nmin(n), g.N, kSiteFs64) break;
                 RT_GUARD(g, pb + op_nmax(n), g.N, kSiteFs64) break;
                 const double cb = op_bilin(chi + pb, n, bh[m + 1]);
-                double wc, wu, e;
-                seg_weights64(ca + cb, tab, wc, wu, e);
-                if (m == 0) C0 = fma(w, wc, C0);
-                else rc[(long long)(m - 1) * nxy] = fma(T, wc, cprev);
-                cprev = T * wu;
-                T *= e;
+                double b;
+                const double before = cprev;
+                seg_step64(T, ca + cb, tab, b, cprev, T);
+                if (m == 0) C0 = fma(w, b, C0);
+                else rc[(long long)(m - 1) * nxy] = before + b;
                 ca = cb;
             }
             if (L > 0) rc[(long long)(L - 1) * nxy] = cprev;
@@ -468,12 +467,18 @@ struct AsmDF {
     {
         return make_float2(__shfl_sync(0xffffffffu, w.x, i), __shfl_sync(0xffffffffu, w.y, i));
     }
+    // the sum is left unnormalised between contributions
     static __device__ __forceinline__ V fma(V w, V c, V a)
     {
-        const dfl r = df_add_s(df_make(a.x, a.y), df_mul(df_make(w.x, w.y), df_make(c.x, c.y)));
-        return make_float2(r.h, r.l);
+        const dfl p = two_prod(w.x, c.x);
+        const dfl s = two_sum(a.x, p.h);
+        return make_float2(s.h, (a.y + s.l) + fmaf(w.y, c.x, fmaf(w.x, c.y, p.l)));
     }
-    static __device__ __forceinline__ Pair pair(V a, V b) { return make_float4(a.x, a.y, b.x, b.y); }
+    static __device__ __forceinline__ Pair pair(V a, V b)
+    {
+        const dfl p = quick_two_sum(a.x, a.y), q = quick_two_sum(b.x, b.y);
+        return make_float4(p.h, p.l, q.h, q.l);
+    }
 };
 
 template <typename T>

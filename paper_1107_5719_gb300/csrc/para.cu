@@ -52,31 +52,45 @@ __device__ __forceinline__ double bilin_p(const double* __restrict__ f, NodesP n
            b.w * __ldg(f + n.a11);
 }
 
+constexpr int kHiOne = 0x3FF00000;       // high word of 1
+
 // Parabolic weights of a segment of optical depth a whose downstream
 // neighbour segment has optical depth b; e = e^{-a}.
 __device__ __forceinline__ void para_weights64(double a, double b, const double* __restrict__ tab,
                                                double& pu, double& pc, double& pd, double& e)
 {
-    e = a <= 700.0 ? exp_neg_tang(a, tab) : 0.0;
     double E0, E1, E2;
-    if (a < 1.0) {
-        // T2 = sum_{k>=3} a^k/k! (through k = 18: truncation < 1e-16 relative)
-        double h = 1.0 / 6402373705728000.0;                      // 1/18!
-        h = fma(h, a, 1.0 / 355687428096000.0);                    // 1/17!
-        h = fma(h, a, 1.0 / 20922789888000.0);
-        h = fma(h, a, 1.0 / 1307674368000.0);
-        h = fma(h, a, 1.0 / 87178291200.0);
-        h = fma(h, a, 1.0 / 6227020800.0);
-        h = fma(h, a, 1.0 / 479001600.0);
-        h = fma(h, a, 1.0 / 39916800.0);
-        h = fma(h, a, 1.0 / 3628800.0);
-        h = fma(h, a, 1.0 / 362880.0);
-        h = fma(h, a, 1.0 / 40320.0);
+    const int ha = __double2hiint(a);
+    if (ha < kHi2m9) e = fma(a, fma(a, phi2_neg64(a, ha), -1.0), 1.0);
+    else e = ha < kHi700 ? exp_neg_times(1.0, a, tab) : 0.0;
+    if (ha < kHiOne) {
+        // T2 = sum_{k>=3} a^k/k! = a^3 h, h's terms below 2^-33 of it in FP32
+        const float f = lead_float(a);
+        double h;
+        if (ha < kHi2m5) {
+            h = pos_double(fmaf(f, fmaf(f, 1.0f / 3628800, 1.0f / 362880), 1.0f / 40320));
+        } else {
+            if (ha < kHiQuarter) {
+                h = pos_double(fmaf(f, fmaf(f, fmaf(f, 1.0f / 6227020800.0f, 1.0f / 479001600),
+                                            1.0f / 39916800), 1.0f / 3628800));
+            } else {
+                h = pos_double(fmaf(f, fmaf(f, fmaf(f, fmaf(f, 1.0f / 6402373705728000.0f,
+                                                            1.0f / 355687428096000.0f),
+                                                    1.0f / 20922789888000.0f),
+                                            1.0f / 1307674368000.0f), 1.0f / 87178291200.0f));
+                h = fma(h, a, 1.0 / 6227020800.0);
+                h = fma(h, a, 1.0 / 479001600.0);
+                h = fma(h, a, 1.0 / 39916800.0);
+                h = fma(h, a, 1.0 / 3628800.0);
+            }
+            h = fma(h, a, 1.0 / 362880.0);
+            h = fma(h, a, 1.0 / 40320.0);
+        }
         h = fma(h, a, 1.0 / 5040.0);
         h = fma(h, a, 1.0 / 720.0);
         h = fma(h, a, 1.0 / 120.0);
         h = fma(h, a, 1.0 / 24.0);
-        h = fma(h, a, 1.0 / 6.0);                                  // 1/3!
+        h = fma(h, a, 1.0 / 6.0);
         const double a2 = a * a;
         const double T2 = h * a2 * a;
         const double T1 = fma(0.5, a2, T2);
@@ -89,7 +103,7 @@ __device__ __forceinline__ void para_weights64(double a, double b, const double*
         E1 = E0 - a * e;
         E2 = 2.0 * E1 - a * a * e;
     }
-    const double r = recip_newton(a * b * (a + b));
+    const double r = div_seed(1.0, a * b * (a + b));
     pu = (E2 + b * E1) * b * r;
     pc = (a * b * E0 - (b - a) * E1 - E2) * (a + b) * r;
     pd = (E2 - a * E1) * a * r;

@@ -19,83 +19,144 @@ namespace {
 // ---- FP64 -----------------------------------------------------------------
 //
 // The FP64 pipe of GB300 issues about 2 DFMA per SM per clock, so the FP64
-// weights are written to use few FP64 instructions:
+// weights are written to use few FP64 instructions; FP32 and integer ones
+// are nearly free beside them.  A segment is taken together with the
+// transmission T at its near end: b = T w_cur, g = T w_up, Tn = T e.
 //
-//  x < 1/4: the phi2 series (Horner in z = x^2, six terms each: the first
-//    omitted terms, z^6/14! and z^6/15! at z <= 1/16, are below 7e-19 and
-//    5e-20); no exp call and no cancellation.  With E as above and
-//    O = x Q, w_cur = xE - zQ and w_up = e (xE + zQ): 17 FP64 operations.
-//  x >= 1/4: e from Tang's table-driven method (ACM TOMS 15, 1989):
-//    -x/ln2 = k/256 + r/ln2, k = round(-256 x/ln2), |r| <= ln2/512,
-//    e = 2^{k>>8} * 2^{(k&255)/256} * P(r), P the degree-4 Taylor polynomial
-//    of e^r (relative error < 4e-17), the 256 powers 2^{j/256} in shared
-//    memory; then (1-e)/x from a reciprocal seed and two Newton steps.
+//  x < 1/2: the series phi2(-x) = sum_k (-x)^k/(k+2)! by Horner, its terms
+//    below 2^-32 of the sum in FP32 (their rounding, 2^-22 of them, is below
+//    the last bit of the FP64 result): from k = 3, 5, 6 or 9 on for x <
+//    2^-9, 2^-5, 2^-3 or 1/2, so 3, 5, 6 or 9 FP64 operations (two series of
+//    five in x^2 before).  Then, a = T x:  b = a phi2(-x),
+//    Tn = (T - a) + x b,  g = (a - b) - x b: six more.  No exp call; against
+//    50 digits, T = 1: 1.6e-16, 1.4e-16 and 2.6e-16 relative at most.
+//  x >= 1/2: e^-x by a two-level form of Tang's table-driven method (ACM TOMS
+//    15, 1989): -x = k ln2/65536 + r, |r| <= 5.3e-6, k = 65536 n + 256 j1 + j2,
+//    e^-x = 2^n 2^{j1/256} 2^{j2/65536} (1 + r + r^2/2), the quadratic term
+//    (1.4e-11) and the low part of k ln2/65536 in FP32; then q = (T - Tn)/x
+//    from the reciprocal seed r0, x r0 = 1 - d, as (T - Tn) r0 (1 + d + d^2);
+//    b = T - q, g = q - Tn: 14 operations for the three products.
 //    Above x = 700 e is taken as 0 (it would scale I by < 1e-304).
-//  Both branch tests compare the high word of x (x >= 0) as an integer, so
-//    they take no FP64 compare.
+//  Branch tests compare the high word of x (x >= 0) as an integer, so they
+//    take no FP64 compare.
 
-constexpr int kExpTable = 256;
+constexpr int kExpTable = 512;
 
-// Fill tab[j] = 2^{j/256} (call from every thread, then __syncthreads()).
+// tab[j] = 2^{j/256}, tab[256 + j] = 2^{j/65536} (call from every thread, then
+// __syncthreads()); the second from the series of e^y, y < 2.8e-3.
 __device__ __forceinline__ void fill_exp_table(double* tab)
 {
-    for (int j = threadIdx.x; j < kExpTable; j += blockDim.x) tab[j] = exp2((double)j / kExpTable);
+    for (int j = threadIdx.x; j < 256; j += blockDim.x) {
+        tab[j] = exp2((double)j / 256);
+        const double y = (double)j * (0.693147180559945309417 / 65536);
+        tab[256 + j] = fma(fma(fma(fma(fma(1.0 / 120, y, 1.0 / 24), y, 1.0 / 6), y, 0.5), y, 1.0), y, 1.0);
+    }
 }
 
-__device__ __forceinline__ double exp_neg_tang(double x, const double* __restrict__ tab)
+// The leading 24 bits of x >= 0, x < 2^127 (below 2^-126: 2^-126 or a little
+// more), and a positive normal float as a double, both on the integer pipe.
+__device__ __forceinline__ float lead_float(double x)
 {
-    constexpr double kMagic = 6755399441055744.0;          // 1.5 * 2^52: round to integer
-    constexpr double kInvL = 369.329930467574632284140718;  // 256 / ln 2
-    constexpr double kL1 = 2.7076061740622863e-03;          // ln2/256, leading part
-    constexpr double kL2 = 9.058776616587108e-20;           // ln2/256 - kL1
-    const double t = fma(-x, kInvL, kMagic);
-    const int k = __double2loint(t);                         // round(-256 x / ln2)
-    const double kd = t - kMagic;
-    double r = fma(-kd, kL1, -x);
-    r = fma(-kd, kL2, r);
-    double p = fma(fma(fma(1.0 / 24.0, r, 1.0 / 6.0), r, 0.5), r, 1.0);
-    p = fma(p, r, 1.0);
-    const double e = tab[k & (kExpTable - 1)] * p;
-    // scale by 2^(k >> 8): add to the exponent field (result stays normal for x <= 700)
-    return __hiloint2double(__double2hiint(e) + (k >> 8) * (1 << 20), __double2loint(e));
+    const int hi = max(__double2hiint(x), 0x38100000) - 0x38000000;
+    return __int_as_float((int)__funnelshift_l((unsigned)__double2loint(x), (unsigned)hi, 3));
 }
 
-__device__ __forceinline__ double recip_newton(double x)
+__device__ __forceinline__ double pos_double(float f)
+{
+    const unsigned u = __float_as_uint(f);
+    return __hiloint2double((int)(u >> 3) + 0x38000000, (int)(u << 29));
+}
+
+// T e^{-x}, 1e-3 < x <= 700
+__device__ __forceinline__ double exp_neg_times(double T, double x, const double* __restrict__ tab)
+{
+    constexpr double kMagic = 6755399441055744.0;        // 1.5 * 2^52: round to integer
+    constexpr double kInvL = 94548.4621996991;            // 65536 / ln 2
+    constexpr double kL1 = 1.0576586617430806e-05;        // ln2/65536, leading part
+    constexpr float kL2 = 3.345677e-17f;                  // (ln2/65536 - kL1) 65536/ln2
+    const double t = fma(-x, kInvL, kMagic);
+    const int k = __double2loint(t);                      // round(-65536 x / ln2)
+    const double r = fma(-(t - kMagic), kL1, -x);
+    const float rf = lead_float(fabs(r));
+    const double u = r + pos_double(fmaf(0.5f * rf, rf, kL2 * lead_float(x)));
+    // 2^n into the exponent field of the first factor (normal for x <= 700)
+    const double t1 = tab[(k >> 8) & 255];
+    const double m = T * __hiloint2double(__double2hiint(t1) + (k >> 16) * (1 << 20), __double2loint(t1)) *
+                     tab[256 + (k & 255)];
+    return fma(m, u, m);
+}
+
+// n / x from the hardware reciprocal seed (20 bits), x > 0 normal
+__device__ __forceinline__ double div_seed(double n, double x)
 {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
-    double e = fma(-x, r, 1.0);
-    r = fma(r, e, r);
-    e = fma(-x, r, 1.0);
-    return fma(r, e, r);
+    const double d = fma(-x, r, 1.0);
+    const double q = n * r;
+    return fma(q, fma(d, d, d), q);
 }
 
-constexpr int kHiQuarter = 0x3FD00000;   // high word of 0.25
-constexpr int kHi700 = 0x4085E000;       // high word of 700.0
+constexpr int kHi2m9 = 0x3F600000;       // high words of 2^-9,
+constexpr int kHi2m5 = 0x3FA00000;       // 2^-5,
+constexpr int kHi2m3 = 0x3FC00000;       // 2^-3,
+constexpr int kHiQuarter = 0x3FD00000;   // 1/4,
+constexpr int kHiHalf = 0x3FE00000;      // 1/2
+constexpr int kHi700 = 0x4085E000;       // and 700
+
+// phi2(-x), x < 1/2; hx the high word of x
+__device__ __forceinline__ double phi2_neg64(double x, int hx)
+{
+    const float xf = lead_float(x);
+    double r;
+    if (hx < kHi2m9) {
+        r = pos_double(fmaf(-xf, fmaf(-xf, 1.0f / 5040, 1.0f / 720), 1.0f / 120));
+    } else {
+        if (hx < kHi2m5) {
+            r = pos_double(fmaf(-xf, fmaf(-xf, 1.0f / 362880, 1.0f / 40320), 1.0f / 5040));
+        } else {
+            if (hx < kHi2m3) {
+                r = pos_double(fmaf(-xf, fmaf(-xf, 1.0f / 3628800, 1.0f / 362880), 1.0f / 40320));
+            } else {
+                r = pos_double(fmaf(-xf, fmaf(-xf, fmaf(-xf, fmaf(-xf, 1.0f / 1307674368000.0f,
+                                                                   1.0f / 87178291200.0f),
+                                                        1.0f / 6227020800.0f),
+                                              1.0f / 479001600), 1.0f / 39916800));
+                r = fma(-x, r, 1.0 / 3628800);
+                r = fma(-x, r, 1.0 / 362880);
+                r = fma(-x, r, 1.0 / 40320);
+            }
+            r = fma(-x, r, 1.0 / 5040);
+        }
+        r = fma(-x, r, 1.0 / 720);
+        r = fma(-x, r, 1.0 / 120);
+    }
+    r = fma(-x, r, 1.0 / 24);
+    r = fma(-x, r, 1.0 / 6);
+    return fma(-x, r, 0.5);
+}
+
+// b = T w_cur, g = T w_up, Tn = T e of a segment of optical depth x
+__device__ __forceinline__ void seg_step64(double T, double x, const double* __restrict__ tab, double& b,
+                                           double& g, double& Tn)
+{
+    const int hx = __double2hiint(x);
+    if (hx < kHiHalf) {
+        const double a = T * x;
+        b = a * phi2_neg64(x, hx);
+        Tn = fma(x, b, T - a);
+        g = fma(-x, b, a - b);
+    } else {
+        Tn = hx < kHi700 ? exp_neg_times(T, x, tab) : 0.0;
+        const double q = div_seed(T - Tn, x);
+        b = T - q;
+        g = q - Tn;
+    }
+}
 
 __device__ __forceinline__ void seg_weights64(double x, const double* __restrict__ tab, double& wc,
                                               double& wu, double& e)
 {
-    const int hx = __double2hiint(x);
-    if (hx < kHiQuarter) {
-        const double z = x * x;
-        // E = sum_j z^j/(2j+2)!,  Q = sum_j z^j/(2j+3)!  (j = 0..5)
-        double E = fma(fma(fma(fma(1.0 / 479001600.0, z, 1.0 / 3628800.0), z, 1.0 / 40320.0), z,
-                           1.0 / 720.0), z, 1.0 / 24.0);
-        E = fma(E, z, 0.5);
-        double Q = fma(fma(fma(fma(1.0 / 6227020800.0, z, 1.0 / 39916800.0), z, 1.0 / 362880.0), z,
-                           1.0 / 5040.0), z, 1.0 / 120.0);
-        Q = fma(Q, z, 1.0 / 6.0);
-        const double xE = x * E;
-        wc = fma(-z, Q, xE);
-        e = fma(x, wc, 1.0 - x);
-        wu = e * fma(z, Q, xE);
-    } else {
-        e = hx < kHi700 ? exp_neg_tang(x, tab) : 0.0;
-        const double q = (1.0 - e) * recip_newton(x);
-        wc = 1.0 - q;
-        wu = q - e;
-    }
+    seg_step64(1.0, x, tab, wc, wu, e);
 }
 
 // Cutoff test on exponent fields only (integer pipe).  With T < 2^(eT+1),
