@@ -51,6 +51,7 @@ struct rt_ctx {
     int* d_nsw = nullptr;     // the graph's sweep counter
     int* d_sw = nullptr;      // sweeps of the graph's last OS step (device), and a pinned copy
     int* h_sw = nullptr;
+    bool os_one = false;      // the last step ran as one kernel (launch_os_solve)
     bool use_graphs = true;
     unsigned long long* berr = nullptr;   // checked builds: out-of-bounds record
     int fs_method = RT_FS_LONG;
@@ -1227,7 +1228,7 @@ int build_os_graph(rt_ctx* c, rt_ctx::OsGraph& e, const double* Jfs, const doubl
     if (err == cudaSuccess) {
         // prologue; every call is attempted so that the capture is always ended
         cudaError_t e1 = launch_os_rhs(c->g, c->coef, c->rdiag, Jfs, Jold, c->r, gs, c->stream);
-        cudaError_t e2 = cudaMemsetAsync(c->dlt, 0, sizeof(double) * (max_sweeps + 2), c->stream);
+        cudaError_t e2 = cudaMemsetAsync(c->dlt, 0, sizeof(double) * (max_sweeps + kPassSweeps), c->stream);
         cudaError_t e3 = cudaMemcpyAsync(c->Jb, Jold, sizeof(double) * c->g.N,
                                          cudaMemcpyDeviceToDevice, c->stream);
         cudaError_t e4 = cudaMemsetAsync(c->d_nsw, 0, sizeof(int), c->stream);
@@ -1294,6 +1295,8 @@ int build_os_graph(rt_ctx* c, rt_ctx::OsGraph& e, const double* Jfs, const doubl
     return RT_OK;
 }
 
+int ensure_sweep_words(rt_ctx* c);
+
 // The operator-splitting step as one graph launch, without waiting for it:
 // J_new and the sweep count (c->d_sw) are written on the device.  The
 // caller copies d_sw to h_sw before its next synchronisation and then calls
@@ -1302,12 +1305,8 @@ int run_os_graph(rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew,
                  int max_sweeps)
 {
     int rc;
-    if ((rc = ensure_dlt(c, max_sweeps + 2))) return rc;
-    if (!c->d_nsw) CK(cudaMalloc((void**)&c->d_nsw, sizeof(int)));
-    if (!c->d_sw) {
-        CK(cudaMalloc((void**)&c->d_sw, sizeof(int)));
-        CK(cudaMallocHost((void**)&c->h_sw, sizeof(int)));
-    }
+    if ((rc = ensure_dlt(c, max_sweeps + kPassSweeps)) || (rc = ensure_sweep_words(c))) return rc;
+    c->os_one = false;
     rt_ctx::OsGraph* e = nullptr;
     for (auto& x : c->osg)
         if (x.exec && x.jold == Jold && x.jfs == Jfs && x.jnew == Jnew && x.dlt == c->dlt &&
@@ -1331,16 +1330,77 @@ int run_os_graph(rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew,
     return RT_OK;
 }
 
-// After the synchronisation that follows run_os_graph: the sweep count and
-// the launch counters of that step.
-int os_graph_done(rt_ctx* c)
+// After the synchronisation that follows run_os_graph or run_os_one: the
+// sweep count into *sweeps, and the counters of that step.
+int os_graph_done(rt_ctx* c, int* sweeps)
 {
-    const int sweeps = *c->h_sw;
+    *sweeps = *c->h_sw;
+    if (*sweeps < 0)
+        return fail(c, RT_ETIMEOUT, "a wait of the operator-splitting kernel's blocks gave up");
     const int per = c->os_method == RT_OS_GAUSS_SEIDEL ? 2 : 1;
-    const int passes = (sweeps + 1) / 2;
-    c->stats.launches += 2 + passes * (2 * per + 1);
-    c->stats.jacobi_launches += passes * 2 * per;
-    return sweeps;
+    const int passes = (*sweeps + kPassSweeps - 1) / kPassSweeps;
+    c->stats.launches += c->os_one ? 1 : 2 + passes * (kPassSweeps * per + 1);
+    c->stats.jacobi_launches += c->os_one ? *sweeps * per : passes * kPassSweeps * per;
+    return RT_OK;
+}
+
+// The context's arrays as a task of launch_os_solve (its barrier word behind
+// the deltas).
+OsTask os_task(const rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew, double* dlt,
+               int max_sweeps, int* sweeps, int nblk)
+{
+    OsTask t;
+    t.g = c->g;
+    t.c = c->coef;
+    t.rdiag = c->rdiag;
+    t.Jfs = Jfs;
+    t.Jold = Jold;
+    t.Ja = c->Ja;
+    t.Jb = c->Jb;
+    t.Jn = Jnew;
+    t.dlt = dlt;
+    t.bar = reinterpret_cast<unsigned*>(dlt + max_sweeps);
+    t.sweeps = sweeps;
+    t.nblk = nblk;
+    return t;
+}
+
+int ensure_sweep_words(rt_ctx* c)
+{
+    if (!c->d_nsw) CK(cudaMalloc((void**)&c->d_nsw, sizeof(int)));
+    if (!c->d_sw) {
+        CK(cudaMalloc((void**)&c->d_sw, sizeof(int)));
+        CK(cudaMallocHost((void**)&c->h_sw, sizeof(int)));
+    }
+    return RT_OK;
+}
+
+// The operator-splitting step as one cooperative kernel, without waiting for
+// it, where the grid's blocks are resident together; ran: whether it was
+// launched.
+int run_os_one(rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew, double tol_inner,
+               int max_sweeps, bool& ran)
+{
+    ran = false;
+    OsShape sh;
+    os_solve_shape(c->g.N, c->num_sms, c->os_method == RT_OS_GAUSS_SEIDEL, &sh);
+    if (sh.blocks == 0) return RT_OK;
+    int rc;
+    if ((rc = ensure_dlt(c, max_sweeps + kPassSweeps)) || (rc = ensure_sweep_words(c))) return rc;
+    CK(cudaMemsetAsync(c->dlt, 0, sizeof(double) * (max_sweeps + 1), c->stream));
+    const OsTask t = os_task(c, Jfs, Jold, Jnew, c->dlt, max_sweeps, c->d_sw, sh.blocks);
+    if (c->profiling) CK(cudaEventRecord(c->ev[2], c->stream));
+    const cudaError_t e = launch_os_solve(t, nullptr, nullptr, 1, sh, c->os_method == RT_OS_GAUSS_SEIDEL,
+                                          c->num_sms, max_sweeps, tol_inner, c->stream);
+    if (e == cudaErrorCooperativeLaunchTooLarge) return RT_OK;
+    CK(e);
+    if (c->profiling) {
+        CK(cudaEventRecord(c->ev[3], c->stream));
+        c->jac_pending = true;
+    }
+    CK(cudaMemcpyAsync(c->h_sw, c->d_sw, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    c->os_one = ran = true;
+    return RT_OK;
 }
 
 int run_os(rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew, double tol_inner,
@@ -1351,6 +1411,8 @@ int run_os(rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew, doubl
     if (c->use_graphs) {
         // sweep count after the caller's synchronisation (os_graph_done)
         if (sweeps_out) *sweeps_out = -1;
+        bool ran = false;
+        if ((rc = run_os_one(c, Jfs, Jold, Jnew, tol_inner, max_sweeps, ran)) || ran) return rc;
         return run_os_graph(c, Jfs, Jold, Jnew, tol_inner, max_sweeps);
     }
     if ((rc = ensure_dlt(c, max_sweeps))) return rc;
@@ -1423,7 +1485,7 @@ int os_step(rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew, doub
         CK(cudaMemcpyAsync(Jnew, dnew, sizeof(double) * c->g.N, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     harvest(c);
-    if (ns < 0) ns = os_graph_done(c);
+    if (ns < 0 && (rc = os_graph_done(c, &ns))) return rc;
     if (sweeps) *sweeps = ns;
     return RT_OK;
 }
@@ -1526,7 +1588,7 @@ int solve(rt_ctx* c, double tol, int max_iter, double tol_inner, int max_sweeps,
         c->stats.host_syncs += 1;
         c->stats.iterations += 1;
         harvest(c);
-        if (ns < 0) ns = os_graph_done(c);
+        if (ns < 0 && (rc = os_graph_done(c, &ns))) return rc;
         total_steps += *c->h_steps;
         delta = c->h_scal[2];
         c->ng_last_delta = delta;
@@ -1605,6 +1667,14 @@ struct rt_batch {
     } osg[2];
     int osg_next = 0;
     bool use_graphs = true;
+    // the active problems' solves in one kernel (launch_os_solve), where their
+    // blocks are resident together: tasks and first blocks (device, pinned
+    // copies), deltas and barrier words of all problems
+    OsTask *d_tasks = nullptr, *h_tasks = nullptr;
+    int *d_first = nullptr, *h_first = nullptr;
+    double* d_bdlt = nullptr;
+    int bdlt_cap = 0;               // sweeps per problem it holds
+    bool os_one = false;            // the last step ran that way
     int* d_sweeps = nullptr;        // sweeps of each problem's last OS step
     int* h_sweeps = nullptr;        // pinned
     // Recorded marches: a problem starts iterating once its recording fits
@@ -1772,13 +1842,26 @@ void batch_release(rt_batch* b, int p)
     }
 }
 
-void batch_free_pool(rt_batch* b)
+// Free pooled blocks until at most `keep` bytes are held, the largest first.
+void batch_free_pool(rt_batch* b, long long keep = 0)
 {
-    if (b->rec_pool.empty()) return;
+    long long held = 0;
+    for (auto& blk : b->rec_pool) held += blk.second;
+    if (held <= keep) return;
     cudaStreamSynchronize(b->stream);
-    for (auto& blk : b->rec_pool) cudaFree(blk.first);
-    b->rec_pool.clear();
+    std::sort(b->rec_pool.begin(), b->rec_pool.end(),
+              [](const auto& x, const auto& y) { return x.second < y.second; });
+    while (!b->rec_pool.empty() && held > keep) {
+        held -= b->rec_pool.back().second;
+        cudaFree(b->rec_pool.back().first);
+        b->rec_pool.pop_back();
+    }
 }
+
+// What a batch keeps of its recordings' memory between solves (the blocks of
+// a small batch: allocating and freeing 4 GB of them took 4 of 37 ms per solve
+// of six wavelengths of 41^3 and 20^3); freed with the batch.
+constexpr long long kPoolKeep = 8LL << 30;
 
 void bharvest(rt_batch* b)
 {
@@ -1842,7 +1925,7 @@ cudaError_t build_batch_os_graph(rt_batch* b, const std::vector<int>& act, doubl
         std::vector<cudaGraphNode_t> deps;
         {
             cudaError_t e1 = launch_os_rhs(c->g, c->coef, c->rdiag, c->Jfs, c->J, c->r, gs, st);
-            cudaError_t e2 = cudaMemsetAsync(c->dlt, 0, sizeof(double) * (max_sweeps + 2), st);
+            cudaError_t e2 = cudaMemsetAsync(c->dlt, 0, sizeof(double) * (max_sweeps + kPassSweeps), st);
             cudaError_t e3 = cudaMemcpyAsync(c->Jb, c->J, sizeof(double) * c->g.N,
                                              cudaMemcpyDeviceToDevice, st);
             cudaError_t e4 = cudaMemsetAsync(c->d_nsw, 0, sizeof(int), st);
@@ -2025,15 +2108,74 @@ int batch_fs(rt_batch* b, const std::vector<int>& act)
     return RT_OK;
 }
 
-// Operator-splitting solves of the active problems as one graph launch (no
-// host synchronisation); the sweep counts reach b->d_sweeps.
+// Operator-splitting solves of the active problems in one cooperative kernel,
+// where all their blocks are resident together; ran: whether it was launched.
+int batch_os_one(rt_batch* b, const std::vector<int>& act, double tol_inner, int max_sweeps, bool& ran)
+{
+    ran = false;
+    b->os_one = false;
+    const int P = (int)b->ctx.size(), method = b->ctx[act[0]]->os_method;
+    long long total = 0;
+    for (int p : act) {
+        if (b->ctx[p]->os_method != method) return RT_OK;
+        total += b->ctx[p]->g.N;
+    }
+    OsShape sh;
+    os_solve_shape(total, b->num_sms, method == RT_OS_GAUSS_SEIDEL, &sh);
+    if (sh.blocks == 0) return RT_OK;
+    if (!b->d_tasks) {
+        BCK(cudaMalloc((void**)&b->d_tasks, sizeof(OsTask) * P));
+        BCK(cudaMalloc((void**)&b->d_first, sizeof(int) * P));
+        BCK(cudaMallocHost((void**)&b->h_tasks, sizeof(OsTask) * P));
+        BCK(cudaMallocHost((void**)&b->h_first, sizeof(int) * P));
+    }
+    if (b->bdlt_cap < max_sweeps + 1) {
+        dfree(b->d_bdlt);
+        b->bdlt_cap = 0;
+        BCK(cudaMalloc((void**)&b->d_bdlt, sizeof(double) * (size_t)P * (max_sweeps + 1)));
+        b->bdlt_cap = max_sweeps + 1;
+    }
+    const long long per = (long long)sh.threads * sh.voxels;
+    sh.blocks = 0;
+    for (size_t q = 0; q < act.size(); ++q) {
+        rt_ctx* c = b->ctx[act[q]];
+        const int nblk = (int)((c->g.N + per - 1) / per);
+        b->h_tasks[q] = os_task(c, c->Jfs, c->J, c->Jn, b->d_bdlt + q * (max_sweeps + 1), max_sweeps,
+                                b->d_sweeps + act[q], nblk);
+        b->h_first[q] = sh.blocks;
+        sh.blocks += nblk;
+    }
+    BCK(cudaMemcpyAsync(b->d_tasks, b->h_tasks, sizeof(OsTask) * act.size(), cudaMemcpyHostToDevice,
+                        b->stream));
+    BCK(cudaMemcpyAsync(b->d_first, b->h_first, sizeof(int) * act.size(), cudaMemcpyHostToDevice,
+                        b->stream));
+    BCK(cudaMemsetAsync(b->d_bdlt, 0, sizeof(double) * act.size() * (max_sweeps + 1), b->stream));
+    if (b->profiling) BCK(cudaEventRecord(b->ev[2], b->stream));
+    const cudaError_t e = launch_os_solve(b->h_tasks[0], b->d_tasks, b->d_first, (int)act.size(), sh,
+                                          method == RT_OS_GAUSS_SEIDEL, b->num_sms, max_sweeps, tol_inner,
+                                          b->stream);
+    if (e == cudaErrorCooperativeLaunchTooLarge) return RT_OK;
+    BCK(e);
+    if (b->profiling) {
+        BCK(cudaEventRecord(b->ev[3], b->stream));
+        b->jac_pending = true;
+    }
+    b->os_one = ran = true;
+    return RT_OK;
+}
+
+// Operator-splitting solves of the active problems as one kernel or one graph
+// launch (no host synchronisation); the sweep counts reach b->d_sweeps.
 int batch_os_graph(rt_batch* b, const std::vector<int>& act, double tol_inner, int max_sweeps)
 {
     int rc;
+    for (int p : act)
+        if ((rc = bpass(b, p, ensure_coef(b->ctx[p])))) return rc;
+    bool ran = false;
+    if ((rc = batch_os_one(b, act, tol_inner, max_sweeps, ran)) || ran) return rc;
     for (int p : act) {
         rt_ctx* c = b->ctx[p];
-        if ((rc = bpass(b, p, ensure_coef(c)))) return rc;
-        if ((rc = bpass(b, p, ensure_dlt(c, max_sweeps + 2)))) return rc;
+        if ((rc = bpass(b, p, ensure_dlt(c, max_sweeps + kPassSweeps)))) return rc;
         if (!c->d_nsw) BCK(cudaMalloc((void**)&c->d_nsw, sizeof(int)));
     }
     std::vector<const void*> key = batch_graph_key(b, act, tol_inner, max_sweeps);
@@ -2074,14 +2216,18 @@ int batch_os_graph(rt_batch* b, const std::vector<int>& act, double tol_inner, i
 
 // Launch counts of the graph-driven operator splitting of `act`, from the
 // sweep counts the graph wrote (read after the iteration's synchronisation).
-void batch_os_graph_counts(rt_batch* b, const std::vector<int>& act)
+int batch_os_graph_counts(rt_batch* b, const std::vector<int>& act)
 {
+    if (b->os_one) b->stats.launches += 1;
     for (int p : act) {
+        if (b->h_sweeps[p] < 0)
+            return bfail(b, RT_ETIMEOUT, "problem %d: a wait of the operator-splitting kernel gave up", p);
         const int per = b->ctx[p]->os_method == RT_OS_GAUSS_SEIDEL ? 2 : 1;
-        const int passes = (b->h_sweeps[p] + 1) / 2;
-        b->stats.launches += 2 + passes * (2 * per + 1);
-        b->stats.jacobi_launches += passes * 2 * per;
+        const int passes = (b->h_sweeps[p] + kPassSweeps - 1) / kPassSweeps;
+        b->stats.launches += b->os_one ? 0 : 2 + passes * (kPassSweeps * per + 1);
+        b->stats.jacobi_launches += b->os_one ? b->h_sweeps[p] * per : passes * kPassSweeps * per;
     }
+    return RT_OK;
 }
 
 // Operator-splitting solves of the active problems without graphs; sweeps
@@ -2766,6 +2912,11 @@ int rt_batch_destroy(rt_batch* b)
     free_batch_graphs(b);
     batch_free_pool(b);
     for (rt_ctx* c : b->ctx) rt_destroy(c);
+    if (b->d_tasks) cudaFree(b->d_tasks);
+    if (b->d_first) cudaFree(b->d_first);
+    if (b->h_tasks) cudaFreeHost(b->h_tasks);
+    if (b->h_first) cudaFreeHost(b->h_first);
+    if (b->d_bdlt) cudaFree(b->d_bdlt);
     if (b->d_sweeps) cudaFree(b->d_sweeps);
     if (b->h_sweeps) cudaFreeHost(b->h_sweeps);
     if (b->d_views) cudaFree(b->d_views);
@@ -2965,7 +3116,7 @@ static int batch_solve(rt_batch* b, double tol, int max_iter, double tol_inner, 
         BCK(cudaStreamSynchronize(b->stream));
         b->stats.host_syncs += 1;
         b->stats.iterations += 1;
-        if (b->use_graphs) batch_os_graph_counts(b, act);
+        if (b->use_graphs && (rc = batch_os_graph_counts(b, act))) return rc;
         bharvest(b);
         b->stats.steps += *b->h_steps;
         for (int p : act) {
@@ -2989,7 +3140,7 @@ static int batch_solve(rt_batch* b, double tol, int max_iter, double tol_inner, 
             if (b->converged[p] || b->iters[p] >= max_iter) batch_release(b, p);
         }
     }
-    batch_free_pool(b);
+    batch_free_pool(b, kPoolKeep);
     int nconv = 0;
     for (int p = 0; p < P; ++p) {
         if (iters) iters[p] = b->iters[p];

@@ -524,12 +524,35 @@ cudaError_t launch_gs_sweep(const Geometry& g, const double* coef, const double*
                             const double* J, double* Jn, double* dlt, int n, double tol,
                             cudaStream_t st);
 // One pass of the device-side sweep loop (body of a CUDA graph WHILE node):
-// sweeps *nsw (b1 -> b0) and *nsw + 1 (b0 -> b1), Jacobi or Gauss-Seidel,
-// then *nsw += 2 and the loop condition h = (*nsw < max_sweeps and the last
-// sweep's dlt >= tol).  Same no-op rule and dlt layout as the host loop.
+// sweeps *nsw .. *nsw + kPassSweeps - 1 (b1 -> b0, b0 -> b1, ...), Jacobi or
+// Gauss-Seidel, then *nsw += kPassSweeps and the loop condition h = (*nsw <
+// max_sweeps and the last sweep's dlt >= tol).  Same no-op rule and dlt layout
+// as the host loop; dlt holds max_sweeps + kPassSweeps entries.  Four sweeps
+// per pass: a pass costs about 8 us beside its sweeps.
+constexpr int kPassSweeps = 4;
 cudaError_t launch_sweep_pass(const Geometry& g, const double* coef, const double* r, double* b0,
                               double* b1, double* dlt, int* nsw, int max_sweeps, double tol,
                               bool gs, cudaGraphConditionalHandle h, cudaStream_t st);
+// A whole operator-splitting solve in one cooperative launch (its blocks wait
+// on one another): right-hand side, sweeps to tol or max_sweeps, J_new and
+// the sweep count.  bar and dlt[0..max_sweeps) zeroed before; *sweeps = -1 if
+// a wait gave up.  Several problems (tasks, their first blocks first[q]) run
+// beside each other, each with its own barrier and stopping test.
+struct OsTask {
+    Geometry g;
+    const double *c, *rdiag, *Jfs, *Jold;
+    double *Ja, *Jb, *Jn, *dlt;
+    unsigned* bar;
+    int* sweeps;
+    int nblk;       // blocks of this problem
+};
+struct OsShape {
+    int threads, voxels, blocks;    // per block, per thread; 0 blocks: not used
+};
+void os_solve_shape(long long N, int num_sms, bool gs, OsShape* s);
+cudaError_t launch_os_solve(const OsTask& one, const OsTask* tasks, const int* first, int ntask,
+                            const OsShape& s, bool gs, int num_sms, int max_sweeps, double tol,
+                            cudaStream_t st);
 // After a device-side sweep loop from the buffers Ja (even sweeps) and Jb
 // (odd sweeps): Jn = the iterate of the last sweep that ran (the first n
 // with dlt[n] < tol, else max_sweeps - 1) and *sweeps_out = n + 1 (may be
