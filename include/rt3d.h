@@ -218,8 +218,10 @@ int rt_last_step_count(rt_ctx *ctx, unsigned long long *steps);
  * (default) records when that fits in 60% of the device and leaves 2 GiB
  * free, 0 never records, > 0 records when it fits in max_bytes; otherwise
  * every formal solution marches.  J agrees with the march to rounding (the
- * terms are summed in another order).  Short characteristics ignore the
- * setting.  RT_EINVAL for max_bytes < -1. */
+ * terms are summed in another order).  Short characteristics record the
+ * weights of every (voxel, direction) under the same setting, 24 ndir N bytes
+ * in FP64 and 16 ndir N + 16 N in double-float.  RT_EINVAL for max_bytes <
+ * -1. */
 int rt_set_fs_record(rt_ctx *ctx, long long max_bytes);
 /* Bytes held for the recorded march (0 if none) and whether a recording
  * valid for the current opacities, directions and boundary is held. */

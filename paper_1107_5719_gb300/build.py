@@ -24,7 +24,7 @@ BUILD_CHECKED = os.path.join(HERE, "_build_checked")
 LIB_CHECKED = os.path.join(HERE, "librt3d_checked.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
-SOURCES = ["fs.cu", "fs32.cu", "fsdf.cu", "sc.cu", "para.cu", "op.cu", "os.cu", "api.cu", "noalloc.cu",
+SOURCES = ["fs.cu", "fs32.cu", "fsdf.cu", "sc.cu", "screc.cu", "para.cu", "op.cu", "os.cu", "api.cu", "noalloc.cu",
            "probe.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE]
@@ -40,7 +40,7 @@ def nvcc() -> str:
 def _deps():
     files = [os.path.join(CSRC, s) for s in SOURCES]
     files += [os.path.join(CSRC, "internal.h"), os.path.join(CSRC, "weights.cuh"),
-              os.path.join(CSRC, "df.cuh"),
+              os.path.join(CSRC, "df.cuh"), os.path.join(CSRC, "dfweights.cuh"),
               os.path.join(INCLUDE, "rt3d.h")]
     return files
 

@@ -962,8 +962,53 @@ int fin_record(rt_ctx* c, const double* Jfs, cudaStream_t st)
     return RT_OK;
 }
 
-// Short-characteristics formal solution (FP64 only): J straight from the
-// march's ordered reduction, Lambda* from its own kernel once per opacity.
+// Recorded short characteristics: the view, with the pairs of chi and S behind
+// the weights in the recording's block.
+ScView scview(rt_ctx* c)
+{
+    ScView v{};
+    v.g = c->g;
+    v.chi = c->chi;
+    v.S = c->S;
+    v.B = c->B;
+    v.G = c->gdiff;
+    v.info = c->info;
+    v.off = c->off;
+    v.bw = c->bw;
+    v.bwdf = c->bwdf;
+    if (c->precision == RT_DF64) {
+        char* q = c->rec_mem + up256(sc_rec_bytes(c->g, true));
+        v.chi2 = reinterpret_cast<const float2*>(q);
+        v.S2 = reinterpret_cast<const float2*>(q + up256(8 * c->g.N));
+    }
+    return v;
+}
+
+// Record the weights of the short characteristics, once per opacity, where
+// they fit the budget; use: whether they are held.
+int ensure_sc_rec(rt_ctx* c, bool& use)
+{
+    use = false;
+    if (c->rec_mode == 0) return RT_OK;
+    const bool df = c->precision == RT_DF64;
+    if (!c->rec_valid) {
+        if (!rec_reserve(c, up256(sc_rec_bytes(c->g, df)) + (df ? 2 * up256(8 * c->g.N) : 0))) return RT_OK;
+        const ScView v = scview(c);
+        if (df) {
+            CK(launch_sc_pairs(c->g.N, c->chi, const_cast<float2*>(v.chi2), c->stream));
+            c->stats.launches += 1;
+        }
+        CK(launch_sc_record(v, df, c->rec_mem, c->stream));
+        c->stats.launches += 1;
+        c->rec_op = false;
+        c->rec_valid = true;
+    }
+    use = true;
+    return RT_OK;
+}
+
+// Short-characteristics formal solution: J straight from the march's ordered
+// reduction, Lambda* from its own kernel once per opacity.
 int run_fs_short(rt_ctx* c, double* Jout, bool count_steps)
 {
     int rc = fs_prepare(c);
@@ -971,7 +1016,18 @@ int run_fs_short(rt_ctx* c, double* Jout, bool count_steps)
     if ((rc = ensure_sc(c))) return rc;
     if (count_steps) CK(cudaMemsetAsync(c->d_steps, 0, sizeof(unsigned long long), c->stream));
     if (c->profiling) CK(cudaEventRecord(c->ev[0], c->stream));
-    if (c->precision == RT_DF64)
+    const bool df = c->precision == RT_DF64;
+    bool use = false;
+    if ((rc = ensure_sc_rec(c, use))) return rc;
+    if (use) {
+        const ScView v = scview(c);
+        if (df) {
+            CK(launch_sc_pairs(c->g.N, c->S, const_cast<float2*>(v.S2), c->stream));
+            c->stats.launches += 1;
+        }
+        CK(launch_sc_apply(v, df, c->rec_mem, c->wsum, c->scpart, c->scplanes, Jout,
+                           count_steps ? c->d_steps : nullptr, c->stream));
+    } else if (df)
         CK(launch_scdf(viewdf(c), c->S, c->wsum, c->scpart, (float2*)c->scplanes, Jout,
                        count_steps ? c->d_steps : nullptr, c->stream));
     else
@@ -985,7 +1041,9 @@ int run_fs_short(rt_ctx* c, double* Jout, bool count_steps)
     c->stats.fs_launches += 1;
     c->stats.launches += 2 * chunks;
     if (!c->lstar_valid) {
-        if (c->precision == RT_DF64)
+        if (use)
+            CK(launch_sc_lstar(scview(c), df, c->rec_mem, c->lstar, c->stream));
+        else if (df)
             CK(launch_lstar_df(viewdf(c), true, c->lstar, c->stream));
         else
             CK(launch_lstar_sc64(c->g, c->chi, c->info, c->off, c->bw, c->lstar, c->stream));
@@ -1133,8 +1191,8 @@ int prepare_source(rt_ctx* c, const double* S_in, bool device)
     } else if (c->precision == RT_FP32_SWEEP) {
         CK(launch_pack_pairs(c->g, c->chi, c->S, c->pair, c->plo, c->stream));
         c->stats.launches += 1;
-    } else if (c->precision == RT_DF64 && c->rec_valid && c->rec_op) {
-        // the operator packs its own source planes
+    } else if (c->precision == RT_DF64 && c->rec_valid && (c->rec_op || c->fs_method == RT_FS_SHORT)) {
+        // the operator and the recorded short characteristics pack their own
     } else if (c->precision == RT_DF64) {
         CK(launch_packdf(c->g, c->chi, c->S, c->node4, c->stream));
         c->stats.launches += 1;

@@ -305,6 +305,28 @@ cudaError_t launch_sc64(const Geometry& g, const double* chi, const double* S, c
 cudaError_t launch_lstar_sc64(const Geometry& g, const double* chi, const DirInfo* info,
                               const StepGeo* off, const Bw4d* bw, double* lstar, cudaStream_t st);
 
+// ---- short characteristics with recorded weights (screc.cu) -----------------
+struct ScView {
+    Geometry g;
+    const double *chi, *S, *B, *G;
+    const float2 *chi2, *S2;        // double-float: chi and S as pairs
+    const DirInfo* info;
+    const StepGeo* off;
+    const Bw4d* bw;
+    const float4* bwdf;             // double-float: launch_bw_df
+};
+// Bytes of the recorded weights of every (direction, voxel).
+__host__ __device__ __forceinline__ long long sc_rec_bytes(const Geometry& g, bool df)
+{
+    return (df ? 16LL : 24LL) * g.ndir * g.N;
+}
+cudaError_t launch_sc_pairs(long long N, const double* x, float2* out, cudaStream_t st);
+cudaError_t launch_sc_record(const ScView& p, bool df, void* coef, cudaStream_t st);
+// J of the source p.S; part and gplanes as launch_sc64 (8 bytes per value).
+cudaError_t launch_sc_apply(const ScView& p, bool df, const void* coef, double wsum, void* part,
+                            void* gplanes, double* J, unsigned long long* steps, cudaStream_t st);
+cudaError_t launch_sc_lstar(const ScView& p, bool df, const void* coef, double* lstar, cudaStream_t st);
+
 // ---- FP32-sweep form (fs32.cu) ---------------------------------------------
 // poff[d][m]: offset of the upstream node (x0, y0) of step m from the
 // voxel's own entry in planes of `rows` padded rows of 2nx entries
