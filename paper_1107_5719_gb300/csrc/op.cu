@@ -374,7 +374,7 @@ __global__ void k_op_offsets(Geometry g, OpLists L, const int* __restrict__ cnt,
 // point: T_{L-1} w_up), and per voxel and slot sum_d w_d w_cur,0 and
 // sum_d w_d T_L I_bc (rays that reach the boundary plane).  The lengths are
 // given (k_op_len), so the march carries no intensity, no source and no
-// cutoff test: 24 of the 32 FP64 instructions per step of the march that
+// cutoff test: about 21 FP64 instructions per step of the march that
 // also forms I (the FP64 pipe bounds both).
 __global__ void __launch_bounds__(kOpThreads)
 k_rec64(Geometry g, int r0, const double* __restrict__ chi, const double* __restrict__ B,
@@ -442,7 +442,7 @@ k_rec64(Geometry g, int r0, const double* __restrict__ chi, const double* __rest
 // list order (eight coefficient loads in flight) and stores an entry when its
 // last contribution is in.  Rows past the warp's own rays hold nothing
 // (m > its length) and count as zero.
-constexpr int kAsmRun = 16;      // entries of a run (even)
+constexpr int kAsmRun = 32;      // entries of a run (even)
 
 // The two arithmetics of the coefficients: FP64, or double-float pairs.
 struct AsmF64 {
@@ -482,7 +482,7 @@ struct AsmDF {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(kListThreads)
+__global__ void __launch_bounds__(kListThreads, 4)
 k_op_assemble(Geometry g, int r0, OpLists L, RecOut ro, const int* __restrict__ lmax, int nwp,
               const int* __restrict__ cnt, const int* __restrict__ segb, const int* __restrict__ E,
               const long long* __restrict__ eb, typename T::V* __restrict__ A)
