@@ -1402,10 +1402,9 @@ int os_graph_done(rt_ctx* c, int* sweeps)
     return RT_OK;
 }
 
-// The context's arrays as a task of launch_os_solve (its barrier word behind
-// the deltas).
-OsTask os_task(const rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew, double* dlt,
-               int max_sweeps, int* sweeps, int nblk)
+// The context's arrays as a task of launch_os_solve.
+OsTask os_task(const rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew, double* words,
+               int* sweeps, int nblk)
 {
     OsTask t;
     t.g = c->g;
@@ -1416,8 +1415,7 @@ OsTask os_task(const rt_ctx* c, const double* Jfs, const double* Jold, double* J
     t.Ja = c->Ja;
     t.Jb = c->Jb;
     t.Jn = Jnew;
-    t.dlt = dlt;
-    t.bar = reinterpret_cast<unsigned*>(dlt + max_sweeps);
+    t.words = reinterpret_cast<unsigned long long*>(words);
     t.sweeps = sweeps;
     t.nblk = nblk;
     return t;
@@ -1444,9 +1442,10 @@ int run_os_one(rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew, d
     os_solve_shape(c->g.N, c->num_sms, c->os_method == RT_OS_GAUSS_SEIDEL, &sh);
     if (sh.blocks == 0) return RT_OK;
     int rc;
-    if ((rc = ensure_dlt(c, max_sweeps + kPassSweeps)) || (rc = ensure_sweep_words(c))) return rc;
-    CK(cudaMemsetAsync(c->dlt, 0, sizeof(double) * (max_sweeps + 1), c->stream));
-    const OsTask t = os_task(c, Jfs, Jold, Jnew, c->dlt, max_sweeps, c->d_sw, sh.blocks);
+    const int words = max_sweeps * (c->os_method == RT_OS_GAUSS_SEIDEL ? 2 : 1);
+    if ((rc = ensure_dlt(c, std::max(words, max_sweeps + kPassSweeps))) || (rc = ensure_sweep_words(c))) return rc;
+    CK(cudaMemsetAsync(c->dlt, 0, sizeof(double) * words, c->stream));
+    const OsTask t = os_task(c, Jfs, Jold, Jnew, c->dlt, c->d_sw, sh.blocks);
     if (c->profiling) CK(cudaEventRecord(c->ev[2], c->stream));
     const cudaError_t e = launch_os_solve(t, nullptr, nullptr, 1, sh, c->os_method == RT_OS_GAUSS_SEIDEL,
                                           c->num_sms, max_sweeps, tol_inner, c->stream);
@@ -1727,11 +1726,11 @@ struct rt_batch {
     bool use_graphs = true;
     // the active problems' solves in one kernel (launch_os_solve), where their
     // blocks are resident together: tasks and first blocks (device, pinned
-    // copies), deltas and barrier words of all problems
+    // copies), barrier words of all problems
     OsTask *d_tasks = nullptr, *h_tasks = nullptr;
     int *d_first = nullptr, *h_first = nullptr;
     double* d_bdlt = nullptr;
-    int bdlt_cap = 0;               // sweeps per problem it holds
+    int bdlt_cap = 0;               // words per problem it holds
     bool os_one = false;            // the last step ran that way
     int* d_sweeps = nullptr;        // sweeps of each problem's last OS step
     int* h_sweeps = nullptr;        // pinned
@@ -2187,18 +2186,19 @@ int batch_os_one(rt_batch* b, const std::vector<int>& act, double tol_inner, int
         BCK(cudaMallocHost((void**)&b->h_tasks, sizeof(OsTask) * P));
         BCK(cudaMallocHost((void**)&b->h_first, sizeof(int) * P));
     }
-    if (b->bdlt_cap < max_sweeps + 1) {
+    const int words = max_sweeps * (method == RT_OS_GAUSS_SEIDEL ? 2 : 1);
+    if (b->bdlt_cap < words) {
         dfree(b->d_bdlt);
         b->bdlt_cap = 0;
-        BCK(cudaMalloc((void**)&b->d_bdlt, sizeof(double) * (size_t)P * (max_sweeps + 1)));
-        b->bdlt_cap = max_sweeps + 1;
+        BCK(cudaMalloc((void**)&b->d_bdlt, sizeof(double) * (size_t)P * words));
+        b->bdlt_cap = words;
     }
     const long long per = (long long)sh.threads * sh.voxels;
     sh.blocks = 0;
     for (size_t q = 0; q < act.size(); ++q) {
         rt_ctx* c = b->ctx[act[q]];
         const int nblk = (int)((c->g.N + per - 1) / per);
-        b->h_tasks[q] = os_task(c, c->Jfs, c->J, c->Jn, b->d_bdlt + q * (max_sweeps + 1), max_sweeps,
+        b->h_tasks[q] = os_task(c, c->Jfs, c->J, c->Jn, b->d_bdlt + q * words,
                                 b->d_sweeps + act[q], nblk);
         b->h_first[q] = sh.blocks;
         sh.blocks += nblk;
@@ -2207,7 +2207,7 @@ int batch_os_one(rt_batch* b, const std::vector<int>& act, double tol_inner, int
                         b->stream));
     BCK(cudaMemcpyAsync(b->d_first, b->h_first, sizeof(int) * act.size(), cudaMemcpyHostToDevice,
                         b->stream));
-    BCK(cudaMemsetAsync(b->d_bdlt, 0, sizeof(double) * act.size() * (max_sweeps + 1), b->stream));
+    BCK(cudaMemsetAsync(b->d_bdlt, 0, sizeof(double) * act.size() * words, b->stream));
     if (b->profiling) BCK(cudaEventRecord(b->ev[2], b->stream));
     const cudaError_t e = launch_os_solve(b->h_tasks[0], b->d_tasks, b->d_first, (int)act.size(), sh,
                                           method == RT_OS_GAUSS_SEIDEL, b->num_sms, max_sweeps, tol_inner,

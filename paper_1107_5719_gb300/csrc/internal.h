@@ -557,19 +557,20 @@ cudaError_t launch_sweep_pass(const Geometry& g, const double* coef, const doubl
                               bool gs, cudaGraphConditionalHandle h, cudaStream_t st);
 // A whole operator-splitting solve in one cooperative launch (its blocks wait
 // on one another): right-hand side, sweeps to tol or max_sweeps, J_new and
-// the sweep count.  bar and dlt[0..max_sweeps) zeroed before; *sweeps = -1 if
-// a wait gave up.  Several problems (tasks, their first blocks first[q]) run
+// the sweep count.  words (one per barrier: one per sweep, two of a Gauss-Seidel
+// sweep) zeroed before; *sweeps = -1 if a wait gave up.  Several problems (tasks, their first blocks first[q]) run
 // beside each other, each with its own barrier and stopping test.
 struct OsTask {
     Geometry g;
     const double *c, *rdiag, *Jfs, *Jold;
-    double *Ja, *Jb, *Jn, *dlt;
-    unsigned* bar;
+    double *Ja, *Jb, *Jn;
+    unsigned long long* words;
     int* sweeps;
     int nblk;       // blocks of this problem
 };
 struct OsShape {
     int threads, voxels, blocks;    // per block, per thread; 0 blocks: not used
+    bool coef;                      // coefficients in shared memory
 };
 void os_solve_shape(long long N, int num_sms, bool gs, OsShape* s);
 cudaError_t launch_os_solve(const OsTask& one, const OsTask* tasks, const int* first, int ntask,

@@ -130,6 +130,29 @@ __device__ __forceinline__ void block_rel_max(const bool (&valid)[V], const doub
     if ((threadIdx.x & 31) == 0 && u) atomicMax((unsigned long long*)out, u);
 }
 
+// !(|a - b| / |a| < tol), the quotient formed only where the FP32 estimate f
+// does not decide it: f < lo or hi <= f < inf, lo and hi 2^-18 off tol.
+struct TolTest {
+    double tol;
+    float lo, hi;
+};
+__device__ __forceinline__ TolTest tol_test(double tol)
+{
+    TolTest t{tol, 0.f, __int_as_float(0x7f800000)};
+    if (tol > 1e-30) {
+        t.lo = (float)tol * (1.0f - 3.8e-6f);
+        t.hi = (float)tol * (1.0f + 3.8e-6f);
+    }
+    return t;
+}
+__device__ __forceinline__ bool not_below(double a, double b, const TolTest& t)
+{
+    const float f = rel_screen(a, b);
+    if (f < t.lo) return false;
+    if (f >= t.hi && f < __int_as_float(0x7f800000)) return true;
+    return !(rel_change(a, b) < t.tol);
+}
+
 __global__ void k_source(long long N, const double* __restrict__ eps, const double* __restrict__ B,
                          const double* __restrict__ J, double* __restrict__ S,
                          float* __restrict__ S32, const double* __restrict__ Bbound,
@@ -384,37 +407,93 @@ k_gs_half(Geometry g, const double* __restrict__ c, const double* __restrict__ r
 // of the problem's blocks after each (half) sweep instead of a kernel
 // boundary: on grids whose sweep is shorter than the gap between graph nodes
 // the solve is bound by those gaps (17^3: 10 us per sweep in the graph's
-// WHILE loop).  The coefficients stay in L1 or L2; the iterates are exchanged
-// through L2.  Arithmetic and stopping rule are those of the sweep kernels.
+// WHILE loop).  The iterates are exchanged through L2.  Arithmetic and
+// stopping rule are those of the sweep kernels.
+//
+// A sweep of a small grid is a chain of latencies (17^3, one warp per SM, in
+// cycles): 2000 for the sum, whose 26 dependent FP64 multiply-adds take 68
+// each, 230 for the convergence test, 970 until the stores are visible, 2100
+// for the barrier's atomic and polls, 550 for the fence behind it.  So the
+// neighbours are loaded together before the first of them is used, the
+// coefficients wait in shared memory (SM: the fences empty L1), the test forms
+// no quotient that its FP32 estimate decides (not_below; 1250 before), and the
+// test's result travels in the barrier's word.  Solve to 1e-12, 26 sweeps:
+// 17^3 0.148 -> 0.111 ms, 33^3 0.173 -> 0.149, 65^3 (bound by the FP64 pipe)
+// 0.63 -> 0.56.
 
-// Arrive and wait for the problem's blocks; polls at most kBarPolls times
-// (about a second), then reports failure.
+// Barrier of the problem's blocks: returns how many of them had a voxel that
+// has not met the tolerance (more), or -1 when a wait gave up, after at most
+// kBarPolls polls (about a second).  The word (zero before) counts the
+// arrivals in its low half and those blocks in its high half, so that one
+// atomic and one polled load carry both.
 constexpr int kBarPolls = 1 << 21;
-__device__ __forceinline__ bool os_barrier(unsigned* bar, unsigned target, int* failed)
+__device__ __forceinline__ int os_barrier(unsigned long long* word, int nblk, bool more)
 {
-    __syncthreads();
+    __shared__ int result;
+    const bool any = __syncthreads_or(more);
     if (threadIdx.x == 0) {
         __threadfence();
-        atomicAdd(bar, 1u);
+        atomicAdd(word, any ? (1ull << 32) + 1 : 1ull);
         int n = 0;
-        unsigned v;
-        do {
-            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-        } while (v < target && ++n < kBarPolls);
-        *failed = v < target;
+        unsigned long long v;
+        do
+            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(word) : "memory");
+        while ((int)v < nblk && ++n < kBarPolls);
         __threadfence();
+        result = (int)v < nblk ? -1 : (int)(v >> 32);
     }
     __syncthreads();
-    return !*failed;
+    return result;
 }
 
-template <bool GS, int V>
-__global__ void __launch_bounds__(256, 4)
+// acc + sum over the 26 neighbours as in stencil / gs_update (same order), the
+// coefficients in shared memory cs apart, the neighbours loaded together
+// before the first of them is used.
+template <bool GS>
+__device__ __forceinline__ double os_update(const Geometry& g, const double* c, int cs,
+                                            const double* same, const double* other, int i, int j,
+                                            int k, int colour, double acc)
+{
+    const int nx = g.nx, ny = g.ny, nxy = nx * ny;
+    const int xs[3] = {wrap1(i - 1, nx), i, wrap1(i + 1, nx)};
+    const int ys[3] = {wrap1(j - 1, ny), j, wrap1(j + 1, ny)};
+    double x[27];
+#pragma unroll
+    for (int oz = 0; oz < 3; ++oz) {
+        int kk = k + oz - 1;
+        if (kk < 0 || kk >= g.nz) kk = k;       // read, not used
+#pragma unroll
+        for (int oy = 0; oy < 3; ++oy) {
+            const int row = kk * nxy + ys[oy] * nx;
+#pragma unroll
+            for (int ox = 0; ox < 3; ++ox) {
+                const int o = oz * 9 + oy * 3 + ox;
+                x[o] = 0.0;
+                if (o == 13) continue;
+                const double* src = GS && ((xs[ox] + ys[oy] + kk) & 1) == colour ? same : other;
+                RT_GUARD(g, row + xs[ox], g.N, GS ? kSiteGs : kSiteStencil) continue;
+                x[o] = __ldcg(src + row + xs[ox]);
+            }
+        }
+    }
+#pragma unroll
+    for (int oz = 0; oz < 3; ++oz) {
+        if (k + oz - 1 < 0 || k + oz - 1 >= g.nz) continue;
+#pragma unroll
+        for (int o = oz * 9; o < oz * 9 + 9; ++o)
+            if (o != 13) acc = fma(c[o * cs], x[o], acc);
+    }
+    return acc;
+}
+
+template <bool GS, int V, bool SM>
+__global__ void __launch_bounds__(256, SM ? 2 : 4)
 k_os_solve(OsTask one, const OsTask* __restrict__ tasks, const int* __restrict__ first, int ntask,
            int max_sweeps, double tol)
 {
+    extern __shared__ double coef[];            // SM: [V][27][threads]
     __shared__ OsTask T;
-    __shared__ int failed, sblk;
+    __shared__ int sblk;
     if (threadIdx.x == 0) {
         int q = 0;
         if (tasks) {
@@ -425,7 +504,6 @@ k_os_solve(OsTask one, const OsTask* __restrict__ tasks, const int* __restrict__
             T = one;
             sblk = blockIdx.x;
         }
-        failed = 0;
     }
     __syncthreads();
     const Geometry& g = T.g;
@@ -446,48 +524,50 @@ k_os_solve(OsTask one, const OsTask* __restrict__ tasks, const int* __restrict__
         vi[h] = t - vj[h] * nx;
         ci[h] = GS ? split_index(g, vi[h], vj[h], vk[h]) : at[h];
         rv[h] = cur[h] = old[h] = 0.0;
+        if (SM)                                 // each thread reads its own
+            for (int o = 0; o < 27; ++o)
+                coef[(h * 27 + o) * blockDim.x + threadIdx.x] = __ldg(T.c + o * cs + ci[h]);
         if (mine[h]) {
             rv[h] = T.Jfs[at[h]] * T.rdiag[ci[h]] -
                     stencil<false>(g, T.c, T.Jold, vi[h], vj[h], vk[h], ci[h], cs, 0.0);
             cur[h] = T.Jold[at[h]];
         }
     }
-    unsigned target = 0;
-    int n = 0;
+    const TolTest tt = tol_test(tol);
+    unsigned long long* word = T.words;
+    int n = 0, left = 0;
     for (;; ++n) {
         const double* src = n == 0 ? T.Jold : (n & 1) ? T.Ja : T.Jb;
         double* dst = (n & 1) ? T.Jb : T.Ja;
 #pragma unroll
         for (int h = 0; h < V; ++h) old[h] = cur[h];
-        if (GS) {
-            for (int colour = 0; colour < 2; ++colour) {
-#pragma unroll
-                for (int h = 0; h < V; ++h) {
-                    if (!mine[h] || ((vi[h] + vj[h] + vk[h]) & 1) != colour) continue;
-                    cur[h] = gs_update<true>(g, T.c, src, colour ? dst : src, vi[h], vj[h], vk[h], ci[h],
-                                             colour, rv[h]);
-                    dst[at[h]] = cur[h];
-                }
-                if (colour == 0) {
-                    target += T.nblk;
-                    if (!os_barrier(T.bar, target, &failed)) break;
-                }
+        for (int colour = 0; colour < (GS ? 2 : 1); ++colour) {
+            if (colour) {
+                left = os_barrier(word++, T.nblk, false);
+                if (left < 0) break;
             }
-            if (failed) break;
-        } else {
 #pragma unroll
             for (int h = 0; h < V; ++h) {
-                if (!mine[h]) continue;
-                cur[h] = stencil<true, true>(g, T.c, src, vi[h], vj[h], vk[h], ci[h], cs, rv[h]);
+                if (!mine[h] || (GS && ((vi[h] + vj[h] + vk[h]) & 1) != colour)) continue;
+                const double* other = colour ? dst : src;
+                if (SM)
+                    cur[h] = os_update<GS>(g, coef + h * 27 * blockDim.x + threadIdx.x, blockDim.x, src, other,
+                                           vi[h], vj[h], vk[h], colour, rv[h]);
+                else if (GS)
+                    cur[h] = gs_update<true>(g, T.c, src, other, vi[h], vj[h], vk[h], ci[h], colour, rv[h]);
+                else
+                    cur[h] = stencil<true, true>(g, T.c, src, vi[h], vj[h], vk[h], ci[h], cs, rv[h]);
                 dst[at[h]] = cur[h];
             }
         }
-        block_rel_max<V>(mine, cur, old, T.dlt + n);
-        target += T.nblk;
-        if (!os_barrier(T.bar, target, &failed)) break;
-        if (n + 1 >= max_sweeps || __ldcg(T.dlt + n) < tol) break;
+        if (left < 0) break;
+        bool more = false;
+#pragma unroll
+        for (int h = 0; h < V; ++h) more |= mine[h] && not_below(cur[h], old[h], tt);
+        left = os_barrier(word++, T.nblk, more);
+        if (left <= 0 || n + 1 >= max_sweeps) break;
     }
-    if (failed) {
+    if (left < 0) {
         if (threadIdx.x == 0) *T.sweeps = -1;
         return;
     }
@@ -707,14 +787,19 @@ cudaError_t launch_sweep_pass(const Geometry& g, const double* coef, const doubl
 
 // Threads per block, voxels per thread and blocks for N voxels (0 blocks: the
 // sweeps run as kernels of a graph): few voxels are spread over all SMs, one
-// warp each at least.  Measured per solve to 1e-12 (about 25 sweeps), graph
-// against one kernel: 17^3 0.24 / 0.15 ms, 33^3 0.27 / 0.18, 65^3 0.72 / 0.63
+// warp each at least.  Measured per solve to 1e-12 (20 to 31 sweeps), graph
+// against one kernel: 17^3 0.24 / 0.11 ms, 33^3 0.27 / 0.15, 65^3 0.72 / 0.56
 // (two voxels per thread); Gauss-Seidel, half of whose threads wait in each
-// half sweep, 17^3 0.51 (host loop) / 0.23, but 61 x 45 x 52 0.05 ms slower
-// than the graph, so it stops earlier.
+// half sweep, 17^3 0.51 (host loop) / 0.16, but 61 x 45 x 52 0.05 ms slower
+// than the graph, so it stops earlier.  The coefficients lie in shared memory
+// up to kSmVoxels voxels per SM: 24^3 0.138 without / 0.115 ms with, 33^3
+// 0.151 / 0.150, but 41^3 0.199 / 0.212 and 48^3 0.25 / 0.35, since the
+// threads of two blocks (the registers of 26 neighbours) hide less.
+constexpr int kSmVoxels = 256;
 void os_solve_shape(long long N, int num_sms, bool gs, OsShape* s)
 {
     const long long per = (N + num_sms - 1) / num_sms;      // voxels per SM
+    s->coef = per <= kSmVoxels;
     s->threads = per <= 32 ? 32 : per <= 64 ? 64 : per <= 128 ? 128 : 256;
     s->voxels = per <= 1024 ? 1 : 2;
     const long long b = (N + (long long)s->threads * s->voxels - 1) / ((long long)s->threads * s->voxels);
@@ -722,18 +807,21 @@ void os_solve_shape(long long N, int num_sms, bool gs, OsShape* s)
 }
 
 namespace {
-template <bool GS, int V>
-cudaError_t os_solve(const OsTask& one, const OsTask* tasks, const int* first, int ntask, int blocks,
-                     int threads, int num_sms, int max_sweeps, double tol, cudaStream_t st)
+template <typename K>
+cudaError_t os_launch(K kernel, const OsTask& one, const OsTask* tasks, const int* first, int ntask,
+                      const OsShape& s, int num_sms, int max_sweeps, double tol, cudaStream_t st)
 {
+    const size_t smem = s.coef ? sizeof(double) * 27 * s.voxels * s.threads : 0;
     int per = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_os_solve<GS, V>, threads, 0);
+    cudaError_t e = cudaSuccess;
+    if (smem > 48 * 1024)
+        e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kernel, s.threads, smem);
     if (e != cudaSuccess) return e;
-    if ((long long)per * num_sms < blocks) return cudaErrorCooperativeLaunchTooLarge;
+    if ((long long)per * num_sms < s.blocks) return cudaErrorCooperativeLaunchTooLarge;
     void* args[] = {(void*)&one, (void*)&tasks, (void*)&first, (void*)&ntask, (void*)&max_sweeps,
                     (void*)&tol};
-    return cudaLaunchCooperativeKernel((const void*)k_os_solve<GS, V>, dim3(blocks), dim3(threads), args,
-                                       0, st);
+    return cudaLaunchCooperativeKernel((const void*)kernel, dim3(s.blocks), dim3(s.threads), args, smem, st);
 }
 }  // namespace
 
@@ -741,15 +829,10 @@ cudaError_t launch_os_solve(const OsTask& one, const OsTask* tasks, const int* f
                             const OsShape& s, bool gs, int num_sms, int max_sweeps, double tol,
                             cudaStream_t st)
 {
-    if (gs)
-        return s.voxels == 1 ? os_solve<true, 1>(one, tasks, first, ntask, s.blocks, s.threads, num_sms,
-                                                 max_sweeps, tol, st)
-                             : os_solve<true, 2>(one, tasks, first, ntask, s.blocks, s.threads, num_sms,
-                                                 max_sweeps, tol, st);
-    return s.voxels == 1 ? os_solve<false, 1>(one, tasks, first, ntask, s.blocks, s.threads, num_sms,
-                                              max_sweeps, tol, st)
-                         : os_solve<false, 2>(one, tasks, first, ntask, s.blocks, s.threads, num_sms,
-                                              max_sweeps, tol, st);
+    auto kernel = s.coef        ? (gs ? k_os_solve<true, 1, true> : k_os_solve<false, 1, true>)
+                  : s.voxels == 1 ? (gs ? k_os_solve<true, 1, false> : k_os_solve<false, 1, false>)
+                                  : (gs ? k_os_solve<true, 2, false> : k_os_solve<false, 2, false>);
+    return os_launch(kernel, one, tasks, first, ntask, s, num_sms, max_sweeps, tol, st);
 }
 
 cudaError_t launch_os_select(long long N, const double* dlt, int max_sweeps, double tol,
