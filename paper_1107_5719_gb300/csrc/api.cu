@@ -69,7 +69,7 @@ struct rt_ctx {
     long long rec_mode = -1;
     FsRec rec{};
     Rec32 rec32{};              // the FP32-sweep recording (same memory block)
-    float4* spair = nullptr;    // the replay's source records
+    float2* srec = nullptr;    // the replay's source records
     char* rec_mem = nullptr;
     long long rec_cap = 0;
     bool rec_valid = false;
@@ -224,7 +224,7 @@ void free_rec(rt_ctx* c)
     c->rec32 = Rec32{};
     c->op = OpMap{};
     c->rec_op = false;
-    c->spair = nullptr;
+    c->srec = nullptr;
     c->rec_cap = 0;
     c->rec_valid = false;
 }
@@ -361,7 +361,7 @@ long long rec_need(const rt_ctx* c)
     const long long npair = (long long)c->g.nx * ((c->g.ny + 1) / 2), nwp = (npair + 31) / 32;
     return up256((long long)c->g.ndir * rec32_steps4(c->g.nz) * nwp * 32 * (long long)sizeof(float2)) +
            up256((long long)c->g.ndir * c->g.nz * nwp * (long long)sizeof(int)) + 2 * b_slot +
-           up256(pair_records(c->g) * (long long)sizeof(float4));
+           up256(pair_records(c->g) * (long long)sizeof(float2));
 }
 
 // The ray-by-ray recording: whether this context records and replays its
@@ -406,7 +406,7 @@ int ensure_rec(rt_ctx* c, bool& use)
         const long long b_coef = up256((long long)c->g.ndir * rec32_steps4(c->g.nz) * nwp * 32 *
                                        (long long)sizeof(float2));
         const long long b_lmax = up256((long long)c->g.ndir * c->g.nz * nwp * (long long)sizeof(int));
-        const long long b_sp = up256(pair_records(c->g) * (long long)sizeof(float4));
+        const long long b_sp = up256(pair_records(c->g) * (long long)sizeof(float2));
         if (!rec_reserve(c, b_coef + b_lmax + 2 * b_slot + b_sp)) return RT_OK;
         char* q = c->rec_mem;
         c->rec32.coef = reinterpret_cast<float2*>(q);
@@ -414,7 +414,7 @@ int ensure_rec(rt_ctx* c, bool& use)
         c->rec32.tsum = reinterpret_cast<double*>(q + b_coef + b_lmax);
         c->rec32.bc = reinterpret_cast<double*>(q + b_coef + b_lmax + b_slot);
         c->rec32.nwp = (int)nwp;
-        c->spair = reinterpret_cast<float4*>(q + b_coef + b_lmax + 2 * b_slot);
+        c->srec = reinterpret_cast<float2*>(q + b_coef + b_lmax + 2 * b_slot);
     }
     use = true;
     return RT_OK;
@@ -1135,8 +1135,8 @@ int run_fs(rt_ctx* c, double* Jout, bool count_steps)
             c->stats.launches += 1;
         }
         if (use && c->rec_valid) {
-            CK(launch_pack_spairs(c->g, c->fin == 2 ? c->dS : c->S, c->spair, c->stream));
-            Rep32 rp{c->g, c->spair, c->info, c->poff32, c->bw32, c->rec32, c->partial,
+            CK(launch_pack_srecs(c->g, c->fin == 2 ? c->dS : c->S, c->srec, c->stream));
+            Rep32 rp{c->g, c->srec, c->info, c->poff32, c->bw32, c->rec32, c->partial,
                      c->fin == 2 ? 1 : 0, plane_major32(c->g, c->order32)};
             CK(launch_fs32rep(rp, G, c->threads32, sp, c->stream));
             c->stats.launches += 1;
@@ -1890,7 +1890,7 @@ void batch_release(rt_batch* b, int p)
         c->rec32 = Rec32{};
         c->op = OpMap{};
         c->rec_op = false;
-        c->spair = nullptr;
+        c->srec = nullptr;
         c->rec_valid = false;
     }
     if (c->ow_mem) {
@@ -2071,9 +2071,9 @@ int batch_fs(rt_batch* b, const std::vector<int>& act)
                 c->rec_valid = true;
                 b->stats.launches += 1;
             }
-            BCK(launch_pack_spairs(c->g, c->fin == 2 ? c->dS : c->S, c->spair, b->stream));
+            BCK(launch_pack_srecs(c->g, c->fin == 2 ? c->dS : c->S, c->srec, b->stream));
             b->stats.launches += 1;
-            b->h_rviews[p] = Rep32{c->g, c->spair, c->info, c->poff32, c->bw32, c->rec32,
+            b->h_rviews[p] = Rep32{c->g, c->srec, c->info, c->poff32, c->bw32, c->rec32,
                                    c->partial, c->fin == 2 ? 1 : 0, plane_major32(c->g, c->order32)};
             b->h_rids[rq] = p;
             b->h_rprefix[rq] = rtotal;

@@ -67,14 +67,10 @@ constexpr int kResident32 = kThreads32 * kMinBlocks32;
 // The fused batch launch keeps six blocks (80 registers): at seven it
 // spills in the loop, 171 against 157 ms per launch of 16 x 65^3 problems.
 constexpr int kResidentB32 = kThreads32 * RT_FS32B_MINB;
-#ifndef RT_FS32R_MINB
-#define RT_FS32R_MINB 8
-#endif
-// The replay of the recorded march: eight blocks (64 registers), since its
-// loads wait on memory more than its arithmetic; measured on the 65^3 slab,
-// 6.14 ms per replay against 6.49 at seven blocks (72 registers); at ten
-// blocks it spills 800 bytes per thread.
-constexpr int kResidentR32 = kThreads32 * RT_FS32R_MINB;
+// The replay of the recorded march: eight blocks (64 registers); 65^3 slab
+// 6.06 ms with eight, 6.02 with nine (which spill a little), 6.6 with ten and
+// 6.35 with six.
+constexpr int kResidentR32 = kThreads32 * 8;
 
 
 // poff[d][m] = offset of the upstream node (x0, y0) of step m from the
@@ -117,9 +113,9 @@ __global__ void k_pack_pairs(Geometry g, const double* __restrict__ chi,
     }
 }
 
-// The replay's source records: spair[k][y][x] = {S_hi, S_lo} of the nodes
-// (x mod nx, y mod ny) and (x+1 mod nx, y mod ny), padded as k_pack_pairs.
-__global__ void k_pack_spairs(Geometry g, const double* __restrict__ S, float4* __restrict__ sp)
+// The replay's source records: srec[k][y][x] = {S_hi, S_lo} of the node
+// (x mod nx, y mod ny), padded as k_pack_pairs.
+__global__ void k_pack_srecs(Geometry g, const double* __restrict__ S, float2* __restrict__ sp)
 {
     const int nx = g.nx, ny = g.ny;
     const long long W = 2LL * nx, R = 2LL * ny + 1, P = R * W;
@@ -127,15 +123,12 @@ __global__ void k_pack_spairs(Geometry g, const double* __restrict__ S, float4* 
     for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < n;
          r += (long long)gridDim.x * blockDim.x) {
         const long long k = r / P, rem = r - k * P;
-        const int y = (int)(rem / W), x = (int)(rem - (long long)y * W);
-        int j = y, i0 = x, i1 = x + 1;
+        int j = (int)(rem / W), i = (int)(rem - j * W);
         while (j >= ny) j -= ny;
-        while (i0 >= nx) i0 -= nx;
-        while (i1 >= nx) i1 -= nx;
-        const long long row = (k * ny + j) * (long long)nx;
-        const double s0 = S[row + i0], s1 = S[row + i1];
-        const float h0 = (float)s0, h1 = (float)s1;
-        sp[r] = make_float4(h0, (float)(s0 - (double)h0), h1, (float)(s1 - (double)h1));
+        while (i >= nx) i -= nx;
+        const double s = S[(k * ny + j) * (long long)nx + i];
+        const float h = (float)s;
+        sp[r] = make_float2(h, (float)(s - (double)h));
     }
 }
 
@@ -484,13 +477,21 @@ k_fs32rec(View32 p, float cut, unsigned long long* __restrict__ steps, Rec32 rec
 }
 
 // Replay of the recorded FP32 march (Rec32) for the source packed in
-// p.spair: per pair of voxels and direction, I - S_0 = sum_m c_m (S(p_m) -
+// p.srec: per pair of voxels and direction, I - S_0 = sum_m c_m (S(p_m) -
 // S_0) over the warp's recorded length (difference form, Kahan sum), then
 // per voxel and slot the boundary sums: partial = sum_d w_d (I_d - S_0) +
 // bc - S_0 tsum (bc omitted for zero boundary intensities).  The interpolated
 // differences are formed as in the march (hi differences exact for nearby
 // values, the lo parts added once).
-template <int TB>
+//
+// Bound by the data pipe of L1 (92%): the records are 8 bytes, a row's two
+// nodes read by two loads of which the second hits the lines of the first;
+// with 16-byte records of both nodes L1 was filled with twice the bytes
+// (6.14 ms).  Two pairs per thread, which share a row, read less but leave too
+// few warps (6.24 ms).  U steps of loads in flight per thread: two for one
+// problem (6.06 ms, 6.13 with four), four in the launch of many problems (the
+// batch of six problems of 25^3 to 41^3 33 ms, 35 with two).
+template <int TB, int U>
 __device__ __forceinline__ void replay32(const Rep32& p, int tile, int k0, int zb, int ZB,
                                          unsigned long long* __restrict__ steps)
 {
@@ -505,8 +506,8 @@ __device__ __forceinline__ void replay32(const Rep32& p, int tile, int k0, int z
         const long long va = (long long)k0 * nxy + (long long)j0 * nx + i0;
         const long long W = 2LL * nx, P = (2LL * ny + 1) * W;
         const long long base = k0 * P + j0 * W + i0;
-        const float4* pa = p.spair + base;
-        const float4 ma = pa[0], mb = pa[W];     // {S_hi, S_lo} of the voxels (and x+1)
+        const float2* pa = p.srec + base;
+        const float2 ma = pa[0], mb = pa[W];     // {S_hi, S_lo} of the voxels
         const float sha = ma.x, sla = ma.y, shb = mb.x, slb = mb.y;
         const double S0a = (double)sha + (double)sla, S0b = (double)shb + (double)slb;
         for (int slot = zb; slot < kSlots; slot += ZB) {
@@ -523,14 +524,15 @@ __device__ __forceinline__ void replay32(const Rep32& p, int tile, int k0, int z
                 auto step = [&](int m, float2 c) {
                     const int o = od[m + 1];
                     const float4 b = bd[m + 1];
-                    const float4* q = pa + o;
-                    const float4 u0 = __ldg(q), u1 = __ldg(q + W), u2 = __ldg(q + 2 * W);
-                    const float dha = b.x * (u0.x - sha) + b.y * (u0.z - sha) + b.z * (u1.x - sha) +
-                                      b.w * (u1.z - sha);
-                    const float dla = b.x * u0.y + b.y * u0.w + b.z * u1.y + b.w * u1.w;
-                    const float dhb = b.x * (u1.x - shb) + b.y * (u1.z - shb) + b.z * (u2.x - shb) +
-                                      b.w * (u2.z - shb);
-                    const float dlb = b.x * u1.y + b.y * u1.w + b.z * u2.y + b.w * u2.w;
+                    const float2* q = pa + o;
+                    const float2 u0 = __ldg(q), v0 = __ldg(q + 1), u1 = __ldg(q + W), v1 = __ldg(q + W + 1),
+                                 u2 = __ldg(q + 2 * W), v2 = __ldg(q + 2 * W + 1);
+                    const float dha = b.x * (u0.x - sha) + b.y * (v0.x - sha) + b.z * (u1.x - sha) +
+                                      b.w * (v1.x - sha);
+                    const float dla = b.x * u0.y + b.y * v0.y + b.z * u1.y + b.w * v1.y;
+                    const float dhb = b.x * (u1.x - shb) + b.y * (v1.x - shb) + b.z * (u2.x - shb) +
+                                      b.w * (v2.x - shb);
+                    const float dlb = b.x * u1.y + b.y * v1.y + b.z * u2.y + b.w * v2.y;
                     const float ya = fmaf(c.x, dha + (dla - sla), Ial);
                     const float ta = Ia + ya;
                     Ial = ya - (ta - Ia);
@@ -541,23 +543,27 @@ __device__ __forceinline__ void replay32(const Rep32& p, int tile, int k0, int z
                     Ib = tb;
                 };
                 int m = 0;
-                // whole blocks of four steps without conditions, so that their
-                // loads can be issued together; then the remaining steps
-                for (; m + 4 <= L; m += 4) {
-                    RT_GUARD(g, base + od[m + 4], P * nz, kSiteFs32) break;
-                    RT_GUARD(g, base + od[m + 4] + 2 * W, P * nz, kSiteFs32) break;
+                // U steps at a time without conditions, so that their loads are
+                // issued together, then the remaining ones
+                for (; m + U <= L; m += U) {
+                    RT_GUARD(g, base + od[m + U], P * nz, kSiteFs32) break;
+                    RT_GUARD(g, base + od[m + U] + 2 * W + 1, P * nz, kSiteFs32) break;
                     // the coefficients are read once: streaming loads, so that
                     // they do not displace the source records from the caches
-                    const float4* c4 = reinterpret_cast<const float4*>(rc + rec32_step(m + 1));
-                    const float4 cA = __ldcs(c4), cB = __ldcs(c4 + 1);
-                    step(m, make_float2(cA.x, cA.y));
-                    step(m + 1, make_float2(cA.z, cA.w));
-                    step(m + 2, make_float2(cB.x, cB.y));
-                    step(m + 3, make_float2(cB.z, cB.w));
+                    float4 c[U / 2];
+#pragma unroll
+                    for (int q = 0; q < U / 2; ++q)
+                        c[q] = __ldcs(reinterpret_cast<const float4*>(rc + rec32_step(m + 1)) + q);
+#pragma unroll
+                    for (int q = 0; q < U / 2; ++q) {
+                        step(m + 2 * q, make_float2(c[q].x, c[q].y));
+                        step(m + 2 * q + 1, make_float2(c[q].z, c[q].w));
+                    }
                 }
+#pragma unroll 1
                 for (; m < L; ++m) {
                     RT_GUARD(g, base + od[m + 1], P * nz, kSiteFs32) break;
-                    RT_GUARD(g, base + od[m + 1] + 2 * W, P * nz, kSiteFs32) break;
+                    RT_GUARD(g, base + od[m + 1] + 2 * W + 1, P * nz, kSiteFs32) break;
                     step(m, __ldcs(rc + rec32_step(m + 1)));
                 }
                 nsteps += (unsigned long long)L * (two ? 2ull : 1ull);
@@ -589,7 +595,7 @@ k_fs32rep(Rep32 p, unsigned long long* __restrict__ steps)
     __syncthreads();
     const int tile = p.pmajor ? blockIdx.y : blockIdx.x;
     const int k0 = p.pmajor ? blockIdx.x : blockIdx.y;
-    replay32<TB>(sp, tile, k0, blockIdx.z, gridDim.z, steps);
+    replay32<TB, 2>(sp, tile, k0, blockIdx.z, gridDim.z, steps);
 }
 
 // The replays of many problems in one launch, blocks assigned to problems
@@ -620,7 +626,7 @@ k_fs32rep_batch(const Rep32* __restrict__ views, const int* __restrict__ ids,
     const int zb = (int)(local / ((long long)tiles * p.g.nz));
     const int tile = p.pmajor ? (int)(tk / p.g.nz) : (int)(tk % tiles);
     const int k0 = p.pmajor ? (int)(tk % p.g.nz) : (int)(tk / tiles);
-    replay32<TB>(p, tile, k0, zb, ZB, steps);
+    replay32<TB, 4>(p, tile, k0, zb, ZB, steps);
 }
 
 int tiles32(const Geometry& g, int tb) { return (g.nx * ((g.ny + 1) / 2) + tb - 1) / tb; }
@@ -746,9 +752,9 @@ cudaError_t launch_pack_pairs(const Geometry& g, const double* chi, const double
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack_spairs(const Geometry& g, const double* S, float4* spair, cudaStream_t st)
+cudaError_t launch_pack_srecs(const Geometry& g, const double* S, float2* srec, cudaStream_t st)
 {
-    k_pack_spairs<<<grid1d(pair_records(g), 256), 256, 0, st>>>(g, S, spair);
+    k_pack_srecs<<<grid1d(pair_records(g), 256), 256, 0, st>>>(g, S, srec);
     return cudaGetLastError();
 }
 

@@ -412,12 +412,12 @@ __host__ __device__ __forceinline__ long long rec32_step(int m)
 {
     return (long long)((m - 1) >> 2) * 128 + ((m - 1) & 3);
 }
-// The replay: the source in spair (k_pack_spairs records), the march's
+// The replay: the source in srec (k_pack_srecs records), the march's
 // geometry tables and block order, the recording; zero_bc: the boundary
 // intensities are zero (the finishing stage's source change).
 struct Rep32 {
     Geometry g;
-    const float4* spair;
+    const float2* srec;
     const DirInfo* info;
     const int* poff;
     const float4* bw;
@@ -426,7 +426,7 @@ struct Rep32 {
     int zero_bc;
     int pmajor;
 };
-cudaError_t launch_pack_spairs(const Geometry& g, const double* S, float4* spair, cudaStream_t st);
+cudaError_t launch_pack_srecs(const Geometry& g, const double* S, float2* srec, cudaStream_t st);
 // Record the march of p (cut at `cut`, the caller's stricter cutoff) into rec.
 cudaError_t launch_fs32rec(const View32& p, double cut, int groups, const Rec32& rec,
                            unsigned long long* steps, cudaStream_t st);
