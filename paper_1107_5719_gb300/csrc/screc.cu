@@ -25,7 +25,7 @@ namespace rt3d {
 
 namespace {
 
-constexpr int kRecThreads = 128, kScrThreads = 256;
+constexpr int kRecThreads = 128;
 
 struct ScCorners {
     int a00, a10, a01, a11;
@@ -58,6 +58,10 @@ struct Sc64 {
     };
     using W = Bw4d;
     static constexpr bool kDiff = false;
+    // threads of a block of the apply kernel, nodes in flight per thread:
+    // bound by the FP64 pipe, 65^3 x 1024 formal solution 6.16 ms with 384
+    // threads and one node (6.43 with 256, 6.76 with two nodes)
+    static constexpr int kThreads = 384, kUnroll = 1;
     static constexpr int kTab = kExpTable;
     using T = double;
     static __device__ __forceinline__ void fill(T* t) { fill_exp_table(t); }
@@ -98,6 +102,10 @@ struct ScDF {
     using C = float4;       // {w_cur, e}, each a pair
     using Coef = float4;
     static constexpr bool kDiff = true;
+    // bound by the latency between the barriers of the planes: 65^3 x 1024
+    // formal solution 3.26 ms with 256 threads, 2.75 with 384, 2.51 with 512,
+    // 2.39 with 640, 3.3 with 768 (whose registers leave one block per SM)
+    static constexpr int kThreads = 640, kUnroll = 2;
     struct W {
         float4 h, l;
     };
@@ -235,11 +243,12 @@ k_sc_rec(ScView p, typename A::C* __restrict__ coef)
 }
 
 template <typename A, bool SMEM>
-__global__ void __launch_bounds__(kScrThreads)
+__global__ void __launch_bounds__(A::kThreads)
 k_sc_apply(ScView p, const typename A::C* __restrict__ coef, int d0, typename A::V* __restrict__ part,
            typename A::V* gplanes, unsigned long long* __restrict__ steps)
 {
     using V = typename A::V;
+    constexpr int kScrThreads = A::kThreads;
     extern __shared__ double2 splanes_raw[];
     const Geometry& g = p.g;
     const int nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny;
@@ -275,7 +284,7 @@ k_sc_apply(ScView p, const typename A::C* __restrict__ coef, int d0, typename A:
         const long long ck = ((long long)d * nz + k) * nxy;
         V* outk = out + (long long)k * nxy;
         int i = if0, j = jf;
-#pragma unroll 2
+#pragma unroll (A::kUnroll)
         for (int t = threadIdx.x; t < nxy; t += kScrThreads) {
             const ScCorners c = sc_corners(i, j, o, nx, ny);
             i += di0;
@@ -413,9 +422,9 @@ cudaError_t sc_apply(const ScView& p, const void* coef, double wsum, void* part,
     for (int d0 = 0; d0 < g.ndir; d0 += chunk) {
         const int nd = g.ndir - d0 < chunk ? g.ndir - d0 : chunk;
         if (smem)
-            k_sc_apply<A, true><<<nd, kScrThreads, shm, st>>>(p, c, d0, pt, gp, steps);
+            k_sc_apply<A, true><<<nd, A::kThreads, shm, st>>>(p, c, d0, pt, gp, steps);
         else
-            k_sc_apply<A, false><<<nd, kScrThreads, 0, st>>>(p, c, d0, pt, gp, steps);
+            k_sc_apply<A, false><<<nd, A::kThreads, 0, st>>>(p, c, d0, pt, gp, steps);
         k_sc_sum<A><<<(unsigned)rb, 256, sizeof(typename A::V) * nd, st>>>(p, d0, nd, pt, wsum, J, d0 > 0);
     }
     return cudaGetLastError();
