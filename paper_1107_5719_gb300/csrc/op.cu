@@ -27,11 +27,15 @@
 // and k_op_apply64 evaluates J for a source.
 #include "df.cuh"
 #include "internal.h"
+
+#include <cooperative_groups.h>
 #include "weights.cuh"
 
 namespace rt3d {
 
 namespace {
+namespace cg = cooperative_groups;
+
 
 constexpr int kOpThreads = 128;      // march and length kernels
 constexpr int kListThreads = 256;
@@ -596,19 +600,47 @@ __global__ void k_op_pack(Geometry g, const double* __restrict__ S, double* __re
     }
 }
 
-// J of a source: one block per 32 voxels of a plane, its warps taking four
-// entries at a time in turn (the block streams its coefficients, 8 bytes per
-// FP64 FMA, in order), then the warps' sums and the voxel's own terms in
-// fixed order.
-template <int NW>
-__global__ void __launch_bounds__(NW * 32, NW < 24 ? 24 / NW : 1)
+// The sums of the NW warps of each of a cluster's C blocks added to a, in
+// fixed order, by warp 0 of its first block (true there).
+template <int NW, int C>
+__device__ __forceinline__ bool tile_sum(double (&red)[NW][32], double mine, double& a)
+{
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    red[wid][lane] = mine;
+    if constexpr (C == 1) {
+        __syncthreads();
+        if (wid != 0) return false;
+        for (int w = 0; w < NW; ++w) a += red[w][lane];
+        return true;
+    } else {
+        cg::cluster_group cl = cg::this_cluster();
+        cl.sync();
+        const bool first = cl.block_rank() == 0 && wid == 0;
+        if (first)
+            for (int b = 0; b < C; ++b) {
+                const double* r = cl.map_shared_rank(&red[0][0], b);
+                for (int w = 0; w < NW; ++w) a += r[w * 32 + lane];
+            }
+        cl.sync();      // the blocks stay until their sums are read
+        return first;
+    }
+}
+
+// J of a source: C blocks (a cluster) per 32 voxels of a plane, their warps
+// taking four entries at a time in turn (they stream the coefficients, 8 bytes
+// per FP64 FMA, in order), then the warps' sums and the voxel's own terms in
+// fixed order.  Bound by the FP64 pipe, so by the SM with the most work: tiles are
+// split over a cluster where an SM has few.
+template <int NWB, int C>
+__global__ void __launch_bounds__(NWB * 32, 24 / NWB)
 k_op_apply64(Geometry g, const double* __restrict__ S, const double* __restrict__ sp, OpMap op,
              double* __restrict__ J, unsigned long long* __restrict__ steps)
 {
-    __shared__ double red[NW][32];
+    constexpr int NW = NWB * C;
+    __shared__ double red[NWB][32];
     const int nx = g.nx, nxy = nx * g.ny;
     const int tile = blockIdx.x, k0 = plane_at(g, blockIdx.y);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, wid = blockIdx.z * NWB + (threadIdx.x >> 5);
     const int t = tile * 32 + lane, tc = t < nxy ? t : 0;
     const int j0 = tc / nx, i0 = tc - j0 * nx;
     const long long at = (long long)k0 * 4 * nxy + (long long)j0 * 2 * nx + i0;
@@ -651,15 +683,10 @@ k_op_apply64(Geometry g, const double* __restrict__ S, const double* __restrict_
         acc0 = fma(b.x, __ldg(s + o.z), acc0);
         acc1 = fma(b.y, __ldg(s + o.w), acc1);
     }
-    red[wid][lane] = acc0 + acc1;
-    __syncthreads();
-    if (wid == 0 && t < nxy) {
-        const long long v = (long long)k0 * nxy + t;
-        double a = fma(op.c0[v], S[v], op.bc[v]);
-        for (int w = 0; w < NW; ++w) a += red[w][lane];
-        J[v] = a;
-    }
-    if (steps && tile == 0 && blockIdx.y == 0 && threadIdx.x == 0) atomicAdd(steps, *op.steps);
+    const long long v = (long long)k0 * nxy + tc;
+    double a = fma(op.c0[v], S[v], op.bc[v]);
+    if (tile_sum<NWB, C>(red, acc0 + acc1, a) && t < nxy) J[v] = a;
+    if (steps && tile == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) atomicAdd(steps, *op.steps);
 }
 
 // S as double-float pairs in the padded planes of k_op_pack.
@@ -701,7 +728,7 @@ __device__ __forceinline__ void diff_add_df(float& h, float& l, float ah, float 
 // difference form: J = sum_e A_e (S_e - S_0) + bc + (wsum - ts) S_0.  22
 // FP32 operations and 8 coefficient bytes per entry: bound by memory.
 template <int NW>
-__global__ void __launch_bounds__(NW * 32, NW < 24 ? 32 / NW : 1)
+__global__ void __launch_bounds__(NW * 32, 32 / NW)
 k_op_apply_df(Geometry g, const double* __restrict__ S, const float2* __restrict__ sp, OpMap op,
               double wsum, double* __restrict__ J, unsigned long long* __restrict__ steps)
 {
@@ -746,14 +773,10 @@ k_op_apply_df(Geometry g, const double* __restrict__ S, const float2* __restrict
     }
     for (; q < nq; q += NW)
         quad(__ldg(off + q), __ldcs(A + (long long)q * 64), __ldcs(A + (long long)q * 64 + 32));
-    red[wid][lane] = ((double)h0 + (double)l0) + ((double)h1 + (double)l1);
-    __syncthreads();
-    if (wid == 0 && t < nxy) {
-        const long long v = (long long)k0 * nxy + t;
-        double a = op.bc[v];
-        for (int w = 0; w < NW; ++w) a += red[w][lane];
+    const long long v = (long long)k0 * nxy + tc;
+    double a = op.bc[v];
+    if (tile_sum<NW, 1>(red, ((double)h0 + (double)l0) + ((double)h1 + (double)l1), a) && t < nxy)
         J[v] = fma(wsum - op.ts[v], S[v], a);
-    }
     if (steps && tile == 0 && blockIdx.y == 0 && threadIdx.x == 0) atomicAdd(steps, *op.steps);
 }
 
@@ -908,32 +931,52 @@ cudaError_t launch_op_own(long long N, const double* c0s, const double* bcs, con
     return cudaGetLastError();
 }
 
-// Below this many tiles 16 warps share one (17^3: 28 against 79 us)
-constexpr long long kFewTiles = 152 * 3;
+namespace {
+// The tiles of the grid with clusters of C blocks per tile.
+template <int NWB, int C, typename K, typename... P>
+cudaError_t launch_tiles(K kernel, dim3 tiles, cudaStream_t st, P... p)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(tiles.x, tiles.y, C);
+    cfg.blockDim = dim3(NWB * 32);
+    cfg.stream = st;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = C;
+    cfg.attrs = &at;
+    cfg.numAttrs = C > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, p...);
+}
+}  // namespace
+
+// How many warps share a tile.  FP64 (the SM with the most work ends it):
+// formal solution of 33^3 with 256 directions (1155 tiles) 367 us with one block
+// of eight warps per tile, 343 with two; 48^3 (3456) 1.38 against 1.37 ms, but
+// 65^3 (8645) 4.58 against 4.61; 17^3 (170) like one block of 16 warps.
+// Double-float (memory, one block): 33^3 319 us with eight warps, 269 with 16;
+// 41^3 616 / 555; 48^3 and 65^3 the same.
+constexpr long long kManyTiles = 4096;
 
 cudaError_t launch_op_apply64(const Geometry& g, const double* S, double* sp, const OpMap& op,
                               double* J, unsigned long long* steps, cudaStream_t st)
 {
     k_op_pack<<<op_grid1d(g.N, 256), 256, 0, st>>>(g, S, sp);
-    const dim3 grid(op.nwp, g.nz);
-    if ((long long)op.nwp * g.nz < kFewTiles)
-        k_op_apply64<16><<<grid, 512, 0, st>>>(g, S, sp, op, J, steps);
-    else
-        k_op_apply64<8><<<grid, 256, 0, st>>>(g, S, sp, op, J, steps);
-    return cudaGetLastError();
+    const dim3 tiles(op.nwp, g.nz);
+    if ((long long)op.nwp * g.nz < kManyTiles)
+        return launch_tiles<8, 2>(k_op_apply64<8, 2>, tiles, st, g, S, sp, op, J, steps);
+    return launch_tiles<8, 1>(k_op_apply64<8, 1>, tiles, st, g, S, sp, op, J, steps);
 }
 
 cudaError_t launch_op_apply_df(const Geometry& g, const double* S, double* sp, const OpMap& op,
                                double wsum, double* J, unsigned long long* steps, cudaStream_t st)
 {
-    float2* p = reinterpret_cast<float2*>(sp);
-    k_op_pack_df<<<op_grid1d(g.N, 256), 256, 0, st>>>(g, S, p);
-    const dim3 grid(op.nwp, g.nz);
-    if ((long long)op.nwp * g.nz < kFewTiles)
-        k_op_apply_df<16><<<grid, 512, 0, st>>>(g, S, p, op, wsum, J, steps);
-    else
-        k_op_apply_df<8><<<grid, 256, 0, st>>>(g, S, p, op, wsum, J, steps);
-    return cudaGetLastError();
+    const float2* p = reinterpret_cast<const float2*>(sp);
+    k_op_pack_df<<<op_grid1d(g.N, 256), 256, 0, st>>>(g, S, reinterpret_cast<float2*>(sp));
+    const dim3 tiles(op.nwp, g.nz);
+    if ((long long)op.nwp * g.nz < kManyTiles)
+        return launch_tiles<16, 1>(k_op_apply_df<16>, tiles, st, g, S, p, op, wsum, J, steps);
+    return launch_tiles<8, 1>(k_op_apply_df<8>, tiles, st, g, S, p, op, wsum, J, steps);
 }
 
 cudaError_t launch_op_lstar(const Geometry& g, bool df, const OpLists& L, const OpMap& op,

@@ -130,3 +130,19 @@ def test_large_operator_in_chunks(R, oracle_mod, form):
             J, _ = s.formal_solution(S, want_lstar=False)
             Jo = oracle_mod.mean_intensity_at(q, S, vox)
             assert np.allclose(J.reshape(-1)[vox], Jo, rtol=RTOL, atol=0)
+
+
+@pytest.mark.parametrize("form", ["linear", "df"])
+@pytest.mark.parametrize("nx,ny,nz", [(3, 11, 127), (3, 11, 128), (64, 32, 63), (64, 32, 64), (63, 33, 65)])
+def test_apply_forms_match_march(R, form, nx, ny, nz):
+    """Both sides of the numbers of tiles (254, 256; 4032, 4096, 4225) at which
+    the warps of a tile change, against the march without recording."""
+    p = W.random_slab(nx, ny, nz, n_theta=2, n_phi=3, seed=nz)
+    p.src_order, prec = _form(R, form)
+    S = 0.5 + np.random.default_rng(6).random(p.B.shape)
+    J = {}
+    for record in (-1, 0):
+        with R.Solver(p, precision=prec, record=record) as s:
+            J[record] = s.formal_solution(S, want_lstar=False)[0]
+            assert R.rt_fs_record_info(s.ctx)[1] == (record != 0)
+    assert np.allclose(J[-1], J[0], rtol=RTOL, atol=0)
