@@ -49,9 +49,13 @@ struct rt_ctx {
     } osg[2];
     int osg_next = 0;
     int* d_nsw = nullptr;     // the graph's sweep counter
-    int* d_sw = nullptr;      // sweeps of the graph's last OS step (device), and a pinned copy
+    int* d_sw = nullptr;      // sweeps of the last OS step (behind scal), and a pinned copy
     int* h_sw = nullptr;
     bool os_one = false;      // the last step ran as one kernel (launch_os_solve)
+    // its barrier words: two sets in turn, each zeroed by the solve before the
+    // one that uses it; words in use and of each set not zero
+    unsigned long long* os_words = nullptr;
+    int os_cap = 0, os_set = 0, os_dirty[2] = {0, 0};
     bool use_graphs = true;
     unsigned long long* berr = nullptr;   // checked builds: out-of-bounds record
     int fs_method = RT_FS_LONG;
@@ -76,6 +80,8 @@ struct rt_ctx {
     // the recording assembled into an operator (rec_op), in the same block;
     // its node lists (per quadrature) and the recording's working storage
     bool rec_op = false;
+    bool op_packed = false;     // the source of the coming formal solution is packed
+    bool op_steps = false;      // h_steps holds the recording's steps
     OpMap op{};
     OpLists ol{};
     char* ol_mem = nullptr;
@@ -123,7 +129,7 @@ struct rt_ctx {
     Bw4d* bwh = nullptr;
     float4* bw32 = nullptr;
     double *d_mu = nullptr, *d_phi = nullptr, *d_w = nullptr;
-    // scalars: [0] smax, [1] inner delta, [2] outer delta
+    // scalars: [0] smax, [2] outer delta, [3] smallest source, [4] sweeps (d_sw)
     double* scal = nullptr;
     unsigned long long* d_steps = nullptr;
     double* h_scal = nullptr;               // pinned
@@ -713,6 +719,7 @@ int ensure_op_rec(rt_ctx* c, int G, bool& use)
         c->stats.launches += 1;
     }
     c->rec_op = op;
+    c->op_steps = false;
     c->rec_valid = true;
     use = true;
     return RT_OK;
@@ -1055,7 +1062,27 @@ int run_fs_short(rt_ctx* c, double* Jout, bool count_steps)
     if (count_steps) {
         CK(cudaMemcpyAsync(c->h_steps, c->d_steps, sizeof(unsigned long long),
                            cudaMemcpyDeviceToHost, c->stream));
+        c->op_steps = false;
     }
+    return RT_OK;
+}
+
+// The formal solution comes from an operator that is there already.
+bool op_ready(const rt_ctx* c)
+{
+    return (c->precision == RT_FP64 || c->precision == RT_DF64) && c->fs_method == RT_FS_LONG &&
+           c->rec_mode != 0 && c->rec_valid && c->rec_op;
+}
+
+// The source packed for the operator, where prepare_source has not (the
+// operator was made in between).
+int op_source(rt_ctx* c)
+{
+    if (!c->op_packed) {
+        CK(launch_op_pack(c->g, c->S, nullptr, nullptr, nullptr, c->precision == RT_DF64, c->ow.sp, c->stream));
+        c->stats.launches += 1;
+    }
+    c->op_packed = false;
     return RT_OK;
 }
 
@@ -1069,6 +1096,7 @@ int df_formal(rt_ctx* c, int G, double* Jout, unsigned long long* steps, bool& d
     if (rc) return rc;
     direct = use && c->rec_op;
     if (direct) {
+        if ((rc = op_source(c))) return rc;
         CK(launch_op_apply_df(c->g, c->S, c->ow.sp, c->op, c->wsum, Jout, steps, c->stream));
         c->stats.launches += 1;
     } else if (use) {
@@ -1092,6 +1120,7 @@ int fs64_formal(rt_ctx* c, int G, double* Jout, unsigned long long* steps, bool&
     direct = use && c->rec_op;
     cudaStream_t st = c->stream;
     if (direct) {
+        if ((rc = op_source(c))) return rc;
         CK(launch_op_apply64(c->g, c->S, c->ow.sp, c->op, Jout, steps, st));
         c->stats.launches += 1;
     } else if (use) {
@@ -1112,6 +1141,8 @@ int run_fs(rt_ctx* c, double* Jout, bool count_steps)
     const int G = auto_groups(c);
     int rc = fs_prepare(c);
     if (rc) return rc;
+    // an operator's steps are those of its recording: counted once
+    count_steps = count_steps && !(op_ready(c) && c->op_steps);
     if (count_steps) CK(cudaMemsetAsync(c->d_steps, 0, sizeof(unsigned long long), c->stream));
     const double cut = cut_of(c);
     if (c->profiling) CK(cudaEventRecord(c->ev[0], c->stream));
@@ -1157,13 +1188,25 @@ int run_fs(rt_ctx* c, double* Jout, bool count_steps)
     if (count_steps) {
         CK(cudaMemcpyAsync(c->h_steps, c->d_steps, sizeof(unsigned long long),
                            cudaMemcpyDeviceToHost, c->stream));
+        c->op_steps = direct;
     }
     return RT_OK;
 }
 
-// S = eps B + (1 - eps) J (or the caller's S), then smax; FP32 copy if needed.
+// S = eps B + (1 - eps) J (or the caller's S), then in the form of the next
+// formal solution: packed for the operator (whose cutoffs are made: no smax),
+// else smax and the FP32 or double-float records.
 int prepare_source(rt_ctx* c, const double* S_in, bool device)
 {
+    c->op_packed = op_ready(c);
+    if (c->op_packed) {
+        if (S_in)
+            CK(cudaMemcpyAsync(c->S, S_in, sizeof(double) * c->g.N, kind(device), c->stream));
+        CK(launch_op_pack(c->g, c->S, S_in ? nullptr : c->eps, c->B, c->J, c->precision == RT_DF64, c->ow.sp,
+                          c->stream));
+        c->stats.launches += 1;
+        return RT_OK;
+    }
     const bool bnd = c->g.top_bc || c->g.bottom_bc;
     CK(cudaMemsetAsync(c->scal + 0, 0, sizeof(double), c->stream));
     if (S_in) {
@@ -1191,8 +1234,8 @@ int prepare_source(rt_ctx* c, const double* S_in, bool device)
     } else if (c->precision == RT_FP32_SWEEP) {
         CK(launch_pack_pairs(c->g, c->chi, c->S, c->pair, c->plo, c->stream));
         c->stats.launches += 1;
-    } else if (c->precision == RT_DF64 && c->rec_valid && (c->rec_op || c->fs_method == RT_FS_SHORT)) {
-        // the operator and the recorded short characteristics pack their own
+    } else if (c->precision == RT_DF64 && c->rec_valid && c->fs_method == RT_FS_SHORT) {
+        // the recorded short characteristics pack their own
     } else if (c->precision == RT_DF64) {
         CK(launch_packdf(c->g, c->chi, c->S, c->node4, c->stream));
         c->stats.launches += 1;
@@ -1402,9 +1445,22 @@ int os_graph_done(rt_ctx* c, int* sweeps)
     return RT_OK;
 }
 
+// Two sets of at least `words` zeroed barrier words (the set in turn).
+int ensure_os_words(rt_ctx* c, int words)
+{
+    if (c->os_cap >= words) return RT_OK;
+    const int cap = std::max(words, 1024);
+    c->os_cap = 0;
+    CK(dalloc(c->os_words, 2 * (size_t)cap));
+    CK(cudaMemsetAsync(c->os_words, 0, sizeof(unsigned long long) * 2 * cap, c->stream));
+    c->os_cap = cap;
+    c->os_dirty[0] = c->os_dirty[1] = 0;
+    return RT_OK;
+}
+
 // The context's arrays as a task of launch_os_solve.
-OsTask os_task(const rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew, double* words,
-               int* sweeps, int nblk)
+OsTask os_task(const rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew,
+               unsigned long long* words, int* sweeps, int nblk)
 {
     OsTask t;
     t.g = c->g;
@@ -1415,7 +1471,10 @@ OsTask os_task(const rt_ctx* c, const double* Jfs, const double* Jold, double* J
     t.Ja = c->Ja;
     t.Jb = c->Jb;
     t.Jn = Jnew;
-    t.words = reinterpret_cast<unsigned long long*>(words);
+    t.words = words;
+    t.clear = nullptr;
+    t.nclear = 0;
+    t.zero = nullptr;
     t.sweeps = sweeps;
     t.nblk = nblk;
     return t;
@@ -1424,18 +1483,15 @@ OsTask os_task(const rt_ctx* c, const double* Jfs, const double* Jold, double* J
 int ensure_sweep_words(rt_ctx* c)
 {
     if (!c->d_nsw) CK(cudaMalloc((void**)&c->d_nsw, sizeof(int)));
-    if (!c->d_sw) {
-        CK(cudaMalloc((void**)&c->d_sw, sizeof(int)));
-        CK(cudaMallocHost((void**)&c->h_sw, sizeof(int)));
-    }
     return RT_OK;
 }
 
 // The operator-splitting step as one cooperative kernel, without waiting for
 // it, where the grid's blocks are resident together; ran: whether it was
-// launched.
+// launched.  In a solve it zeroes the outer delta, and the caller copies that
+// and the sweep count back together.
 int run_os_one(rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew, double tol_inner,
-               int max_sweeps, bool& ran)
+               int max_sweeps, bool in_solve, bool& ran)
 {
     ran = false;
     OsShape sh;
@@ -1443,33 +1499,42 @@ int run_os_one(rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew, d
     if (sh.blocks == 0) return RT_OK;
     int rc;
     const int words = max_sweeps * (c->os_method == RT_OS_GAUSS_SEIDEL ? 2 : 1);
-    if ((rc = ensure_dlt(c, std::max(words, max_sweeps + kPassSweeps))) || (rc = ensure_sweep_words(c))) return rc;
-    CK(cudaMemsetAsync(c->dlt, 0, sizeof(double) * words, c->stream));
-    const OsTask t = os_task(c, Jfs, Jold, Jnew, c->dlt, c->d_sw, sh.blocks);
+    if ((rc = ensure_os_words(c, words))) return rc;
+    const int set = c->os_set;
+    OsTask t = os_task(c, Jfs, Jold, Jnew, c->os_words + (long long)set * c->os_cap, c->d_sw, sh.blocks);
+    t.clear = c->os_words + (long long)(set ^ 1) * c->os_cap;
+    t.nclear = c->os_dirty[set ^ 1];
+    if (in_solve) t.zero = c->scal + 2;
     if (c->profiling) CK(cudaEventRecord(c->ev[2], c->stream));
     const cudaError_t e = launch_os_solve(t, nullptr, nullptr, 1, sh, c->os_method == RT_OS_GAUSS_SEIDEL,
                                           c->num_sms, max_sweeps, tol_inner, c->stream);
     if (e == cudaErrorCooperativeLaunchTooLarge) return RT_OK;
     CK(e);
+    c->os_dirty[set ^ 1] = 0;
+    c->os_dirty[set] = words;
+    c->os_set = set ^ 1;
     if (c->profiling) {
         CK(cudaEventRecord(c->ev[3], c->stream));
         c->jac_pending = true;
     }
-    CK(cudaMemcpyAsync(c->h_sw, c->d_sw, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    if (!in_solve)
+        CK(cudaMemcpyAsync(c->h_sw, c->d_sw, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     c->os_one = ran = true;
     return RT_OK;
 }
 
 int run_os(rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew, double tol_inner,
-           int max_sweeps, int* sweeps_out)
+           int max_sweeps, bool in_solve, int* sweeps_out)
 {
+    c->os_one = false;
     int rc = ensure_coef(c);
     if (rc) return rc;
     if (c->use_graphs) {
         // sweep count after the caller's synchronisation (os_graph_done)
         if (sweeps_out) *sweeps_out = -1;
         bool ran = false;
-        if ((rc = run_os_one(c, Jfs, Jold, Jnew, tol_inner, max_sweeps, ran)) || ran) return rc;
+        if ((rc = run_os_one(c, Jfs, Jold, Jnew, tol_inner, max_sweeps, in_solve, ran)) || ran)
+            return rc;
         return run_os_graph(c, Jfs, Jold, Jnew, tol_inner, max_sweeps);
     }
     if ((rc = ensure_dlt(c, max_sweeps))) return rc;
@@ -1537,7 +1602,7 @@ int os_step(rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew, doub
     }
     double* dnew = device ? Jnew : c->S;  // S is free as scratch here
     int ns = 0;
-    if ((rc = run_os(c, dfs, dold, dnew, tol_inner, max_sweeps, &ns))) return rc;
+    if ((rc = run_os(c, dfs, dold, dnew, tol_inner, max_sweeps, false, &ns))) return rc;
     if (!device)
         CK(cudaMemcpyAsync(Jnew, dnew, sizeof(double) * c->g.N, cudaMemcpyDeviceToHost, c->stream));
     CK(cudaStreamSynchronize(c->stream));
@@ -1557,27 +1622,27 @@ int ensure_ng(rt_ctx* c)
 }
 
 // Ng bookkeeping after iteration `it` (1-based) produced J_new in c->Jn from
-// the previous iterate c->J: remember c->J, and when four iterates are held
+// the previous iterate c->J: have c->J remembered (hist: where the kernel that
+// forms the outer delta copies it), and when four iterates are held
 // and it is a multiple of the period, enqueue the weighted sums and the
 // extrapolation of J_new, whose 2x2 system is solved on the device (no
 // host synchronisation; the iterate is left unchanged if it is singular).
-int ng_push(rt_ctx* c, int it)
+int ng_push(rt_ctx* c, int it, double*& hist)
 {
+    hist = nullptr;
     if (!c->ng_period) return RT_OK;
     int rc = ensure_ng(c);
     if (rc) return rc;
     double* t = c->ng_old[2];
     c->ng_old[2] = c->ng_old[1];
     c->ng_old[1] = c->ng_old[0];
-    c->ng_old[0] = t;
-    CK(cudaMemcpyAsync(c->ng_old[0], c->J, sizeof(double) * c->g.N, cudaMemcpyDeviceToDevice,
-                       c->stream));
+    c->ng_old[0] = hist = t;
     if (c->ng_count < 4) ++c->ng_count;
     if (c->ng_count == 4 && it % c->ng_period == 0 &&
         (it == 1 || c->ng_last_delta >= c->ng_min_delta)) {
-        CK(launch_ng_dots(c->g.N, c->Jn, c->ng_old[0], c->ng_old[1], c->ng_old[2], c->ng_part,
+        CK(launch_ng_dots(c->g.N, c->Jn, c->J, c->ng_old[1], c->ng_old[2], c->ng_part,
                           c->ng_out, c->stream));
-        CK(launch_ng_apply(c->g.N, c->ng_out, c->ng_old[0], c->ng_old[1], c->Jn, c->stream));
+        CK(launch_ng_apply(c->g.N, c->ng_out, c->J, c->ng_old[1], c->Jn, c->stream));
         c->stats.launches += 3;
         c->ng_applied += 1;
         c->ng_count = 1;
@@ -1634,13 +1699,15 @@ int solve(rt_ctx* c, double tol, int max_iter, double tol_inner, int max_sweeps,
         if ((rc = prepare_source(c, nullptr, true))) return rc;
         if ((rc = run_fs(c, c->Jfs, true))) return rc;
         int ns = 0;
-        if ((rc = run_os(c, c->Jfs, c->J, c->Jn, tol_inner, max_sweeps, &ns))) return rc;
-        if ((rc = ng_push(c, it + 1))) return rc;
-        CK(cudaMemsetAsync(c->scal + 2, 0, sizeof(double), c->stream));
-        CK(launch_rel_change(c->g.N, c->Jn, c->J, c->scal + 2, c->stream));
+        if ((rc = run_os(c, c->Jfs, c->J, c->Jn, tol_inner, max_sweeps, true, &ns))) return rc;
+        double* hist = nullptr;
+        if ((rc = ng_push(c, it + 1, hist))) return rc;
+        if (!c->os_one) CK(cudaMemsetAsync(c->scal + 2, 0, sizeof(double), c->stream));
+        CK(launch_rel_change(c->g.N, c->Jn, c->J, c->scal + 2, hist, c->stream));
         c->stats.launches += 1;
-        CK(cudaMemcpyAsync(c->h_scal + 2, c->scal + 2, sizeof(double), cudaMemcpyDeviceToHost,
-                           c->stream));
+        // with the sweep count where the step ran as one kernel
+        CK(cudaMemcpyAsync(c->h_scal + 2, c->scal + 2, sizeof(double) * (c->os_one ? 3 : 1),
+                           cudaMemcpyDeviceToHost, c->stream));
         CK(cudaStreamSynchronize(c->stream));
         c->stats.host_syncs += 1;
         c->stats.iterations += 1;
@@ -1729,7 +1796,7 @@ struct rt_batch {
     // copies), barrier words of all problems
     OsTask *d_tasks = nullptr, *h_tasks = nullptr;
     int *d_first = nullptr, *h_first = nullptr;
-    double* d_bdlt = nullptr;
+    unsigned long long* d_bdlt = nullptr;
     int bdlt_cap = 0;               // words per problem it holds
     bool os_one = false;            // the last step ran that way
     int* d_sweeps = nullptr;        // sweeps of each problem's last OS step
@@ -2190,7 +2257,7 @@ int batch_os_one(rt_batch* b, const std::vector<int>& act, double tol_inner, int
     if (b->bdlt_cap < words) {
         dfree(b->d_bdlt);
         b->bdlt_cap = 0;
-        BCK(cudaMalloc((void**)&b->d_bdlt, sizeof(double) * (size_t)P * words));
+        BCK(cudaMalloc((void**)&b->d_bdlt, sizeof(unsigned long long) * (size_t)P * words));
         b->bdlt_cap = words;
     }
     const long long per = (long long)sh.threads * sh.voxels;
@@ -2207,7 +2274,7 @@ int batch_os_one(rt_batch* b, const std::vector<int>& act, double tol_inner, int
                         b->stream));
     BCK(cudaMemcpyAsync(b->d_first, b->h_first, sizeof(int) * act.size(), cudaMemcpyHostToDevice,
                         b->stream));
-    BCK(cudaMemsetAsync(b->d_bdlt, 0, sizeof(double) * act.size() * words, b->stream));
+    BCK(cudaMemsetAsync(b->d_bdlt, 0, sizeof(unsigned long long) * act.size() * words, b->stream));
     if (b->profiling) BCK(cudaEventRecord(b->ev[2], b->stream));
     const cudaError_t e = launch_os_solve(b->h_tasks[0], b->d_tasks, b->d_first, (int)act.size(), sh,
                                           method == RT_OS_GAUSS_SEIDEL, b->num_sms, max_sweeps, tol_inner,
@@ -2373,9 +2440,9 @@ int rt_create(rt_ctx** out, int device, int precision)
     if (cudaSetDevice(device) != cudaSuccess ||
         cudaStreamCreateWithFlags(&c->own_stream, cudaStreamNonBlocking) != cudaSuccess ||
         cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess ||
-        cudaMalloc((void**)&c->scal, 4 * sizeof(double)) != cudaSuccess ||
+        cudaMalloc((void**)&c->scal, 5 * sizeof(double)) != cudaSuccess ||
         cudaMalloc((void**)&c->d_steps, sizeof(unsigned long long)) != cudaSuccess ||
-        cudaMallocHost((void**)&c->h_scal, 4 * sizeof(double)) != cudaSuccess ||
+        cudaMallocHost((void**)&c->h_scal, 5 * sizeof(double)) != cudaSuccess ||
         cudaMallocHost((void**)&c->h_steps, sizeof(unsigned long long)) != cudaSuccess ||
         cudaEventCreate(&c->ev[0]) != cudaSuccess || cudaEventCreate(&c->ev[1]) != cudaSuccess ||
         cudaEventCreate(&c->ev[2]) != cudaSuccess || cudaEventCreate(&c->ev[3]) != cudaSuccess) {
@@ -2383,6 +2450,8 @@ int rt_create(rt_ctx** out, int device, int precision)
         return RT_ECUDA;
     }
     *c->h_steps = 0;
+    c->d_sw = reinterpret_cast<int*>(c->scal + 4);
+    c->h_sw = reinterpret_cast<int*>(c->h_scal + 4);
     c->stream = c->own_stream;
     // the FP32 sweep finishes in double-float by default (rt_set_df_finish)
     c->df_switch = precision == RT_FP32_SWEEP ? kDefaultDfSwitch : 0.0;
@@ -2412,10 +2481,7 @@ int rt_destroy(rt_ctx* c)
     dfree(c->berr);
     if (c->d_nsw) cudaFree(c->d_nsw);
     c->d_nsw = nullptr;
-    if (c->d_sw) cudaFree(c->d_sw);
-    c->d_sw = nullptr;
-    if (c->h_sw) cudaFreeHost(c->h_sw);
-    c->h_sw = nullptr;
+    dfree(c->os_words);
     if (c->h_scal) cudaFreeHost(c->h_scal);
     if (c->h_steps) cudaFreeHost(c->h_steps);
     if (c->h_dlt) cudaFreeHost(c->h_dlt);
@@ -3158,12 +3224,12 @@ static int batch_solve(rt_batch* b, double tol, int max_iter, double tol_inner, 
         else
             rc = batch_os(b, act, tol_inner, max_sweeps);
         if (rc) return rc;
-        for (int p : act)
-            if ((rc = bpass(b, p, ng_push(b->ctx[p], b->iters[p] + 1)))) return rc;
         BCK(cudaMemsetAsync(b->d_delta, 0, sizeof(double) * P, b->stream));
         for (int p : act) {
             rt_ctx* c = b->ctx[p];
-            BCK(launch_rel_change(c->g.N, c->Jn, c->J, b->d_delta + p, b->stream));
+            double* hist = nullptr;
+            if ((rc = bpass(b, p, ng_push(c, b->iters[p] + 1, hist)))) return rc;
+            BCK(launch_rel_change(c->g.N, c->Jn, c->J, b->d_delta + p, hist, b->stream));
             b->stats.launches += 1;
         }
         BCK(cudaMemcpyAsync(b->h_delta, b->d_delta, sizeof(double) * P, cudaMemcpyDeviceToHost,

@@ -280,11 +280,15 @@ cudaError_t launch_op_assemble(const Geometry& g, bool df, int r0, int nplanes, 
 // The voxels' own terms from the slots' (tss: null for FP64).
 cudaError_t launch_op_own(long long N, const double* c0s, const double* bcs, const double* tss,
                           const OpMap& op, cudaStream_t st);
-// J of source S; sp: 4N scratch doubles (S padded).
-cudaError_t launch_op_apply64(const Geometry& g, const double* S, double* sp, const OpMap& op,
+// The source S in the form of the apply kernels: sp, 4N doubles (padded
+// planes, df: pairs).  With eps, S = eps B + (1 - eps) J is formed first.
+cudaError_t launch_op_pack(const Geometry& g, double* S, const double* eps, const double* B,
+                           const double* J, bool df, double* sp, cudaStream_t st);
+// J of source S, packed in sp.
+cudaError_t launch_op_apply64(const Geometry& g, const double* S, const double* sp, const OpMap& op,
                               double* J, unsigned long long* steps, cudaStream_t st);
 // The same in double-float: J = wsum S + sum_e A_e (S(e) - S) + bc - S ts.
-cudaError_t launch_op_apply_df(const Geometry& g, const double* S, double* sp, const OpMap& op,
+cudaError_t launch_op_apply_df(const Geometry& g, const double* S, const double* sp, const OpMap& op,
                                double wsum, double* J, unsigned long long* steps, cudaStream_t st);
 cudaError_t launch_op_lstar(const Geometry& g, bool df, const OpLists& L, const OpMap& op,
                             const int* cnt, const int* segb, double* lstar, cudaStream_t st);
@@ -558,13 +562,16 @@ cudaError_t launch_sweep_pass(const Geometry& g, const double* coef, const doubl
 // A whole operator-splitting solve in one cooperative launch (its blocks wait
 // on one another): right-hand side, sweeps to tol or max_sweeps, J_new and
 // the sweep count.  words (one per barrier: one per sweep, two of a Gauss-Seidel
-// sweep) zeroed before; *sweeps = -1 if a wait gave up.  Several problems (tasks, their first blocks first[q]) run
+// sweep) zeroed before; clear[0..nclear) and *zero (may be null) are zeroed;
+// *sweeps = -1 if a wait gave up.  Several problems (tasks, their first blocks first[q]) run
 // beside each other, each with its own barrier and stopping test.
 struct OsTask {
     Geometry g;
     const double *c, *rdiag, *Jfs, *Jold;
     double *Ja, *Jb, *Jn;
-    unsigned long long* words;
+    unsigned long long *words, *clear;
+    int nclear;
+    double* zero;
     int* sweeps;
     int nblk;       // blocks of this problem
 };
@@ -598,8 +605,8 @@ cudaError_t launch_ng_dots(long long N, const double* x0, const double* x1, cons
 // when the system is singular.
 cudaError_t launch_ng_apply(long long N, const double* s5, const double* x1, const double* x2,
                             double* x0, cudaStream_t st);
-// *delta = max |Jn - Jo| / |Jn|
+// *delta (zero before) = max |Jn - Jo| / |Jn|; Jo is copied to hist (may be null)
 cudaError_t launch_rel_change(long long N, const double* Jn, const double* Jo, double* delta,
-                              cudaStream_t st);
+                              double* hist, cudaStream_t st);
 
 }  // namespace rt3d

@@ -581,22 +581,47 @@ __global__ void k_op_own(long long N, const double* __restrict__ c0s, const doub
     }
 }
 
-// S in planes padded to 2ny x 2nx by periodic copies, so that an entry's node
-// is at one offset from every voxel of the plane.
-__global__ void k_op_pack(Geometry g, const double* __restrict__ S, double* __restrict__ sp)
+// s, in planes padded to 2ny x 2nx by periodic copies, at voxel v: an entry's
+// node is then at one offset from every voxel of the plane.
+template <typename V>
+__device__ __forceinline__ void pad_store(const Geometry& g, long long v, V s, V* __restrict__ sp)
 {
     const int nx = g.nx, ny = g.ny;
     const long long W = 2LL * nx, P = 4LL * nx * ny;
+    const int i = (int)(v % nx), j = (int)((v / nx) % ny);
+    V* p = sp + v / ((long long)nx * ny) * P + (long long)j * W + i;
+    p[0] = s;
+    p[nx] = s;
+    p[(long long)ny * W] = s;
+    p[(long long)ny * W + nx] = s;
+}
+__device__ __forceinline__ void op_value(double s, double& x) { x = s; }
+__device__ __forceinline__ void op_value(double s, float2& x)
+{
+    const dfl q = df_from_double(s);
+    x = make_float2(q.h, q.l);
+}
+
+// The source in the apply kernel's form (V: double, or double-float pairs).
+// With eps the source is formed here and written to S, in place of a kernel
+// before this one (a kernel of a small grid costs its launch, 3 us).
+template <typename V>
+__global__ void k_op_pack(Geometry g, double* __restrict__ S, const double* __restrict__ eps,
+                          const double* __restrict__ B, const double* __restrict__ J, V* __restrict__ sp)
+{
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < g.N;
          v += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(v % nx), j = (int)((v / nx) % ny);
-        const long long k = v / ((long long)nx * ny);
-        const double s = S[v];
-        double* p = sp + k * P + (long long)j * W + i;
-        p[0] = s;
-        p[nx] = s;
-        p[(long long)ny * W] = s;
-        p[(long long)ny * W + nx] = s;
+        double s;
+        if (eps) {
+            const double e = eps[v];
+            s = fma(e, B[v], (1.0 - e) * J[v]);
+            S[v] = s;
+        } else {
+            s = S[v];
+        }
+        V x;
+        op_value(s, x);
+        pad_store(g, v, x, sp);
     }
 }
 
@@ -687,25 +712,6 @@ k_op_apply64(Geometry g, const double* __restrict__ S, const double* __restrict_
     double a = fma(op.c0[v], S[v], op.bc[v]);
     if (tile_sum<NWB, C>(red, acc0 + acc1, a) && t < nxy) J[v] = a;
     if (steps && tile == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x == 0) atomicAdd(steps, *op.steps);
-}
-
-// S as double-float pairs in the padded planes of k_op_pack.
-__global__ void k_op_pack_df(Geometry g, const double* __restrict__ S, float2* __restrict__ sp)
-{
-    const int nx = g.nx, ny = g.ny;
-    const long long W = 2LL * nx, P = 4LL * nx * ny;
-    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < g.N;
-         v += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(v % nx), j = (int)((v / nx) % ny);
-        const long long k = v / ((long long)nx * ny);
-        const dfl q = df_from_double(S[v]);
-        const float2 s = make_float2(q.h, q.l);
-        float2* p = sp + k * P + (long long)j * W + i;
-        p[0] = s;
-        p[nx] = s;
-        p[(long long)ny * W] = s;
-        p[(long long)ny * W + nx] = s;
-    }
 }
 
 // h + l += (ah + al) ((sh + sl) - (s0h + s0l)): the difference of the high
@@ -958,21 +964,30 @@ cudaError_t launch_tiles(K kernel, dim3 tiles, cudaStream_t st, P... p)
 // 41^3 616 / 555; 48^3 and 65^3 the same.
 constexpr long long kManyTiles = 4096;
 
-cudaError_t launch_op_apply64(const Geometry& g, const double* S, double* sp, const OpMap& op,
+cudaError_t launch_op_pack(const Geometry& g, double* S, const double* eps, const double* B,
+                           const double* J, bool df, double* sp, cudaStream_t st)
+{
+    const unsigned n = op_grid1d(g.N, 256);
+    if (df)
+        k_op_pack<<<n, 256, 0, st>>>(g, S, eps, B, J, reinterpret_cast<float2*>(sp));
+    else
+        k_op_pack<<<n, 256, 0, st>>>(g, S, eps, B, J, sp);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_op_apply64(const Geometry& g, const double* S, const double* sp, const OpMap& op,
                               double* J, unsigned long long* steps, cudaStream_t st)
 {
-    k_op_pack<<<op_grid1d(g.N, 256), 256, 0, st>>>(g, S, sp);
     const dim3 tiles(op.nwp, g.nz);
     if ((long long)op.nwp * g.nz < kManyTiles)
         return launch_tiles<8, 2>(k_op_apply64<8, 2>, tiles, st, g, S, sp, op, J, steps);
     return launch_tiles<8, 1>(k_op_apply64<8, 1>, tiles, st, g, S, sp, op, J, steps);
 }
 
-cudaError_t launch_op_apply_df(const Geometry& g, const double* S, double* sp, const OpMap& op,
+cudaError_t launch_op_apply_df(const Geometry& g, const double* S, const double* sp, const OpMap& op,
                                double wsum, double* J, unsigned long long* steps, cudaStream_t st)
 {
     const float2* p = reinterpret_cast<const float2*>(sp);
-    k_op_pack_df<<<op_grid1d(g.N, 256), 256, 0, st>>>(g, S, reinterpret_cast<float2*>(sp));
     const dim3 tiles(op.nwp, g.nz);
     if ((long long)op.nwp * g.nz < kManyTiles)
         return launch_tiles<16, 1>(k_op_apply_df<16>, tiles, st, g, S, p, op, wsum, J, steps);

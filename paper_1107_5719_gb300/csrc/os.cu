@@ -533,6 +533,9 @@ k_os_solve(OsTask one, const OsTask* __restrict__ tasks, const int* __restrict__
             cur[h] = T.Jold[at[h]];
         }
     }
+    // the words of the solve after this one (no kernel between them to do it)
+    for (int q = sblk * blockDim.x + threadIdx.x; q < T.nclear; q += T.nblk * blockDim.x) T.clear[q] = 0;
+    if (T.zero && sblk == 0 && threadIdx.x == 0) *T.zero = 0.0;
     const TolTest tt = tol_test(tol);
     unsigned long long* word = T.words;
     int n = 0, left = 0;
@@ -617,12 +620,14 @@ __global__ void k_os_select(long long N, const double* __restrict__ dlt, int max
 }
 
 __global__ void k_rel_change(long long N, const double* __restrict__ Jn,
-                             const double* __restrict__ Jo, double* __restrict__ delta)
+                             const double* __restrict__ Jo, double* __restrict__ delta,
+                             double* __restrict__ hist)
 {
     double m = 0.0;
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < N;
          v += (long long)gridDim.x * blockDim.x) {
-        const double a = nonneg((Jn[v] - Jo[v]) / Jn[v]);
+        const double o = Jo[v], a = nonneg((Jn[v] - o) / Jn[v]);
+        if (hist) hist[v] = o;
         if (!(a <= m)) m = a;
     }
     block_max_to(m, delta);
@@ -872,9 +877,9 @@ cudaError_t launch_ng_apply(long long N, const double* s5, const double* x1, con
 }
 
 cudaError_t launch_rel_change(long long N, const double* Jn, const double* Jo, double* delta,
-                              cudaStream_t st)
+                              double* hist, cudaStream_t st)
 {
-    k_rel_change<<<grid_1d(N, 256), 256, 0, st>>>(N, Jn, Jo, delta);
+    k_rel_change<<<grid_1d(N, 256), 256, 0, st>>>(N, Jn, Jo, delta, hist);
     return cudaGetLastError();
 }
 

@@ -146,3 +146,32 @@ def test_apply_forms_match_march(R, form, nx, ny, nz):
             J[record] = s.formal_solution(S, want_lstar=False)[0]
             assert R.rt_fs_record_info(s.ctx)[1] == (record != 0)
     assert np.allclose(J[-1], J[0], rtol=RTOL, atol=0)
+
+
+@pytest.mark.parametrize("form", FORMS)
+def test_steps_are_counted_per_formal_solution(R, form):
+    """Every formal solution adds the steps of its recording, also after new
+    opacities and after formal solutions that are marched."""
+    p = W.random_slab(9, 8, 12, n_theta=4, n_phi=6, seed=8)
+    q = W.random_slab(9, 8, 12, n_theta=4, n_phi=6, seed=9, chi_decades=5.0)
+    p.src_order, prec = _form(R, form)
+    q.src_order = p.src_order
+
+    def steps(s, n):
+        R.rt_reset_stats(s.ctx)
+        for _ in range(n):
+            s.formal_solution(p.B, want_lstar=False)
+        return R.rt_get_stats(s.ctx)["steps"]
+
+    with R.Solver(q, precision=prec) as s:
+        one_q = steps(s, 1)
+    with R.Solver(p, precision=prec) as s:
+        one_p = steps(s, 1)
+        assert one_p != one_q and steps(s, 3) == 3 * one_p
+        R.rt_set_opacity(s.ctx, q.chi)
+        assert steps(s, 1) == one_q and steps(s, 2) == 2 * one_q
+        R.rt_set_fs_record(s.ctx, 0)
+        marched = steps(s, 1)
+        R.rt_set_fs_record(s.ctx, -1)
+        assert steps(s, 2) == 2 * one_q
+    assert 0 < marched <= one_q

@@ -38,3 +38,20 @@ def test_one_kernel_equals_host_loop(R, method, nx, ny, nz, tol, max_sweeps):
             out[graphs] = s.os_step(Jfs, p.B, tol_inner=tol, max_sweeps=max_sweeps)
     assert out[True][1] == out[False][1]
     assert np.array_equal(out[True][0], out[False][0])
+
+
+@pytest.mark.parametrize("method", [0, 1], ids=["jacobi", "gauss_seidel"])
+def test_solves_of_different_lengths_in_turn(R, method):
+    """The barrier words of a solve are those that the one before it zeroed:
+    fewer and more sweeps in turn, and more than the words held at first."""
+    p = W.random_slab(7, 6, 8, n_theta=2, n_phi=4, seed=3, eps_range=(1e-3, 1.0))
+    runs = [(0.0, 3), (0.0, 40), (1e-12, 300), (0.0, 1), (0.0, 2600), (0.0, 5), (1e-6, 50), (0.0, 1100)]
+    out = {}
+    for graphs in (True, False):
+        with R.Solver(p, os_method=method) as s:
+            R.rt_set_graphs(s.ctx, graphs)
+            Jfs, _ = s.formal_solution(p.B)
+            out[graphs] = [s.os_step(Jfs, p.B, tol_inner=t, max_sweeps=m) for t, m in runs]
+    for (Jg, ng), (Jh, nh) in zip(out[True], out[False]):
+        assert ng == nh
+        assert np.array_equal(Jg, Jh)
