@@ -38,10 +38,14 @@ sys.path.insert(0, ROOT)
 # division (8: Newton from a reciprocal seed, 4 FMA), w_cur and w_up (2),
 # the intensity update (5) and the transmission update (1).
 FLOPS_PER_STEP_FP64 = 49
-# Replay of the recorded FP64 march, per step: the bilinear interpolation
-# of S (one multiply and three FMA, 7 flops) and I += c S (one FMA, 2): five
-# FP64 instructions; 8 coefficient bytes streamed from memory.
-FLOPS_PER_STEP_FP64_REPLAY = 9
+# Operator of the recorded FP64 march, per recorded step: the rays' steps meet
+# in 2.24 distinct nodes per step (65^3 slab, 32 x 32 directions), each one FMA
+# and 8 coefficient bytes streamed from memory.
+OP_ENTRIES_PER_STEP = 2.24
+FLOPS_PER_STEP_FP64_REPLAY = 2 * OP_ENTRIES_PER_STEP
+# Recording march (k_rec64), FP64 flops executed per step (ncu: 10.0 FMA, 5.4
+# additions, 3.5 multiplications).
+FLOPS_PER_STEP_FP64_RECORD = 29
 # Peak FP64 of GB300 from the profiling recipe's figure (1.25 TFLOP/s,
 # i.e. 152 SMs x 2 DFMA/clk x 2 flops x 2.07 GHz).
 PEAK_FP64_TFLOPS = 1.25
@@ -62,10 +66,10 @@ FLOPS_SERIES_FP32 = 61
 FLOPS_PER_STEP_FP32 = FLOPS_CLOSED_FP32     # lower bound: every step on the closed form
 # Replay of the recorded FP32 march, per voxel-step: 20 flops for the
 # interpolated source difference, 5 for the Kahan update; DRAM bytes per
-# replayed voxel-step from ncu on the 33^3 slab (4 coefficient bytes, the
-# blocks of four steps padded, and the source records)
+# replayed voxel-step from ncu on the 65^3 slab with 144 directions (4
+# coefficient bytes, the blocks of four steps padded, and the source records)
 FLOPS_PER_STEP_FP32_REPLAY = 25
-REPLAY32_DRAM_BYTES_PER_STEP = 5.48
+REPLAY32_DRAM_BYTES_PER_STEP = 4.84
 # Thread instructions per step of k_fs32d (ncu, 65^3 slab, 32 x 32 directions)
 INSTR_PER_STEP_FP32 = 74.2
 # FP32 peak from unit counts and clock: 152 SMs x 128 FP32 lanes x 2 x 2.07 GHz.
@@ -74,13 +78,14 @@ PEAK_FP32_TFLOPS = 80.5
 # capture of the current kernel: chi, S, B and the direction tables stay
 # L2-resident, so the march reads 7.8 MB per launch from DRAM and writes none.
 TRAFFIC_FS64_SLAB65 = 7805184
-# DRAM bytes per k_fs64rep launch on slab65: 8.35 bytes per replayed step
-# (ncu on the 33^3 slab, whose recording fits a capture) x 3.576e9 steps
-TRAFFIC_FS64REP_SLAB65 = 29843233564
-# The double-float march executes 398 thread instructions per step (ncu,
-# slab65); its bound is instruction issue: 152 SMs x 4 schedulers x 32 lanes
+# DRAM bytes per k_op_apply64 launch on slab65: 7.9 bytes per multiply-add (ncu
+# on the 33^3 slab, whose operator fits a capture) x 2.30 of them per step (with
+# the padding of the lists) x 3.571e9 steps
+TRAFFIC_OP_SLAB65 = 64885070000
+# The double-float march executes 375 thread instructions per step (ncu,
+# 33^3 slab); its bound is instruction issue: 152 SMs x 4 schedulers x 32 lanes
 # x 2.07 GHz = 40.3e12 thread instructions/s.
-INSTR_PER_STEP_DF64 = 398
+INSTR_PER_STEP_DF64 = 375
 PEAK_ISSUE_TINST = 40.3
 
 # HBM bandwidth of the GB300s: the driver's measured copy
@@ -329,9 +334,9 @@ def march_rate(R, p, precision, dev, stream, launches=5, record=0):
 
 def record_rate(R, p, dev, stream, reps=2):
     """The recorded FP64 march on problem p: device time of a recording
-    formal solution (the march that records, then the replay that gives J)
-    and of replays alone, with their steps; new opacities before each
-    recording.  Source S = eps B + (1 - eps) B."""
+    formal solution (lengths, recording march, assembly, then the operator
+    that gives J) and of formal solutions by the operator alone, with the
+    recording's steps; new opacities before each recording.  Source S = eps B + (1 - eps) B."""
     import torch
     S = torch.from_numpy(p.eps * p.B + (1 - p.eps) * p.B).to(dev)
     chi = torch.from_numpy(p.chi).to(dev)
@@ -367,7 +372,7 @@ def record_rate(R, p, dev, stream, reps=2):
     rep_steps = rep["steps"] / reps
     out.update(replay_ms=rep_ms, replay_steps=rep_steps,
                record_ms=both["fs_ms"] / reps - rep_ms,
-               record_steps=both["steps"] / reps - rep_steps)
+               record_steps=both["steps"] / reps)
     return out
 
 
@@ -465,9 +470,9 @@ def run_only(args, dev, R):
 def fp32_replay_roofline(r32):
     """The replay of the recorded FP32 march: per voxel-step the
     interpolated source difference (4 differences, 4 + 4 products and sums:
-    20 flops) and the Kahan update (5), 4 coefficient bytes streamed; it
-    waits on its loads (ncu: long-scoreboard stalls), so both the HBM
-    fraction of its coefficient stream and its FP32 rate are given."""
+    20 flops) and the Kahan update (5), 4 coefficient bytes streamed; the
+    data pipe of L1 bounds it, so both the HBM fraction of its coefficient
+    stream and its FP32 rate are given."""
     ms, n = r32["ms_per_launch"], r32["steps_per_launch"]
     gbs = REPLAY32_DRAM_BYTES_PER_STEP * n / (ms / 1e3) / 1e9
     tfl = FLOPS_PER_STEP_FP32_REPLAY * n / (ms / 1e3) / 1e12
@@ -477,8 +482,8 @@ def fp32_replay_roofline(r32):
             "dram_bytes_per_step": REPLAY32_DRAM_BYTES_PER_STEP,
             "flops_per_step": FLOPS_PER_STEP_FP32_REPLAY,
             "achieved_tflops": round(tfl, 3), "frac_of_fp32_peak": round(tfl / PEAK_FP32_TFLOPS, 4),
-            "note": "latency-bound (ncu on the 33^3 slab: long-scoreboard stalls 10 per issue, "
-                    "issue 37%); DRAM bytes per step from that capture"}
+            "note": "ncu (65^3, 144 directions): bound by the data pipe of L1 (90% busy); DRAM "
+                    "bytes per step from that capture"}
 
 
 def fp32_roofline(m32, probe):
@@ -550,31 +555,32 @@ def run_ours(args):
     except R.RtError:
         probe = {"fp64_tflops": None, "fp32_tflops": None}
 
-    # dominant kernel: the replay of the recorded FP64 march (every formal
-    # solution of a solve evaluates J from the recording; the first one
-    # also records it), timed alone; the recording march beside it
+    # dominant kernel: the operator of the recorded FP64 march (every formal
+    # solution of a solve evaluates J from it; the first one also records
+    # and assembles it), timed alone; the recording beside it
     rec = record_rate(R, p, dev, stream)
     iters = st["iterations"] / args.steps
     if rec["recorded"]:
         rep_ms, rep_steps = rec["replay_ms"], rec["replay_steps"]
         achieved = FLOPS_PER_STEP_FP64_REPLAY * rep_steps / (rep_ms / 1e3) / 1e12
-        roofline = {"kernel": "k_fs64rep (replay of the recorded FP64 march)", "bound": "alu",
+        roofline = {"kernel": "k_op_apply64 (operator of the recorded FP64 march)", "bound": "alu",
                     "achieved": round(achieved, 4), "peak": PEAK_FP64_TFLOPS, "unit": "TFLOP/s",
                     "frac": round(achieved / PEAK_FP64_TFLOPS, 4),
-                    "traffic": TRAFFIC_FS64REP_SLAB65 if args.workload == "slab65" else None,
+                    "traffic": TRAFFIC_OP_SLAB65 if args.workload == "slab65" else None,
                     "flops_per_step": FLOPS_PER_STEP_FP64_REPLAY,
-                    "fp64_instructions_per_step": 5,
-                    "coefficient_bytes_per_step": 8,
-                    "hbm_gbs_coefficients": round(8 * rep_steps / (rep_ms / 1e3) / 1e9, 1),
+                    "fp64_instructions_per_step": OP_ENTRIES_PER_STEP,
+                    "coefficient_bytes_per_step": 8 * OP_ENTRIES_PER_STEP,
+                    "hbm_gbs_coefficients": round(8 * OP_ENTRIES_PER_STEP * rep_steps
+                                                  / (rep_ms / 1e3) / 1e9, 1),
                     "steps_per_launch": round(rep_steps),
                     "ms_per_launch": round(rep_ms, 4),
                     "share_of_step": round(rep_ms * iters / (my_ms / args.steps), 4),
-                    "record": {"kernel": "k_fs64<true> (the march, recording)",
+                    "record": {"kernel": "k_op_len, k_rec64, k_op_assemble (recording)",
                                "ms": round(rec["record_ms"], 3),
                                "steps": round(rec["record_steps"]),
-                               "achieved_tflops": round(FLOPS_PER_STEP_FP64 * rec["record_steps"]
+                               "achieved_tflops": round(FLOPS_PER_STEP_FP64_RECORD * rec["record_steps"]
                                                         / (rec["record_ms"] / 1e3) / 1e12, 4),
-                               "flops_per_step": FLOPS_PER_STEP_FP64,
+                               "flops_per_step": FLOPS_PER_STEP_FP64_RECORD,
                                "bytes_held": rec["bytes"]}}
     else:
         fs_ms = st["fs_ms"] / max(st["fs_launches"], 1)
@@ -628,12 +634,12 @@ def run_ours(args):
         stdf = rdf["stats"]
         msdf = float(sum(rdf["times"]))
         # the march (every formal solution of an unrecorded context) and the
-        # replay of its recording, each timed alone
+        # operator of its recording, each timed alone
         mdf = march_rate(R, p, R.RT_DF64, dev, stream)
         repdf = march_rate(R, p, R.RT_DF64, dev, stream, record=-1)
         eq = FLOPS_PER_STEP_FP64 * mdf["steps_per_launch"] / (mdf["ms_per_launch"] / 1e3) / 1e12
         df64 = {"value": round(RP.weak_throughput(args.df64_steps, msdf)[0], 6), "unit": "solves/s",
-                "form": "double-float, the march recorded once per opacity and replayed",
+                "form": "double-float, the march recorded once per opacity as an operator",
                 "ms_per_step": round(msdf / args.df64_steps, 3),
                 "iters_per_solve": stdf["fs_launches"] / args.df64_steps,
                 "march": mdf, "replay": repdf,
@@ -683,7 +689,7 @@ def run_ours(args):
         stpa = rpa["stats"]
         mspa = float(sum(rpa["times"]))
         para = {"value": round(RP.weak_throughput(args.para_steps, mspa)[0], 6), "unit": "solves/s",
-                "form": "FP64, the march recorded once per opacity and replayed",
+                "form": "FP64, the march recorded once per opacity as an operator",
                 "ms_per_step": round(mspa / args.para_steps, 3),
                 "iters_per_solve": stpa["fs_launches"] / args.para_steps,
                 "ms_per_fs_launch": round(stpa["fs_ms"] / max(stpa["fs_launches"], 1), 4),
@@ -855,8 +861,9 @@ def os_sweep_roofline(R, dev, sweeps=200):
                        "hbm_frac": out["slab129"]["frac_of_hbm"],
                        "peak_source": "unit counts and clock (FP64); HBM: measured copy "
                                       "bandwidth (MEASURED_PEAKS.json hbm_gbs)",
-                       "note": "ncu: FP64 pipe 90% busy (26 stencil FMAs and the "
-                               "convergence test, ~36 FP64 instructions per voxel), DRAM "
+                       "note": "ncu: FP64 pipe 92% busy (26 stencil FMAs and the "
+                               "convergence test, its quotients only where they can be "
+                               "the largest), DRAM "
                                "traffic = the algorithmic 232 B per voxel, so the FP64 pipe, "
                                "not HBM, bounds the sweep on this GPU; slab65's sweep is "
                                "L2-resident"}

@@ -293,8 +293,11 @@ int rt_set_precision(rt_ctx *ctx, int precision);
  * whose WHILE node runs the sweeps and their convergence test on the
  * device, so the host launches it without waiting; an outer iteration of
  * rt_solve waits for the GPU once (for delta and the sweep count) instead
- * of once per chunk of sweeps.  Results are identical either way (same
- * kernels, same sweep count).  on = 0 selects the host-driven loop. */
+ * of once per chunk of sweeps.  Grids of up to 2048 voxels per SM
+ * (Gauss-Seidel 600) run the step as one cooperative kernel in place of the
+ * graph; a wait of its blocks that gives up (about a second) returns
+ * RT_ETIMEOUT.  Results are identical either way (same arithmetic, same sweep
+ * count).  on = 0 selects the host-driven loop. */
 int rt_set_graphs(rt_ctx *ctx, int on);
 
 /* Automatic finishing stage for RT_FP32_SWEEP contexts: within rt_solve,
@@ -518,7 +521,8 @@ int rt_batch_set_fs_record(rt_batch *batch, long long max_bytes);
  * sweeps to tol_inner or max_sweeps, the pick of the last sweep's iterate),
  * so the host launches once and waits once per iteration (Ng runs on the
  * device too); the graph is rebuilt when the set of active problems
- * changes.  on == 0: the sweeps are enqueued from the host in growing chunks
+ * changes.  While the active problems together have up to 2048 voxels per SM
+ * (Gauss-Seidel 600) one cooperative kernel takes its place.  on == 0: the sweeps are enqueued from the host in growing chunks
  * with one wait per chunk.  Results are identical. */
 int rt_batch_set_graphs(rt_batch *batch, int on);
 /* As rt_set_ng, for every problem of the batch. */

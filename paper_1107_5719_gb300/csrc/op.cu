@@ -27,15 +27,14 @@
 // and k_op_apply64 evaluates J for a source.
 #include "df.cuh"
 #include "internal.h"
+#include "weights.cuh"
 
 #include <cooperative_groups.h>
-#include "weights.cuh"
 
 namespace rt3d {
 
 namespace {
 namespace cg = cooperative_groups;
-
 
 constexpr int kOpThreads = 128;      // march and length kernels
 constexpr int kListThreads = 256;
