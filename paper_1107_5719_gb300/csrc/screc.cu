@@ -410,8 +410,9 @@ cudaError_t sc_apply(const ScView& p, const void* coef, double wsum, void* part,
     const size_t shm = 16 * (size_t)g.nx * g.ny;
     const bool smem = sc_scratch_planes(g) == 0;
     if (smem) {
+        // one value for all grids: contexts of several threads set it
         cudaError_t e = cudaFuncSetAttribute(k_sc_apply<A, true>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return e;
     }
     long long rb = (g.N + 255) / 256;
