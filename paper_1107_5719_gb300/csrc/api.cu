@@ -80,7 +80,7 @@ struct rt_ctx {
     // the recording assembled into an operator (rec_op), in the same block;
     // its node lists (per quadrature) and the recording's working storage
     bool rec_op = false;
-    bool op_packed = false;     // the source of the coming formal solution is packed
+    bool op_packed = false;     // the source of the coming formal solution is packed (operator, replay)
     bool op_steps = false;      // h_steps holds the recording's steps
     OpMap op{};
     OpLists ol{};
@@ -1074,6 +1074,26 @@ bool op_ready(const rt_ctx* c)
            c->rec_mode != 0 && c->rec_valid && c->rec_op;
 }
 
+// The FP32 sweep replays a recording that is there already (the finishing
+// stage's reference marches).
+bool rep_ready(const rt_ctx* c)
+{
+    return c->precision == RT_FP32_SWEEP && c->fs_method == RT_FS_LONG && c->rec_mode != 0 && c->rec_valid &&
+           c->fin != 1;
+}
+
+// The source records of the replay, where prepare_source has not formed them
+// (the recording was made in between, from S).
+int rep_source(rt_ctx* c)
+{
+    if (!c->op_packed) {
+        CK(launch_pack_srecs(c->g, c->S, nullptr, nullptr, nullptr, nullptr, nullptr, c->srec, c->stream));
+        c->stats.launches += 1;
+    }
+    c->op_packed = false;
+    return RT_OK;
+}
+
 // The source packed for the operator, where prepare_source has not (the
 // operator was made in between).
 int op_source(rt_ctx* c)
@@ -1166,7 +1186,7 @@ int run_fs(rt_ctx* c, double* Jout, bool count_steps)
             c->stats.launches += 1;
         }
         if (use && c->rec_valid) {
-            CK(launch_pack_srecs(c->g, c->fin == 2 ? c->dS : c->S, c->srec, c->stream));
+            if ((rc = rep_source(c))) return rc;
             Rep32 rp{c->g, c->srec, c->info, c->poff32, c->bw32, c->rec32, c->partial,
                      c->fin == 2 ? 1 : 0, plane_major32(c->g, c->order32)};
             CK(launch_fs32rep(rp, G, c->threads32, sp, c->stream));
@@ -1194,11 +1214,20 @@ int run_fs(rt_ctx* c, double* Jout, bool count_steps)
 }
 
 // S = eps B + (1 - eps) J (or the caller's S), then in the form of the next
-// formal solution: packed for the operator (whose cutoffs are made: no smax),
-// else smax and the FP32 or double-float records.
-int prepare_source(rt_ctx* c, const double* S_in, bool device)
+// formal solution: packed for the operator or the replay (whose cutoffs are
+// made: no smax), else (march: always) smax and the FP32 or double-float records.
+int prepare_source(rt_ctx* c, const double* S_in, bool device, bool march)
 {
-    c->op_packed = op_ready(c);
+    c->op_packed = !march && op_ready(c);
+    if (!march && rep_ready(c)) {
+        if (S_in)
+            CK(cudaMemcpyAsync(c->S, S_in, sizeof(double) * c->g.N, kind(device), c->stream));
+        CK(launch_pack_srecs(c->g, c->S, S_in ? nullptr : c->eps, c->B, c->J,
+                             c->fin == 2 ? c->S_ref : nullptr, c->dS, c->srec, c->stream));
+        c->stats.launches += 1;
+        c->op_packed = true;
+        return RT_OK;
+    }
     if (c->op_packed) {
         if (S_in)
             CK(cudaMemcpyAsync(c->S, S_in, sizeof(double) * c->g.N, kind(device), c->stream));
@@ -1222,15 +1251,10 @@ int prepare_source(rt_ctx* c, const double* S_in, bool device)
         CK(launch_delta_source(c->g.N, c->S, c->S_ref, c->dS, c->stream));
         CK(cudaMemsetAsync(c->scal + 0, 0, sizeof(double), c->stream));
         CK(launch_absmax(c->g.N, c->dS, nullptr, c->scal + 0, nullptr, c->stream));
-        if (!c->rec_valid) {   // the replay packs its own source records
-            CK(launch_pack_pairs(c->g, c->chi, c->dS, c->pair, c->plo, c->stream));
-            c->stats.launches += 1;
-        }
-        c->stats.launches += 2;
+        CK(launch_pack_pairs(c->g, c->chi, c->dS, c->pair, c->plo, c->stream));
+        c->stats.launches += 3;
     } else if (c->precision == RT_FP32_SWEEP && c->fin == 1) {
         // the reference formal solution packs its own double-float nodes
-    } else if (c->precision == RT_FP32_SWEEP && c->rec_valid) {
-        // the replay packs its own source records
     } else if (c->precision == RT_FP32_SWEEP) {
         CK(launch_pack_pairs(c->g, c->chi, c->S, c->pair, c->plo, c->stream));
         c->stats.launches += 1;
@@ -1268,7 +1292,7 @@ int formal_solution(rt_ctx* c, const double* S, double* Jfs_out, double* lstar_o
     if (rc) return rc;
     if ((rc = need_all(c))) return rc;
     if (!Jfs_out) return fail(c, RT_EINVAL, "J_fs is NULL");
-    if ((rc = prepare_source(c, S, device))) return rc;
+    if ((rc = prepare_source(c, S, device, false))) return rc;
     if ((rc = run_fs(c, c->Jfs, true))) return rc;
     const cudaMemcpyKind out = device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
     CK(cudaMemcpyAsync(Jfs_out, c->Jfs, sizeof(double) * c->g.N, out, c->stream));
@@ -1696,7 +1720,7 @@ int solve(rt_ctx* c, double tol, int max_iter, double tol_inner, int max_sweeps,
     bool converged = false;
     unsigned long long total_steps = 0;
     while (it < max_iter) {
-        if ((rc = prepare_source(c, nullptr, true))) return rc;
+        if ((rc = prepare_source(c, nullptr, true, false))) return rc;
         if ((rc = run_fs(c, c->Jfs, true))) return rc;
         int ns = 0;
         if ((rc = run_os(c, c->Jfs, c->J, c->Jn, tol_inner, max_sweeps, true, &ns))) return rc;
@@ -2112,7 +2136,7 @@ int batch_fs(rt_batch* b, const std::vector<int>& act)
     std::vector<char> direct(b->ctx.size(), 0);     // J is in c->Jfs already
     for (int p : act) {
         rt_ctx* c = b->ctx[p];
-        if ((rc = bpass(b, p, prepare_source(c, nullptr, true)))) return rc;
+        if ((rc = bpass(b, p, prepare_source(c, nullptr, true, false)))) return rc;
         if ((rc = bpass(b, p, fs_prepare(c)))) return rc;
     }
     const int G = batch_groups(b, act);
@@ -2138,8 +2162,7 @@ int batch_fs(rt_batch* b, const std::vector<int>& act)
                 c->rec_valid = true;
                 b->stats.launches += 1;
             }
-            BCK(launch_pack_srecs(c->g, c->fin == 2 ? c->dS : c->S, c->srec, b->stream));
-            b->stats.launches += 1;
+            if ((rc = bpass(b, p, rep_source(c)))) return rc;
             b->h_rviews[p] = Rep32{c->g, c->srec, c->info, c->poff32, c->bw32, c->rec32,
                                    c->partial, c->fin == 2 ? 1 : 0, plane_major32(c->g, c->order32)};
             b->h_rids[rq] = p;
@@ -2732,7 +2755,7 @@ static int fs32_branch_counts(rt_ctx* c, const double* S, unsigned long long* st
     if (!steps || !series) return fail(c, RT_EINVAL, "steps or series is NULL");
     if (c->precision != RT_FP32_SWEEP || c->fs_method != RT_FS_LONG)
         return fail(c, RT_EINVAL, "branch counts need the FP32-sweep long-characteristics march");
-    if ((rc = prepare_source(c, S, false))) return rc;
+    if ((rc = prepare_source(c, S, false, true))) return rc;
     if ((rc = fs_prepare(c))) return rc;
     CK(launch_pack_pairs(c->g, c->chi, c->S, c->pair, c->plo, c->stream));
     unsigned long long* d = nullptr;

@@ -114,21 +114,39 @@ __global__ void k_pack_pairs(Geometry g, const double* __restrict__ chi,
 }
 
 // The replay's source records: srec[k][y][x] = {S_hi, S_lo} of the node
-// (x mod nx, y mod ny), padded as k_pack_pairs.
-__global__ void k_pack_srecs(Geometry g, const double* __restrict__ S, float2* __restrict__ sp)
+// (x mod nx, y mod ny), padded as k_pack_pairs.  With eps the source is formed
+// here and written to S; with Sref the records hold S - Sref, also written to
+// dS (one kernel per formal solution where there were up to four, 4 us each on
+// small grids).
+__global__ void k_pack_srecs(Geometry g, double* __restrict__ S, const double* __restrict__ eps,
+                             const double* __restrict__ B, const double* __restrict__ J,
+                             const double* __restrict__ Sref, double* __restrict__ dS,
+                             float2* __restrict__ sp)
 {
     const int nx = g.nx, ny = g.ny;
-    const long long W = 2LL * nx, R = 2LL * ny + 1, P = R * W;
-    const long long n = P * g.nz;
-    for (long long r = blockIdx.x * (long long)blockDim.x + threadIdx.x; r < n;
-         r += (long long)gridDim.x * blockDim.x) {
-        const long long k = r / P, rem = r - k * P;
-        int j = (int)(rem / W), i = (int)(rem - j * W);
-        while (j >= ny) j -= ny;
-        while (i >= nx) i -= nx;
-        const double s = S[(k * ny + j) * (long long)nx + i];
+    const long long W = 2LL * nx, P = (2LL * ny + 1) * W;
+    for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < g.N;
+         v += (long long)gridDim.x * blockDim.x) {
+        double s;
+        if (eps) {
+            const double e = eps[v];
+            s = fma(e, B[v], (1.0 - e) * J[v]);
+            S[v] = s;
+        } else {
+            s = S[v];
+        }
+        if (Sref) {
+            s -= Sref[v];
+            dS[v] = s;
+        }
         const float h = (float)s;
-        sp[r] = make_float2(h, (float)(s - (double)h));
+        const float2 r = make_float2(h, (float)(s - (double)h));
+        const int i = (int)(v % nx), j = (int)((v / nx) % ny);
+        float2* p = sp + v / ((long long)nx * ny) * P + i;
+        for (long long y = j; y <= 2LL * ny; y += ny) {
+            p[y * W] = r;
+            p[y * W + nx] = r;
+        }
     }
 }
 
@@ -752,9 +770,11 @@ cudaError_t launch_pack_pairs(const Geometry& g, const double* chi, const double
     return cudaGetLastError();
 }
 
-cudaError_t launch_pack_srecs(const Geometry& g, const double* S, float2* srec, cudaStream_t st)
+cudaError_t launch_pack_srecs(const Geometry& g, double* S, const double* eps, const double* B,
+                              const double* J, const double* Sref, double* dS, float2* srec,
+                              cudaStream_t st)
 {
-    k_pack_srecs<<<grid1d(pair_records(g), 256), 256, 0, st>>>(g, S, srec);
+    k_pack_srecs<<<grid1d(g.N, 256), 256, 0, st>>>(g, S, eps, B, J, Sref, dS, srec);
     return cudaGetLastError();
 }
 

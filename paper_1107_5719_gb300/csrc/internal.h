@@ -430,7 +430,11 @@ struct Rep32 {
     int zero_bc;
     int pmajor;
 };
-cudaError_t launch_pack_srecs(const Geometry& g, const double* S, float2* srec, cudaStream_t st);
+// Source records of S, or with Sref of dS = S - Sref; with eps,
+// S = eps B + (1 - eps) J is formed first.
+cudaError_t launch_pack_srecs(const Geometry& g, double* S, const double* eps, const double* B,
+                              const double* J, const double* Sref, double* dS, float2* srec,
+                              cudaStream_t st);
 // Record the march of p (cut at `cut`, the caller's stricter cutoff) into rec.
 cudaError_t launch_fs32rec(const View32& p, double cut, int groups, const Rec32& rec,
                            unsigned long long* steps, cudaStream_t st);
