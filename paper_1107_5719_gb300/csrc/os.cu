@@ -412,34 +412,36 @@ k_gs_half(Geometry g, const double* __restrict__ c, const double* __restrict__ r
 //
 // A sweep of a small grid is a chain of latencies (17^3, one warp per SM, in
 // cycles): 2000 for the sum, whose 26 dependent FP64 multiply-adds take 68
-// each, 230 for the convergence test, 970 until the stores are visible, 2100
-// for the barrier's atomic and polls, 550 for the fence behind it.  So the
+// each, 230 for the convergence test, and 3600 for the barrier with a fence on
+// either side (970 until the stores are visible, 2100 for the atomic and the
+// polls, 550), 2800 with a releasing atomic and acquiring polls.  So the
 // neighbours are loaded together before the first of them is used, the
 // coefficients wait in shared memory (SM: the fences empty L1), the test forms
 // no quotient that its FP32 estimate decides (not_below; 1250 before), and the
 // test's result travels in the barrier's word.  Solve to 1e-12, 26 sweeps:
-// 17^3 0.148 -> 0.111 ms, 33^3 0.173 -> 0.149, 65^3 (bound by the FP64 pipe)
-// 0.63 -> 0.56.
+// 17^3 0.148 -> 0.100 ms, 33^3 0.173 -> 0.136, 65^3 (bound by the FP64 pipe)
+// 0.63 -> 0.55.
 
 // Barrier of the problem's blocks: returns how many of them had a voxel that
 // has not met the tolerance (more), or -1 when a wait gave up, after at most
 // kBarPolls polls (about a second).  The word (zero before) counts the
 // arrivals in its low half and those blocks in its high half, so that one
-// atomic and one polled load carry both.
+// atomic and one polled load carry both.  The block's stores come before its
+// releasing atomic (block barrier, then release), its later loads after the
+// acquiring load.
 constexpr int kBarPolls = 1 << 21;
 __device__ __forceinline__ int os_barrier(unsigned long long* word, int nblk, bool more)
 {
     __shared__ int result;
     const bool any = __syncthreads_or(more);
     if (threadIdx.x == 0) {
-        __threadfence();
-        atomicAdd(word, any ? (1ull << 32) + 1 : 1ull);
+        asm volatile("red.release.gpu.global.add.u64 [%0], %1;"
+                     :: "l"(word), "l"(any ? (1ull << 32) + 1 : 1ull) : "memory");
         int n = 0;
         unsigned long long v;
         do
-            asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(word) : "memory");
+            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(word) : "memory");
         while ((int)v < nblk && ++n < kBarPolls);
-        __threadfence();
         result = (int)v < nblk ? -1 : (int)(v >> 32);
     }
     __syncthreads();
@@ -793,9 +795,9 @@ cudaError_t launch_sweep_pass(const Geometry& g, const double* coef, const doubl
 // Threads per block, voxels per thread and blocks for N voxels (0 blocks: the
 // sweeps run as kernels of a graph): few voxels are spread over all SMs, one
 // warp each at least.  Measured per solve to 1e-12 (20 to 31 sweeps), graph
-// against one kernel: 17^3 0.24 / 0.11 ms, 33^3 0.27 / 0.15, 65^3 0.72 / 0.56
+// against one kernel: 17^3 0.24 / 0.10 ms, 33^3 0.27 / 0.14, 65^3 0.72 / 0.55
 // (two voxels per thread); Gauss-Seidel, half of whose threads wait in each
-// half sweep, 17^3 0.51 (host loop) / 0.16, but 61 x 45 x 52 0.05 ms slower
+// half sweep, 17^3 0.51 (host loop) / 0.15, but 61 x 45 x 52 0.05 ms slower
 // than the graph, so it stops earlier.  The coefficients lie in shared memory
 // up to kSmVoxels voxels per SM: 24^3 0.138 without / 0.115 ms with, 33^3
 // 0.151 / 0.150, but 41^3 0.199 / 0.212 and 48^3 0.25 / 0.35, since the
