@@ -441,34 +441,31 @@ k_rec64(Geometry g, int r0, const double* __restrict__ chi, const double* __rest
 // A of the planes of rank r0 + blockIdx.y: one block per 32 voxels, the
 // lanes of its warps the voxels.  A warp takes a run of entries of a list and
 // walks their contributions, which are consecutive: 32 at a time, each lane
-// looks up one contribution's row, then the warp adds them eight by eight in
-// list order (eight coefficient loads in flight) and stores an entry when its
-// last contribution is in.  Rows past the warp's own rays hold nothing
-// (m > its length) and count as zero.
+// looks one up and leaves its weight, row and entry in shared memory, then the
+// warp adds them eight by eight in list order (eight coefficient loads in
+// flight) and stores an entry when its last contribution is in.  Rows past the
+// warp's own rays hold nothing (m > its length) and count as zero.
+// FP64: bound by the FP64 pipe (81% busy; 33^3 with 256 directions 0.66 ms).  With
+// the contributions passed by shuffles and the entries stored in pairs it took
+// 2.5 times the instructions (0.74 ms; double-float 0.77 against 0.50).
 constexpr int kAsmRun = 32;      // entries of a run (even)
+constexpr int kAsmShared = 8 * 24 * 1024;    // the lengths of 24 Ki directions
 
 // The two arithmetics of the coefficients: FP64, or double-float pairs.
 struct AsmF64 {
     using V = double;
-    using Pair = double2;
     static __device__ __forceinline__ V zero() { return 0.0; }
     static __device__ __forceinline__ V weight(double w) { return w; }
-    static __device__ __forceinline__ V shfl(V w, int i) { return __shfl_sync(0xffffffffu, w, i); }
     static __device__ __forceinline__ V fma(V w, V c, V a) { return ::fma(w, c, a); }
-    static __device__ __forceinline__ Pair pair(V a, V b) { return make_double2(a, b); }
+    static __device__ __forceinline__ V entry(V a) { return a; }
 };
 struct AsmDF {
     using V = float2;
-    using Pair = float4;
     static __device__ __forceinline__ V zero() { return make_float2(0.f, 0.f); }
     static __device__ __forceinline__ V weight(double w)
     {
         const dfl q = df_from_double(w);
         return make_float2(q.h, q.l);
-    }
-    static __device__ __forceinline__ V shfl(V w, int i)
-    {
-        return make_float2(__shfl_sync(0xffffffffu, w.x, i), __shfl_sync(0xffffffffu, w.y, i));
     }
     // the sum is left unnormalised between contributions
     static __device__ __forceinline__ V fma(V w, V c, V a)
@@ -477,10 +474,10 @@ struct AsmDF {
         const dfl s = two_sum(a.x, p.h);
         return make_float2(s.h, (a.y + s.l) + fmaf(w.y, c.x, fmaf(w.x, c.y, p.l)));
     }
-    static __device__ __forceinline__ Pair pair(V a, V b)
+    static __device__ __forceinline__ V entry(V a)
     {
-        const dfl p = quick_two_sum(a.x, a.y), q = quick_two_sum(b.x, b.y);
-        return make_float4(p.h, p.l, q.h, q.l);
+        const dfl p = quick_two_sum(a.x, a.y);
+        return make_float2(p.h, p.l);
     }
 };
 
@@ -491,7 +488,14 @@ k_op_assemble(Geometry g, int r0, OpLists L, RecOut ro, const int* __restrict__ 
               const long long* __restrict__ eb, typename T::V* __restrict__ A)
 {
     using V = typename T::V;
-    using Pair = typename T::Pair;
+    // a contribution as every lane reads it: weight, row (kNoRow: none), element
+    // of the entry that it completes (kOpen: none)
+    struct __align__(16) Step {
+        V wb;
+        unsigned row, out;
+    };
+    constexpr unsigned kNoRow = ~0u, kOpen = ~0u;
+    __shared__ Step steps[kListThreads / 32][32];
     extern __shared__ int2 lr[];     // [ndir] {length, first row}
     const int nz = g.nz, nxy = g.nx * g.ny;
     const int k0 = plane_at(g, r0 + blockIdx.y), tile = blockIdx.x;
@@ -502,54 +506,58 @@ k_op_assemble(Geometry g, int r0, OpLists L, RecOut ro, const int* __restrict__ 
         lr[d] = make_int2(lmax[((long long)d * nz + k0) * nwp + tile],
                           ro.rowbase[(long long)k0 * g.ndir + d]);
     __syncthreads();
-    const V* c = reinterpret_cast<const V*>(ro.base) + ro.prow[k0] * nxy + (live ? t : 0);
-    Pair* out = reinterpret_cast<Pair*>(A + eb[k0] * (long long)nwp * 32) +
-                (long long)tile * (E[k0] / 2) * 32 + lane;
+    const char* c = reinterpret_cast<const char*>(reinterpret_cast<const V*>(ro.base) + ro.prow[k0] * nxy +
+                                                  (live ? t : 0));
+    const unsigned row_bytes = (unsigned)(nxy * sizeof(V));
+    V* out = A + eb[k0] * (long long)nwp * 32 + (long long)tile * E[k0] * 32 + 2 * lane;
+    Step* mine = steps[wid];
     int run = wid;                   // runs go round the warps, across the lists
     for (int q = blockIdx.z; q < 2 * nz; q += gridDim.z) {
         const int n = cnt[(long long)k0 * 2 * nz + q];
         if (n == 0) continue;
         const int m = q < nz ? q : q - nz;
-        Pair* oq = out + (long long)(segb[(long long)k0 * 2 * nz + q] / 2) * 32;
+        V* oq = out + (long long)segb[(long long)k0 * 2 * nz + q] * 32;
         const int* us = L.ustart + (long long)q * (L.ucap + 1);
         const OpContrib* ct = L.contrib + (long long)q * L.icap;
         const int runs = (n + kAsmRun - 1) / kAsmRun;
         for (; run < runs; run += nw) {
             const int js = us[run * kAsmRun], je = us[min(n, (run + 1) * kAsmRun)];
-            V acc = T::zero(), even = T::zero();
+            V acc = T::zero();
             for (int jb = js; jb < je; jb += 32) {
-                V wb = T::zero();
-                int row = -1, ul0 = 0;
+                Step p{T::zero(), kNoRow, kOpen};
                 if (jb + lane < je) {
                     const OpContrib k = ct[jb + lane];
-                    const int2 p = lr[k.d];
-                    if (m <= p.x || m == 0) row = p.y + m - 1 + ro.para;
-                    wb = T::weight(k.wb);
-                    ul0 = k.ul;
+                    const int2 r = lr[k.d];
+                    if (m <= r.x || m == 0) p.row = r.y + m - 1 + ro.para;
+                    p.wb = T::weight(k.wb);
+                    // entry k.ul >> 1, in pairs of 32 x 2 elements
+                    if (k.ul & 1) p.out = (unsigned)(k.ul >> 2) * 64 + ((k.ul >> 1) & 1);
                 }
+                __syncwarp();
+                mine[lane] = p;
+                __syncwarp();
                 const int nj = min(32, je - jb);
                 for (int i = 0; i < nj; i += 8) {
                     V cv[8];
 #pragma unroll
                     for (int h = 0; h < 8; ++h) {
-                        const int r = __shfl_sync(0xffffffffu, row, i + h);
-                        cv[h] = r >= 0 ? __ldg(c + (long long)r * nxy) : T::zero();
+                        const unsigned r = mine[i + h].row;
+                        cv[h] = T::zero();
+                        if (live && r != kNoRow)
+                            cv[h] = __ldg(reinterpret_cast<const V*>(c + (unsigned long long)r * row_bytes));
                     }
 #pragma unroll
                     for (int h = 0; h < 8; ++h) {
-                        acc = T::fma(T::shfl(wb, i + h), cv[h], acc);
-                        const int ul = __shfl_sync(0xffffffffu, ul0, i + h);
-                        if (ul & 1) {       // entry ul >> 1 is complete
-                            if (!live) acc = T::zero();
-                            if (ul & 2) oq[(long long)(ul >> 2) * 32] = T::pair(even, acc);
-                            else even = acc;
+                        const Step x = mine[i + h];
+                        acc = T::fma(x.wb, cv[h], acc);
+                        if (x.out != kOpen) {
+                            oq[x.out] = T::entry(acc);
                             acc = T::zero();
                         }
                     }
                 }
             }
-            if ((n & 1) && (run + 1) * kAsmRun >= n)
-                oq[(long long)(n >> 1) * 32] = T::pair(even, T::zero());
+            if ((n & 1) && (run + 1) * kAsmRun >= n) oq[(long long)(n >> 1) * 64 + 1] = T::zero();
         }
         run -= runs;
     }
@@ -557,7 +565,7 @@ k_op_assemble(Geometry g, int r0, OpLists L, RecOut ro, const int* __restrict__ 
     const int qz = 2 * nz - 1;
     const int tail = (segb[(long long)k0 * 2 * nz + qz] + cnt[(long long)k0 * 2 * nz + qz] + 1) / 2;
     for (int p = tail + wid; p < E[k0] / 2; p += nw)
-        out[(long long)p * 32] = T::pair(T::zero(), T::zero());
+        out[(long long)p * 64] = out[(long long)p * 64 + 1] = T::zero();
 }
 
 // c0[v] = sum over slots of c0s; bc[v] and ts[v] (when given) likewise (slot
@@ -907,10 +915,11 @@ cudaError_t launch_op_assemble(const Geometry& g, bool df, int r0, int nplanes, 
 {
     const size_t shm = sizeof(int2) * (size_t)g.ndir;
     if (shm > 48 * 1024) {
+        // one value for all quadratures: contexts of several threads set it
         cudaError_t e = df ? cudaFuncSetAttribute(k_op_assemble<AsmDF>,
-                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm)
+                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, kAsmShared)
                            : cudaFuncSetAttribute(k_op_assemble<AsmF64>,
-                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
+                                                  cudaFuncAttributeMaxDynamicSharedMemorySize, kAsmShared);
         if (e != cudaSuccess) return e;
     }
     // few tiles: several blocks share a tile's lists, so that every SM has
