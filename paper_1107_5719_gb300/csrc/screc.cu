@@ -345,17 +345,21 @@ k_sc_sum(ScView p, int d0, int nd, const typename A::V* __restrict__ part, doubl
 
 // Lambda* from the recorded weights (see k_lstar_sc64): per direction w_cur at
 // the voxel and, at the corners c of its upstream point, b_c (w_up + e
-// w_cur(c)), w_cur(c) read from c's own record (0 on the entry plane).
+// w_cur(c)), w_cur(c) read from c's own record (0 on the entry plane).  FP64
+// reads the voxel's own weights as well (65^3 x 1024: 4.9 ms, 14.4 forming them
+// again); double-float, whose record has no w_up, forms them.
 template <typename A>
 __global__ void __launch_bounds__(kRecThreads)
 k_sc_lstar(ScView p, const typename A::C* __restrict__ coef, double* __restrict__ lstar)
 {
     using V = typename A::V;
     __shared__ V lam[27][kRecThreads];
-    __shared__ typename A::T tab[A::kTab];
+    __shared__ typename A::T tab[A::kDiff ? A::kTab : 1];
     for (int q = 0; q < 27; ++q) lam[q][threadIdx.x] = A::zero();
-    A::fill(tab);
-    __syncthreads();
+    if (A::kDiff) {
+        A::fill(tab);
+        __syncthreads();
+    }
     const Geometry& g = p.g;
     const int nxy = g.nx * g.ny, nz = g.nz;
     const int t = blockIdx.x * kRecThreads + threadIdx.x, k = blockIdx.y;
@@ -369,11 +373,18 @@ k_sc_lstar(ScView p, const typename A::C* __restrict__ coef, double* __restrict_
         if (ku < 0 || ku >= nz) continue;
         const ScCorners c = sc_corners(i, j, p.off[(long long)d * nz + 1], g.nx, g.ny);
         if (!sc_inside(g, c, kSiteLstarSc)) continue;
-        const V* u = chi + (long long)ku * nxy;
         const auto b = A::weights(p, d);
         V wc, wu, e;
-        A::segment(A::depth(di, A::bilin(b, __ldg(u + c.a00), __ldg(u + c.a10), __ldg(u + c.a01),
-                                         __ldg(u + c.a11)), me), tab, wc, wu, e);
+        if constexpr (A::kDiff) {
+            const V* u = chi + (long long)ku * nxy;
+            A::segment(A::depth(di, A::bilin(b, __ldg(u + c.a00), __ldg(u + c.a10), __ldg(u + c.a01),
+                                             __ldg(u + c.a11)), me), tab, wc, wu, e);
+        } else {
+            const auto own = A::load(coef, g.ndir * g.N, ((long long)d * nz + k) * nxy + t);
+            wc = own.a.x;
+            e = own.a.y;
+            wu = own.u;
+        }
         const V wd = A::make(di.w);
         lam[13][threadIdx.x] = A::add(lam[13][threadIdx.x], A::mul(wd, wc));
         const bool deeper = ku != (di.sgn > 0 ? 0 : nz - 1);
