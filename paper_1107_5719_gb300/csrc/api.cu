@@ -56,6 +56,9 @@ struct rt_ctx {
     // one that uses it; words in use and of each set not zero
     unsigned long long* os_words = nullptr;
     int os_cap = 0, os_set = 0, os_dirty[2] = {0, 0};
+    // where that kernel forms the outer delta and copies J_old to, in a solve's
+    // iterations without extrapolation (null: it does not)
+    double *os_delta = nullptr, *os_hist = nullptr;
     bool use_graphs = true;
     unsigned long long* berr = nullptr;   // checked builds: out-of-bounds record
     int fs_method = RT_FS_LONG;
@@ -1499,6 +1502,8 @@ OsTask os_task(const rt_ctx* c, const double* Jfs, const double* Jold, double* J
     t.clear = nullptr;
     t.nclear = 0;
     t.zero = nullptr;
+    t.delta = c->os_delta;
+    t.hist = c->os_hist;
     t.sweeps = sweeps;
     t.nblk = nblk;
     return t;
@@ -1645,16 +1650,20 @@ int ensure_ng(rt_ctx* c)
     return RT_OK;
 }
 
-// Ng bookkeeping after iteration `it` (1-based) produced J_new in c->Jn from
-// the previous iterate c->J: have c->J remembered (hist: where the kernel that
-// forms the outer delta copies it), and when four iterates are held
-// and it is a multiple of the period, enqueue the weighted sums and the
-// extrapolation of J_new, whose 2x2 system is solved on the device (no
-// host synchronisation; the iterate is left unchanged if it is singular).
-int ng_push(rt_ctx* c, int it, double*& hist)
+// Ng bookkeeping of iteration `it` (1-based), before its operator splitting
+// produces J_new in c->Jn from c->J: c->J is remembered (hist: where the
+// kernel that forms the outer delta copies it), and the iteration
+// extrapolates (due) when four iterates are held and it is a multiple of the
+// period.  Otherwise the operator-splitting kernel may form the delta itself.
+int ng_begin(rt_ctx* c, int it, double* delta, double*& hist, bool& due)
 {
     hist = nullptr;
-    if (!c->ng_period) return RT_OK;
+    due = false;
+    c->os_delta = c->os_hist = nullptr;
+    if (!c->ng_period) {
+        c->os_delta = delta;
+        return RT_OK;
+    }
     int rc = ensure_ng(c);
     if (rc) return rc;
     double* t = c->ng_old[2];
@@ -1662,8 +1671,22 @@ int ng_push(rt_ctx* c, int it, double*& hist)
     c->ng_old[1] = c->ng_old[0];
     c->ng_old[0] = hist = t;
     if (c->ng_count < 4) ++c->ng_count;
-    if (c->ng_count == 4 && it % c->ng_period == 0 &&
-        (it == 1 || c->ng_last_delta >= c->ng_min_delta)) {
+    due = c->ng_count == 4 && it % c->ng_period == 0 &&
+          (it == 1 || c->ng_last_delta >= c->ng_min_delta);
+    c->os_delta = due ? nullptr : delta;
+    c->os_hist = due ? nullptr : hist;
+    return RT_OK;
+}
+
+// After the operator splitting (in one kernel: one): where the extrapolation is
+// due, the weighted sums and the extrapolation of J_new, whose 2x2 system is
+// solved on the device (no host synchronisation; the iterate is left unchanged
+// if it is singular); then the outer delta, unless that kernel has formed it.
+int ng_end(rt_ctx* c, bool one, bool due, double* delta, double* hist)
+{
+    const bool formed = one && c->os_delta;
+    c->os_delta = c->os_hist = nullptr;
+    if (due) {
         CK(launch_ng_dots(c->g.N, c->Jn, c->J, c->ng_old[1], c->ng_old[2], c->ng_part,
                           c->ng_out, c->stream));
         CK(launch_ng_apply(c->g.N, c->ng_out, c->J, c->ng_old[1], c->Jn, c->stream));
@@ -1671,7 +1694,18 @@ int ng_push(rt_ctx* c, int it, double*& hist)
         c->ng_applied += 1;
         c->ng_count = 1;
     }
+    if (!formed) {
+        CK(launch_rel_change(c->g.N, c->Jn, c->J, delta, hist, c->stream));
+        c->stats.launches += 1;
+    }
     return RT_OK;
+}
+
+// After an iteration that failed: no history, no delta in the next solve.
+void ng_forget(rt_ctx* c)
+{
+    c->ng_count = 1;
+    c->os_delta = c->os_hist = nullptr;
 }
 
 // Switch between the FP32 sweep and the double-float march (see rt_set_precision).
@@ -1723,12 +1757,15 @@ int solve(rt_ctx* c, double tol, int max_iter, double tol_inner, int max_sweeps,
         if ((rc = prepare_source(c, nullptr, true, false))) return rc;
         if ((rc = run_fs(c, c->Jfs, true))) return rc;
         int ns = 0;
-        if ((rc = run_os(c, c->Jfs, c->J, c->Jn, tol_inner, max_sweeps, true, &ns))) return rc;
         double* hist = nullptr;
-        if ((rc = ng_push(c, it + 1, hist))) return rc;
+        bool due = false;
+        if ((rc = ng_begin(c, it + 1, c->scal + 2, hist, due))) return rc;
+        if ((rc = run_os(c, c->Jfs, c->J, c->Jn, tol_inner, max_sweeps, true, &ns))) {
+            ng_forget(c);
+            return rc;
+        }
         if (!c->os_one) CK(cudaMemsetAsync(c->scal + 2, 0, sizeof(double), c->stream));
-        CK(launch_rel_change(c->g.N, c->Jn, c->J, c->scal + 2, hist, c->stream));
-        c->stats.launches += 1;
+        if ((rc = ng_end(c, c->os_one, due, c->scal + 2, hist))) return rc;
         // with the sweep count where the step ran as one kernel
         CK(cudaMemcpyAsync(c->h_scal + 2, c->scal + 2, sizeof(double) * (c->os_one ? 3 : 1),
                            cudaMemcpyDeviceToHost, c->stream));
@@ -3242,18 +3279,26 @@ static int batch_solve(rt_batch* b, double tol, int max_iter, double tol_inner, 
             if (b->admitted[p] && !b->converged[p] && b->iters[p] < max_iter) act.push_back(p);
         if (act.empty()) break;
         if ((rc = batch_fs(b, act))) return rc;
-        if (b->use_graphs)
-            rc = batch_os_graph(b, act, tol_inner, max_sweeps);
-        else
-            rc = batch_os(b, act, tol_inner, max_sweeps);
-        if (rc) return rc;
         BCK(cudaMemsetAsync(b->d_delta, 0, sizeof(double) * P, b->stream));
+        std::vector<double*> hist(P, nullptr);
+        std::vector<char> due(P, 0);
+        rc = RT_OK;
         for (int p : act) {
-            rt_ctx* c = b->ctx[p];
-            double* hist = nullptr;
-            if ((rc = bpass(b, p, ng_push(c, b->iters[p] + 1, hist)))) return rc;
-            BCK(launch_rel_change(c->g.N, c->Jn, c->J, b->d_delta + p, hist, b->stream));
-            b->stats.launches += 1;
+            bool d = false;
+            if ((rc = bpass(b, p, ng_begin(b->ctx[p], b->iters[p] + 1, b->d_delta + p, hist[p], d)))) break;
+            due[p] = d;
+        }
+        b->os_one = false;
+        if (rc == RT_OK)
+            rc = b->use_graphs ? batch_os_graph(b, act, tol_inner, max_sweeps)
+                               : batch_os(b, act, tol_inner, max_sweeps);
+        if (rc) {
+            for (int p : act) ng_forget(b->ctx[p]);
+            return rc;
+        }
+        for (int p : act) {
+            if ((rc = bpass(b, p, ng_end(b->ctx[p], b->os_one, due[p], b->d_delta + p, hist[p])))) return rc;
+            b->stats.launches += b->os_one && !due[p] ? 0 : 1;
         }
         BCK(cudaMemcpyAsync(b->h_delta, b->d_delta, sizeof(double) * P, cudaMemcpyDeviceToHost,
                             b->stream));

@@ -567,6 +567,8 @@ cudaError_t launch_sweep_pass(const Geometry& g, const double* coef, const doubl
 // on one another): right-hand side, sweeps to tol or max_sweeps, J_new and
 // the sweep count.  words (one per barrier: one per sweep, two of a Gauss-Seidel
 // sweep) zeroed before; clear[0..nclear) and *zero (may be null) are zeroed;
+// delta (may be null; zero before, or zeroed by this launch): max |Jn - Jold| /
+// |Jn|, and Jold copied to hist (may be null);
 // *sweeps = -1 if a wait gave up.  Several problems (tasks, their first blocks first[q]) run
 // beside each other, each with its own barrier and stopping test.
 struct OsTask {
@@ -575,7 +577,7 @@ struct OsTask {
     double *Ja, *Jb, *Jn;
     unsigned long long *words, *clear;
     int nclear;
-    double* zero;
+    double *zero, *delta, *hist;
     int* sweeps;
     int nblk;       // blocks of this problem
 };

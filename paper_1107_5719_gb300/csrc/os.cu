@@ -576,9 +576,19 @@ k_os_solve(OsTask one, const OsTask* __restrict__ tasks, const int* __restrict__
         if (threadIdx.x == 0) *T.sweeps = -1;
         return;
     }
+    double change = 0.0;
 #pragma unroll
     for (int h = 0; h < V; ++h)
-        if (mine[h]) T.Jn[at[h]] = cur[h];
+        if (mine[h]) {
+            T.Jn[at[h]] = cur[h];
+            if (T.delta) {
+                const double o = T.Jold[at[h]], a = nonneg((cur[h] - o) / cur[h]);
+                if (T.hist) T.hist[at[h]] = o;
+                if (!(a <= change)) change = a;
+            }
+        }
+    // the zero of *delta came before the first barrier
+    if (T.delta) block_max_to(change, T.delta);
     if (sblk == 0 && threadIdx.x == 0) *T.sweeps = n + 1;
 }
 
