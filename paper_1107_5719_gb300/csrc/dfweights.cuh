@@ -3,21 +3,21 @@
 #pragma once
 
 #include "df.cuh"
+#include "exptable.cuh"
 
 namespace rt3d {
 namespace {
 
 constexpr int kExpTableDF = 256;
 
-// tab[j] = 2^{-j/256} and tab[256 + j] = 1 - 2^{-j/256} (the latter from
-// expm1, so accurate relative to itself), as double-float pairs (call from
-// all threads, then sync)
+// tab[j] = 2^{-j/256} and tab[256 + j] = 1 - 2^{-j/256} (accurate relative to
+// itself), as double-float pairs (call from all threads, then sync)
+__device__ const exptable::TableDF g_exp_table_df = exptable::table_df();
+
 __device__ __forceinline__ void fill_exp_table_df(dfl* tab)
 {
-    for (int j = threadIdx.x; j < kExpTableDF; j += blockDim.x) {
-        tab[j] = df_from_double(exp2(-(double)j / kExpTableDF));
-        tab[kExpTableDF + j] = df_from_double(-expm1(-(double)j * (0.693147180559945309417 / kExpTableDF)));
-    }
+    for (int j = threadIdx.x; j < 2 * kExpTableDF; j += blockDim.x)
+        tab[j] = dfl{__ldg(&g_exp_table_df.v[j][0]), __ldg(&g_exp_table_df.v[j][1])};
 }
 
 // e^{-x} and 1 - e^{-x} for 0.05 <= x <= 80 (Tang's table-driven method in

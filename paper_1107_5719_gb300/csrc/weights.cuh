@@ -13,6 +13,8 @@
 
 #include <cuda_runtime.h>
 
+#include "exptable.cuh"
+
 namespace rt3d {
 namespace {
 
@@ -43,14 +45,12 @@ namespace {
 constexpr int kExpTable = 512;
 
 // tab[j] = 2^{j/256}, tab[256 + j] = 2^{j/65536} (call from every thread, then
-// __syncthreads()); the second from the series of e^y, y < 2.8e-3.
+// __syncthreads())
+__device__ const exptable::Table64 g_exp_table = exptable::table64();
+
 __device__ __forceinline__ void fill_exp_table(double* tab)
 {
-    for (int j = threadIdx.x; j < 256; j += blockDim.x) {
-        tab[j] = exp2((double)j / 256);
-        const double y = (double)j * (0.693147180559945309417 / 65536);
-        tab[256 + j] = fma(fma(fma(fma(fma(1.0 / 120, y, 1.0 / 24), y, 1.0 / 6), y, 0.5), y, 1.0), y, 1.0);
-    }
+    for (int j = threadIdx.x; j < kExpTable; j += blockDim.x) tab[j] = __ldg(&g_exp_table.v[j]);
 }
 
 // The leading 24 bits of x >= 0, x < 2^127 (below 2^-126: 2^-126 or a little
