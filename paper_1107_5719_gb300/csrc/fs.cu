@@ -274,31 +274,43 @@ __global__ void k_plane_mean(Geometry g, const double* __restrict__ chi, double*
 }
 
 // Estimated march work of every plane (w[k]) and the planes by decreasing
-// work (order[rank] = plane).  One block.
-__global__ void k_plane_rank(int nz, double dz, const double* __restrict__ mean,
-                             double* __restrict__ w, int* __restrict__ order)
+// work (order[rank] = plane).  One block; eight lanes to a plane, six of them
+// one walk each (36 planes: 9.8 us, 23.3 with one thread to a plane).
+constexpr int kRankThreads = 1024;
+__global__ void __launch_bounds__(kRankThreads)
+k_plane_rank(int nz, double dz, const double* __restrict__ mean, double* w, int* __restrict__ order)
 {
     constexpr double kTauEnd = 40.0;
-    const double amu[3] = {1.0, 0.5, 0.2};
-    for (int k0 = threadIdx.x; k0 < nz; k0 += blockDim.x) {
-        double work = 0.0;
-        for (int q = 0; q < 3; ++q) {
-            const double hs = dz / (2.0 * amu[q]);
-            for (int s = -1; s <= 1; s += 2) {
-                double tau = 0.0;
-                int n = 1;   // per-characteristic overhead, about one step
-                for (int k = k0; k - s >= 0 && k - s < nz && tau <= kTauEnd; k -= s, ++n)
-                    tau += hs * (mean[k] + mean[k - s]);
-                work += n;
+    const int lane = threadIdx.x & 7, first = threadIdx.x >> 3, step = kRankThreads / 8;
+    const int rounds = (nz + step - 1) / step;
+    for (int r = 0; r < rounds; ++r) {
+        const int k0 = first + r * step;
+        int n = 0;
+        if (k0 < nz && lane < 6) {
+            const double amu = lane < 2 ? 1.0 : lane < 4 ? 0.5 : 0.2;
+            const double hs = dz / (2.0 * amu);
+            const int s = lane & 1 ? 1 : -1;
+            double tau = 0.0, here = mean[k0];
+            n = 1;       // per-characteristic overhead, about one step
+            for (int k = k0; k - s >= 0 && k - s < nz && tau <= kTauEnd; k -= s, ++n) {
+                const double next = mean[k - s];
+                tau += hs * (here + next);
+                here = next;
             }
         }
-        w[k0] = work;
+        for (int h = 4; h > 0; h >>= 1) n += __shfl_xor_sync(0xffffffffu, n, h);
+        if (k0 < nz && lane == 0) w[k0] = n;
     }
     __syncthreads();
-    for (int k0 = threadIdx.x; k0 < nz; k0 += blockDim.x) {
+    for (int r = 0; r < rounds; ++r) {
+        const int k0 = first + r * step;
         int rank = 0;
-        for (int j = 0; j < nz; ++j) rank += (w[j] > w[k0]) || (w[j] == w[k0] && j < k0);
-        order[rank] = k0;
+        if (k0 < nz) {
+            const double mine = w[k0];
+            for (int j = lane; j < nz; j += 8) rank += (w[j] > mine) || (w[j] == mine && j < k0);
+        }
+        for (int h = 4; h > 0; h >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, h);
+        if (k0 < nz && lane == 0) order[rank] = k0;
     }
 }
 
@@ -431,7 +443,7 @@ cudaError_t launch_plane_order(const Geometry& g, double dz, const double* chi, 
                                int* order, cudaStream_t st)
 {
     k_plane_mean<<<g.nz, 256, 0, st>>>(g, chi, scratch);
-    k_plane_rank<<<1, 256, 0, st>>>(g.nz, dz, scratch, scratch + g.nz, order);
+    k_plane_rank<<<1, kRankThreads, 0, st>>>(g.nz, dz, scratch, scratch + g.nz, order);
     return cudaGetLastError();
 }
 
