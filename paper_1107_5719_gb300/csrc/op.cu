@@ -483,8 +483,13 @@ constexpr int kAsmRun = 32;      // entries of a run (even)
 constexpr int kAsmShared = 8 * 24 * 1024;    // the lengths of 24 Ki directions
 
 // The two arithmetics of the coefficients: FP64, or double-float pairs.
+// kBlocks: of an SM (double-float waits for its coefficients more than for a
+// pipe: 38 x 46 x 36 with 198 directions 732 us with four, 684 with five, more
+// with six, which spill; FP64 is bound by its pipe, 65^3 solve 430.9 ms with
+// four, 432.0 with five).
 struct AsmF64 {
     using V = double;
+    static constexpr int kBlocks = 4;
     static __device__ __forceinline__ V zero() { return 0.0; }
     static __device__ __forceinline__ V weight(double w) { return w; }
     static __device__ __forceinline__ V fma(V w, V c, V a) { return ::fma(w, c, a); }
@@ -492,6 +497,7 @@ struct AsmF64 {
 };
 struct AsmDF {
     using V = float2;
+    static constexpr int kBlocks = 5;
     static __device__ __forceinline__ V zero() { return make_float2(0.f, 0.f); }
     static __device__ __forceinline__ V weight(double w)
     {
@@ -513,7 +519,7 @@ struct AsmDF {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(kListThreads, 4)
+__global__ void __launch_bounds__(kListThreads, T::kBlocks)
 k_op_assemble(Geometry g, int r0, OpLists L, RecOut ro, const int* __restrict__ lmax, int nwp,
               const int* __restrict__ cnt, const int* __restrict__ segb, const int* __restrict__ E,
               const long long* __restrict__ eb, typename T::V* __restrict__ A)
