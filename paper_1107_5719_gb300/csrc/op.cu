@@ -912,7 +912,15 @@ cudaError_t launch_op_lengths(const Geometry& g, const double* chi, const double
         k_op_pack_len<false><<<op_grid1d(g.N, 256), 256, 0, st>>>(g, chi, S, smax, node);
     // two bits beyond the cutoff cover the FP32 rounding of tau and I
     const float lcut = cut > 0.0 ? (float)(-log2(cut)) + 2.0f + (float)extra_bits : INFINITY;
-    const dim3 grid((g.nx * g.ny + kOpThreads - 1) / kOpThreads, groups, g.nz);
+    // The directions are shared by more blocks than the march's (a ray here is
+    // short, and the last wave of long blocks half empty): twice its groups, and
+    // more until every SM has 32 blocks.  17^3 with 256 directions (FP64): solve 2.81
+    // -> 2.76 ms; 33^3: first formal solution 4.09 -> 4.03; 38 x 46 x 36 with 198 (double-float) 2.26 ->
+    // 2.22; half the march's groups 4.13 and 2.27; four times as the rule's.
+    const int blocks = (g.nx * g.ny + kOpThreads - 1) / kOpThreads;
+    int share = 2 * groups;
+    while (share < g.ndir && (long long)blocks * g.nz * share < 152 * 32) share *= 2;
+    const dim3 grid(blocks, share, g.nz);
     if (own)
         k_op_len<true><<<grid, kOpThreads, 0, st>>>(g, node, S, smax, info, poff, bw32, lcut, lmax, nwp);
     else
