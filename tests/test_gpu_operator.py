@@ -57,6 +57,23 @@ def _form(R, form):
     return (1 if form == "parabolic" else 0, R.RT_DF64 if form == "df" else R.RT_FP64)
 
 
+@pytest.mark.parametrize("form", ["linear", "df"])
+@pytest.mark.parametrize("nz", [127, 128, 129, 257])
+def test_tall_grids_match_oracle(R, oracle_mod, nz, form):
+    """The kernels that share planes, distances and directions among lanes:
+    planes on both sides of one round of the plane order (128), more slots
+    than a block has warps, 35 directions of a sign (more than 32 lanes)."""
+    p = W.random_slab(3, 4, nz, n_theta=10, n_phi=7, seed=nz)
+    _, prec = _form(R, form)
+    S = 0.5 + np.random.default_rng(6).random(p.B.shape)
+    J0 = oracle_mod.formal_solution(p, S)[0]
+    for record in (-1, 0):
+        with R.Solver(p, precision=prec, record=record) as s:
+            J, _ = s.formal_solution(S, want_lstar=False)
+            assert R.rt_fs_record_info(s.ctx)[1] == (record != 0)
+        assert np.allclose(J, J0, rtol=RTOL, atol=0)
+
+
 @pytest.mark.parametrize("form", FORMS)
 @pytest.mark.parametrize("name", PROBLEMS)
 def test_operator_matches_oracle(R, oracle_mod, name, form):
