@@ -94,10 +94,12 @@ __device__ __forceinline__ float rel_screen(double a, double b)
 
 // Maximum over the block of |a - b| / |a| into *out (zeroed before), a the new
 // and b the old values of each thread's V voxels (valid: it has them).  The
-// FP64 quotient (rel_change, seven operations) is formed only by the warps
-// with an FP32 estimate within 2^-18 of the block's largest, so the result is
-// the maximum of the FP64 quotients at a fraction of their cost: the FP64
-// pipe bounds the sweep (129^3: 114 us with the screening, 139 us without).
+// FP64 quotient (rel_change, seven operations) is formed only for the voxels
+// without an estimate and those whose FP32 estimate lies within 2^-18 of the
+// block's largest (of the finite ones: a voxel without an estimate says nothing
+// about the others), so the result is the maximum of the FP64 quotients at a
+// fraction of their cost: the FP64 pipe bounds the sweep (129^3: 114 us with
+// the screening, 139 us without).
 template <int V>
 __device__ __forceinline__ void block_rel_max(const bool (&valid)[V], const double (&a)[V],
                                               const double (&b)[V], double* out)
@@ -107,19 +109,22 @@ __device__ __forceinline__ void block_rel_max(const bool (&valid)[V], const doub
     float f[V], fm = 0.f;
 #pragma unroll
     for (int h = 0; h < V; ++h) {
-        f[h] = valid[h] ? rel_screen(a[h], b[h]) : 0.f;
-        fm = fmaxf(fm, f[h]);
+        f[h] = valid[h] ? rel_screen(a[h], b[h]) : -1.f;
+        if (f[h] < __int_as_float(0x7f800000)) fm = fmaxf(fm, f[h]);
     }
     __syncthreads();
     const int m = __reduce_max_sync(0xffffffffu, __float_as_int(fm));    // >= 0: ordered as ints
     if ((threadIdx.x & 31) == 0) atomicMax(&top, m);
     __syncthreads();
     const float t = __int_as_float(top) * (1.0f - 3.8e-6f);
-    if (!__any_sync(0xffffffffu, fm >= t)) return;
+    bool form = false;
+#pragma unroll
+    for (int h = 0; h < V; ++h) form |= f[h] >= t;
+    if (!__any_sync(0xffffffffu, form)) return;
     unsigned long long u = 0;
 #pragma unroll
     for (int h = 0; h < V; ++h)
-        if (valid[h] && f[h] >= t) {
+        if (f[h] >= t) {
             const unsigned long long o = (unsigned long long)__double_as_longlong(rel_change(a[h], b[h]));
             u = o > u ? o : u;
         }
