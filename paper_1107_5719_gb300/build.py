@@ -41,7 +41,7 @@ def _deps():
     files = [os.path.join(CSRC, s) for s in SOURCES]
     files += [os.path.join(CSRC, "internal.h"), os.path.join(CSRC, "weights.cuh"),
               os.path.join(CSRC, "df.cuh"), os.path.join(CSRC, "dfweights.cuh"),
-              os.path.join(CSRC, "exptable.cuh"),
+              os.path.join(CSRC, "exptable.cuh"), os.path.join(CSRC, "osbarrier.cuh"),
               os.path.join(INCLUDE, "rt3d.h")]
     return files
 

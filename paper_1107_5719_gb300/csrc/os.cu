@@ -23,6 +23,7 @@
 // like the values; max is independent of the order, so results are
 // reproducible.
 #include "internal.h"
+#include "osbarrier.cuh"
 
 namespace rt3d {
 
@@ -427,30 +428,49 @@ k_gs_half(Geometry g, const double* __restrict__ c, const double* __restrict__ r
 // 17^3 0.148 -> 0.100 ms, 33^3 0.173 -> 0.136, 65^3 (bound by the FP64 pipe)
 // 0.63 -> 0.55.
 
-// Barrier of the problem's blocks: returns how many of them had a voxel that
-// has not met the tolerance (more), or -1 when a wait gave up, after at most
-// kBarPolls polls (about a second).  The word (zero before) counts the
-// arrivals in its low half and those blocks in its high half, so that one
-// atomic and one polled load carry both.  The block's stores come before its
-// releasing atomic (block barrier, then release), its later loads after the
-// acquiring load.
+// Barrier of the problem's blocks (bar_wait): returns how many of them had a
+// voxel that has not met the tolerance (more), or a negative number when a wait
+// gave up, after at most kBarPolls polls (about a second).  The block's stores
+// come before its releasing atomic (block barrier, then release), its later
+// loads after the acquiring load.
 constexpr int kBarPolls = 1 << 21;
+struct BarWord {
+    unsigned long long* p;
+    __device__ __forceinline__ void arrive(unsigned long long x)
+    {
+        asm volatile("red.release.gpu.global.add.u64 [%0], %1;" :: "l"(p), "l"(x) : "memory");
+    }
+    __device__ __forceinline__ unsigned long long load()
+    {
+        unsigned long long v;
+        asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+        return v;
+    }
+    __device__ __forceinline__ unsigned long long cas(unsigned long long seen, unsigned long long x)
+    {
+        unsigned long long v;
+        asm volatile("atom.acquire.gpu.global.cas.b64 %0, [%1], %2, %3;"
+                     : "=l"(v) : "l"(p), "l"(seen), "l"(x) : "memory");
+        return v;
+    }
+};
 __device__ __forceinline__ int os_barrier(unsigned long long* word, int nblk, bool more)
 {
     __shared__ int result;
     const bool any = __syncthreads_or(more);
-    if (threadIdx.x == 0) {
-        asm volatile("red.release.gpu.global.add.u64 [%0], %1;"
-                     :: "l"(word), "l"(any ? (1ull << 32) + 1 : 1ull) : "memory");
-        int n = 0;
-        unsigned long long v;
-        do
-            asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(word) : "memory");
-        while ((int)v < nblk && ++n < kBarPolls);
-        result = (int)v < nblk ? -1 : (int)(v >> 32);
-    }
+    if (threadIdx.x == 0) result = bar_wait(BarWord{word}, nblk, any, kBarPolls);
     __syncthreads();
     return result;
+}
+
+// Whether the last barrier, at which a wait gave up, was passed all the same
+// (bar_settle): the same answer in all blocks.
+__device__ __noinline__ bool os_settled(unsigned long long* word, int nblk, bool last_sweep)
+{
+    __shared__ int left;
+    if (threadIdx.x == 0) left = bar_settle(BarWord{word}, nblk);
+    __syncthreads();
+    return left == 0 || (left > 0 && last_sweep);
 }
 
 // acc + sum over the 26 neighbours as in stencil / gs_update (same order), the
@@ -577,8 +597,9 @@ k_os_solve(OsTask one, const OsTask* __restrict__ tasks, const int* __restrict__
         left = os_barrier(word++, T.nblk, more);
         if (left <= 0 || n + 1 >= max_sweeps) break;
     }
-    if (left < 0) {
-        if (threadIdx.x == 0) *T.sweeps = -1;
+    // (Gauss-Seidel: a barrier between the colours is never the last)
+    if (left < 0 && ((GS && ((word - T.words) & 1)) || !os_settled(word - 1, T.nblk, n + 1 >= max_sweeps))) {
+        if (sblk == 0 && threadIdx.x == 0) *T.sweeps = -1;
         return;
     }
     double change = 0.0;
