@@ -1773,7 +1773,10 @@ int solve(rt_ctx* c, double tol, int max_iter, double tol_inner, int max_sweeps,
         c->stats.host_syncs += 1;
         c->stats.iterations += 1;
         harvest(c);
-        if (ns < 0 && (rc = os_graph_done(c, &ns))) return rc;
+        if (ns < 0 && (rc = os_graph_done(c, &ns))) {
+            ng_forget(c);       // its history may not have been written
+            return rc;
+        }
         total_steps += *c->h_steps;
         delta = c->h_scal[2];
         c->ng_last_delta = delta;
@@ -3308,7 +3311,10 @@ static int batch_solve(rt_batch* b, double tol, int max_iter, double tol_inner, 
         BCK(cudaStreamSynchronize(b->stream));
         b->stats.host_syncs += 1;
         b->stats.iterations += 1;
-        if (b->use_graphs && (rc = batch_os_graph_counts(b, act))) return rc;
+        if (b->use_graphs && (rc = batch_os_graph_counts(b, act))) {
+            for (int p : act) ng_forget(b->ctx[p]);     // histories may not have been written
+            return rc;
+        }
         bharvest(b);
         b->stats.steps += *b->h_steps;
         for (int p : act) {
