@@ -140,7 +140,7 @@ struct rt_ctx {
     // per-sweep deltas of one Jacobi solve (device) and a pinned copy
     double* dlt = nullptr;
     double* h_dlt = nullptr;
-    int dlt_cap = 0;
+    long long dlt_cap = 0;
     unsigned long long last_steps = 0;
 
     // Ng acceleration: period (0 = off), older iterates, reduction scratch
@@ -1318,11 +1318,12 @@ int ensure_coef(rt_ctx* c)
     return RT_OK;
 }
 
-int ensure_dlt(rt_ctx* c, int max_sweeps)
+int ensure_dlt(rt_ctx* c, long long max_sweeps)
 {
     if (c->dlt_cap >= max_sweeps) return RT_OK;
-    int cap = max_sweeps < 1024 ? 1024 : max_sweeps;
+    const long long cap = std::max(max_sweeps, 1024LL);
     free_os_graphs(c);          // they hold the old dlt pointer
+    c->dlt_cap = 0;
     CK(dalloc(c->dlt, (size_t)cap));
     if (c->h_dlt) cudaFreeHost(c->h_dlt);
     c->h_dlt = nullptr;
@@ -1356,7 +1357,7 @@ int build_os_graph(rt_ctx* c, rt_ctx::OsGraph& e, const double* Jfs, const doubl
     if (err == cudaSuccess) {
         // prologue; every call is attempted so that the capture is always ended
         cudaError_t e1 = launch_os_rhs(c->g, c->coef, c->rdiag, Jfs, Jold, c->r, gs, c->stream);
-        cudaError_t e2 = cudaMemsetAsync(c->dlt, 0, sizeof(double) * (max_sweeps + kPassSweeps), c->stream);
+        cudaError_t e2 = cudaMemsetAsync(c->dlt, 0, sizeof(double) * ((size_t)max_sweeps + kPassSweeps), c->stream);
         cudaError_t e3 = cudaMemcpyAsync(c->Jb, Jold, sizeof(double) * c->g.N,
                                          cudaMemcpyDeviceToDevice, c->stream);
         cudaError_t e4 = cudaMemsetAsync(c->d_nsw, 0, sizeof(int), c->stream);
@@ -1433,7 +1434,7 @@ int run_os_graph(rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew,
                  int max_sweeps)
 {
     int rc;
-    if ((rc = ensure_dlt(c, max_sweeps + kPassSweeps)) || (rc = ensure_sweep_words(c))) return rc;
+    if ((rc = ensure_dlt(c, (long long)max_sweeps + kPassSweeps)) || (rc = ensure_sweep_words(c))) return rc;
     c->os_one = false;
     rt_ctx::OsGraph* e = nullptr;
     for (auto& x : c->osg)
@@ -1470,6 +1471,17 @@ int os_graph_done(rt_ctx* c, int* sweeps)
     c->stats.launches += c->os_one ? 1 : 2 + passes * (kPassSweeps * per + 1);
     c->stats.jacobi_launches += c->os_one ? *sweeps * per : passes * kPassSweeps * per;
     return RT_OK;
+}
+
+// Barrier words that the one-kernel solves use at most (of a set; of all problems
+// of a batch): 32 MB.  Above them the sweeps run as a graph, which needs a word per sweep too
+// but does not zero them in a kernel of few blocks.
+constexpr long long kBarWords = 1LL << 22;
+
+// Barriers of a solve.
+long long os_barriers(const rt_ctx* c, int max_sweeps)
+{
+    return (long long)max_sweeps * (c->os_method == RT_OS_GAUSS_SEIDEL ? 2 : 1);
 }
 
 // Two sets of at least `words` zeroed barrier words (the set in turn).
@@ -1526,8 +1538,9 @@ int run_os_one(rt_ctx* c, const double* Jfs, const double* Jold, double* Jnew, d
     OsShape sh;
     os_solve_shape(c->g.N, c->num_sms, c->os_method == RT_OS_GAUSS_SEIDEL, &sh);
     if (sh.blocks == 0) return RT_OK;
+    if (os_barriers(c, max_sweeps) > kBarWords) return RT_OK;
     int rc;
-    const int words = max_sweeps * (c->os_method == RT_OS_GAUSS_SEIDEL ? 2 : 1);
+    const int words = (int)os_barriers(c, max_sweeps);
     if ((rc = ensure_os_words(c, words))) return rc;
     const int set = c->os_set;
     OsTask t = os_task(c, Jfs, Jold, Jnew, c->os_words + (long long)set * c->os_cap, c->d_sw, sh.blocks);
@@ -2113,7 +2126,7 @@ cudaError_t build_batch_os_graph(rt_batch* b, const std::vector<int>& act, doubl
         std::vector<cudaGraphNode_t> deps;
         {
             cudaError_t e1 = launch_os_rhs(c->g, c->coef, c->rdiag, c->Jfs, c->J, c->r, gs, st);
-            cudaError_t e2 = cudaMemsetAsync(c->dlt, 0, sizeof(double) * (max_sweeps + kPassSweeps), st);
+            cudaError_t e2 = cudaMemsetAsync(c->dlt, 0, sizeof(double) * ((size_t)max_sweeps + kPassSweeps), st);
             cudaError_t e3 = cudaMemcpyAsync(c->Jb, c->J, sizeof(double) * c->g.N,
                                              cudaMemcpyDeviceToDevice, st);
             cudaError_t e4 = cudaMemsetAsync(c->d_nsw, 0, sizeof(int), st);
@@ -2309,14 +2322,12 @@ int batch_os_one(rt_batch* b, const std::vector<int>& act, double tol_inner, int
     }
     OsShape sh;
     os_solve_shape(total, b->num_sms, method == RT_OS_GAUSS_SEIDEL, &sh);
-    if (sh.blocks == 0) return RT_OK;
-    if (!b->d_tasks) {
-        BCK(cudaMalloc((void**)&b->d_tasks, sizeof(OsTask) * P));
-        BCK(cudaMalloc((void**)&b->d_first, sizeof(int) * P));
-        BCK(cudaMallocHost((void**)&b->h_tasks, sizeof(OsTask) * P));
-        BCK(cudaMallocHost((void**)&b->h_first, sizeof(int) * P));
-    }
-    const int words = max_sweeps * (method == RT_OS_GAUSS_SEIDEL ? 2 : 1);
+    if (sh.blocks == 0 || P * os_barriers(b->ctx[act[0]], max_sweeps) > kBarWords) return RT_OK;
+    if (!b->d_tasks) BCK(cudaMalloc((void**)&b->d_tasks, sizeof(OsTask) * P));
+    if (!b->d_first) BCK(cudaMalloc((void**)&b->d_first, sizeof(int) * P));
+    if (!b->h_tasks) BCK(cudaMallocHost((void**)&b->h_tasks, sizeof(OsTask) * P));
+    if (!b->h_first) BCK(cudaMallocHost((void**)&b->h_first, sizeof(int) * P));
+    const int words = (int)os_barriers(b->ctx[act[0]], max_sweeps);
     if (b->bdlt_cap < words) {
         dfree(b->d_bdlt);
         b->bdlt_cap = 0;
@@ -2363,7 +2374,7 @@ int batch_os_graph(rt_batch* b, const std::vector<int>& act, double tol_inner, i
     if ((rc = batch_os_one(b, act, tol_inner, max_sweeps, ran)) || ran) return rc;
     for (int p : act) {
         rt_ctx* c = b->ctx[p];
-        if ((rc = bpass(b, p, ensure_dlt(c, max_sweeps + kPassSweeps)))) return rc;
+        if ((rc = bpass(b, p, ensure_dlt(c, (long long)max_sweeps + kPassSweeps)))) return rc;
         if (!c->d_nsw) BCK(cudaMalloc((void**)&c->d_nsw, sizeof(int)));
     }
     std::vector<const void*> key = batch_graph_key(b, act, tol_inner, max_sweeps);

@@ -28,9 +28,9 @@ lib.fake_solves.argtypes = [C.c_int, C.c_double]
 lib.fake_live.restype = lib.fake_peak.restype = C.c_longlong
 GB = 1 << 30
 def counts():
-    n = (C.c_int * 6)()
+    n = (C.c_int * 7)()
     lib.fake_counts(n)
-    return dict(zip(("solves", "graphs", "marches", "applies", "lengths", "ng"), n))
+    return dict(zip(("solves", "graphs", "marches", "applies", "lengths", "ng", "outside"), n))
 """
 
 

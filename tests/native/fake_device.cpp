@@ -13,7 +13,8 @@
 namespace {
 std::map<void*, size_t> g_mem;
 long long g_total = 284LL << 30, g_live = 0, g_peak = 0, g_fail_lo = 1, g_fail_hi = 0;
-int g_sweeps = 5, g_solves = 0, g_graphs = 0, g_marches = 0, g_applies = 0, g_lengths = 0, g_ng = 0;
+int g_sweeps = 5, g_solves = 0, g_graphs = 0, g_marches = 0, g_applies = 0, g_lengths = 0, g_ng = 0,
+    g_outside = 0;
 double g_delta = 0.5;
 int g_entries = 64, g_rows = 64;        // of every plane of an operator
 }  // namespace
@@ -32,12 +33,12 @@ long long fake_peak(int reset)
     return p;
 }
 // {one-kernel solves, graph launches, marches, applied operators, length marches,
-// extrapolations} since the last call
+// extrapolations, barrier words outside their allocation} since the last call
 void fake_counts(int* n)
 {
-    const int c[6] = {g_solves, g_graphs, g_marches, g_applies, g_lengths, g_ng};
+    const int c[7] = {g_solves, g_graphs, g_marches, g_applies, g_lengths, g_ng, g_outside};
     std::memcpy(n, c, sizeof c);
-    g_solves = g_graphs = g_marches = g_applies = g_lengths = g_ng = 0;
+    g_solves = g_graphs = g_marches = g_applies = g_lengths = g_ng = g_outside = 0;
 }
 
 cudaError_t cudaMalloc(void** p, size_t n)
@@ -83,6 +84,11 @@ cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind)
 }
 cudaError_t cudaMemsetAsync(void* d, int x, size_t n, cudaStream_t)
 {
+    if (!x && n >= 1 << 24 && (size_t)d % 4096 == 0) {      // without touching the pages
+        madvise(d, n / 4096 * 4096, MADV_DONTNEED);
+        d = (char*)d + n / 4096 * 4096;
+        n %= 4096;
+    }
     std::memset(d, x, n);
     return cudaSuccess;
 }
@@ -93,8 +99,24 @@ const char* cudaGetErrorString(cudaError_t e)
     return e == cudaErrorMemoryAllocation ? "out of memory" : "error";
 }
 cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return ++g_graphs, cudaSuccess; }
+cudaError_t cudaGraphAddNode(cudaGraphNode_t*, cudaGraph_t, const cudaGraphNode_t*, const cudaGraphEdgeData*,
+                             size_t, cudaGraphNodeParams* p)
+{
+    static cudaGraph_t body[1];
+    p->conditional.phGraph_out = body;
+    return cudaSuccess;
+}
 
 }  // extern "C"
+
+// Whether [p, p + n) lies in one allocation.
+static bool inside(const void* p, long long n)
+{
+    auto it = g_mem.upper_bound(const_cast<void*>(p));
+    if (it == g_mem.begin()) return false;
+    --it;
+    return n >= 0 && (char*)p + n <= (char*)it->first + it->second;
+}
 
 namespace rt3d {
 
@@ -151,12 +173,14 @@ cudaError_t launch_fsdf(const ViewDF&, double, int, unsigned long long*, cudaStr
 {
     return ++g_marches, cudaSuccess;
 }
-cudaError_t launch_os_solve(const OsTask& one, const OsTask* tasks, const int*, int ntask, const OsShape&, bool,
-                            int, int, double, cudaStream_t)
+cudaError_t launch_os_solve(const OsTask& one, const OsTask* tasks, const int*, int ntask, const OsShape&, bool gs,
+                            int, int max_sweeps, double, cudaStream_t)
 {
     ++g_solves;
     for (int q = 0; q < (tasks ? ntask : 1); ++q) {
         const OsTask& t = tasks ? tasks[q] : one;
+        g_outside += !inside(t.words, 8LL * max_sweeps * (gs ? 2 : 1)) ||
+                     (t.nclear && !inside(t.clear, 8LL * t.nclear));
         *t.sweeps = g_sweeps;
         if (t.delta) *t.delta = g_delta;
     }
