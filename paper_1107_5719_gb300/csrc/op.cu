@@ -892,8 +892,9 @@ cudaError_t launch_op_lists(const Geometry& g, const DirInfo* info, const StepGe
 {
     const size_t shm = scratch ? 0 : sizeof(int) * (size_t)g.nx * g.ny;
     if (shm > 40 * 1024) {
+        // one value for all planes: contexts of several threads set it
         cudaError_t e = cudaFuncSetAttribute(k_op_lists, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)shm);
+                                             (int)sizeof(int) * kListSmemNodes);
         if (e != cudaSuccess) return e;
     }
     k_op_lists<<<2 * g.nz, kListThreads, shm, st>>>(g, info, off, bw, dn, L, scratch);

@@ -34,31 +34,45 @@ def counts():
 """
 
 
-def build(folder):
-    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
-    if not os.path.exists(nvcc):
+def sh(*cmd):
+    return subprocess.run(cmd, check=True, capture_output=True, text=True, timeout=600).stdout
+
+
+def nvcc():
+    path = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    if not os.path.exists(path):
         pytest.skip("nvcc not available")
+    return path
 
-    def sh(*cmd):
-        return subprocess.run(cmd, check=True, capture_output=True, text=True, timeout=600).stdout
 
-    api, fake, stubs = (os.path.join(folder, n) for n in ("api.o", "fake.o", "stubs.c"))
-    flags = ["-std=c++17", "-O1", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include")]
-    sh(nvcc, *flags, "-c", os.path.join(CSRC, "api.cu"), "-o", api)
-    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc))), "include")
-    sh("g++", "-std=c++17", "-O1", "-w", "-fPIC", "-I", cuda, "-c",
-       os.path.join(HERE, "native", "fake_device.cpp"), "-o", fake)
+def compile_cpp(name, obj):
+    """native/<name> against the CUDA headers alone."""
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(nvcc()))), "include")
+    sh("g++", "-std=c++17", "-O1", "-w", "-fPIC", "-I", cuda, "-c", os.path.join(HERE, "native", name), "-o", obj)
+    return obj
 
+
+def stubs(objs, folder, also=()):
+    """Functions that return 0 for the CUDA calls and launches (and `also`) that
+    the objects call and none of them defines."""
     def symbols(which):
-        return {line.split()[-1] for o in (api, fake) for line in sh("nm", which, o).splitlines() if line.strip()}
+        return {line.split()[-1] for o in objs for line in sh("nm", which, o).splitlines() if line.strip()}
 
-    names = {n for n in symbols("-u") if n.startswith(("cuda", "__cuda", "_ZN4rt3d"))} | set(exported_names())
-    names = sorted(names - symbols("--defined-only"))
-    with open(stubs, "w") as f:
-        f.writelines(f"long {n}(void) {{ return 0; }}\n" for n in names)
+    names = {n for n in symbols("-u") if n.startswith(("cuda", "__cuda", "_ZN4rt3d"))} | set(also)
+    src = os.path.join(folder, "stubs.c")
+    with open(src, "w") as f:
+        f.writelines(f"long {n}(void) {{ return 0; }}\n" for n in sorted(names - symbols("--defined-only")))
+    sh("gcc", "-w", "-fPIC", "-c", src, "-o", src + ".o")
+    return src + ".o"
+
+
+def build(folder):
+    api = os.path.join(folder, "api.o")
+    sh(nvcc(), "-std=c++17", "-O1", "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-c",
+       os.path.join(CSRC, "api.cu"), "-o", api)
+    objs = [api, compile_cpp("fake_device.cpp", os.path.join(folder, "fake.o"))]
     lib = os.path.join(folder, "librt3d_fake.so")
-    sh("gcc", "-w", "-fPIC", "-c", stubs, "-o", stubs + ".o")
-    sh("g++", "-shared", "-o", lib, api, fake, stubs + ".o", "-Wl,-Bsymbolic")
+    sh("g++", "-shared", "-o", lib, *objs, stubs(objs, folder, exported_names()), "-Wl,-Bsymbolic")
     return lib
 
 
