@@ -217,7 +217,12 @@ int rt_last_step_count(rt_ctx *ctx, unsigned long long *steps);
  * 128 N + the source records (65^3 x 1024: 38.9 GB).  max_bytes: -1
  * (default) records when that fits in 60% of the device and leaves 2 GiB
  * free, 0 never records, > 0 records when it fits in max_bytes; otherwise
- * every formal solution marches.  J agrees with the march to rounding (the
+ * every formal solution marches; it also marches when the device has no memory
+ * for what a recording takes beside that block (FP64 and double-float: about
+ * 224 N + 4 ndir nz (ceil(nx ny/32) + 3) + 16 nz^2 bytes of working storage
+ * from the first recording on and, with as many directions up as down, 84 ndir
+ * nz + 16 nz min(nx ny, 2 ndir) bytes of node lists per quadrature; without the
+ * lists the coefficients are kept ray by ray).  J agrees with the march to rounding (the
  * terms are summed in another order).  Short characteristics record the
  * weights of every (voxel, direction) under the same setting, 24 ndir N bytes
  * in FP64 and 16 ndir N + 16 N in double-float.  RT_EINVAL for max_bytes <

@@ -574,14 +574,24 @@ int ensure_op_work(rt_ctx* c)
 double cut_of(const rt_ctx* c);
 ViewDF viewdf(rt_ctx* c);
 
+// rc of an allocation that a recording can do without: no memory is no error.
+bool no_memory(rt_ctx* c, int rc)
+{
+    if (rc != RT_ENOMEM) return false;
+    c->err.clear();
+    cudaGetLastError();
+    return true;
+}
+
 // Below this bound on an operator's bytes its exact size is not asked for:
 // the recording runs without a host wait.
 constexpr long long kOpNoWait = 64LL << 20;
 
 // Record the march of the current source (FP64, linear or parabolic, or
 // double-float) and assemble its operator, or keep it ray by ray where the
-// operator would take more memory (op_budget).  use: whether a recording is
-// held afterwards.
+// operator would take more memory (op_budget) or its lists get none.  use:
+// whether a recording is held afterwards (not where the block or the working
+// storage gets no memory: the march runs).
 int ensure_op_rec(rt_ctx* c, int G, bool& use)
 {
     use = false;
@@ -591,10 +601,19 @@ int ensure_op_rec(rt_ctx* c, int G, bool& use)
         use = true;
         return RT_OK;
     }
-    const long long limit = std::max(rec_limit(c), c->rec_cap);
+    long long limit = std::max(rec_limit(c), c->rec_cap);
     if (need > limit) return RT_OK;
     int rc;
-    if ((rc = ensure_op_work(c))) return rc;
+    if (!c->ow_mem) {
+        if ((rc = ensure_op_work(c))) return no_memory(c, rc) ? RT_OK : rc;
+        // what is left beside it
+        limit = std::max(rec_limit(c), c->rec_cap);
+        if (need > limit) {
+            CK(cudaStreamSynchronize(c->stream));
+            free_op_work(c);
+            return RT_OK;
+        }
+    }
     const Geometry& g = c->g;
     const bool para = c->src_order == RT_SRC_PARABOLIC, df = c->precision == RT_DF64;
     const long long nxy = (long long)g.nx * g.ny, nwp = op_tiles(c);
@@ -610,8 +629,11 @@ int ensure_op_rec(rt_ctx* c, int G, bool& use)
     for (int k = 0; k < g.nz; ++k) order[k] = k;
     std::vector<int> first{0, g.nz};    // ranks of the chunks' first planes
     long long entries = 0, rows = 0, chunk = 0;
+    if (op && (rc = ensure_op_lists(c))) {
+        if (!no_memory(c, rc)) return rc;
+        op = false;
+    }
     if (op) {
-        if ((rc = ensure_op_lists(c))) return rc;
         CK(launch_op_counts(g, c->ol, para, w.Lp, w.rowbase, w.cnt, w.segb, w.E, w.rows, st));
         c->stats.launches += 1;
         op_bounds(c, para, &eb, &prow, entries, rows);

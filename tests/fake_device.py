@@ -23,14 +23,13 @@ sys.path.insert(0, {root!r})
 from paper_1107_5719_gb300 import rt3d as R, workloads as W
 lib = R.load({lib!r})
 lib.fake_memory.argtypes = [C.c_longlong]
-lib.fake_fail.argtypes = [C.c_longlong, C.c_longlong]
 lib.fake_solves.argtypes = [C.c_int, C.c_double]
 lib.fake_live.restype = lib.fake_peak.restype = C.c_longlong
 GB = 1 << 30
 def counts():
-    n = (C.c_int * 7)()
+    n = (C.c_int * 8)()
     lib.fake_counts(n)
-    return dict(zip(("solves", "graphs", "marches", "applies", "lengths", "ng", "outside"), n))
+    return dict(zip(("solves", "graphs", "marches", "applies", "lengths", "ng", "outside", "replays"), n))
 """
 
 

@@ -1,6 +1,6 @@
 // A device in host memory for tests of the library's host code (csrc/api.cu) where no
 // GPU is wanted: device allocations are counted against a total that the test
-// sets, those of chosen sizes fail, and the kernels whose results steer the host
+// sets, a chosen one fails, and the kernels whose results steer the host
 // code write what the test says.  Every other kernel launch and CUDA call that
 // api.cu makes is a stub that returns 0 (fake_device.py writes them).
 #include "../../paper_1107_5719_gb300/csrc/internal.h"
@@ -12,9 +12,10 @@
 
 namespace {
 std::map<void*, size_t> g_mem;
-long long g_total = 284LL << 30, g_live = 0, g_peak = 0, g_fail_lo = 1, g_fail_hi = 0;
+long long g_total = 284LL << 30, g_live = 0, g_peak = 0;
 int g_sweeps = 5, g_solves = 0, g_graphs = 0, g_marches = 0, g_applies = 0, g_lengths = 0, g_ng = 0,
-    g_outside = 0;
+    g_outside = 0, g_replays = 0, g_nth = -1;
+cudaError_t g_last = cudaSuccess;
 double g_delta = 0.5;
 int g_entries = 64, g_rows = 64;        // of every plane of an operator
 }  // namespace
@@ -22,7 +23,9 @@ int g_entries = 64, g_rows = 64;        // of every plane of an operator
 extern "C" {
 
 void fake_memory(long long total) { g_total = total; }
-void fake_fail(long long lo, long long hi) { g_fail_lo = lo; g_fail_hi = hi; }
+// the n-th allocation from here fails (-1: none; it is -1 again once it has)
+void fake_fail(int n) { g_nth = n; }
+int fake_failed(void) { return g_nth < 0; }
 void fake_solves(int sweeps, double delta) { g_sweeps = sweeps; g_delta = delta; }
 void fake_operator(int entries, int rows) { g_entries = entries; g_rows = rows; }
 long long fake_live(void) { return g_live; }
@@ -33,21 +36,23 @@ long long fake_peak(int reset)
     return p;
 }
 // {one-kernel solves, graph launches, marches, applied operators, length marches,
-// extrapolations, barrier words outside their allocation} since the last call
+// extrapolations, barrier words outside their allocation, ray-by-ray replays} since the
+// last call
 void fake_counts(int* n)
 {
-    const int c[7] = {g_solves, g_graphs, g_marches, g_applies, g_lengths, g_ng, g_outside};
+    const int c[8] = {g_solves, g_graphs, g_marches, g_applies, g_lengths, g_ng, g_outside, g_replays};
     std::memcpy(n, c, sizeof c);
-    g_solves = g_graphs = g_marches = g_applies = g_lengths = g_ng = g_outside = 0;
+    g_solves = g_graphs = g_marches = g_applies = g_lengths = g_ng = g_outside = g_replays = 0;
 }
 
 cudaError_t cudaMalloc(void** p, size_t n)
 {
     *p = nullptr;
-    if (((long long)n >= g_fail_lo && (long long)n <= g_fail_hi) || g_live + (long long)n > g_total)
-        return cudaErrorMemoryAllocation;
+    const bool chosen = g_nth == 0;
+    if (g_nth >= 0) --g_nth;
+    if (chosen || g_live + (long long)n > g_total) return g_last = cudaErrorMemoryAllocation;
     void* m = mmap(nullptr, n, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
-    if (m == MAP_FAILED) return cudaErrorMemoryAllocation;
+    if (m == MAP_FAILED) return g_last = cudaErrorMemoryAllocation;
     g_mem[m] = n;
     g_live += (long long)n;
     if (g_live > g_peak) g_peak = g_live;
@@ -91,6 +96,12 @@ cudaError_t cudaMemsetAsync(void* d, int x, size_t n, cudaStream_t)
     }
     std::memset(d, x, n);
     return cudaSuccess;
+}
+cudaError_t cudaGetLastError(void)
+{
+    const cudaError_t e = g_last;
+    g_last = cudaSuccess;
+    return e;
 }
 cudaError_t cudaGetDeviceCount(int* n) { return *n = 1, cudaSuccess; }
 cudaError_t cudaDeviceGetAttribute(int* v, cudaDeviceAttr, int) { return *v = 152, cudaSuccess; }
@@ -151,27 +162,36 @@ cudaError_t launch_op_lengths(const Geometry&, const double*, const double*, con
                               const int*, const float4*, double, int, bool, int, float2*, int*, int, int*,
                               unsigned long long*, cudaStream_t)
 {
-    return ++g_lengths, cudaSuccess;
+    return ++g_lengths, cudaGetLastError();
 }
 cudaError_t launch_op_apply64(const Geometry&, const double*, const double*, const OpMap&, double*,
                               unsigned long long*, cudaStream_t)
 {
-    return ++g_applies, cudaSuccess;
+    return ++g_applies, cudaGetLastError();
 }
 cudaError_t launch_op_apply_df(const Geometry&, const double*, const double*, const OpMap&, double, double*,
                                unsigned long long*, cudaStream_t)
 {
-    return ++g_applies, cudaSuccess;
+    return ++g_applies, cudaGetLastError();
 }
 cudaError_t launch_fs64(const Geometry&, const double*, const double*, const double*, const double*,
                         const DirInfo*, const StepGeo*, const Bw4d*, const Bw4d*, const double*, double, int,
                         double*, unsigned long long*, cudaStream_t)
 {
-    return ++g_marches, cudaSuccess;
+    return ++g_marches, cudaGetLastError();
+}
+cudaError_t launch_fs64rep(const Geometry&, const double*, const DirInfo*, const StepGeo*, const Bw4d*, const FsRec&,
+                           int, double*, unsigned long long*, cudaStream_t)
+{
+    return ++g_replays, cudaGetLastError();
+}
+cudaError_t launch_fsdfrep(const ViewDF&, const Rec32&, int, unsigned long long*, cudaStream_t)
+{
+    return ++g_replays, cudaGetLastError();
 }
 cudaError_t launch_fsdf(const ViewDF&, double, int, unsigned long long*, cudaStream_t)
 {
-    return ++g_marches, cudaSuccess;
+    return ++g_marches, cudaGetLastError();
 }
 cudaError_t launch_os_solve(const OsTask& one, const OsTask* tasks, const int*, int ntask, const OsShape&, bool gs,
                             int, int max_sweeps, double, cudaStream_t)

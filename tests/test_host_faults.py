@@ -1,5 +1,5 @@
 """The host code on a device in host memory (fake_device.py): waits that gave up,
-numbers of sweeps up to the largest."""
+numbers of sweeps up to the largest, allocations that fail."""
 
 import pytest
 
@@ -66,4 +66,38 @@ for method in (0, 1):
         one = 3 * sweeps * (1 + method) <= 1 << 22
         assert n["outside"] == 0 and (n["solves"] == 2) == one and (n["graphs"] == 2) != one, (method, sweeps, n)
         R.rt_batch_destroy(b)
+""")
+
+
+@pytest.mark.parametrize("form", ["fp64", "df64", "parabolic", "short"])
+def test_recording_that_gets_no_memory_marches(lib, form):
+    """Each allocation of a first formal solution with recording fails in turn: the
+    formal solution marches, or replays ray by ray, and the next one records."""
+    fake_device.run(lib, f"""
+form = {form!r}
+p = W.random_slab(9, 8, 12, n_theta=4, n_phi=6, seed=1)
+p.src_order = int(form == "parabolic")
+kw = dict(precision=R.RT_DF64 if form == "df64" else R.RT_FP64,
+          fs_method=R.RT_FS_SHORT if form == "short" else R.RT_FS_LONG)
+n = tried = 0
+while True:
+    with R.Solver(p, record=0, **kw) as s:
+        s.formal_solution(p.B)          # the buffers of every formal solution
+        R.rt_set_fs_record(s.ctx, -1)
+        counts()
+        lib.fake_fail(n)
+        s.formal_solution(p.B)
+        if not lib.fake_failed():
+            lib.fake_fail(-1)
+            break
+        first = counts()
+        s.formal_solution(p.B)
+        assert R.rt_fs_record_info(s.ctx)[1], n
+        if form in ("fp64", "df64"):
+            assert first["marches"] + first["replays"] == 1 and not first["applies"], (n, first)
+            again = counts()
+            assert again["applies"] == (first["marches"]) and again["replays"] == first["replays"], (n, again)
+    n += 1
+assert n >= (1 if form == "short" else 3), n
+assert lib.fake_live() == 0
 """)
