@@ -511,14 +511,22 @@ int rt_batch_set_block_order(rt_batch *batch, int order);
  * afterwards (FP32 sweep: all replays in one fused launch), exactly as a
  * single solve does, so the batch's iterates stay bit-identical to single
  * solves.  A problem starts iterating once its recording fits in the
- * budget beside the recordings held (max_bytes: -1 (default) 60% of the
- * device, while what the unconverged problems still allocate at their
- * finishing stage and 4 GiB stay free; 0 no recordings; > 0 a byte
- * limit), and returns the memory when
+ * budget beside what the running problems hold or may still take (max_bytes:
+ * -1 (default) 60% of the device, while what the unconverged problems still
+ * allocate, at their finishing stage too, and 4 GiB stay free; 0 no
+ * recordings; > 0 a byte limit), and returns the memory when
  * it converges or reaches max_iter; problems run in waves when the budget
  * holds fewer than all (65^3 x 1024 directions, FP32 sweep: 39 GB each).
- * A problem whose recording could never fit marches from the start.
- * Releases the recordings held.  RT_EINVAL for max_bytes < -1. */
+ * FP64 and double-float problems may take what an operator can need, at most
+ * half as much again as the ray-by-ray recording (at least 4, at most 24 GiB
+ * more), until they have recorded; then they hold what theirs takes.  Where the
+ * budget is below that, or nothing is running whose memory could be waited for,
+ * they get the ray-by-ray recording's bytes.
+ * A problem whose recording could never fit marches from the start, and so does
+ * one whose memory the device does not have.  The batch keeps up to 8 GiB of the
+ * returned memory for its next solve.
+ * This call releases the recordings held and the memory kept.  RT_EINVAL for
+ * max_bytes < -1. */
 int rt_batch_set_fs_record(rt_batch *batch, long long max_bytes);
 /* on != 0 (the default): every outer iteration runs the operator-splitting
  * solves of all active problems (Sect. 2.3) as ONE CUDA graph, one

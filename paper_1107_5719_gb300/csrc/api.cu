@@ -488,6 +488,23 @@ long long rec_ask(const rt_ctx* c, long long need)
     return std::max(need, std::min(most, op_budget(c, need)));
 }
 
+// Bytes of a context's node lists and of its working storage.
+long long op_list_bytes(const rt_ctx* c)
+{
+    const long long nxy = (long long)c->g.nx * c->g.ny, Q = 2LL * c->g.nz;
+    const long long icap = 4LL * std::max(c->dpos, c->g.ndir - c->dpos), ucap = std::min(nxy, icap);
+    return up256(4LL * c->g.ndir) + up256(4 * Q) + up256(4 * Q * ucap) + up256(4 * Q * (ucap + 1)) +
+           up256(4 * Q * icap) + up256(4LL * c->g.ndir * c->g.nz) +
+           up256((long long)sizeof(OpContrib) * Q * icap) + 256;
+}
+
+long long op_work_bytes(const rt_ctx* c)
+{
+    const long long T = (long long)c->g.ndir * c->g.nz, Q = 2LL * c->g.nz * c->g.nz;
+    return up256(32 * c->g.N) + up256(4 * T * op_tiles(c)) + 3 * up256(4 * T) + 2 * up256(4 * Q) +
+           4 * up256(8LL * c->g.nz) + 256 + 3 * up256(8LL * kSlots * c->g.N);
+}
+
 // Node lists of the context's directions, built at the first recording.
 int ensure_op_lists(rt_ctx* c)
 {
@@ -502,10 +519,9 @@ int ensure_op_lists(rt_ctx* c)
     const long long b_dord = up256(4LL * g.ndir), b_cnt = up256(4 * Q),
                     b_node = up256(4 * Q * L.ucap), b_start = up256(4 * Q * (L.ucap + 1)),
                     b_item = up256(4 * Q * L.icap), b_pos = up256(4LL * g.ndir * g.nz),
-                    b_con = up256((long long)sizeof(OpContrib) * Q * L.icap), b_l = 256;
-    const long long total = b_dord + b_cnt + b_node + b_start + b_item + b_pos + b_con + b_l;
+                    b_con = up256((long long)sizeof(OpContrib) * Q * L.icap);
     char* m = nullptr;
-    CK(cudaMalloc((void**)&m, (size_t)total));
+    CK(cudaMalloc((void**)&m, (size_t)op_list_bytes(c)));
     char* q = m;
     int* dord = reinterpret_cast<int*>(q); q += b_dord;
     L.dord = dord;
@@ -548,7 +564,7 @@ int ensure_op_work(rt_ctx* c)
                     b_q = up256(4 * Q), b_z = up256(8LL * g.nz),
                     b_slot = up256(8LL * kSlots * g.N);
     char* m = nullptr;
-    CK(cudaMalloc((void**)&m, (size_t)(b_sp + b_lmax + 3 * b_t + 2 * b_q + 4 * b_z + 256 + 3 * b_slot)));
+    CK(cudaMalloc((void**)&m, (size_t)op_work_bytes(c)));
     c->ow_mem = m;
     auto& w = c->ow;
     w.sp = reinterpret_cast<double*>(m); m += b_sp;
@@ -1960,6 +1976,81 @@ int batch_groups(const rt_batch* b, const std::vector<int>& act)
     return G;
 }
 
+// Free pooled blocks until at most `keep` bytes are held, the largest first;
+// not block `pick`.
+void batch_free_pool(rt_batch* b, long long keep = 0, char* pick = nullptr)
+{
+    long long held = 0;
+    for (auto& blk : b->rec_pool) held += blk.second;
+    if (held <= keep) return;
+    cudaStreamSynchronize(b->stream);
+    std::sort(b->rec_pool.begin(), b->rec_pool.end(),
+              [](const auto& x, const auto& y) { return x.second < y.second; });
+    for (size_t i = b->rec_pool.size(); i-- > 0 && held > keep;) {
+        if (b->rec_pool[i].first == pick) continue;
+        held -= b->rec_pool[i].second;
+        cudaFree(b->rec_pool[i].first);
+        b->rec_pool.erase(b->rec_pool.begin() + i);
+    }
+}
+
+// What the batch's recordings may take: `used` of `limit` bytes are held or
+// promised to the admitted problems that have not recorded yet; automatic:
+// `reserve` of the `free_now` bytes of the device (less what is promised) stay free.
+struct RecBudget {
+    long long limit = 0, used = 0, reserve = 0, free_now = 0;
+    bool automatic = false;
+};
+
+// Give problem c up to `want` bytes for its recording, with a pooled block to
+// start from, where the budget has them; blocks it cannot use go back to the
+// device where that makes the room.  op: what it will take is known when it
+// records (ensure_op_rec), at most `want`; else it takes them now.
+bool batch_take(rt_batch* b, rt_ctx* c, long long want, bool op, RecBudget& m)
+{
+    // the smallest block that holds it; for an operator else the largest
+    int pick = -1;
+    long long pooled = 0;
+    for (size_t i = 0; i < b->rec_pool.size(); ++i) {
+        const long long cap = b->rec_pool[i].second, best = pick < 0 ? 0 : b->rec_pool[pick].second;
+        pooled += cap;
+        if (cap >= want ? best < want || cap < best : op && cap > best) pick = (int)i;
+    }
+    char* mem = pick < 0 ? nullptr : b->rec_pool[pick].first;
+    long long cap = pick < 0 ? 0 : b->rec_pool[pick].second;
+    const long long work = op && !c->ow_mem ? op_work_bytes(c) : 0;
+    auto room = [&](long long have, long long freed) {
+        const long long grow = std::max(want - have, 0LL);
+        return m.used + grow <= m.limit + freed &&
+               (!m.automatic || grow + work + m.reserve <= m.free_now + freed);
+    };
+    if (!room(cap, 0)) {
+        if (!room(cap, pooled - cap)) {
+            if (!room(0, pooled)) return false;
+            mem = nullptr;
+            cap = 0;
+        }
+        batch_free_pool(b, cap, mem);
+        m.used -= pooled - cap;
+        m.free_now += pooled - cap;
+    }
+    for (size_t i = 0; mem && i < b->rec_pool.size(); ++i)
+        if (b->rec_pool[i].first == mem) {
+            b->rec_pool.erase(b->rec_pool.begin() + i);
+            c->rec_mem = mem;
+            c->rec_cap = cap;
+            break;
+        }
+    c->rec_mode = std::max(want, cap);
+    if (!op) {
+        bool use = false;
+        if (ensure_rec(c, use) != RT_OK || !use) return false;
+    }
+    m.used += std::max(want - cap, 0LL);
+    m.free_now -= std::max(want - cap, 0LL) + work;
+    return true;
+}
+
 // Admit waiting problems (in launch order) whose recorded march fits in the
 // batch's budget beside the recordings held; a problem whose form does not
 // record, or whose recording could never fit, starts at once and marches.
@@ -1967,74 +2058,55 @@ int batch_groups(const rt_batch* b, const std::vector<int>& act)
 // too, so that the solve always progresses.
 int batch_admit(rt_batch* b, int max_iter)
 {
-    long long limit = b->rec_mode, reserve = 0, free_now = 0;
-    if (limit < 0) {
+    RecBudget m;
+    m.limit = b->rec_mode;
+    m.automatic = b->rec_mode < 0;
+    bool running = false;
+    for (auto& blk : b->rec_pool) m.used += blk.second;
+    if (m.automatic) {
         // automatic: recordings up to 60% of the device, each admitted only
         // while what the unconverged problems still allocate (Ng's iterates;
-        // at their finishing stage the reference's double-float node planes
-        // and tables, S_ref, J_ref and the source change) stays free beside
-        // it, with 4 GiB to spare
+        // node lists; at their finishing stage the reference's double-float
+        // node planes and tables, S_ref, J_ref and the source change) stays
+        // free beside it, with 4 GiB to spare
         size_t fr = 0, tot = 0;
         BCK(cudaMemGetInfo(&fr, &tot));
-        limit = (long long)(0.6 * (double)tot);
-        reserve = 4LL << 30;
-        for (size_t p = 0; p < b->ctx.size(); ++p) {
-            const rt_ctx* c = b->ctx[p];
-            if (b->converged[p] || c->S_ref) continue;
-            reserve += 24 * c->g.N + (c->node4 ? 0 : 64 * c->g.N) +
-                       (c->ng_old[0] ? 0 : 24 * c->g.N) +     // Ng's older iterates
-                       36LL * c->g.ndir * c->g.nz + (1LL << 20);
-        }
-        free_now = (long long)fr;
+        m.limit = (long long)(0.6 * (double)tot);
+        m.free_now = (long long)fr;
+        m.reserve = 4LL << 30;
     }
-    long long used = 0;
-    bool running = false;
     for (size_t p = 0; p < b->ctx.size(); ++p) {
-        used += b->ctx[p]->rec_cap;
-        if (b->admitted[p] && !b->converged[p] && b->iters[p] < max_iter) running = true;
+        const rt_ctx* c = b->ctx[p];
+        const bool op = c->precision != RT_FP32_SWEEP;
+        if (m.automatic && !b->converged[p] && !c->S_ref)
+            m.reserve += 24 * c->g.N + (c->node4 ? 0 : 64 * c->g.N) +
+                         (c->ng_old[0] ? 0 : 24 * c->g.N) +     // Ng's older iterates
+                         36LL * c->g.ndir * c->g.nz + (1LL << 20);
+        if (m.automatic && !b->converged[p] && op && !c->ol_mem && op_fits(c))
+            m.reserve += op_list_bytes(c);
+        m.used += c->rec_cap;
+        if (!b->admitted[p] || b->converged[p] || b->iters[p] >= max_iter) continue;
+        running = true;
+        if (c->rec_valid || c->rec_mode <= c->rec_cap) continue;
+        m.used += c->rec_mode - c->rec_cap;         // promised
+        m.free_now -= c->rec_mode - c->rec_cap + (op && !c->ow_mem ? op_work_bytes(c) : 0);
     }
-    for (auto& blk : b->rec_pool) used += blk.second;
     for (int p : b->order) {
         rt_ctx* c = b->ctx[p];
         if (b->admitted[p] || b->converged[p] || b->iters[p] >= max_iter) continue;
-        // room for the assembled operator of an FP64 problem where the
-        // budget allows it at all, else for the ray-by-ray recording
-        long long need = rec_need(c);
-        if (need > 0 && c->precision != RT_FP32_SWEEP && rec_ask(c, need) <= limit)
-            need = rec_ask(c, need);
-        // a pooled block that holds the recording
-        int pick = -1;
-        for (size_t i = 0; i < b->rec_pool.size(); ++i)
-            if (b->rec_pool[i].second >= need &&
-                (pick < 0 || b->rec_pool[i].second < b->rec_pool[pick].second))
-                pick = (int)i;
-        if (b->rec_mode != 0 && need > 0 && pick >= 0) {
-            c->rec_mem = b->rec_pool[pick].first;
-            c->rec_cap = b->rec_pool[pick].second;
-            b->rec_pool.erase(b->rec_pool.begin() + pick);
-            c->rec_mode = c->rec_cap;
-            bool use = false;
-            const int rc = ensure_rec(c, use);
-            if (rc) return bfail(b, rc, "problem %d: %s", p, rt_last_error(c));
-        } else if (b->rec_mode == 0 || need == 0 || need > limit) {
+        const bool op = c->precision != RT_FP32_SWEEP;
+        const long long need = rec_need(c);
+        if (b->rec_mode == 0 || need == 0 || need > m.limit) {
             c->rec_mode = 0;                      // marches
-        } else if (used + need <= limit && (reserve == 0 || need + reserve <= free_now)) {
-            c->rec_mode = need;
-            bool use = false;
-            const int rc = ensure_rec(c, use);
-            if (rc) return bfail(b, rc, "problem %d: %s", p, rt_last_error(c));
-            if (use) {
-                used += c->rec_cap;
-                free_now -= c->rec_cap;
-            } else if (running) {
-                continue;                         // wait for memory
-            } else {
-                c->rec_mode = 0;
-            }
-        } else if (running) {
-            continue;                             // wait for memory
         } else {
-            c->rec_mode = 0;
+            // room for the assembled operator where the budget allows it at
+            // all, else (or where nothing runs whose memory could be waited for)
+            // for the ray-by-ray recording
+            const long long ask = op && rec_ask(c, need) <= m.limit ? rec_ask(c, need) : need;
+            if (!batch_take(b, c, ask, op, m)) {
+                if (running) continue;            // wait for memory
+                if (ask == need || !batch_take(b, c, need, op, m)) c->rec_mode = 0;
+            }
         }
         b->admitted[p] = 1;
         running = true;
@@ -2062,22 +2134,6 @@ void batch_release(rt_batch* b, int p)
     if (c->ow_mem) {
         cudaStreamSynchronize(b->stream);
         free_op_work(c);
-    }
-}
-
-// Free pooled blocks until at most `keep` bytes are held, the largest first.
-void batch_free_pool(rt_batch* b, long long keep = 0)
-{
-    long long held = 0;
-    for (auto& blk : b->rec_pool) held += blk.second;
-    if (held <= keep) return;
-    cudaStreamSynchronize(b->stream);
-    std::sort(b->rec_pool.begin(), b->rec_pool.end(),
-              [](const auto& x, const auto& y) { return x.second < y.second; });
-    while (!b->rec_pool.empty() && held > keep) {
-        held -= b->rec_pool.back().second;
-        cudaFree(b->rec_pool.back().first);
-        b->rec_pool.pop_back();
     }
 }
 
@@ -2313,6 +2369,10 @@ int batch_fs(rt_batch* b, const std::vector<int>& act)
                                          : fs64_formal(c, G, c->Jfs, b->d_steps, d);
             if ((rc = bpass(b, p, rc))) return rc;
             direct[p] = d;
+            if (!c->rec_valid && c->rec_mode != 0) {    // no memory: marches from here on
+                batch_release(b, p);
+                c->rec_mode = 0;
+            }
             b->stats.fs_launches += 1;
             b->stats.launches += 1;
         }
@@ -3368,7 +3428,10 @@ static int batch_solve(rt_batch* b, double tol, int max_iter, double tol_inner, 
                 c->ng_min_delta = 0.0;
                 c->ng_count = 1;
             }
-            if (b->converged[p] || b->iters[p] >= max_iter) batch_release(b, p);
+            if (b->converged[p] || b->iters[p] >= max_iter) {
+                batch_release(b, p);
+                b->admitted[p] = 0;             // a later solve admits it again
+            }
         }
     }
     batch_free_pool(b, kPoolKeep);

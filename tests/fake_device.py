@@ -24,8 +24,16 @@ from paper_1107_5719_gb300 import rt3d as R, workloads as W
 lib = R.load({lib!r})
 lib.fake_memory.argtypes = [C.c_longlong]
 lib.fake_solves.argtypes = [C.c_int, C.c_double]
-lib.fake_live.restype = lib.fake_peak.restype = C.c_longlong
+lib.fake_large.argtypes = [C.c_longlong]
+lib.fake_live.restype = lib.fake_peak.restype = lib.fake_large.restype = C.c_longlong
 GB = 1 << 30
+up = lambda b: (b + 255) // 256 * 256
+
+def rays(p):
+    # bytes of a ray-by-ray recording of p in FP64 or double-float
+    N, D, nxy = p.nvox, p.ndir, p.nx * p.ny
+    return up(4 * D * nxy * p.nz * (p.nz - 1)) + up(4 * D * p.nz * ((nxy + 31) // 32)) + 2 * up(64 * N)
+
 def counts():
     n = (C.c_int * 8)()
     lib.fake_counts(n)

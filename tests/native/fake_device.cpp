@@ -12,7 +12,7 @@
 
 namespace {
 std::map<void*, size_t> g_mem;
-long long g_total = 284LL << 30, g_live = 0, g_peak = 0;
+long long g_total = 284LL << 30, g_live = 0, g_peak = 0, g_large = 1LL << 60, g_large_live = 0, g_large_peak = 0;
 int g_sweeps = 5, g_solves = 0, g_graphs = 0, g_marches = 0, g_applies = 0, g_lengths = 0, g_ng = 0,
     g_outside = 0, g_replays = 0, g_nth = -1;
 cudaError_t g_last = cudaSuccess;
@@ -28,6 +28,17 @@ void fake_fail(int n) { g_nth = n; }
 int fake_failed(void) { return g_nth < 0; }
 void fake_solves(int sweeps, double delta) { g_sweeps = sweeps; g_delta = delta; }
 void fake_operator(int entries, int rows) { g_entries = entries; g_rows = rows; }
+// the peak of the allocations of at least `bytes` since the last call, which
+// sets that size
+long long fake_large(long long bytes)
+{
+    const long long p = g_large_peak;
+    g_large = bytes;
+    g_large_live = 0;
+    for (auto& m : g_mem) g_large_live += (long long)m.second >= g_large ? m.second : 0;
+    g_large_peak = g_large_live;
+    return p;
+}
 long long fake_live(void) { return g_live; }
 long long fake_peak(int reset)
 {
@@ -56,6 +67,8 @@ cudaError_t cudaMalloc(void** p, size_t n)
     g_mem[m] = n;
     g_live += (long long)n;
     if (g_live > g_peak) g_peak = g_live;
+    if ((long long)n >= g_large) g_large_live += (long long)n;
+    if (g_large_live > g_large_peak) g_large_peak = g_large_live;
     *p = m;
     return cudaSuccess;
 }
@@ -66,6 +79,7 @@ cudaError_t cudaFree(void* p)
     if (it == g_mem.end()) return cudaErrorInvalidValue;
     munmap(p, it->second);
     g_live -= (long long)it->second;
+    if ((long long)it->second >= g_large) g_large_live -= (long long)it->second;
     g_mem.erase(it);
     return cudaSuccess;
 }
@@ -188,6 +202,12 @@ cudaError_t launch_fs64rep(const Geometry&, const double*, const DirInfo*, const
 cudaError_t launch_fsdfrep(const ViewDF&, const Rec32&, int, unsigned long long*, cudaStream_t)
 {
     return ++g_replays, cudaGetLastError();
+}
+cudaError_t launch_fs32rep_batch(const Rep32*, const int*, const long long*, int n, long long, int, int,
+                                 unsigned long long*, cudaStream_t)
+{
+    g_replays += n;
+    return cudaGetLastError();
 }
 cudaError_t launch_fsdf(const ViewDF&, double, int, unsigned long long*, cudaStream_t)
 {

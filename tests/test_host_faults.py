@@ -1,5 +1,5 @@
 """The host code on a device in host memory (fake_device.py): waits that gave up,
-numbers of sweeps up to the largest, allocations that fail."""
+numbers of sweeps up to the largest, allocations that fail, budgets of batches."""
 
 import pytest
 
@@ -100,4 +100,94 @@ while True:
     n += 1
 assert n >= (1 if form == "short" else 3), n
 assert lib.fake_live() == 0
+""")
+
+
+@pytest.mark.parametrize("form", ["fp64", "df64"])
+def test_batch_keeps_its_budget(lib, form):
+    """Problems of two sizes whose operators take more than their ray-by-ray
+    recordings, under budgets from one such recording to several operators, solved
+    three times: what is held never exceeds the budget, and every problem records."""
+    fake_device.run(lib, f"""
+prec = R.RT_DF64 if {form!r} == "df64" else R.RT_FP64
+small = W.random_slab(16, 12, 10, n_theta=4, n_phi=6, seed=1)
+large = W.random_slab(20, 16, 12, n_theta=4, n_phi=6, seed=2)
+probs = [small, large, small, large, small, large]
+sizes = []
+for p in (small, large):
+    with R.Solver(p, precision=prec) as s:
+        s.formal_solution(p.B)
+        sizes.append(R.rt_fs_record_info(s.ctx)[0])
+        assert sizes[-1] > rays(p)
+lib.fake_solves(5, 1e-9)
+need = rays(large)
+budgets = [need, need + 1000, sizes[1], sizes[1] + rays(small), sizes[1] + need, sizes[1] + sizes[0], 2 * sizes[1],
+           2 * sizes[1] + need, 3 * sizes[1] + sizes[0], 20 * sizes[1]]
+for budget in budgets:
+    b = R.rt_batch_create(probs, precision=prec)
+    R.rt_batch_set_fs_record(b, budget)
+    lib.fake_large(int(0.8 * rays(small)))
+    counts()
+    for solve in range(3):
+        lib.fake_solves(5, 1e-9)
+        r = R.rt_batch_solve(b, len(probs))
+        assert r["converged"]
+        n = counts()
+        assert n["marches"] == 0 and n["applies"] + n["replays"] == len(probs), (budget, solve, n)
+        if budget >= sizes[1]:
+            assert n["replays"] == 0, (budget, solve, n)
+        held = lib.fake_large(int(0.8 * rays(small)))
+        assert held <= budget, (budget, solve, held)
+        R.rt_batch_reset(b, rebuild_lstar=True)
+    R.rt_batch_destroy(b)
+assert lib.fake_live() == 0
+""")
+
+
+def test_batch_that_stops_and_goes_on_keeps_its_budget(lib):
+    """Problems that reach max_iter and go on in a later solve are admitted
+    again, within the budget."""
+    fake_device.run(lib, """
+p = W.random_slab(16, 12, 10, n_theta=4, n_phi=6, seed=1)
+with R.Solver(p) as s:
+    s.formal_solution(p.B)
+    one = R.rt_fs_record_info(s.ctx)[0]
+b = R.rt_batch_create([p] * 5, precision=0)
+R.rt_batch_set_fs_record(b, 2 * one)
+lib.fake_large(int(0.8 * rays(p)))
+lib.fake_solves(5, 0.5)
+counts()
+for it in (2, 3, 5):
+    R.rt_batch_solve(b, 5, tol=0.0, max_iter=it)
+n = counts()
+assert n["marches"] == n["replays"] == 0 and n["applies"] == 25, n
+assert lib.fake_large(1 << 60) <= 2 * one
+R.rt_batch_destroy(b)
+""")
+
+
+@pytest.mark.parametrize("form", ["fp64", "df64", "fp32"])
+def test_batch_automatic_budget_leaves_its_reserve(lib, form):
+    """The automatic budget on devices with little room: 4 GiB stay free."""
+    fake_device.run(lib, f"""
+prec = dict(fp64=R.RT_FP64, df64=R.RT_DF64, fp32=R.RT_FP32_SWEEP)[{form!r}]
+p = W.random_slab(16, 12, 10, n_theta=4, n_phi=6, seed=1)
+lib.fake_solves(5, 1e-9)
+recorded = []
+for mb in (3, 8, 16, 32, 64, 128, 256):
+    lib.fake_memory(400 * GB)
+    b = R.rt_batch_create([p] * 6, precision=prec)
+    total = lib.fake_live() + 4 * GB + (mb << 20)
+    lib.fake_memory(total)
+    lib.fake_peak(1)
+    counts()
+    for solve in range(2):
+        assert R.rt_batch_solve(b, 6)["converged"]
+        R.rt_batch_reset(b, rebuild_lstar=True)
+    n = counts()
+    recorded.append(n["applies"] + n["replays"])
+    if recorded[-1]:
+        assert total - lib.fake_peak(0) >= 4 * GB, (mb, recorded[-1])
+    R.rt_batch_destroy(b)
+assert recorded[-1] == 12 and recorded == sorted(recorded)
 """)
