@@ -144,34 +144,63 @@ k_op_lists(Geometry g, const DirInfo* __restrict__ info, const StepGeo* __restri
         const int* u = uofi + 4 * q;
         L.posmax[(long long)dl[q] * nz + m] = max(max(u[0], u[1]), max(u[2], u[3])) + 1;
     }
-    // contributions: counts, their prefix sums, then the entries
-    for (int u = threadIdx.x; u < U; u += kListThreads) {
-        int c = 0;
-        for (int i = 0; i < n; ++i) c += uofi[i] == u;
-        ustart[u + 1] = c;
-    }
     __syncthreads();
+    // contributions: counts, their prefix sums, then the entries in item order (in
+    // time linear in the items; every thread looking through all items for its
+    // nodes took 3.8 ms for 33 planes of 4096 directions, and the first formal
+    // solution after a quadrature in double-float 32.4 ms against 29.4)
+    int* next = first;           // its nodes are looked up
+    for (int u = threadIdx.x; u < U; u += kListThreads) next[u] = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < n; i += kListThreads) atomicAdd(&next[uofi[i]], 1);
+    __syncthreads();
+    base = 0;
+    for (int u0 = 0; u0 < U; u0 += kListThreads) {
+        const int u = u0 + threadIdx.x, v = u < U ? next[u] : 0;
+        int x = v;
+        for (int h = 1; h < 32; h <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, h);
+            if (lane >= h) x += y;
+        }
+        if (lane == 31) wsum[wid] = x;
+        __syncthreads();
+        int pre = base, tot = 0;
+        for (int w = 0; w < kListThreads / 32; ++w) {
+            if (w < wid) pre += wsum[w];
+            tot += wsum[w];
+        }
+        if (u < U) {
+            ustart[u] = next[u] = pre + x - v;
+            if (u == U - 1) ustart[U] = pre + x;
+        }
+        base += tot;
+        __syncthreads();
+    }
     if (threadIdx.x == 0) {
-        ustart[0] = 0;
-        int s = 0;
-        for (int u = 0; u < U; ++u) {
-            s += ustart[u + 1];
-            ustart[u + 1] = s;
-        }
         L.ucount[row] = U;
+        if (U == 0) ustart[0] = 0;
     }
-    __syncthreads();
-    for (int u = threadIdx.x; u < U; u += kListThreads) {
-        int j = ustart[u];
-        const int last = ustart[u + 1] - 1;
-        for (int i = 0; i < n; ++i) {
-            if (uofi[i] != u) continue;
-            const int d = dl[i >> 2], q = i & 3;
-            const Bw4d b = m == 0 ? dn[d].b : bw[(long long)d * nz + m];
-            const double v = q == 0 ? b.x : q == 1 ? b.y : q == 2 ? b.z : b.w;
-            ct[j] = OpContrib{info[d].w * v, d, 2 * u + (j == last)};
-            ++j;
+    // the places, 32 items at a time: an item comes after those of its node in
+    // lower lanes and in earlier rounds
+    if (wid == 0)
+        for (int i0 = 0; i0 < n; i0 += 32) {
+            const int i = i0 + lane, u = i < n ? uofi[i] : -1;
+            const unsigned same = __match_any_sync(0xffffffffu, u);
+            const int j = u < 0 ? 0 : next[u] + __popc(same & ((1u << lane) - 1));
+            __syncwarp();
+            if (u >= 0) {
+                if (lane == __ffs(same) - 1) next[u] += __popc(same);
+                ct[j].d = i;
+                ct[j].ul = 2 * u + (j == ustart[u + 1] - 1);
+            }
+            __syncwarp();
         }
+    __syncthreads();
+    for (int j = threadIdx.x; j < n; j += kListThreads) {
+        const int i = ct[j].d, d = dl[i >> 2], q = i & 3;
+        const Bw4d b = m == 0 ? dn[d].b : bw[(long long)d * nz + m];
+        ct[j].wb = info[d].w * (q == 0 ? b.x : q == 1 ? b.y : q == 2 ? b.z : b.w);
+        ct[j].d = d;
     }
 }
 
