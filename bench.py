@@ -39,8 +39,8 @@ sys.path.insert(0, ROOT)
 # the intensity update (5) and the transmission update (1).
 FLOPS_PER_STEP_FP64 = 49
 # Operator of the recorded FP64 march, per recorded step: the rays' steps meet
-# in 2.24 distinct nodes per step (65^3 slab, 32 x 32 directions), each one FMA
-# and 8 coefficient bytes streamed from memory.
+# in 2.24 distinct nodes per step (65^3 slab, 32 x 32 directions; counted for that
+# workload alone), each one FMA and 8 coefficient bytes streamed from memory.
 OP_ENTRIES_PER_STEP = 2.24
 FLOPS_PER_STEP_FP64_REPLAY = 2 * OP_ENTRIES_PER_STEP
 # Recording march (k_rec64), FP64 flops executed per step (ncu: 10.0 FMA, 5.4
@@ -467,6 +467,25 @@ def run_only(args, dev, R):
     print(json.dumps({"only": name, name: out}), flush=True)
 
 
+def op_roofline(workload, rec):
+    """Roofline of the operator's application: rates only for the workload whose
+    entries per step were counted."""
+    ms, steps = rec["replay_ms"], rec["replay_steps"]
+    counted = workload == "slab65"
+    tfl = FLOPS_PER_STEP_FP64_REPLAY * steps / (ms / 1e3) / 1e12 if counted else None
+    return {"kernel": "k_op_apply64 (operator of the recorded FP64 march)", "bound": "alu",
+            "achieved": round(tfl, 4) if counted else None, "peak": PEAK_FP64_TFLOPS, "unit": "TFLOP/s",
+            "frac": round(tfl / PEAK_FP64_TFLOPS, 4) if counted else None,
+            "traffic": TRAFFIC_OP_SLAB65 if counted else None,
+            "flops_per_step": FLOPS_PER_STEP_FP64_REPLAY if counted else None,
+            "fp64_instructions_per_step": OP_ENTRIES_PER_STEP if counted else None,
+            "coefficient_bytes_per_step": 8 * OP_ENTRIES_PER_STEP if counted else None,
+            "hbm_gbs_coefficients": round(8 * OP_ENTRIES_PER_STEP * steps / (ms / 1e3) / 1e9, 1)
+            if counted else None,
+            "steps_per_launch": round(steps),
+            "ms_per_launch": round(ms, 4)}
+
+
 def fp32_replay_roofline(r32):
     """The replay of the recorded FP32 march: per voxel-step the
     interpolated source difference (4 differences, 4 + 4 products and sums:
@@ -561,20 +580,8 @@ def run_ours(args):
     rec = record_rate(R, p, dev, stream)
     iters = st["iterations"] / args.steps
     if rec["recorded"]:
-        rep_ms, rep_steps = rec["replay_ms"], rec["replay_steps"]
-        achieved = FLOPS_PER_STEP_FP64_REPLAY * rep_steps / (rep_ms / 1e3) / 1e12
-        roofline = {"kernel": "k_op_apply64 (operator of the recorded FP64 march)", "bound": "alu",
-                    "achieved": round(achieved, 4), "peak": PEAK_FP64_TFLOPS, "unit": "TFLOP/s",
-                    "frac": round(achieved / PEAK_FP64_TFLOPS, 4),
-                    "traffic": TRAFFIC_OP_SLAB65 if args.workload == "slab65" else None,
-                    "flops_per_step": FLOPS_PER_STEP_FP64_REPLAY,
-                    "fp64_instructions_per_step": OP_ENTRIES_PER_STEP,
-                    "coefficient_bytes_per_step": 8 * OP_ENTRIES_PER_STEP,
-                    "hbm_gbs_coefficients": round(8 * OP_ENTRIES_PER_STEP * rep_steps
-                                                  / (rep_ms / 1e3) / 1e9, 1),
-                    "steps_per_launch": round(rep_steps),
-                    "ms_per_launch": round(rep_ms, 4),
-                    "share_of_step": round(rep_ms * iters / (my_ms / args.steps), 4),
+        roofline = {**op_roofline(args.workload, rec),
+                    "share_of_step": round(rec["replay_ms"] * iters / (my_ms / args.steps), 4),
                     "record": {"kernel": "k_op_len, k_rec64, k_op_assemble (recording)",
                                "ms": round(rec["record_ms"], 3),
                                "steps": round(rec["record_steps"]),
@@ -596,8 +603,8 @@ def run_ours(args):
     roofline.update({
         "peak_source": "unit counts and clock: 152 SMs x 2 DFMA/clk x 2 flops x 2.07 GHz",
         "peak_measured": round(probe["fp64_tflops"], 4) if probe["fp64_tflops"] else None,
-        "frac_of_measured": round(achieved / probe["fp64_tflops"], 4)
-        if probe["fp64_tflops"] else None,
+        "frac_of_measured": round(roofline["achieved"] / probe["fp64_tflops"], 4)
+        if probe["fp64_tflops"] and roofline["achieved"] else None,
         "peak_measured_source": "rt_probe_peaks: register-resident DFMA chains on every "
                                 "SM, CUDA events"})
 
