@@ -222,7 +222,10 @@ int rt_last_step_count(rt_ctx *ctx, unsigned long long *steps);
  * 224 N + 4 ndir nz (ceil(nx ny/32) + 3) + 16 nz^2 bytes of working storage
  * from the first recording on and, with as many directions up as down, 84 ndir
  * nz + 16 nz min(nx ny, 2 ndir) bytes of node lists per quadrature; without the
- * lists the coefficients are kept ray by ray).  J agrees with the march to rounding (the
+ * lists the coefficients are kept ray by ray).  A recording pays from the second
+ * or third formal solution on the same opacities; a program that makes one per
+ * opacity does best with 0 (65^3 x 512 directions, double-float: 21 ms in place
+ * of 37).  J agrees with the march to rounding (the
  * terms are summed in another order).  Short characteristics record the
  * weights of every (voxel, direction) under the same setting, 24 ndir N bytes
  * in FP64 and 16 ndir N + 16 N in double-float.  RT_EINVAL for max_bytes <
@@ -300,7 +303,8 @@ int rt_set_precision(rt_ctx *ctx, int precision);
  * rt_solve waits for the GPU once (for delta and the sweep count) instead
  * of once per chunk of sweeps.  Grids of up to 2048 voxels per SM
  * (Gauss-Seidel 600) run the step as one cooperative kernel in place of the
- * graph; a wait of its blocks that gives up (about a second) returns
+ * graph, unless max_sweeps allows more than 4 Mi barriers (one a sweep,
+ * Gauss-Seidel two); a wait of its blocks that gives up (about a second) returns
  * RT_ETIMEOUT.  Results are identical either way (same arithmetic, same sweep
  * count).  on = 0 selects the host-driven loop. */
 int rt_set_graphs(rt_ctx *ctx, int on);
@@ -535,7 +539,7 @@ int rt_batch_set_fs_record(rt_batch *batch, long long max_bytes);
  * so the host launches once and waits once per iteration (Ng runs on the
  * device too); the graph is rebuilt when the set of active problems
  * changes.  While the active problems together have up to 2048 voxels per SM
- * (Gauss-Seidel 600) one cooperative kernel takes its place.  on == 0: the sweeps are enqueued from the host in growing chunks
+ * (Gauss-Seidel 600) and 4 Mi barriers one cooperative kernel takes its place.  on == 0: the sweeps are enqueued from the host in growing chunks
  * with one wait per chunk.  Results are identical. */
 int rt_batch_set_graphs(rt_batch *batch, int on);
 /* As rt_set_ng, for every problem of the batch. */

@@ -147,7 +147,7 @@ k_op_lists(Geometry g, const DirInfo* __restrict__ info, const StepGeo* __restri
     __syncthreads();
     // contributions: counts, their prefix sums, then the entries in item order (in
     // time linear in the items; every thread looking through all items for its
-    // nodes took 3.8 ms for 33 planes of 4096 directions, and the first formal
+    // nodes took 3.4 ms for 33 planes of 4096 directions, and the first formal
     // solution after a quadrature in double-float 32.4 ms against 29.4)
     int* next = first;           // its nodes are looked up
     for (int u = threadIdx.x; u < U; u += kListThreads) next[u] = 0;
