@@ -2022,7 +2022,7 @@ bool batch_take(rt_batch* b, rt_ctx* c, long long want, bool op, RecBudget& m)
     auto room = [&](long long have, long long freed) {
         const long long grow = std::max(want - have, 0LL);
         return m.used + grow <= m.limit + freed &&
-               (!m.automatic || grow + work + m.reserve <= m.free_now + freed);
+               (!m.automatic || grow + work == 0 || grow + work + m.reserve <= m.free_now + freed);
     };
     if (!room(cap, 0)) {
         if (!room(cap, pooled - cap)) {

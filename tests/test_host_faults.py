@@ -191,3 +191,21 @@ for mb in (3, 8, 16, 32, 64, 128, 256):
     R.rt_batch_destroy(b)
 assert recorded[-1] == 12 and recorded == sorted(recorded)
 """)
+
+
+def test_batch_uses_its_own_block_on_a_full_device(lib):
+    """A pooled block that holds the recording takes no memory: it is used also where
+    less than the reserve is free."""
+    fake_device.run(lib, """
+p = W.random_slab(16, 12, 10, n_theta=4, n_phi=6, seed=1)
+lib.fake_solves(5, 1e-9)
+lib.fake_memory(400 * GB)
+b = R.rt_batch_create([p] * 3, precision=R.RT_FP32_SWEEP)
+R.rt_batch_solve(b, 3)
+assert counts()["replays"] == 3
+R.rt_batch_reset(b, rebuild_lstar=True)
+lib.fake_memory(lib.fake_live() + 3 * GB)
+R.rt_batch_solve(b, 3)
+assert counts()["replays"] == 3
+R.rt_batch_destroy(b)
+""")
