@@ -201,7 +201,8 @@ int rt_last_step_count(rt_ctx *ctx, unsigned long long *steps);
  * that the directions give the same node of the same voxel are added up
  * once, and a formal solution is one multiply-add per (voxel, node) (Lambda*
  * is read off them); where that takes more memory than the coefficients
- * themselves and half as much again (at least 4, at most 24 GiB more), they
+ * themselves and half as much again (at least 4, at most 24 GiB more; another
+ * eighth, at least 2 GiB, while it is made), they
  * are kept ray by ray and S is interpolated at every step.  The parabolic
  * source also keeps the coefficient of S at the downstream point per
  * (voxel, direction).  The FP32 sweep records FP32 coefficients of

@@ -23,6 +23,7 @@ sys.path.insert(0, {root!r})
 from paper_1107_5719_gb300 import rt3d as R, workloads as W
 lib = R.load({lib!r})
 lib.fake_memory.argtypes = [C.c_longlong]
+lib.fake_operator.argtypes = [C.c_int, C.c_int, C.c_ulonglong]
 lib.fake_solves.argtypes = [C.c_int, C.c_double]
 lib.fake_large.argtypes = [C.c_longlong]
 lib.fake_live.restype = lib.fake_peak.restype = lib.fake_large.restype = C.c_longlong
@@ -35,9 +36,9 @@ def rays(p):
     return up(4 * D * nxy * p.nz * (p.nz - 1)) + up(4 * D * p.nz * ((nxy + 31) // 32)) + 2 * up(64 * N)
 
 def counts():
-    n = (C.c_int * 8)()
+    n = (C.c_int * 9)()
     lib.fake_counts(n)
-    return dict(zip(("solves", "graphs", "marches", "applies", "lengths", "ng", "outside", "replays"), n))
+    return dict(zip(("solves", "graphs", "marches", "applies", "lengths", "ng", "outside", "replays", "chunks"), n))
 """
 
 

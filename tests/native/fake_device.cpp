@@ -14,7 +14,8 @@ namespace {
 std::map<void*, size_t> g_mem;
 long long g_total = 284LL << 30, g_live = 0, g_peak = 0, g_large = 1LL << 60, g_large_live = 0, g_large_peak = 0;
 int g_sweeps = 5, g_solves = 0, g_graphs = 0, g_marches = 0, g_applies = 0, g_lengths = 0, g_ng = 0,
-    g_outside = 0, g_replays = 0, g_nth = -1;
+    g_outside = 0, g_replays = 0, g_chunks = 0, g_nth = -1;
+unsigned long long g_steps = 1ull << 40;
 cudaError_t g_last = cudaSuccess;
 double g_delta = 0.5;
 int g_entries = 64, g_rows = 64;        // of every plane of an operator
@@ -27,7 +28,12 @@ void fake_memory(long long total) { g_total = total; }
 void fake_fail(int n) { g_nth = n; }
 int fake_failed(void) { return g_nth < 0; }
 void fake_solves(int sweeps, double delta) { g_sweeps = sweeps; g_delta = delta; }
-void fake_operator(int entries, int rows) { g_entries = entries; g_rows = rows; }
+void fake_operator(int entries, int rows, unsigned long long steps)
+{
+    g_entries = entries;
+    g_rows = rows;
+    g_steps = steps;
+}
 // the peak of the allocations of at least `bytes` since the last call, which
 // sets that size
 long long fake_large(long long bytes)
@@ -47,13 +53,13 @@ long long fake_peak(int reset)
     return p;
 }
 // {one-kernel solves, graph launches, marches, applied operators, length marches,
-// extrapolations, barrier words outside their allocation, ray-by-ray replays} since the
-// last call
+// extrapolations, barrier words outside their allocation, ray-by-ray replays,
+// recording marches (one a chunk of planes)} since the last call
 void fake_counts(int* n)
 {
-    const int c[8] = {g_solves, g_graphs, g_marches, g_applies, g_lengths, g_ng, g_outside, g_replays};
+    const int c[9] = {g_solves, g_graphs, g_marches, g_applies, g_lengths, g_ng, g_outside, g_replays, g_chunks};
     std::memcpy(n, c, sizeof c);
-    g_solves = g_graphs = g_marches = g_applies = g_lengths = g_ng = g_outside = g_replays = 0;
+    g_solves = g_graphs = g_marches = g_applies = g_lengths = g_ng = g_outside = g_replays = g_chunks = 0;
 }
 
 cudaError_t cudaMalloc(void** p, size_t n)
@@ -174,8 +180,9 @@ cudaError_t launch_op_counts(const Geometry& g, const OpLists&, bool, const int*
 }
 cudaError_t launch_op_lengths(const Geometry&, const double*, const double*, const double*, const DirInfo*,
                               const int*, const float4*, double, int, bool, int, float2*, int*, int, int*,
-                              unsigned long long*, cudaStream_t)
+                              unsigned long long* steps, cudaStream_t)
 {
+    *steps = g_steps;
     return ++g_lengths, cudaGetLastError();
 }
 cudaError_t launch_op_apply64(const Geometry&, const double*, const double*, const OpMap&, double*,
@@ -193,6 +200,17 @@ cudaError_t launch_fs64(const Geometry&, const double*, const double*, const dou
                         double*, unsigned long long*, cudaStream_t)
 {
     return ++g_marches, cudaGetLastError();
+}
+cudaError_t launch_rec64(const Geometry&, int, int, const double*, const double*, const double*, const DirInfo*,
+                         const StepGeo*, const Bw4d*, const Bw4d*, const RecOut&, const int*, int, int, double*,
+                         double*, cudaStream_t)
+{
+    return ++g_chunks, cudaGetLastError();
+}
+cudaError_t launch_recdf(const ViewDF&, int, int, const RecOut&, const int*, int, int, double*, double*, double*,
+                         cudaStream_t)
+{
+    return ++g_chunks, cudaGetLastError();
 }
 cudaError_t launch_fs64rep(const Geometry&, const double*, const DirInfo*, const StepGeo*, const Bw4d*, const FsRec&,
                            int, double*, unsigned long long*, cudaStream_t)

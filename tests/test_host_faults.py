@@ -1,5 +1,6 @@
 """The host code on a device in host memory (fake_device.py): waits that gave up,
-numbers of sweeps up to the largest, allocations that fail, budgets of batches."""
+numbers of sweeps up to the largest, allocations that fail, budgets of batches,
+chunks of a recording."""
 
 import pytest
 
@@ -208,4 +209,25 @@ lib.fake_memory(lib.fake_live() + 3 * GB)
 R.rt_batch_solve(b, 3)
 assert counts()["replays"] == 3
 R.rt_batch_destroy(b)
+""")
+
+
+@pytest.mark.parametrize("form", ["fp64", "df64"])
+def test_operator_near_its_budget_is_recorded_in_large_chunks(lib, form):
+    """33^3 with 256 directions, ray by ray 1.1 GiB, so an operator of up to 5.1 GiB: one
+    of 4.6 records its 1 GiB of coefficients at once, not a few planes at a time;
+    where max_bytes leaves less beside it, in chunks; above the budget ray by ray."""
+    fake_device.run(lib, f"""
+prec = R.RT_DF64 if {form!r} == "df64" else R.RT_FP64
+p = W.slab_65(n=33, n_theta=16, n_phi=16)
+own = lambda entries: entries * 33 * 35 * 32 * 8
+for entries, record, chunks, applies in ((16704, -1, 1, 1), (16704, own(16704) + GB // 2, 14, 1),
+                                         (18720, -1, 1, 0)):
+    lib.fake_operator(entries, 3735, 1 << 40)
+    with R.Solver(p, precision=prec, record=record) as s:
+        counts()
+        s.formal_solution(p.B)
+        n = counts()
+    assert n["applies"] == applies and n["replays"] == 1 - applies, (entries, record, n)
+    assert n["chunks"] == 1 if chunks == 1 else n["chunks"] >= 12, (entries, record, n)
 """)
