@@ -202,7 +202,8 @@ int rt_last_step_count(rt_ctx *ctx, unsigned long long *steps);
  * once, and a formal solution is one multiply-add per (voxel, node) (Lambda*
  * is read off them); where that takes more memory than the coefficients
  * themselves and half as much again (at least 4, at most 24 GiB more; another
- * eighth, at least 2 GiB, while it is made), they
+ * eighth, at least 2 GiB, while it is made), or where a medium opaque but for a few
+ * columns gives it more terms than the rays have steps worth (7 to 8.5 each), they
  * are kept ray by ray and S is interpolated at every step.  The parabolic
  * source also keeps the coefficient of S at the downstream point per
  * (voxel, direction).  The FP32 sweep records FP32 coefficients of

@@ -484,6 +484,19 @@ long long op_budget(const rt_ctx* c, long long need)
 // 55.0 in FP64, 15.5 and 44.9 with it.
 long long op_chunk(long long need) { return std::max(need / 8, 2LL << 30); }
 
+// Entries per recorded step up to which the operator is the faster form.  The
+// entries of a plane are those of its longest rays, for all its voxels: where a
+// medium is opaque but for a few columns they outnumber the steps, and the
+// ray-by-ray replay does less.  45^3 x 256, operator over rays, formal solution and
+// solve: slab with noise (2.8 entries per step) 0.53 and 0.67 in FP64, 0.59 and 0.71 in
+// double-float; opaque with a column of 8% of the sides clear (6.9 and 7.2) 1.10
+// and 1.01, 0.95 and 0.98; 10% (8.0 and 8.3) 1.25 and 1.11, 1.06 and 1.07; 25% (9.0 and
+// 9.2) 1.41 and 1.53, 1.34 and 1.50; parabolic 7.1: 0.85 and 0.91, 8.8: 1.05 and 1.00.
+double op_worth(const rt_ctx* c)
+{
+    return c->src_order == RT_SRC_PARABOLIC ? 8.5 : c->precision == RT_DF64 ? 7.5 : 7.0;
+}
+
 // The most memory a recording of this context asks for.
 long long rec_ask(const rt_ctx* c, long long need)
 {
@@ -612,7 +625,8 @@ constexpr long long kOpNoWait = 64LL << 20;
 
 // Record the march of the current source (FP64, linear or parabolic, or
 // double-float) and assemble its operator, or keep it ray by ray where the
-// operator would take more memory (op_budget) or its lists get no memory.  use: whether a recording is held afterwards (not where the block or
+// operator would take more memory (op_budget) or time (op_worth) or its lists get
+// no memory.  use: whether a recording is held afterwards (not where the block or
 // the working storage gets no memory: the march runs).
 int ensure_op_rec(rt_ctx* c, int G, bool& use)
 {
@@ -664,6 +678,8 @@ int ensure_op_rec(rt_ctx* c, int G, bool& use)
         if (op_bytes(c, entries) + chunk > std::min(room, kOpNoWait)) {
             // the size it really has, and chunks of planes
             std::vector<int> E(g.nz), R(g.nz);
+            unsigned long long steps = 0;
+            CK(cudaMemcpyAsync(&steps, w.steps, sizeof steps, cudaMemcpyDeviceToHost, st));
             CK(cudaMemcpyAsync(E.data(), w.E, sizeof(int) * g.nz, cudaMemcpyDeviceToHost, st));
             CK(cudaMemcpyAsync(R.data(), w.rows, sizeof(int) * g.nz, cudaMemcpyDeviceToHost, st));
             if (g.zorder)
@@ -683,7 +699,8 @@ int ensure_op_rec(rt_ctx* c, int G, bool& use)
             // a chunk as large as it should be, or the whole
             long long cb = std::min(rows, std::max(most, op_chunk(need) / row)) * row;
             if (own + up256(cb) > room) cb = std::max(most, rows / 12) * row;
-            if (own + up256(cb) > room || own > op_budget(c, need)) {
+            if (own + up256(cb) > room || own > op_budget(c, need) ||
+                (double)entries * (double)(nwp * 32) > op_worth(c) * (double)steps) {
                 op = false;
             } else {
                 first.assign(1, 0);

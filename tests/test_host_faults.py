@@ -231,3 +231,23 @@ for entries, record, chunks, applies in ((16704, -1, 1, 1), (16704, own(16704) +
     assert n["applies"] == applies and n["replays"] == 1 - applies, (entries, record, n)
     assert n["chunks"] == 1 if chunks == 1 else n["chunks"] >= 12, (entries, record, n)
 """)
+
+
+def test_operator_is_kept_while_its_entries_are_worth_it(lib):
+    """On both sides of the entries per step up to which the operator is the faster
+    form: 7 in FP64, 7.5 in double-float, 8.5 for the parabolic source."""
+    fake_device.run(lib, """
+entries = 3200
+lanes = entries * 33 * 35 * 32
+for form, worth in (("fp64", 7.0), ("df64", 7.5), ("parabolic", 8.5)):
+    p = W.slab_65(n=33, n_theta=16, n_phi=16)
+    p.src_order = int(form == "parabolic")
+    for ratio in (worth - 0.01, worth + 0.01, 1e6):
+        lib.fake_operator(entries, 100, int(lanes / ratio))
+        with R.Solver(p, precision=R.RT_DF64 if form == "df64" else R.RT_FP64) as s:
+            counts()
+            s.formal_solution(p.B)
+            n = counts()
+        kept = ratio < worth
+        assert (n["applies"], n["replays"]) == ((1, 0) if kept else (0, 1)), (form, ratio, n)
+""")
