@@ -2805,7 +2805,7 @@ static int set_chi(rt_ctx* c, const double* chi, bool device)
     // before any march that reads it)
     CK(launch_plane_order(c->g, c->dz, c->chi, c->zscratch, c->zorder, c->stream));
     c->g.zorder = c->zorder;
-    c->stats.launches += 2;
+    c->stats.launches += c->g.nz <= kRankOne ? 2 : 3;
     c->have_chi = true;
     c->lstar_valid = c->coef_valid = c->gdiff_valid = c->rec_valid = false;
     return RT_OK;

@@ -273,45 +273,62 @@ __global__ void k_plane_mean(Geometry g, const double* __restrict__ chi, double*
     if (threadIdx.x == 0) mean[blockIdx.x] = red[0] / nxy;
 }
 
-// Estimated march work of every plane (w[k]) and the planes by decreasing
-// work (order[rank] = plane).  One block; eight lanes to a plane, six of them
-// one walk each (36 planes: 9.8 us, 23.3 with one thread to a plane).
-constexpr int kRankThreads = 1024;
-__global__ void __launch_bounds__(kRankThreads)
-k_plane_rank(int nz, double dz, const double* __restrict__ mean, double* w, int* __restrict__ order)
+// Estimated march work of the planes (w[k]), eight lanes to a plane, six of them
+// one walk each, and a plane's rank by decreasing work (order[rank] = plane).
+__device__ __forceinline__ void plane_work(int k0, int lane, int nz, double dz,
+                                           const double* __restrict__ mean, double* w)
 {
     constexpr double kTauEnd = 40.0;
-    const int lane = threadIdx.x & 7, first = threadIdx.x >> 3, step = kRankThreads / 8;
-    const int rounds = (nz + step - 1) / step;
-    for (int r = 0; r < rounds; ++r) {
-        const int k0 = first + r * step;
-        int n = 0;
-        if (k0 < nz && lane < 6) {
-            const double amu = lane < 2 ? 1.0 : lane < 4 ? 0.5 : 0.2;
-            const double hs = dz / (2.0 * amu);
-            const int s = lane & 1 ? 1 : -1;
-            double tau = 0.0, here = mean[k0];
-            n = 1;       // per-characteristic overhead, about one step
-            for (int k = k0; k - s >= 0 && k - s < nz && tau <= kTauEnd; k -= s, ++n) {
-                const double next = mean[k - s];
-                tau += hs * (here + next);
-                here = next;
-            }
+    int n = 0;
+    if (k0 < nz && lane < 6) {
+        const double amu = lane < 2 ? 1.0 : lane < 4 ? 0.5 : 0.2;
+        const double hs = dz / (2.0 * amu);
+        const int s = lane & 1 ? 1 : -1;
+        double tau = 0.0, here = mean[k0];
+        n = 1;       // per-characteristic overhead, about one step
+        for (int k = k0; k - s >= 0 && k - s < nz && tau <= kTauEnd; k -= s, ++n) {
+            const double next = mean[k - s];
+            tau += hs * (here + next);
+            here = next;
         }
-        for (int h = 4; h > 0; h >>= 1) n += __shfl_xor_sync(0xffffffffu, n, h);
-        if (k0 < nz && lane == 0) w[k0] = n;
     }
+    for (int h = 4; h > 0; h >>= 1) n += __shfl_xor_sync(0xffffffffu, n, h);
+    if (k0 < nz && lane == 0) w[k0] = n;
+}
+
+__device__ __forceinline__ void plane_rank(int k0, int lane, int nz, const double* w, int* __restrict__ order)
+{
+    int rank = 0;
+    if (k0 < nz) {
+        const double mine = w[k0];
+        for (int j = lane; j < nz; j += 8) rank += (w[j] > mine) || (w[j] == mine && j < k0);
+    }
+    for (int h = 4; h > 0; h >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, h);
+    if (k0 < nz && lane == 0) order[rank] = k0;
+}
+
+// Up to 64 planes: both in one block (36 planes: 9.8 us, 23.3 with one thread to a
+// plane).  Above, where one SM's FP64 pipe would do all the walks, a kernel each of
+// blocks of 32 planes: setting the opacity of 128 planes of 5 x 5 takes 42 us (65 with
+// one block, 74 with a block of one thread to a plane), of 1000 0.16 ms (1.84, 1.21),
+// of 20000 4.4 ms (449, 323).
+constexpr int kRankThreads = 8 * kRankOne, kRankTall = 256;
+__global__ void __launch_bounds__(kRankThreads)
+k_plane_order(int nz, double dz, const double* __restrict__ mean, double* w, int* __restrict__ order)
+{
+    plane_work(threadIdx.x >> 3, threadIdx.x & 7, nz, dz, mean, w);
     __syncthreads();
-    for (int r = 0; r < rounds; ++r) {
-        const int k0 = first + r * step;
-        int rank = 0;
-        if (k0 < nz) {
-            const double mine = w[k0];
-            for (int j = lane; j < nz; j += 8) rank += (w[j] > mine) || (w[j] == mine && j < k0);
-        }
-        for (int h = 4; h > 0; h >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, h);
-        if (k0 < nz && lane == 0) order[rank] = k0;
-    }
+    plane_rank(threadIdx.x >> 3, threadIdx.x & 7, nz, w, order);
+}
+__global__ void __launch_bounds__(kRankTall)
+k_plane_work(int nz, double dz, const double* __restrict__ mean, double* w)
+{
+    plane_work((blockIdx.x * kRankTall + threadIdx.x) >> 3, threadIdx.x & 7, nz, dz, mean, w);
+}
+__global__ void __launch_bounds__(kRankTall)
+k_plane_rank(int nz, const double* __restrict__ w, int* __restrict__ order)
+{
+    plane_rank((blockIdx.x * kRankTall + threadIdx.x) >> 3, threadIdx.x & 7, nz, w, order);
 }
 
 __global__ void k_sum_groups(long long N, const double* __restrict__ partial,
@@ -443,7 +460,14 @@ cudaError_t launch_plane_order(const Geometry& g, double dz, const double* chi, 
                                int* order, cudaStream_t st)
 {
     k_plane_mean<<<g.nz, 256, 0, st>>>(g, chi, scratch);
-    k_plane_rank<<<1, kRankThreads, 0, st>>>(g.nz, dz, scratch, scratch + g.nz, order);
+    double* w = scratch + g.nz;
+    if (g.nz <= kRankOne) {
+        k_plane_order<<<1, kRankThreads, 0, st>>>(g.nz, dz, scratch, w, order);
+    } else {
+        const int blocks = (8 * g.nz + kRankTall - 1) / kRankTall;
+        k_plane_work<<<blocks, kRankTall, 0, st>>>(g.nz, dz, scratch, w);
+        k_plane_rank<<<blocks, kRankTall, 0, st>>>(g.nz, w, order);
+    }
     return cudaGetLastError();
 }
 

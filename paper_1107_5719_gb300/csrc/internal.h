@@ -117,6 +117,7 @@ cudaError_t launch_dir_tables(const Geometry& g, double dx, double dy, double dz
 // index).  scratch: 2 nz doubles.  Light planes dispatched last fill the end
 // of the launch, where otherwise a partial wave of heavy blocks would run
 // alone.
+constexpr int kRankOne = 64;    // planes up to which it takes two kernels, above three
 cudaError_t launch_plane_order(const Geometry& g, double dz, const double* chi, double* scratch,
                                int* order, cudaStream_t st);
 
