@@ -242,13 +242,12 @@ k_sc_rec(ScView p, typename A::C* __restrict__ coef)
     }
 }
 
-template <typename A, bool SMEM>
-__global__ void __launch_bounds__(A::kThreads)
+template <typename A, bool SMEM, int kScrThreads>
+__global__ void __launch_bounds__(kScrThreads)
 k_sc_apply(ScView p, const typename A::C* __restrict__ coef, int d0, typename A::V* __restrict__ part,
            typename A::V* gplanes, unsigned long long* __restrict__ steps)
 {
     using V = typename A::V;
-    constexpr int kScrThreads = A::kThreads;
     extern __shared__ double2 splanes_raw[];
     const Geometry& g = p.g;
     const int nx = g.nx, ny = g.ny, nz = g.nz, nxy = nx * ny;
@@ -412,17 +411,20 @@ cudaError_t sc_record(const ScView& p, void* coef, cudaStream_t st)
     return cudaGetLastError();
 }
 
-template <typename A>
+// T threads: not more warps than a plane has work for, so that more directions share
+// an SM (formal solution of 9 x 9 x 129 with 4096 directions 2.36 ms with 640 threads, 1.36
+// with 128 in double-float, 2.35 and 1.70 in FP64; the march without a recording takes
+// 2.17 and 4.2).  A constant: with the number from blockDim 65^3 x 1024 took 7% longer.
+template <typename A, bool SMEM, int T>
 cudaError_t sc_apply(const ScView& p, const void* coef, double wsum, void* part, void* gplanes, double* J,
                      unsigned long long* steps, cudaStream_t st)
 {
     const Geometry& g = p.g;
     const int chunk = sc_chunk(g);
-    const size_t shm = 16 * (size_t)g.nx * g.ny;
-    const bool smem = sc_scratch_planes(g) == 0;
-    if (smem) {
+    const size_t shm = SMEM ? 16 * (size_t)g.nx * g.ny : 0;
+    if (shm > 40 * 1024) {
         // one value for all grids: contexts of several threads set it
-        cudaError_t e = cudaFuncSetAttribute(k_sc_apply<A, true>,
+        cudaError_t e = cudaFuncSetAttribute(k_sc_apply<A, SMEM, T>,
                                              cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         if (e != cudaSuccess) return e;
     }
@@ -433,13 +435,21 @@ cudaError_t sc_apply(const ScView& p, const void* coef, double wsum, void* part,
     auto* gp = static_cast<typename A::V*>(gplanes);
     for (int d0 = 0; d0 < g.ndir; d0 += chunk) {
         const int nd = g.ndir - d0 < chunk ? g.ndir - d0 : chunk;
-        if (smem)
-            k_sc_apply<A, true><<<nd, A::kThreads, shm, st>>>(p, c, d0, pt, gp, steps);
-        else
-            k_sc_apply<A, false><<<nd, A::kThreads, 0, st>>>(p, c, d0, pt, gp, steps);
+        k_sc_apply<A, SMEM, T><<<nd, T, shm, st>>>(p, c, d0, pt, gp, steps);
         k_sc_sum<A><<<(unsigned)rb, 256, sizeof(typename A::V) * nd, st>>>(p, d0, nd, pt, wsum, J, d0 > 0);
     }
     return cudaGetLastError();
+}
+
+template <typename A>
+cudaError_t sc_apply_any(const ScView& p, const void* coef, double wsum, void* part, void* gplanes, double* J,
+                         unsigned long long* steps, cudaStream_t st)
+{
+    const int nxy = p.g.nx * p.g.ny;
+    if (sc_scratch_planes(p.g)) return sc_apply<A, false, A::kThreads>(p, coef, wsum, part, gplanes, J, steps, st);
+    if (nxy <= 128) return sc_apply<A, true, 128>(p, coef, wsum, part, gplanes, J, steps, st);
+    if (nxy <= 256) return sc_apply<A, true, 256>(p, coef, wsum, part, gplanes, J, steps, st);
+    return sc_apply<A, true, A::kThreads>(p, coef, wsum, part, gplanes, J, steps, st);
 }
 
 }  // namespace
@@ -460,8 +470,8 @@ cudaError_t launch_sc_record(const ScView& p, bool df, void* coef, cudaStream_t 
 cudaError_t launch_sc_apply(const ScView& p, bool df, const void* coef, double wsum, void* part,
                             void* gplanes, double* J, unsigned long long* steps, cudaStream_t st)
 {
-    return df ? sc_apply<ScDF>(p, coef, wsum, part, gplanes, J, steps, st)
-              : sc_apply<Sc64>(p, coef, wsum, part, gplanes, J, steps, st);
+    return df ? sc_apply_any<ScDF>(p, coef, wsum, part, gplanes, J, steps, st)
+              : sc_apply_any<Sc64>(p, coef, wsum, part, gplanes, J, steps, st);
 }
 
 cudaError_t launch_sc_lstar(const ScView& p, bool df, const void* coef, double* lstar, cudaStream_t st)
