@@ -36,9 +36,9 @@ def rays(p):
     return up(4 * D * nxy * p.nz * (p.nz - 1)) + up(4 * D * p.nz * ((nxy + 31) // 32)) + 2 * up(64 * N)
 
 def counts():
-    n = (C.c_int * 9)()
+    n = (C.c_int * 10)()
     lib.fake_counts(n)
-    return dict(zip(("solves", "graphs", "marches", "applies", "lengths", "ng", "outside", "replays", "chunks"), n))
+    return dict(zip(("solves", "graphs", "marches", "applies", "lengths", "ng", "outside", "replays", "chunks", "mallocs"), n))
 """
 
 

@@ -14,7 +14,7 @@ namespace {
 std::map<void*, size_t> g_mem;
 long long g_total = 284LL << 30, g_live = 0, g_peak = 0, g_large = 1LL << 60, g_large_live = 0, g_large_peak = 0;
 int g_sweeps = 5, g_solves = 0, g_graphs = 0, g_marches = 0, g_applies = 0, g_lengths = 0, g_ng = 0,
-    g_outside = 0, g_replays = 0, g_chunks = 0, g_nth = -1;
+    g_outside = 0, g_replays = 0, g_chunks = 0, g_mallocs = 0, g_nth = -1;
 unsigned long long g_steps = 1ull << 40;
 cudaError_t g_last = cudaSuccess;
 double g_delta = 0.5;
@@ -54,17 +54,19 @@ long long fake_peak(int reset)
 }
 // {one-kernel solves, graph launches, marches, applied operators, length marches,
 // extrapolations, barrier words outside their allocation, ray-by-ray replays,
-// recording marches (one a chunk of planes)} since the last call
+// recording marches (one a chunk of planes), device allocations} since the last call
 void fake_counts(int* n)
 {
-    const int c[9] = {g_solves, g_graphs, g_marches, g_applies, g_lengths, g_ng, g_outside, g_replays, g_chunks};
+    const int c[10] = {g_solves, g_graphs, g_marches, g_applies, g_lengths,
+                       g_ng, g_outside, g_replays, g_chunks, g_mallocs};
     std::memcpy(n, c, sizeof c);
-    g_solves = g_graphs = g_marches = g_applies = g_lengths = g_ng = g_outside = g_replays = g_chunks = 0;
+    g_solves = g_graphs = g_marches = g_applies = g_lengths = g_ng = g_outside = g_replays = g_chunks = g_mallocs = 0;
 }
 
 cudaError_t cudaMalloc(void** p, size_t n)
 {
     *p = nullptr;
+    ++g_mallocs;
     const bool chosen = g_nth == 0;
     if (g_nth >= 0) --g_nth;
     if (chosen || g_live + (long long)n > g_total) return g_last = cudaErrorMemoryAllocation;

@@ -1,6 +1,6 @@
 """The host code on a device in host memory (fake_device.py): waits that gave up,
 numbers of sweeps up to the largest, allocations that fail, budgets of batches,
-chunks of a recording."""
+chunks of a recording, blocks kept over a change of the quadrature."""
 
 import pytest
 
@@ -250,4 +250,25 @@ for form, worth in (("fp64", 7.0), ("df64", 7.5), ("parabolic", 8.5)):
             n = counts()
         kept = ratio < worth
         assert (n["applies"], n["replays"]) == ((1, 0) if kept else (0, 1)), (form, ratio, n)
+""")
+
+
+@pytest.mark.parametrize("form", ["fp64", "df64"])
+def test_recording_keeps_its_blocks_over_a_quadrature(lib, form):
+    """A quadrature of the same or a somewhat smaller size takes the blocks of the
+    one before; a much smaller or a larger one its own; a grid frees them."""
+    fake_device.run(lib, f"""
+prec = R.RT_DF64 if {form!r} == "df64" else R.RT_FP64
+p = W.random_slab(20, 18, 40, n_theta=32, n_phi=32, seed=1)
+with R.Solver(p, precision=prec) as s:
+    s.formal_solution(p.B)
+    for n_theta, n_phi, new in ((32, 32, 0), (32, 24, 0), (32, 32, 0), (4, 2, 1), (32, 32, 1)):
+        R.rt_set_quadrature(s.ctx, *W.quadrature(n_theta, n_phi))
+        counts()
+        s.formal_solution(p.B)
+        n = counts()
+        assert n["applies"] == 1
+        # the recording's block itself where it has to grow; lists and working storage
+        assert n["mallocs"] <= 1 if new == 0 else n["mallocs"] >= new, (n_theta, n_phi, n)
+assert lib.fake_live() == 0
 """)
