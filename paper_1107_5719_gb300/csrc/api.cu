@@ -617,11 +617,12 @@ int ensure_op_work(rt_ctx* c)
     w.poff = reinterpret_cast<int*>(m); m += b_t;
     w.cnt = reinterpret_cast<int*>(m); m += b_q;
     w.segb = reinterpret_cast<int*>(m); m += b_q;
+    // (the host copies the steps, E and the rows together)
+    w.steps = reinterpret_cast<unsigned long long*>(m); m += 256;
     w.E = reinterpret_cast<int*>(m); m += b_z;
     w.rows = reinterpret_cast<int*>(m); m += b_z;
     w.eb = reinterpret_cast<long long*>(m); m += b_z;
     w.prow = reinterpret_cast<long long*>(m); m += b_z;
-    w.steps = reinterpret_cast<unsigned long long*>(m); m += 256;
     w.c0s = reinterpret_cast<double*>(m); m += b_slot;
     w.bcs = reinterpret_cast<double*>(m); m += b_slot;
     w.tss = reinterpret_cast<double*>(m);
@@ -704,16 +705,15 @@ int ensure_op_rec(rt_ctx* c, int G, bool& use)
         if (op_bytes(c, entries) + chunk > std::min(room, kOpNoWait)) {
             bounds = false;
             // the size it really has, and chunks of planes
-            std::vector<int> E(g.nz), R(g.nz);
-            unsigned long long steps = 0;
-            CK(cudaMemcpyAsync(&steps, w.steps, sizeof steps, cudaMemcpyDeviceToHost, st));
-            CK(cudaMemcpyAsync(E.data(), w.E, sizeof(int) * g.nz, cudaMemcpyDeviceToHost, st));
-            CK(cudaMemcpyAsync(R.data(), w.rows, sizeof(int) * g.nz, cudaMemcpyDeviceToHost, st));
-            if (g.zorder)
-                CK(cudaMemcpyAsync(order.data(), g.zorder, sizeof(int) * g.nz,
-                                   cudaMemcpyDeviceToHost, st));
+            const char* from = reinterpret_cast<const char*>(w.steps);
+            std::vector<char> host(reinterpret_cast<const char*>(w.rows + g.nz) - from);
+            CK(cudaMemcpyAsync(host.data(), from, host.size(), cudaMemcpyDeviceToHost, st));
             CK(cudaStreamSynchronize(st));
             c->stats.host_syncs += 1;
+            unsigned long long steps;
+            std::memcpy(&steps, host.data(), sizeof steps);
+            const int* E = reinterpret_cast<const int*>(host.data() + (reinterpret_cast<const char*>(w.E) - from));
+            const int* R = E + (w.rows - w.E);
             entries = rows = 0;
             long long most = 0;
             for (int k = 0; k < g.nz; ++k) {
@@ -730,6 +730,12 @@ int ensure_op_rec(rt_ctx* c, int G, bool& use)
                 (double)entries * (double)(nwp * 32) > op_worth(c) * (double)steps) {
                 op = false;
             } else {
+                if (g.zorder && cb < rows * row) {
+                    CK(cudaMemcpyAsync(order.data(), g.zorder, sizeof(int) * g.nz,
+                                       cudaMemcpyDeviceToHost, st));
+                    CK(cudaStreamSynchronize(st));
+                    c->stats.host_syncs += 1;
+                }
                 first.assign(1, 0);
                 long long at = 0;
                 for (int r = 0; r < g.nz; ++r) {
